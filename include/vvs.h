@@ -15,7 +15,7 @@
  * General rules
  *   - Every function returns VVS_OK (0) or a negative vvs_status.  Host-side argument errors
  *     are returned before anything is launched.  No exceptions.  Process-wide state is limited
- *     to per-device kernel attributes set once and the scratch array of vvs_decide_noalloc.
+ *     to per-device kernel attributes set once and the status word of vvs_decide_noalloc.
  *   - "device" pointers are CUDA device memory of the context's GPU, owned by the caller,
  *     16-byte aligned unless stated otherwise.  "host" pointers are ordinary host memory.
  *     The library never frees caller memory and keeps no reference to host arrays after a
@@ -270,10 +270,10 @@ int vvs_decide(vvs_ctx* ctx, const float* target_probs, int32_t n_rows_per_seq, 
  * vvs_decide without a context and without any allocation.  Some callers may not call
  * cudaMalloc at all: code that runs inside a serving process whose allocator reserved the whole
  * GPU at start-up, a plugin whose host forbids allocations, or a latency-critical loop that
- * cannot afford the device-wide synchronisation an allocation implies.  For them the scratch of
- * the decision kernels lives in one fixed array in device memory that is part of the library
- * image: about 325 KB held on every GPU that loads the library, until the process exits.  The
- * function calls no cudaMalloc / cudaFree and no allocating library routine.
+ * cannot afford the device-wide synchronisation an allocation implies.  The decision kernel keeps
+ * what lies between its steps in registers and shared memory; the only device memory of its own is
+ * one status word that is part of the library image.  The function calls no cudaMalloc / cudaFree
+ * and no allocating library routine.
  *
  * Capacity (larger sizes return VVS_ERR_SHAPE): n_images <= 64, n_draft_max <= 16,
  * nbr_k <= 64, vocab <= 65536.
@@ -284,13 +284,11 @@ int vvs_decide(vvs_ctx* ctx, const float* target_probs, int32_t n_rows_per_seq, 
  * Arguments are those of vvs_decide, with what a context would carry passed explicitly: vocab,
  * vocab_offset, and the CSR neighbour table (device int32, may be NULL in strict mode).
  * status_bits: optional device int32 the VVS_DEV_* bits are OR-ed into (caller clears it);
- * NULL = a private word inside the scratch array, cleared by each call and not readable.
+ * NULL = a private word of the library, not readable.
  *
- * The first call on each device looks up the array's device address (cudaGetSymbolAddress, with
- * that device current) and caches it; make that first call outside any stream capture.  All
- * calls on a device share the one array, which still holds the previous call's values (each
- * call rewrites what it reads): two calls whose kernels may overlap on the GPU (different
- * streams without ordering, or several host threads) race on it and must be serialised. */
+ * The first call on each device that passes no status_bits looks up the word's device address
+ * (cudaGetSymbolAddress, with that device current) and caches it; make that call outside any stream
+ * capture.  Calls on different streams do not interfere. */
 #define VVS_NOALLOC_MAX_IMAGES 64
 #define VVS_NOALLOC_MAX_DRAFTS 16
 #define VVS_NOALLOC_MAX_NBR_K 64

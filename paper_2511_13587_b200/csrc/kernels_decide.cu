@@ -403,4 +403,253 @@ void launch_sample(const Workspace& ws, const DecideParams& p, cudaStream_t s) {
   sample_kernel<<<p.n_images, kSampleChunk, 0, s>>>(ws, p, n_chunks);
 }
 
+// ---------------------------------------------------------------------------------------------
+// The whole decision of an image in one kernel: softmax statistics (when the rows are logits), acceptance,
+// residual masses, inverse CDF.  A cluster of S CTAs per image: every CTA takes the acceptance decision for
+// itself (a few dozen gathered values: cheaper than an exchange), then sums its contiguous part of the codebook, warp
+// by warp in index order; the part sums are read through distributed shared memory and the one warp whose part
+// holds the sample point walks it.  Replaces finalize / gather / accept / select / residual / sample, six launches
+// of 3-7 us each on a few hundred kilobytes: the work is a chain of four dependent round trips to L2.
+namespace {
+
+constexpr int kDecideThreads = 256, kDecideWarps = kDecideThreads / 32;
+
+__device__ __forceinline__ double ld_cluster_f64(const double* local, uint32_t rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(local), r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
+  return v;
+}
+
+// LOGITS: rows hold guided logits, statistics come from the [n_tiles, n_rows] softmax partials; else probabilities.
+template <bool LOGITS>
+__global__ void __launch_bounds__(kDecideThreads) decide_kernel(Workspace ws, DecideParams p, const float* __restrict__ rows,
+                                                                int n_tiles, int n_rows) {
+  __shared__ float s_m[32], s_inv[32];
+  __shared__ double s_ratio[32];
+  __shared__ double s_w[2][kDecideWarps];            // masses of this CTA's warps: residual, target
+  __shared__ double s_seg[2];
+  __shared__ double s_lo, s_t, s_total;
+  __shared__ int s_n, s_kind, s_part, s_use_p;
+  const int b = blockIdx.y, S = (int)gridDim.x, rank = (int)blockIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int K = p.n_draft_max, V = p.vocab;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  // ---- statistics of the image's rows: M = max_t m_t, S = sum_t s_t exp(m_t - M) ------------------------------------
+  if (LOGITS) {
+    for (int r = warp; r < p.rows_per_seq; r += kDecideWarps) {
+      const int row = b * p.rows_per_seq + r;
+      float mx = -CUDART_INF_F;
+      for (int t = lane; t < n_tiles; t += 32) mx = fmaxf(mx, ws.part_m[(size_t)t * n_rows + row]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      float sum = 0.f;
+      for (int t = lane; t < n_tiles; t += 32) sum += ws.part_s[(size_t)t * n_rows + row] * expf(ws.part_m[(size_t)t * n_rows + row] - mx);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if (lane == 0) {
+        s_m[r] = mx;
+        s_inv[r] = 1.f / sum;
+        if (rank == 0) {
+          ws.stat_m[row] = mx;
+          ws.stat_inv[row] = 1.f / sum;
+        }
+      }
+    }
+    __syncthreads();
+  }
+
+  // ---- acceptance ratios, a warp per draft ---------------------------------------------------------------------------
+  int nd = p.n_draft ? p.n_draft[b] : K;
+  if (nd < 0 || nd > K) {
+    if (tid == 0) atomicOr(ws.status, VVS_DEV_BAD_ARG);
+    nd = nd < 0 ? 0 : K;
+  }
+  for (int i = warp; i < nd; i += kDecideWarps) {
+    double ratio = 0.0;
+    const int x = p.drafts[(size_t)b * p.drafts_ld + i] - p.vocab_offset;
+    if (x < 0 || x >= V) {
+      if (lane == 0) atomicOr(ws.status, VVS_DEV_BAD_TOKEN);
+    } else {
+      const int r = p.first_row + i;
+      const float* row = rows + ((size_t)b * p.rows_per_seq + r) * V;
+      const float m = LOGITS ? s_m[r] : 0.f, inv = LOGITS ? s_inv[r] : 1.f;
+      const double qx = (double)p.draft_probs[((size_t)b * K + i) * V + x];
+      double mass = (double)(LOGITS ? prob_of(row[x], m, inv) : row[x]);
+      if (p.mode == VVS_MODE_RELAXED && p.nbr_k > 1) {
+        const int beg = p.row_ptr[x], len = p.row_ptr[x + 1] - beg;
+        if (len < 1 && lane == 0) atomicOr(ws.status, VVS_DEV_BAD_NEIGHBOUR);
+        const int kk = min(p.nbr_k, len);
+        int j_end;
+        mass += pooled_prefix(kk, (double)p.delta, lane, [&](int j) {
+          const int c = p.col[beg + j];
+          if (c < 0 || c >= V) {
+            atomicOr(ws.status, VVS_DEV_BAD_NEIGHBOUR);
+            return 0.0;
+          }
+          return (double)(LOGITS ? prob_of(row[c], m, inv) : row[c]);
+        }, &j_end);
+      }
+      ratio = qx > 0.0 ? fmin(1.0, mass / qx) : (mass > 0.0 ? 1.0 : 0.0);
+    }
+    if (lane == 0) s_ratio[i] = ratio;
+  }
+  __syncthreads();
+  if (warp == 0) {                                    // accepted prefix: the first lane whose test fails
+    const double u = lane < nd ? (double)p.uniforms[(size_t)b * (K + 1) + lane] : 0.0;
+    const bool pass = lane < nd && u < s_ratio[lane];
+    const unsigned fails = ~__ballot_sync(0xffffffffu, pass);
+    const int n = fails ? min(__ffs(fails) - 1, nd) : nd;
+    if (lane == 0) {
+      s_n = n;
+      s_kind = n < nd ? 0 : 1;
+    }
+    if (rank == 0) {
+      if (lane < K) {
+        const bool judged = lane < nd && lane <= n;
+        if (p.margins) p.margins[(size_t)b * (K + 1) + lane] = judged ? (float)fabs(u - s_ratio[lane]) : CUDART_INF_F;
+        if (p.accept_mask) p.accept_mask[(size_t)b * K + lane] = lane < n ? 1 : 0;
+      }
+      if (lane == 0) p.accept_len[b] = n;
+      if (lane < p.n_cfg) {
+        const int r = lane * p.n_images + b;
+        if (p.new_len && p.cache_len) p.new_len[r] = p.cache_len[r] + p.n_forced + n;
+        if (p.n_commit) p.n_commit[r] = p.n_forced + n;
+      }
+    }
+  }
+  __syncthreads();
+
+  // ---- masses of this CTA's part, a contiguous range per warp ------------------------------------------------------
+  const int n = s_n, r_sel = p.first_row + n;
+  const bool has_row = r_sel < p.rows_per_seq;
+  const float* p_row = rows + ((size_t)b * p.rows_per_seq + (has_row ? r_sel : 0)) * V;
+  const float* q_row = p.draft_probs + ((size_t)b * K + (s_kind == 0 ? n : 0)) * V;
+  const float m = LOGITS ? s_m[has_row ? r_sel : 0] : 0.f, inv = LOGITS ? s_inv[has_row ? r_sel : 0] : 1.f;
+  const int per = (V + S * kDecideWarps - 1) / (S * kDecideWarps), at = (rank * kDecideWarps + warp) * per;
+  const int v0 = min(V, at), v1 = min(V, at + per), kind = s_kind;
+  auto target = [&](int j) { return LOGITS ? prob_of(p_row[j], m, inv) : p_row[j]; };
+  double sr = 0.0, sp = 0.0;
+  if (has_row) {
+#pragma unroll 8
+    for (int j = v0 + lane; j < v1; j += 32) {
+      const float pr = target(j);
+      sr += (double)(kind != 0 ? pr : fmaxf(0.f, pr - q_row[j]));
+      sp += (double)pr;
+    }
+  }
+  sr = warp_sum_d(sr);
+  sp = warp_sum_d(sp);
+  if (lane == 0) {
+    s_w[0][warp] = sr;
+    s_w[1][warp] = sp;
+  }
+  __syncthreads();
+  if (tid < 2) {
+    double s = 0.0;
+    for (int w = 0; w < kDecideWarps; ++w) s += s_w[tid][w];
+    s_seg[tid] = s;
+  }
+  if (S > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  else __syncthreads();
+  if (warp == 0) {
+    double seg[2] = {0.0, 0.0};
+    if (lane < S) {
+      seg[0] = S > 1 ? ld_cluster_f64(&s_seg[0], lane) : s_seg[0];
+      seg[1] = S > 1 ? ld_cluster_f64(&s_seg[1], lane) : s_seg[1];
+    }
+    const double total_r = warp_sum_d(seg[0]), total_p = warp_sum_d(seg[1]);
+    const int use_p = total_r > 0.0 ? 0 : 1;          // p == q numerically: fall back to the target row itself
+    const double val = seg[use_p], total = use_p ? total_p : total_r;
+    const double t = (double)p.uniforms[(size_t)b * (K + 1) + K] * total;
+    const double incl = warp_incl_scan_d(val, lane);
+    const unsigned hit = __ballot_sync(0xffffffffu, lane < S && incl > t), nz = __ballot_sync(0xffffffffu, val > 0.0);
+    const int part = hit ? __ffs(hit) - 1 : nz ? 31 - __clz(nz) : 0;
+    const double lo = __shfl_sync(0xffffffffu, incl - val, part);
+    if (lane == 0) {
+      s_lo = lo; s_t = t; s_total = total; s_use_p = use_p;
+      s_part = has_row && total > 0.0 ? part : -1;
+    }
+  }
+  if (S > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // (waited for at the end)
+  __syncthreads();
+  // ---- the sample point: smallest index whose cumulative mass exceeds t, in the part that holds it -----------------
+  if (s_part < 0) {
+    if (rank == 0 && tid == 0) {
+      p.next_token[b] = -1;
+      if (p.margins) p.margins[(size_t)b * (K + 1) + K] = CUDART_INF_F;
+    }
+  } else if (s_part == rank) {
+    const int eff = s_use_p ? 1 : kind;
+    const double* w_mass = s_w[s_use_p];
+    int sel = -1, last_nz = 0;
+    double lo = s_lo, sel_lo = lo, nz_lo = lo;
+    for (int w = 0; w < kDecideWarps; ++w) {
+      if (w_mass[w] > 0.0) { last_nz = w; nz_lo = lo; }
+      if (lo + w_mass[w] > s_t) { sel = w; sel_lo = lo; break; }
+      lo += w_mass[w];
+    }
+    if (sel < 0) { sel = last_nz; sel_lo = nz_lo; }
+    if (warp == sel) {
+      double run = sel_lo, pick_lo = 0.0, pick_hi = 0.0;
+      int pick = -1;
+      bool found = false;
+      for (int j0 = v0; j0 < v1 && !found; j0 += 32) {
+        const int j = j0 + lane;
+        const float pr = j < v1 ? target(j) : 0.f;
+        const double val = j < v1 ? (double)(eff != 0 ? pr : fmaxf(0.f, pr - q_row[j])) : 0.0;
+        const double inc = warp_incl_scan_d(val, lane), cdf = run + inc;
+        const unsigned over = __ballot_sync(0xffffffffu, j < v1 && cdf > s_t), nz = __ballot_sync(0xffffffffu, val > 0.0);
+        const int src = over ? __ffs(over) - 1 : nz ? 31 - __clz(nz) : -1;
+        if (src >= 0) {
+          pick = j0 + src;
+          pick_hi = __shfl_sync(0xffffffffu, cdf, src);
+          pick_lo = pick_hi - __shfl_sync(0xffffffffu, val, src);
+        }
+        found = over != 0;
+        run += __shfl_sync(0xffffffffu, inc, 31);
+      }
+      if (lane == 0) {
+        p.next_token[b] = pick < 0 ? -1 : p.vocab_offset + pick;
+        if (p.margins && pick >= 0)
+          p.margins[(size_t)b * (K + 1) + K] = (float)(fmin(fabs(s_t - pick_lo), fabs(pick_hi - s_t)) / s_total);
+      }
+    }
+  }
+  if (S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // nobody leaves while its sums may be read
+}
+
+}  // namespace
+
+// Parts of a codebook: 2048 codes or more each, eight CTAs (the portable cluster) at most -- fewer where the images
+// alone fill the GPU.
+int launch_decide(const float* rows, bool logits, int n_tiles, int n_rows, const Workspace& ws, const DecideParams& p, bool pdl,
+                  cudaStream_t s) {
+  int S = 1;
+  while (S < 8 && p.vocab >= 2048 * 2 * S) S *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(S, p.n_images, 1);
+  cfg.blockDim = dim3(kDecideThreads, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  int na = 0;
+  if (S > 1) {
+    attr[na].id = cudaLaunchAttributeClusterDimension;
+    attr[na].val.clusterDim.x = S;
+    attr[na].val.clusterDim.y = 1;
+    attr[na++].val.clusterDim.z = 1;
+  }
+  if (pdl) {
+    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[na++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = na;
+  const cudaError_t e = logits ? cudaLaunchKernelEx(&cfg, decide_kernel<true>, ws, p, rows, n_tiles, n_rows)
+                               : cudaLaunchKernelEx(&cfg, decide_kernel<false>, ws, p, rows, n_tiles, n_rows);
+  return e == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
+}
+
 }  // namespace vvs

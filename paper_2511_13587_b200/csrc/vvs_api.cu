@@ -92,7 +92,12 @@ size_t layout(const vvs_model_desc& d, Workspace& ws, char* base) {
   if (d.dtype == VVS_DTYPE_BF16 && d.n_layers > 0) c.take(ws.anc_mask, M * 4);
   c.take(ws.tree_res, (size_t)2 * d.max_rows * V * 8);
   c.take(ws.tree_path, (size_t)d.max_rows * 32 * 4);
-  if (d.dtype == VVS_DTYPE_BF16 && !std::getenv("VVS_DEBUG_GENERIC")) c.take(ws.logits_small, (M < 64 ? M : 64) * V * 4);
+  if (d.dtype == VVS_DTYPE_BF16 && !std::getenv("VVS_DEBUG_GENERIC")) {
+    // guided logits of a call: 64 decision rows always, more as long as the buffer stays under a gigabyte
+    const size_t cap = ((size_t)1 << 30) / (V * 4);
+    ws.logit_rows = (int)(M < 64 ? M : cap < 64 ? 64 : M < cap ? M : cap);
+    c.take(ws.logits_small, (size_t)ws.logit_rows * V * 4);
+  }
   return (c.off + 255) & ~size_t(255);
 }
 
@@ -182,17 +187,26 @@ int run_decisions(vvs_ctx* ctx, const T* hid, int rows_per_seq, int first_row, c
     LmHeadArgs la{};
     la.v = V; la.k = md.d_model; la.bt = BT; la.n_cfg = C; la.tm_a = &ctx->lm_map; la.tm_b = &tm_hid;
     la.pdl = ctx->use_pdl; la.n_sms = ctx->n_sms; la.cfg_scale = a->cfg_scale; la.inv_temp = 1.f / a->temperature;
-    // few decision rows: the guided logits are written out (under a megabyte at 9 rows) and the
-    // sampled row is read back from them; otherwise a second pass over the head recomputes it
-    float* lbuf = o->target_probs ? o->target_probs : (BT <= 64 ? ws.logits_small : nullptr);
+    // The guided logits are written out (they mostly stay in L2: 0.6 MB at 9 rows, 19 MB at 288 rows of 16384 codes) and
+    // the decision kernel gathers and samples from them.  Only calls too large for the buffer recompute the sampled
+    // rows by a second pass over the head and pick the gathered logits in its epilogue (which at 576 feature rows of
+    // a 4096-wide, 16384-code head with 64 neighbours took 278 us per call against X with the logits written).
+    float* lbuf = o->target_probs ? o->target_probs : (BT <= ws.logit_rows ? ws.logits_small : nullptr);
+    const bool fused = lbuf && !p.adjusted;
     la.part_m = ws.part_m; la.part_s = ws.part_s; la.logits_out = lbuf; la.status = ws.status;
-    la.rows_per_seq = rows_per_seq; la.first_row = first_row; la.n_draft_max = p.n_draft_max;
+    la.rows_per_seq = rows_per_seq; la.first_row = first_row; la.n_draft_max = fused ? 0 : p.n_draft_max;
     la.vocab_offset = md.vocab_offset; la.relaxed = (p.mode == VVS_MODE_RELAXED && p.nbr_k > 1) ? 1 : 0;
     la.nbr_k = p.nbr_k; la.kmax = p.kmax; la.drafts_ld = drafts_ld; la.drafts = drafts;
     la.row_ptr = p.row_ptr; la.col = p.col; la.l_tok = ws.l_tok; la.l_nbr = ws.l_nbr;
     int rc = VVS_OK;
     VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_lmhead_tc(la, s));
     if (rc != VVS_OK) return rc;
+    if (fused) {
+      VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(lbuf, true, (V + 127) / 128, BT, ws, p, ctx->use_pdl, s));
+      if (rc == VVS_OK && o->target_probs)
+        VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(o->target_probs, ws, o->target_probs, BT, V, s));
+      return rc != VVS_OK ? rc : cudaGetLastError() == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
+    }
     VVS_LAUNCH(VVS_PROF_OTHER, launch_finalize_stats(ws, (V + 127) / 128, BT, s));
     VVS_LAUNCH(VVS_PROF_OTHER, launch_accept(ws, p, s));
     if (lbuf) {
@@ -220,6 +234,13 @@ int run_decisions(vvs_ctx* ctx, const T* hid, int rows_per_seq, int first_row, c
   VVS_LAUNCH(VVS_PROF_OTHER, launch_guide(ws.logits_raw, ws.logits, B, C, rows_per_seq, V, a->cfg_scale,
                                           1.f / a->temperature, s));
   VVS_LAUNCH(VVS_PROF_OTHER, launch_row_stats(ws.logits, ws.part_m, ws.part_s, BT, V, s));
+  if (!p.adjusted) {
+    int rc = VVS_OK;
+    VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(ws.logits, true, 1, BT, ws, p, false, s));
+    if (rc == VVS_OK && o->target_probs)
+      VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(ws.logits, ws, o->target_probs, BT, V, s));
+    return rc != VVS_OK ? rc : cudaGetLastError() == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
+  }
   VVS_LAUNCH(VVS_PROF_OTHER, launch_finalize_stats(ws, 1, BT, s));
   if (p.n_draft_max > 0) VVS_LAUNCH(VVS_PROF_OTHER, launch_gather_logits(ws.logits, ws, p, s));
   VVS_LAUNCH(VVS_PROF_OTHER, launch_accept(ws, p, s));
@@ -888,6 +909,10 @@ int vvs_decide(vvs_ctx* ctx, const float* target_probs, int32_t n_rows_per_seq, 
   }
   DecideParams p = decide_params(ctx, n_rows_per_seq, first_row, drafts, a->n_draft_max, a, o, false);
   p.direct_probs = target_probs;
+  if (!p.adjusted) {
+    VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(target_probs, false, 0, 0, ws, p, false, s));
+    return rc;
+  }
   if (p.n_draft_max > 0) VVS_LAUNCH(VVS_PROF_OTHER, launch_gather_logits(target_probs, ws, p, s));
   VVS_LAUNCH(VVS_PROF_OTHER, launch_accept(ws, p, s));
   if (p.adjusted) VVS_LAUNCH(VVS_PROF_OTHER, launch_adjust_target(ws, p, s));   // copies the row, then adjusts it
