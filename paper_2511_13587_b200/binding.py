@@ -17,6 +17,11 @@ if not os.path.exists(_LIB_PATH):
         f"{_LIB_PATH} is missing: build it first (python -m paper_2511_13587_b200.build, or "
         "__graft_entry__.build()).  There is no fallback path.")
 lib = C.CDLL(_LIB_PATH)
+try:
+    from . import _native  # linked against the library loaded above
+except ImportError as e:
+    raise ImportError("the package's _native module is missing or stale: build it first (python -m "
+                      "paper_2511_13587_b200.build, or __graft_entry__.build()).") from e
 
 VVS_OK = 0
 VVS_DTYPE_FP32, VVS_DTYPE_BF16 = 0, 1
@@ -186,73 +191,18 @@ def vvs_bind_neighbors(ctx: int, row_ptr: torch.Tensor, col: torch.Tensor) -> No
     _keepalive[ctx]["nbr"] = (row_ptr, col)
 
 
-def _args(n_images, n_cfg, n_forced, n_draft_max, block, n_draft, kv_k, kv_v, kv_rows, cache_len,
-          cache_len_host, draft_probs, uniforms, cfg_scale, temperature, mode, nbr_k, delta,
-          tree_parent=None, adjusted_residual=False):
-    return vvs_verify_args(int(n_images), int(n_cfg), int(n_forced), int(n_draft_max), _ptr(block),
-                           _ptr(n_draft), _ptr(kv_k), _ptr(kv_v), int(kv_rows), _ptr(cache_len),
-                           _ptr(cache_len_host), _ptr(draft_probs), _ptr(uniforms), float(cfg_scale),
-                           float(temperature), int(mode), int(nbr_k), float(delta), _ptr(tree_parent),
-                           int(adjusted_residual))
-
-
-def _out(accept_len, next_token, new_len, n_commit, accept_mask, target_probs, hidden, margins,
-         accept_path=None):
-    return vvs_verify_out(_ptr(accept_len), _ptr(next_token), _ptr(new_len), _ptr(n_commit), _ptr(accept_mask),
-                          _ptr(target_probs), _ptr(hidden), _ptr(accept_path), _ptr(margins))
-
-
-def vvs_verify(ctx: int, *, n_images, n_cfg, n_forced, n_draft_max, block, kv_k, kv_v, kv_rows,
-               cache_len, draft_probs, uniforms, accept_len, next_token, new_len, n_draft=None,
-               cache_len_host=None, cfg_scale=1.0, temperature=1.0, mode=VVS_MODE_STRICT, nbr_k=1,
-               delta=float("inf"), n_commit=None, accept_mask=None, target_probs=None, hidden=None,
-               margins=None, tree_parent=None, accept_path=None, adjusted_residual=False, stream=None) -> None:
-    a = _args(n_images, n_cfg, n_forced, n_draft_max, block, n_draft, kv_k, kv_v, kv_rows, cache_len,
-              cache_len_host, draft_probs, uniforms, cfg_scale, temperature, mode, nbr_k, delta, tree_parent,
-              adjusted_residual)
-    o = _out(accept_len, next_token, new_len, n_commit, accept_mask, target_probs, hidden, margins, accept_path)
-    _check(lib.vvs_verify(ctx, C.byref(a), C.byref(o), _stream(stream)), "vvs_verify")
-
-
-def vvs_epilogue(ctx: int, *, hidden_in, n_rows_per_seq, first_row, drafts, n_images, n_cfg,
-                 n_draft_max, draft_probs, uniforms, accept_len, next_token, n_draft=None,
-                 cfg_scale=1.0, temperature=1.0, mode=VVS_MODE_STRICT, nbr_k=1, delta=float("inf"),
-                 accept_mask=None, target_probs=None, margins=None, adjusted_residual=False,
-                 stream=None) -> None:
-    a = _args(n_images, n_cfg, 1, n_draft_max, None, n_draft, None, None, 0, None, None, draft_probs,
-              uniforms, cfg_scale, temperature, mode, nbr_k, delta, None, adjusted_residual)
-    o = _out(accept_len, next_token, None, None, accept_mask, target_probs, None, margins)
-    _check(lib.vvs_epilogue(ctx, _ptr(hidden_in), int(n_rows_per_seq), int(first_row), _ptr(drafts),
-                            C.byref(a), C.byref(o), _stream(stream)), "vvs_epilogue")
-
-
-def vvs_decide(ctx: int, *, target_probs, n_rows_per_seq, first_row, drafts, n_images, n_draft_max,
-               draft_probs, uniforms, accept_len, next_token, n_draft=None, mode=VVS_MODE_STRICT,
-               nbr_k=1, delta=float("inf"), accept_mask=None, margins=None, tree_parent=None,
-               accept_path=None, adjusted_residual=False, stream=None) -> None:
-    a = _args(n_images, 1, 1, n_draft_max, None, n_draft, None, None, 0, None, None, draft_probs,
-              uniforms, 1.0, 1.0, mode, nbr_k, delta, tree_parent, adjusted_residual)
-    o = _out(accept_len, next_token, None, None, accept_mask, None, None, margins, accept_path)
-    _check(lib.vvs_decide(ctx, _ptr(target_probs), int(n_rows_per_seq), int(first_row), _ptr(drafts),
-                          C.byref(a), C.byref(o), _stream(stream)), "vvs_decide")
-
-
-def vvs_decide_noalloc(*, target_probs, vocab, vocab_offset, n_rows_per_seq, first_row, drafts,
-                       n_images, n_draft_max, draft_probs, uniforms, accept_len, next_token,
-                       nbr_row_ptr=None, nbr_col=None, n_draft=None, mode=VVS_MODE_STRICT, nbr_k=1,
-                       delta=float("inf"), accept_mask=None, margins=None, status_bits=None,
-                       tree_parent=None, accept_path=None, adjusted_residual=False, stream=None) -> None:
-    """vvs_decide for callers that must not allocate device memory: no context, scratch in a fixed
-    device array inside the library (limits: 64 images, 16 drafts, 64 neighbours, vocab 65536;
-    chains only: tree_parent / accept_path are refused).  Calls on one device share that array
-    and must not overlap on the GPU."""
-    a = _args(n_images, 1, 1, n_draft_max, None, n_draft, None, None, 0, None, None, draft_probs,
-              uniforms, 1.0, 1.0, mode, nbr_k, delta, tree_parent, adjusted_residual)
-    o = _out(accept_len, next_token, None, None, accept_mask, None, None, margins, accept_path)
-    _check(lib.vvs_decide_noalloc(_ptr(target_probs), int(vocab), int(vocab_offset), int(n_rows_per_seq),
-                                  int(first_row), _ptr(drafts), _ptr(nbr_row_ptr), _ptr(nbr_col),
-                                  C.byref(a), C.byref(o), _ptr(status_bits), _stream(stream)),
-           "vvs_decide_noalloc")
+# The calls a decoding loop makes per step are marshalled natively, csrc/binding_native.c (keyword arguments named as
+# the fields of the C structures, `ctx` first; a call through ctypes costs 6-10 us of host time).
+_native.setup(VvsError, torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+vvs_verify = _native.vvs_verify
+vvs_epilogue = _native.vvs_epilogue
+vvs_decide = _native.vvs_decide
+vvs_decide_noalloc = _native.vvs_decide_noalloc
+vvs_feature_cache_reset = _native.vvs_feature_cache_reset
+vvs_feature_cache_store = _native.vvs_feature_cache_store
+vvs_feature_cache_fetch = _native.vvs_feature_cache_fetch
+vvs_skip_decide = _native.vvs_skip_decide
+vvs_select_unverified = _native.vvs_select_unverified
 
 
 def vvs_selftest_bounded_wait(ctx: int, stream=None):
@@ -267,44 +217,6 @@ def make_fcache(feat: torch.Tensor, fpos: torch.Tensor, newest: torch.Tensor) ->
     fc = vvs_fcache(_ptr(feat), _ptr(fpos), _ptr(newest), int(feat.shape[0]), int(feat.shape[1]))
     fc._keep = (feat, fpos, newest)
     return fc
-
-
-def vvs_feature_cache_reset(ctx: int, fc: vvs_fcache, stream=None) -> None:
-    _check(lib.vvs_feature_cache_reset(ctx, C.byref(fc), _stream(stream)), "vvs_feature_cache_reset")
-
-
-def vvs_feature_cache_store(ctx: int, fc: vvs_fcache, hidden, n_rows_per_seq, base_pos, n_store,
-                            stream=None) -> None:
-    _check(lib.vvs_feature_cache_store(ctx, C.byref(fc), _ptr(hidden), int(n_rows_per_seq),
-                                       _ptr(base_pos), _ptr(n_store), _stream(stream)),
-           "vvs_feature_cache_store")
-
-
-def vvs_feature_cache_fetch(ctx: int, fc: vvs_fcache, skip_mask, n_images, gamma, gamma_max,
-                            staleness, out, out_pos, stream=None) -> None:
-    _check(lib.vvs_feature_cache_fetch(ctx, C.byref(fc), _ptr(skip_mask), int(n_images), _ptr(gamma),
-                                       int(gamma_max), int(staleness), _ptr(out), _ptr(out_pos),
-                                       _stream(stream)), "vvs_feature_cache_fetch")
-
-
-def vvs_skip_decide(ctx: int, paths, path_len, codebook, last_verified, stride: int, alpha: float,
-                    threshold: float, decision, similarity, stream=None) -> None:
-    """Alg. 1 / Eq. 2 of the paper: paths int32 [B, N, L], path_len int32 [B, N] or None,
-    codebook float32 [V, dim], last_verified uint8 [B] or None -> decision uint8 [B], similarity
-    float32 [B]."""
-    b, n, l = paths.shape
-    v, dim = codebook.shape
-    _check(lib.vvs_skip_decide(ctx, _ptr(paths), _ptr(path_len), int(b), int(n), int(l), _ptr(codebook), int(v),
-                               int(dim), _ptr(last_verified), int(stride), float(alpha), float(threshold),
-                               _ptr(decision), _ptr(similarity), _stream(stream)), "vvs_skip_decide")
-
-
-def vvs_select_unverified(ctx: int, paths, path_len, uniforms, out_path, out_gamma, out_tokens, stream=None) -> None:
-    """Sec. 4.2 / Eq. 3: uniform draw of one candidate path per image, cut to gamma tokens."""
-    b, n, l = paths.shape
-    _check(lib.vvs_select_unverified(ctx, _ptr(paths), _ptr(path_len), int(b), int(n), int(l), _ptr(uniforms),
-                                     _ptr(out_path), _ptr(out_gamma), _ptr(out_tokens), _stream(stream)),
-           "vvs_select_unverified")
 
 
 def vvs_device_status(ctx: int, stream=None, raise_on_error: bool = False) -> int:

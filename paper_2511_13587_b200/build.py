@@ -1,4 +1,5 @@
-"""Builds the CUDA library (sm_100a) in-tree with nvcc: csrc/*.cu -> lib/libvvs.so.
+"""Builds the CUDA library (sm_100a) in-tree with nvcc: csrc/*.cu -> lib/libvvs.so, and the CPython
+entry points that marshal its calls: csrc/binding_native.c -> _native.so.
 
 nvcc cross-compiles without a GPU.  Objects go to _build/ (not committed); the shared library
 stays inside the package so that it travels with the source tree."""
@@ -7,6 +8,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -15,6 +17,8 @@ CSRC = os.path.join(PKG, "csrc")
 LIB_DIR = os.path.join(PKG, "lib")
 LIB = os.path.join(LIB_DIR, "libvvs.so")
 OBJ_DIR = os.path.join(PKG, "_build")
+NATIVE_SRC = os.path.join(CSRC, "binding_native.c")
+NATIVE = os.path.join(PKG, "_native.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -69,7 +73,21 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
+    build_native(force)
     return LIB
+
+
+def build_native(force: bool = False) -> str:
+    """The extension module finds libvvs.so next to it (rpath), so both travel with the source tree."""
+    newest = max(os.path.getmtime(p) for p in (NATIVE_SRC, os.path.join(ROOT, "include", "vvs.h")))
+    if force or not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < newest:
+        cmd = [os.environ.get("CC", "gcc"), "-shared", "-fPIC", "-O2", "-std=c11", "-Wall", "-I", sysconfig.get_paths()["include"],
+               "-I", os.path.join(ROOT, "include"), NATIVE_SRC, "-o", NATIVE, "-L", LIB_DIR, "-l:libvvs.so",
+               "-Wl,-rpath,$ORIGIN/lib"]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError(f"gcc failed for {NATIVE_SRC}:\n{r.stdout}\n{r.stderr}")
+    return NATIVE
 
 
 if __name__ == "__main__":
