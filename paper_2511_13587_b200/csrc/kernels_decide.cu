@@ -435,7 +435,8 @@ __global__ void __launch_bounds__(kDecideThreads) decide_kernel(Workspace ws, De
   const int b = blockIdx.y, S = (int)gridDim.x, rank = (int)blockIdx.x;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int K = p.n_draft_max, V = p.vocab;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  grid_dep_launch();
+  grid_dep_wait();
 
   // ---- statistics of the image's rows: M = max_t m_t, S = sum_t s_t exp(m_t - M) ------------------------------------
   if (LOGITS) {

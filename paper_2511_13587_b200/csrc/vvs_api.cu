@@ -910,7 +910,7 @@ int vvs_decide(vvs_ctx* ctx, const float* target_probs, int32_t n_rows_per_seq, 
   DecideParams p = decide_params(ctx, n_rows_per_seq, first_row, drafts, a->n_draft_max, a, o, false);
   p.direct_probs = target_probs;
   if (!p.adjusted) {
-    VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(target_probs, false, 0, 0, ws, p, false, s));
+    VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(target_probs, false, 0, 0, ws, p, ctx->use_pdl, s));
     return rc;
   }
   if (p.n_draft_max > 0) VVS_LAUNCH(VVS_PROF_OTHER, launch_gather_logits(target_probs, ws, p, s));

@@ -38,6 +38,25 @@ inline cudaError_t ensure_dynamic_smem(const void* kernel, int bytes) {
   return e;
 }
 
+// Launch with optional programmatic dependent launch: the kernel may start while the one before it in the stream is
+// draining and orders itself by griddepcontrol.wait, which every kernel launched this way executes first.
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, bool pdl, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, fn, P(args)...);
+}
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Scratch memory of a context.  Row index m of an activation matrix is r * T + t with
 // r = c * B + b (cond sequences first).  "Decision rows" are (b, t) pairs: index b * T + t.
 struct Workspace {
