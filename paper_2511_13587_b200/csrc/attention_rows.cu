@@ -374,10 +374,6 @@ int launch_hd(const AttentionRowsArgs& a, cudaStream_t s) {
 
 }  // namespace
 
-bool attention_rows_applicable(const vvs_model_desc& md, int t_len) {
-  return md.dtype == VVS_DTYPE_BF16 && (md.head_dim == 64 || md.head_dim == 128) && t_len >= 1 && t_len <= kMaxT;
-}
-
 int launch_attention_rows(const AttentionRowsArgs& a, cudaStream_t s) {
   if (a.hd == 64) return launch_hd<64>(a, s);
   if (a.hd == 128) return launch_hd<128>(a, s);

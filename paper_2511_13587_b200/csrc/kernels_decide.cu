@@ -188,6 +188,8 @@ void launch_accept(const Workspace& ws, const DecideParams& p, cudaStream_t s) {
 __global__ void probs_kernel(const float* __restrict__ logits, const float* __restrict__ stat_m,
                              const float* __restrict__ stat_inv, float* __restrict__ probs, int v) {
   size_t row = blockIdx.y;
+  grid_dep_launch();
+  grid_dep_wait();
   float m = stat_m[row], inv = stat_inv[row];
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < v) probs[row * v + j] = prob_of(logits[row * v + j], m, inv);
@@ -195,9 +197,8 @@ __global__ void probs_kernel(const float* __restrict__ logits, const float* __re
 
 // probs may alias logits (in-place normalisation)
 void launch_probs_from_logits(const float* logits, const Workspace& ws, float* probs, int n_rows,
-                              int v, cudaStream_t s) {
-  dim3 grid((v + 255) / 256, n_rows);
-  probs_kernel<<<grid, 256, 0, s>>>(logits, ws.stat_m, ws.stat_inv, probs, v);
+                              int v, bool pdl, cudaStream_t s) {
+  launch_kernel(probs_kernel, dim3((v + 255) / 256, n_rows), dim3(256), 0, pdl, s, logits, ws.stat_m, ws.stat_inv, probs, v);
 }
 
 // target probabilities of the row each image samples from, out of stored guided logits

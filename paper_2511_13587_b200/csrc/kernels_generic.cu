@@ -76,6 +76,8 @@ __global__ void embed_kernel(const T* __restrict__ tok_emb, const int32_t* __res
   int m = blockIdx.x;
   int r = m / t_len, t = m % t_len;
   int b = r % n_images;
+  grid_dep_launch();
+  grid_dep_wait();
   int tok = block[b * t_len + t];
   bool ok = tok >= 0 && tok < tok_rows;
   if (!ok && threadIdx.x == 0) atomicOr(status, VVS_DEV_BAD_TOKEN);
@@ -97,6 +99,8 @@ template <typename T>
 __global__ void rmsnorm_kernel(const float* __restrict__ x, const T* __restrict__ scale,
                                T* __restrict__ out, int d, float eps) {
   __shared__ float red[32];
+  grid_dep_launch();
+  grid_dep_wait();
   const float* row = x + (size_t)blockIdx.x * d;
   float ss = 0.f;
   for (int i = threadIdx.x; i < d; i += blockDim.x) ss += row[i] * row[i];
@@ -204,8 +208,8 @@ __global__ void __launch_bounds__(128) rmsnorm_row_block_kernel(const float* __r
 }
 
 template <typename T>
-void launch_rmsnorm(const float* x, const T* scale, T* out, int m, int d, float eps, cudaStream_t s) {
-  rmsnorm_kernel<T><<<m, 256, 0, s>>>(x, scale, out, d, eps);
+void launch_rmsnorm(const float* x, const T* scale, T* out, int m, int d, float eps, cudaStream_t s, bool pdl) {
+  launch_kernel(rmsnorm_kernel<T>, dim3(m), dim3(256), 0, pdl, s, x, scale, out, d, eps);
 }
 
 static cudaError_t launch_dependent(const void* fn, dim3 grid, dim3 block, void** args, bool pdl, cudaStream_t s) {
@@ -233,189 +237,284 @@ void launch_rmsnorm_rows(const float* x, const __nv_bfloat16* scale, __nv_bfloat
 }
 
 // ---------------------------------------------------------------------------------------------
-// c[m, n] (+)= sum_k a[m, k] * w[n, k].  One warp per weight row n, MT activation rows per pass.
-template <typename T, int MT>
-__global__ void gemm_nt_kernel(const T* __restrict__ a, const T* __restrict__ w,
-                               float* __restrict__ c, int m, int n, int k, int ldc, int accumulate) {
-  constexpr int VEC = VecOf<T>::n;
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int col = blockIdx.x * (blockDim.x >> 5) + warp;
-  int m0 = blockIdx.y * MT;
-  if (col >= n) return;
-  float acc[MT];
+// Projections on the CUDA cores: acc[m, n] = sum_k a[m, k] * w[n, k], one warp per weight row (or pair of rows), MT
+// activation rows per pass, with what surrounds a projection folded in:
+//   QKV     a = norm(x) * scale; rotation of q and k pairs, q to its buffer, k and v to cache slots L_r + t
+//   GATEUP  a = norm(x) * scale; silu(gate) * up
+//   ADD     residual x += acc
+//   STORE   plain product
+// A small model's step is a chain of dependent kernels of a few microseconds each, so what counts is their number
+// (five per layer instead of ten) and the loads in a row inside one: weights are requested before
+// griddepcontrol.wait, the activation rows of all their pieces together.  (Tiny float32 step of 5 rows: 128 -> 66 us.)
+template <typename T>
+struct RowGemm {
+  int m, n, k;                 // n: warps' worth of columns (pairs for QKV)
+  const T* a;                  // ADD, STORE: activations [m, k]
+  const float* x_in;           // QKV, GATEUP: residual rows [m, k]
+  const T* scale; float eps;
+  const T* w; const T* w2;     // GATEUP: gate, up
+  float* c; int ldc;           // ADD, STORE
+  T* act;                      // GATEUP [m, n]
+  T* q; T* kv_k; T* kv_v;      // QKV
+  const float* inv_freq; const int32_t* cache_len; int32_t* status;
+  int d, n_heads, hd, s_max, rope_mode, grid_w, n_prefix, layer, kv_rows, t_len;
+};
+
+template <typename T, int EPI>
+__global__ void __launch_bounds__(128) row_gemm_kernel(const RowGemm<T> p) {
+  constexpr int VEC = VecOf<T>::n, MT = 8;
+  constexpr bool NORM = EPI == ROW_QKV || EPI == ROW_GATEUP;
+  constexpr int NW = NORM ? 2 : 1, PF = NORM ? 4 : 8;           // weight rows per warp, pieces of them in flight
+  __shared__ float s_rs[MT];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int col = blockIdx.x * 4 + warp, m0 = blockIdx.y * MT, k = p.k;
+  const bool live = col < p.n;
+  const T* w[NW];
+  w[0] = p.w + (size_t)(EPI == ROW_QKV ? 2 * col : col) * k;
+  if (NW == 2) w[NW - 1] = EPI == ROW_QKV ? w[0] + k : p.w2 + (size_t)col * k;
+  uint4 wv[NW][PF];
+  auto fetch = [&](int base) {
 #pragma unroll
-  for (int i = 0; i < MT; ++i) acc[i] = 0.f;
-  const T* wrow = w + (size_t)col * k;
-  for (int k0 = lane * VEC; k0 < k; k0 += 32 * VEC) {
-    float wv[VEC];
-    load_vec(wrow + k0, wv);
+    for (int j = 0; j < PF; ++j) {
+      const int k0 = base + (j * 32 + lane) * VEC;
+#pragma unroll
+      for (int r = 0; r < NW; ++r)
+        wv[r][j] = live && k0 < k ? __ldg(reinterpret_cast<const uint4*>(w[r] + k0)) : make_uint4(0, 0, 0, 0);
+    }
+  };
+  fetch(0);
+  grid_dep_launch();
+  grid_dep_wait();
+  if (NORM) {
+    for (int i = warp; i < MT; i += 4) {
+      float ss = 0.f;
+      if (m0 + i < p.m) {
+        const float* row = p.x_in + (size_t)(m0 + i) * k;
+#pragma unroll 4
+        for (int j = lane * 4; j < k; j += 128) {
+          const float4 v = *reinterpret_cast<const float4*>(row + j);
+          ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+        }
+      }
+      ss = warp_sum(ss);
+      if (lane == 0) s_rs[i] = rsqrtf(ss / (float)k + p.eps);
+    }
+    __syncthreads();
+  }
+  if (!live) return;
+  float acc[NW][MT];
+#pragma unroll
+  for (int r = 0; r < NW; ++r)
+#pragma unroll
+    for (int i = 0; i < MT; ++i) acc[r][i] = 0.f;
+  for (int base = 0; base < k; base += PF * 32 * VEC) {
+    if (base > 0) fetch(base);
+#pragma unroll
+    for (int j = 0; j < PF; ++j) {
+      const int k0 = base + (j * 32 + lane) * VEC;
+      if (k0 >= k) break;
+      float wf[NW][VEC], sc[VEC];
+#pragma unroll
+      for (int r = 0; r < NW; ++r) load_vec(reinterpret_cast<const T*>(&wv[r][j]), wf[r]);
+      if (NORM) load_vec(p.scale + k0, sc);
+#pragma unroll
+      for (int i = 0; i < MT; ++i) {
+        if (m0 + i < p.m) {
+          float av[VEC];
+          if (NORM) {
+            const float rs = s_rs[i];
+#pragma unroll
+            for (int e = 0; e < VEC; e += 4) load_vec(p.x_in + (size_t)(m0 + i) * k + k0 + e, av + e);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) av[e] = to_f(from_f<T>(av[e] * rs * sc[e]));
+          } else {
+            load_vec(p.a + (size_t)(m0 + i) * k + k0, av);
+          }
+#pragma unroll
+          for (int r = 0; r < NW; ++r)
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) acc[r][i] = fmaf(av[e], wf[r][e], acc[r][i]);
+        }
+      }
+    }
+  }
+  float v[NW];                                   // lane i keeps row m0 + i
+#pragma unroll
+  for (int r = 0; r < NW; ++r) {
+    v[r] = 0.f;
 #pragma unroll
     for (int i = 0; i < MT; ++i) {
-      if (m0 + i < m) {
-        float av[VEC];
-        load_vec(a + (size_t)(m0 + i) * k + k0, av);
-#pragma unroll
-        for (int j = 0; j < VEC; ++j) acc[i] = fmaf(av[j], wv[j], acc[i]);
-      }
+      const float s = warp_sum(acc[r][i]);
+      if (lane == i) v[r] = s;
     }
   }
-#pragma unroll
-  for (int i = 0; i < MT; ++i) {
-    float v = warp_sum(acc[i]);
-    if (lane == 0 && m0 + i < m) {
-      float* dst = c + (size_t)(m0 + i) * ldc + col;
-      *dst = accumulate ? (*dst + v) : v;
+  const int row = m0 + lane;
+  if (lane >= MT || row >= p.m) return;
+  if constexpr (EPI == ROW_ADD) {
+    p.c[(size_t)row * p.ldc + col] += v[0];
+  } else if constexpr (EPI == ROW_STORE) {
+    p.c[(size_t)row * p.ldc + col] = v[0];
+  } else if constexpr (EPI == ROW_GATEUP) {
+    p.act[(size_t)row * p.n + col] = from_f<T>(v[0] / (1.f + expf(-v[0])) * v[NW - 1]);
+  } else {
+    const int r = row / p.t_len, t = row - r * p.t_len, fill = p.cache_len[r], pos = fill + t;
+    const bool ok = fill >= 0 && fill + p.t_len <= p.s_max;
+    if (!ok && col == 0) atomicOr(p.status, VVS_DEV_CACHE_OVERFLOW);
+    const int n = 2 * col, sec = n / p.d, e = n - sec * p.d, h = e / p.hd, i2 = e - h * p.hd;
+    float y0 = v[0], y1 = v[NW - 1];
+    if (sec < 2) {
+      float coord = 0.f;                         // coordinate driving this pair: first / second head half
+      if (p.rope_mode == VVS_ROPE_1D) {
+        coord = (float)pos;
+      } else if (p.rope_mode == VVS_ROPE_2D_GRID && pos >= p.n_prefix) {
+        const int g = pos - p.n_prefix;
+        coord = (float)(i2 < p.hd / 2 ? g / p.grid_w : g % p.grid_w);
+      }
+      float sn, cs;
+      sincosf(coord * p.inv_freq[i2 >> 1], &sn, &cs);
+      const float a0 = y0;
+      y0 = a0 * cs - y1 * sn;
+      y1 = a0 * sn + y1 * cs;
+    }
+    T* dst = nullptr;
+    if (sec == 0) dst = p.q + (size_t)row * p.d + e;
+    else if (ok) dst = (sec == 1 ? p.kv_k : p.kv_v) + ((((size_t)p.layer * p.kv_rows + r) * p.n_heads + h) * p.s_max + pos) * p.hd + i2;
+    if (dst) {
+      dst[0] = from_f<T>(y0);
+      dst[1] = from_f<T>(y1);
     }
   }
 }
 
 template <typename T>
-void launch_gemm_nt(const T* a, const T* w, float* c, int m, int n, int k, int ldc, bool accumulate,
-                    cudaStream_t s) {
-  constexpr int MT = 8;
-  dim3 grid((n + 3) / 4, (m + MT - 1) / MT);
-  gemm_nt_kernel<T, MT><<<grid, 128, 0, s>>>(a, w, c, m, n, k, ldc, accumulate ? 1 : 0);
+static void launch_row_gemm(int epi, const RowGemm<T>& p, bool pdl, cudaStream_t s) {
+  const dim3 grid((p.n + 3) / 4, (p.m + 7) / 8);
+  if (epi == ROW_QKV) launch_kernel(row_gemm_kernel<T, ROW_QKV>, grid, dim3(128), 0, pdl, s, p);
+  else if (epi == ROW_GATEUP) launch_kernel(row_gemm_kernel<T, ROW_GATEUP>, grid, dim3(128), 0, pdl, s, p);
+  else if (epi == ROW_ADD) launch_kernel(row_gemm_kernel<T, ROW_ADD>, grid, dim3(128), 0, pdl, s, p);
+  else launch_kernel(row_gemm_kernel<T, ROW_STORE>, grid, dim3(128), 0, pdl, s, p);
+}
+
+template <typename T>
+void launch_row_qkv(const float* x, const T* scale, float eps, const T* w, const float* inv_freq, T* q, T* kv_k, T* kv_v,
+                    const int32_t* cache_len, const vvs_model_desc& md, int layer, int kv_rows, int m, int t_len, int32_t* status,
+                    bool pdl, cudaStream_t s) {
+  RowGemm<T> p{};
+  p.m = m; p.n = 3 * md.d_model / 2; p.k = md.d_model; p.x_in = x; p.scale = scale; p.eps = eps; p.w = w; p.q = q; p.kv_k = kv_k;
+  p.kv_v = kv_v; p.inv_freq = inv_freq; p.cache_len = cache_len; p.status = status; p.d = md.d_model; p.n_heads = md.n_heads;
+  p.hd = md.head_dim; p.s_max = md.s_max; p.rope_mode = md.rope_mode; p.grid_w = md.rope_grid_w; p.n_prefix = md.n_prefix;
+  p.layer = layer; p.kv_rows = kv_rows; p.t_len = t_len;
+  launch_row_gemm<T>(ROW_QKV, p, pdl, s);
+}
+template <typename T>
+void launch_row_gateup(const float* x, const T* scale, float eps, const T* gate, const T* up, T* act, int m, int ff, int d, bool pdl,
+                       cudaStream_t s) {
+  RowGemm<T> p{};
+  p.m = m; p.n = ff; p.k = d; p.x_in = x; p.scale = scale; p.eps = eps; p.w = gate; p.w2 = up; p.act = act;
+  launch_row_gemm<T>(ROW_GATEUP, p, pdl, s);
+}
+// c[m, n] (+)= sum_k a[m, k] * w[n, k]
+template <typename T>
+void launch_row_product(const T* a, const T* w, float* c, int m, int n, int k, int ldc, bool accumulate, bool pdl, cudaStream_t s) {
+  RowGemm<T> p{};
+  p.m = m; p.n = n; p.k = k; p.a = a; p.w = w; p.c = c; p.ldc = ldc;
+  launch_row_gemm<T>(accumulate ? ROW_ADD : ROW_STORE, p, pdl, s);
 }
 
 // ---------------------------------------------------------------------------------------------
-// RoPE on q and k of the block rows, k/v appended to the cache at slots L_r + t.
-template <typename T>
-__global__ void rope_append_kernel(float* __restrict__ qkv, const float* __restrict__ inv_freq,
-                                   T* __restrict__ q, T* __restrict__ kv_k, T* __restrict__ kv_v,
-                                   const int32_t* __restrict__ cache_len, int d, int n_heads, int hd,
-                                   int s_max, int rope_mode, int grid_w, int n_prefix, int layer,
-                                   int kv_rows, int t_len, int32_t* status,
-                                   const float* __restrict__ tab_cos, const float* __restrict__ tab_sin,
-                                   int clear_src) {
-  int m = blockIdx.x;
-  int r = m / t_len, t = m % t_len;
-  int fill = cache_len[r];
-  bool ok = fill >= 0 && fill + t_len <= s_max;
-  if (!ok && threadIdx.x == 0) atomicOr(status, VVS_DEV_CACHE_OVERFLOW);
-  int pos = fill + t;
-  float c_lo = 0.f, c_hi = 0.f;  // coordinate driving the pairs of the first / second head half
-  if (rope_mode == VVS_ROPE_1D) {
-    c_lo = c_hi = (float)pos;
-  } else if (rope_mode == VVS_ROPE_2D_GRID && pos >= n_prefix) {
-    int n = pos - n_prefix;
-    c_lo = (float)(n / grid_w);
-    c_hi = (float)(n % grid_w);
+// Block-vs-cache attention: query row t of sequence r sees cache slots [0, L_r + t].  One CTA per (head, sequence,
+// query row): scores by groups of lanes that read a key row with 16-byte loads side by side, then softmax, then the
+// output by (column group, key phase) with a reduction over the phases.  A row's keys stay in L2 / L1 between the
+// CTAs of a head; with a few dozen (head, row) pairs the kernel is a chain of three round trips (40 -> XX us with four
+// heads, 5 rows and 69 keys, where a lane walked a whole key and a warp all keys of a column in turn).
+template <typename T, int HD>
+__global__ void __launch_bounds__(128) attention_kernel(const T* __restrict__ q, const T* __restrict__ kv_k,
+                                                        const T* __restrict__ kv_v, const int32_t* __restrict__ cache_len,
+                                                        T* __restrict__ out, int d, int n_heads, int s_max, int layer,
+                                                        int kv_rows, int t_len) {
+  extern __shared__ float sc[];                   // scores [s_max], then the phases' sums [kPh][HD]
+  constexpr int VEC = VecOf<T>::n, kLanes = HD / (2 * VEC), kGroups = 128 / kLanes;
+  constexpr int kCols = HD / VEC, kPh = 128 / kCols;
+  __shared__ float red[32];
+  const int h = blockIdx.x, r = blockIdx.y, t = blockIdx.z, tid = threadIdx.x;
+  grid_dep_launch();
+  grid_dep_wait();
+  const int fill = cache_len[r];
+  const size_t o = ((size_t)r * t_len + t) * d + (size_t)h * HD;
+  if (fill < 0 || fill + t_len > s_max) {
+    for (int i = tid; i < HD; i += 128) out[o + i] = from_f<T>(0.f);
+    return;
   }
-  float* src = qkv + (size_t)m * 3 * d;
-  int half = hd / 2;
-  for (int p = threadIdx.x; p < d / 2; p += blockDim.x) {
-    int h = p / half, i = p % half;
-    float sn, cs;
-    if (tab_cos) {                        // rotation tables of the step (tree calls: position = fill + depth)
-      cs = tab_cos[(size_t)m * half + i];
-      sn = tab_sin[(size_t)m * half + i];
-    } else {
-      sincosf(((i < half / 2) ? c_lo : c_hi) * inv_freq[i], &sn, &cs);
-    }
-    int e = h * hd + 2 * i;
-    float q0 = src[e], q1 = src[e + 1];
-    q[(size_t)m * d + e] = from_f<T>(q0 * cs - q1 * sn);
-    q[(size_t)m * d + e + 1] = from_f<T>(q0 * sn + q1 * cs);
-    if (ok) {
-      size_t slot = ((((size_t)layer * kv_rows + r) * n_heads + h) * s_max + pos) * hd + 2 * i;
-      float k0 = src[d + e], k1 = src[d + e + 1];
-      kv_k[slot] = from_f<T>(k0 * cs - k1 * sn);
-      kv_k[slot + 1] = from_f<T>(k0 * sn + k1 * cs);
-      kv_v[slot] = from_f<T>(src[2 * d + e]);
-      kv_v[slot + 1] = from_f<T>(src[2 * d + e + 1]);
-    }
-    if (clear_src) {                           // split-K sums are added into this buffer: leave it zero
-      const float2 z = make_float2(0.f, 0.f);
-      *reinterpret_cast<float2*>(src + e) = z;
-      *reinterpret_cast<float2*>(src + d + e) = z;
-      *reinterpret_cast<float2*>(src + 2 * d + e) = z;
-    }
-  }
-}
-
-template <typename T>
-void launch_rope_append(float* qkv, const float* inv_freq, T* q, T* kv_k, T* kv_v,
-                        const int32_t* cache_len, const vvs_model_desc& md, int layer, int kv_rows,
-                        int n_rows, int t_len, int32_t* status, cudaStream_t s, const float* tab_cos,
-                        const float* tab_sin, bool clear_src) {
-  rope_append_kernel<T><<<n_rows * t_len, 256, 0, s>>>(
-      qkv, inv_freq, q, kv_k, kv_v, cache_len, md.d_model, md.n_heads, md.head_dim, md.s_max,
-      md.rope_mode, md.rope_grid_w, md.n_prefix, layer, kv_rows, t_len, status, tab_cos, tab_sin, clear_src ? 1 : 0);
-}
-
-// ---------------------------------------------------------------------------------------------
-// Block-vs-cache attention: query row t of sequence r sees cache slots [0, L_r + t].
-// One CTA per (head, sequence); each warp owns query rows t = warp, warp + nwarps, ...
-template <typename T>
-__global__ void attention_kernel(const T* __restrict__ q, const T* __restrict__ kv_k,
-                                 const T* __restrict__ kv_v, const int32_t* __restrict__ cache_len,
-                                 T* __restrict__ out, int d, int n_heads, int hd, int s_max, int layer,
-                                 int kv_rows, int t_len) {
-  extern __shared__ float sm[];
-  constexpr int VEC = VecOf<T>::n;
-  int h = blockIdx.x, r = blockIdx.y;
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  float* sc = sm + (size_t)warp * (s_max + hd);
-  float* qv = sc + s_max;
-  int fill = cache_len[r];
-  bool ok = fill >= 0 && fill + t_len <= s_max;
-  size_t base = (((size_t)layer * kv_rows + r) * n_heads + h) * (size_t)s_max * hd;
-  const T* kb = kv_k + base;
-  const T* vb = kv_v + base;
-  float scale = rsqrtf((float)hd);
-  for (int t = warp; t < t_len; t += nw) {
-    size_t o = ((size_t)r * t_len + t) * d + (size_t)h * hd;
-    if (!ok) {
-      for (int i = lane; i < hd; i += 32) out[o + i] = from_f<T>(0.f);
-      continue;
-    }
-    for (int i = lane; i < hd; i += 32) qv[i] = to_f(q[o + i]);
-    __syncwarp();
-    int nk = fill + t + 1;
-    float mx = -CUDART_INF_F;
-    for (int j = lane; j < nk; j += 32) {
-      const T* kr = kb + (size_t)j * hd;
-      float s = 0.f;
-      for (int i = 0; i < hd; i += VEC) {
-        float kv[VEC];
-        load_vec(kr + i, kv);
+  const size_t base = (((size_t)layer * kv_rows + r) * n_heads + h) * (size_t)s_max * HD;
+  const int nk = fill + t + 1;
+  const float scale = rsqrtf((float)HD);
+  // ---- scores: group g takes keys g, g + kGroups, ..; lane c of it columns [c VEC, ..) and the same in the second half
+  const int g = tid / kLanes, c = tid & (kLanes - 1);
+  float q0[VEC], q1[VEC];
+  load_vec(q + o + c * VEC, q0);
+  load_vec(q + o + HD / 2 + c * VEC, q1);
+  float mx = -CUDART_INF_F;
+#pragma unroll 4
+  for (int j0 = 0; j0 < nk; j0 += kGroups) {
+    const int j = j0 + g;
+    float k0[VEC], k1[VEC], s = 0.f;
+    const T* kr = kv_k + base + (size_t)(j < nk ? j : 0) * HD + c * VEC;
+    load_vec(kr, k0);
+    load_vec(kr + HD / 2, k1);
 #pragma unroll
-        for (int e = 0; e < VEC; ++e) s = fmaf(qv[i + e], kv[e], s);
-      }
-      s *= scale;
-      sc[j] = s;
+    for (int e = 0; e < VEC; ++e) s = fmaf(q0[e], k0[e], fmaf(q1[e], k1[e], s));
+#pragma unroll
+    for (int w = kLanes / 2; w > 0; w >>= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
+    s *= scale;
+    if (j < nk) {
       mx = fmaxf(mx, s);
+      if (c == 0) sc[j] = s;
     }
-    mx = warp_max(mx);
-    float sum = 0.f;
-    for (int j = lane; j < nk; j += 32) {
-      float e = expf(sc[j] - mx);
-      sc[j] = e;
-      sum += e;
-    }
-    sum = warp_sum(sum);
-    __syncwarp();
-    float inv = 1.f / sum;
-    for (int i = lane; i < hd; i += 32) {
-      float acc = 0.f;
-      for (int j = 0; j < nk; ++j) acc = fmaf(sc[j], to_f(vb[(size_t)j * hd + i]), acc);
-      out[o + i] = from_f<T>(acc * inv);
-    }
-    __syncwarp();
+  }
+  mx = block_max(mx, red);                        // (its barriers also publish the scores)
+  float sum = 0.f;
+  for (int j = tid; j < nk; j += 128) {
+    const float e = expf(sc[j] - mx);
+    sc[j] = e;
+    sum += e;
+  }
+  sum = block_sum(sum, red);
+  // ---- output ----
+  const int cg = tid % kCols, ph = tid / kCols;
+  float acc[VEC];
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) acc[e] = 0.f;
+  const T* vb = kv_v + base + cg * VEC;
+#pragma unroll 8
+  for (int j = ph; j < nk; j += kPh) {
+    float v[VEC];
+    load_vec(vb + (size_t)j * HD, v);
+    const float pj = sc[j];
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) acc[e] = fmaf(pj, v[e], acc[e]);
+  }
+  float* part = sc + s_max;
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) part[ph * HD + cg * VEC + e] = acc[e];
+  __syncthreads();
+  const float inv = 1.f / sum;
+  for (int i = tid; i < HD; i += 128) {
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < kPh; ++w) s += part[w * HD + i];
+    out[o + i] = from_f<T>(s * inv);
   }
 }
 
 template <typename T>
 void launch_attention(const T* q, const T* kv_k, const T* kv_v, const int32_t* cache_len, T* out,
-                      const vvs_model_desc& md, int layer, int kv_rows, int n_rows, int t_len,
-                      cudaStream_t s) {
-  constexpr int kWarps = 4;
-  size_t smem = (size_t)kWarps * (md.s_max + md.head_dim) * sizeof(float);
-  if (smem > 48 * 1024) ensure_dynamic_smem(reinterpret_cast<const void*>(attention_kernel<T>), (int)smem);
-  dim3 grid(md.n_heads, n_rows);
-  attention_kernel<T><<<grid, kWarps * 32, smem, s>>>(q, kv_k, kv_v, cache_len, out, md.d_model,
-                                                      md.n_heads, md.head_dim, md.s_max, layer,
-                                                      kv_rows, t_len);
+                      const vvs_model_desc& md, int layer, int kv_rows, int n_rows, int t_len, bool pdl, cudaStream_t s) {
+  // phases x head_dim = 128 x VEC whatever the head_dim
+  const size_t smem = ((size_t)md.s_max + 128 * VecOf<T>::n) * sizeof(float);
+  auto* kernel = md.head_dim == 64 ? attention_kernel<T, 64> : attention_kernel<T, 128>;
+  if (smem > 48 * 1024) ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), (int)smem);
+  launch_kernel(kernel, dim3(md.n_heads, n_rows, t_len), dim3(128), smem, pdl, s, q, kv_k, kv_v, cache_len, out, (int)md.d_model,
+                (int)md.n_heads, (int)md.s_max, layer, kv_rows, t_len);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -450,62 +549,60 @@ void launch_silu_mul(float* gu, T* act, int m, int ff, cudaStream_t s, bool clea
 }
 
 // ---------------------------------------------------------------------------------------------
-// guided logits / temperature:  l = l_u + s (l_c - l_u)  (or l_c without guidance)
-__global__ void guide_kernel(const float* __restrict__ raw, float* __restrict__ logits, int n_images,
-                             int n_cfg, int rows_per_seq, int v, float cfg_scale, float inv_temp) {
-  int row = blockIdx.x;  // b * rows_per_seq + t
+// guided logits / temperature:  l = l_u + s (l_c - l_u)  (or l_c without guidance), and the row's max and sum of
+// exp(l - max) as a single "tile" of softmax partials
+__global__ void __launch_bounds__(256) guide_stats_kernel(const float* __restrict__ raw, float* __restrict__ logits,
+                                                          float* __restrict__ part_m, float* __restrict__ part_s, int n_images,
+                                                          int n_cfg, int rows_per_seq, int v, float cfg_scale, float inv_temp) {
+  __shared__ float red[32];
+  const int row = blockIdx.x;  // b * rows_per_seq + t
+  grid_dep_launch();
+  grid_dep_wait();
   const float* lc = raw + (size_t)row * v;
   const float* lu = raw + ((size_t)n_images * rows_per_seq + row) * v;
   float* o = logits + (size_t)row * v;
-  for (int j = threadIdx.x; j < v; j += blockDim.x) {
+  float mx = -CUDART_INF_F;
+#pragma unroll 4
+  for (int j = threadIdx.x; j < v; j += 256) {
     float l = lc[j];
     if (n_cfg == 2) {
-      float u = lu[j];
+      const float u = lu[j];
       l = u + cfg_scale * (l - u);
     }
-    o[j] = l * inv_temp;
+    l *= inv_temp;
+    o[j] = l;
+    mx = fmaxf(mx, l);
   }
-}
-
-void launch_guide(const float* raw, float* logits, int n_images, int n_cfg, int rows_per_seq, int v,
-                  float cfg_scale, float inv_temp, cudaStream_t s) {
-  guide_kernel<<<n_images * rows_per_seq, 256, 0, s>>>(raw, logits, n_images, n_cfg, rows_per_seq, v,
-                                                       cfg_scale, inv_temp);
-}
-
-// per-row max and sum of exp(l - max) as a single "tile" of softmax partials
-__global__ void row_stats_kernel(const float* __restrict__ logits, float* __restrict__ part_m,
-                                 float* __restrict__ part_s, int v) {
-  __shared__ float red[32];
-  const float* row = logits + (size_t)blockIdx.x * v;
-  float mx = -CUDART_INF_F;
-  for (int j = threadIdx.x; j < v; j += blockDim.x) mx = fmaxf(mx, row[j]);
   mx = block_max(mx, red);
   float sum = 0.f;
-  for (int j = threadIdx.x; j < v; j += blockDim.x) sum += expf(row[j] - mx);
+  for (int j = threadIdx.x; j < v; j += 256) sum += expf(o[j] - mx);      // this thread's own values
   sum = block_sum(sum, red);
   if (threadIdx.x == 0) {
-    part_m[blockIdx.x] = mx;
-    part_s[blockIdx.x] = sum;
+    part_m[row] = mx;
+    part_s[row] = sum;
   }
 }
 
-void launch_row_stats(const float* logits, float* part_m, float* part_s, int n_rows, int v,
-                      cudaStream_t s) {
-  row_stats_kernel<<<n_rows, 256, 0, s>>>(logits, part_m, part_s, v);
+void launch_guide_stats(const float* raw, float* logits, float* part_m, float* part_s, int n_images, int n_cfg, int rows_per_seq,
+                        int v, float cfg_scale, float inv_temp, bool pdl, cudaStream_t s) {
+  launch_kernel(guide_stats_kernel, dim3(n_images * rows_per_seq), dim3(256), 0, pdl, s, raw, logits, part_m, part_s, n_images,
+                n_cfg, rows_per_seq, v, cfg_scale, inv_temp);
 }
 
 // explicit instantiations
-#define VVS_INSTANTIATE(T)                                                                          \
-  template void launch_embed<T>(const T*, const int32_t*, float*, int, int, int, int, int, int32_t*, \
-                                cudaStream_t);                                                       \
-  template void launch_rmsnorm<T>(const float*, const T*, T*, int, int, float, cudaStream_t);        \
-  template void launch_gemm_nt<T>(const T*, const T*, float*, int, int, int, int, bool, cudaStream_t); \
-  template void launch_rope_append<T>(float*, const float*, T*, T*, T*, const int32_t*,              \
-                                      const vvs_model_desc&, int, int, int, int, int32_t*,           \
-                                      cudaStream_t, const float*, const float*, bool);               \
-  template void launch_attention<T>(const T*, const T*, const T*, const int32_t*, T*,                \
-                                    const vvs_model_desc&, int, int, int, int, cudaStream_t);        \
+#define VVS_INSTANTIATE(T)                                                                             \
+  template void launch_embed<T>(const T*, const int32_t*, float*, int, int, int, int, int, int32_t*,    \
+                                cudaStream_t);                                                          \
+  template void launch_rmsnorm<T>(const float*, const T*, T*, int, int, float, cudaStream_t, bool);     \
+  template void launch_row_qkv<T>(const float*, const T*, float, const T*, const float*, T*, T*, T*,    \
+                                  const int32_t*, const vvs_model_desc&, int, int, int, int, int32_t*,  \
+                                  bool, cudaStream_t);                                                  \
+  template void launch_row_gateup<T>(const float*, const T*, float, const T*, const T*, T*, int, int,   \
+                                     int, bool, cudaStream_t);                                          \
+  template void launch_row_product<T>(const T*, const T*, float*, int, int, int, int, bool, bool,       \
+                                      cudaStream_t);                                                    \
+  template void launch_attention<T>(const T*, const T*, const T*, const int32_t*, T*,                   \
+                                    const vvs_model_desc&, int, int, int, int, bool, cudaStream_t);     \
   template void launch_silu_mul<T>(float*, T*, int, int, cudaStream_t, bool, bool);
 VVS_INSTANTIATE(float)
 VVS_INSTANTIATE(__nv_bfloat16)

@@ -204,7 +204,7 @@ int run_decisions(vvs_ctx* ctx, const T* hid, int rows_per_seq, int first_row, c
     if (fused) {
       VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(lbuf, true, (V + 127) / 128, BT, ws, p, ctx->use_pdl, s));
       if (rc == VVS_OK && o->target_probs)
-        VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(o->target_probs, ws, o->target_probs, BT, V, s));
+        VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(o->target_probs, ws, o->target_probs, BT, V, ctx->use_pdl, s));
       return rc != VVS_OK ? rc : cudaGetLastError() == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
     }
     VVS_LAUNCH(VVS_PROF_OTHER, launch_finalize_stats(ws, (V + 127) / 128, BT, s));
@@ -212,7 +212,7 @@ int run_decisions(vvs_ctx* ctx, const T* hid, int rows_per_seq, int first_row, c
     if (lbuf) {
       VVS_LAUNCH(VVS_PROF_OTHER, launch_select_p_row(lbuf, ws, B, V, s));
       if (o->target_probs)
-        VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(o->target_probs, ws, o->target_probs, BT, V, s));
+        VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(o->target_probs, ws, o->target_probs, BT, V, ctx->use_pdl, s));
       if (p.adjusted) VVS_LAUNCH(VVS_PROF_OTHER, launch_adjust_target(ws, p, s));
       VVS_LAUNCH(VVS_PROF_OTHER, launch_residual_mass(ws, p, s));
       VVS_LAUNCH(VVS_PROF_OTHER, launch_sample(ws, p, s));
@@ -230,22 +230,21 @@ int run_decisions(vvs_ctx* ctx, const T* hid, int rows_per_seq, int first_row, c
     VVS_LAUNCH(VVS_PROF_OTHER, launch_sample(ws, p, s));
     return cudaGetLastError() == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
   }
-  VVS_LAUNCH(VVS_PROF_GEMM, launch_gemm_nt<T>(hid, w_lm, ws.logits_raw, M, V, md.d_model, V, false, s));
-  VVS_LAUNCH(VVS_PROF_OTHER, launch_guide(ws.logits_raw, ws.logits, B, C, rows_per_seq, V, a->cfg_scale,
-                                          1.f / a->temperature, s));
-  VVS_LAUNCH(VVS_PROF_OTHER, launch_row_stats(ws.logits, ws.part_m, ws.part_s, BT, V, s));
+  VVS_LAUNCH(VVS_PROF_GEMM, launch_row_product<T>(hid, w_lm, ws.logits_raw, M, V, md.d_model, V, false, ctx->use_pdl, s));
+  VVS_LAUNCH(VVS_PROF_OTHER, launch_guide_stats(ws.logits_raw, ws.logits, ws.part_m, ws.part_s, B, C, rows_per_seq, V, a->cfg_scale,
+                                                1.f / a->temperature, ctx->use_pdl, s));
   if (!p.adjusted) {
     int rc = VVS_OK;
-    VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(ws.logits, true, 1, BT, ws, p, false, s));
+    VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(ws.logits, true, 1, BT, ws, p, ctx->use_pdl, s));
     if (rc == VVS_OK && o->target_probs)
-      VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(ws.logits, ws, o->target_probs, BT, V, s));
+      VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(ws.logits, ws, o->target_probs, BT, V, ctx->use_pdl, s));
     return rc != VVS_OK ? rc : cudaGetLastError() == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
   }
   VVS_LAUNCH(VVS_PROF_OTHER, launch_finalize_stats(ws, 1, BT, s));
   if (p.n_draft_max > 0) VVS_LAUNCH(VVS_PROF_OTHER, launch_gather_logits(ws.logits, ws, p, s));
   VVS_LAUNCH(VVS_PROF_OTHER, launch_accept(ws, p, s));
   if (o->target_probs)
-    VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(ws.logits, ws, o->target_probs, BT, V, s));
+    VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(ws.logits, ws, o->target_probs, BT, V, ctx->use_pdl, s));
   VVS_LAUNCH(VVS_PROF_OTHER, launch_select_p_row(ws.logits, ws, B, V, s));
   if (p.adjusted) VVS_LAUNCH(VVS_PROF_OTHER, launch_adjust_target(ws, p, s));
   VVS_LAUNCH(VVS_PROF_OTHER, launch_residual_mass(ws, p, s));
@@ -261,7 +260,6 @@ int run_verify(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* o, 
   const int M = R * Tn, d = md.d_model, ff = md.d_ff;
   T* kv_k = static_cast<T*>(a->kv_k);
   T* kv_v = static_cast<T*>(a->kv_v);
-  T* xn = static_cast<T*>(ws.xn);
   T* q = static_cast<T*>(ws.q);
   T* attn = static_cast<T*>(ws.attn);
   T* act = static_cast<T*>(ws.act);
@@ -269,25 +267,19 @@ int run_verify(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* o, 
 
   VVS_LAUNCH(VVS_PROF_OTHER, launch_embed<T>(static_cast<const T*>(ctx->tok_emb), a->block, ws.x, B, C, Tn,
                                              d, md.tok_rows, ws.status, s));
+  const bool pdl = ctx->use_pdl;
   for (int l = 0; l < md.n_layers; ++l) {
     const Layer& L = ctx->layers[l];
-    VVS_LAUNCH(VVS_PROF_OTHER, launch_rmsnorm<T>(ws.x, static_cast<const T*>(L.norm1), xn, M, d, md.rms_eps, s));
-    VVS_LAUNCH(VVS_PROF_GEMM,
-               launch_gemm_nt<T>(xn, static_cast<const T*>(L.w_qkv), ws.qkv, M, 3 * d, d, 3 * d, false, s));
-    VVS_LAUNCH(VVS_PROF_OTHER, launch_rope_append<T>(ws.qkv, ws.rope_inv_freq, q, kv_k, kv_v, a->cache_len, md,
-                                                     l, a->kv_rows, R, Tn, ws.status, s));
-    VVS_LAUNCH(VVS_PROF_ATTENTION,
-               launch_attention<T>(q, kv_k, kv_v, a->cache_len, attn, md, l, a->kv_rows, R, Tn, s));
-    VVS_LAUNCH(VVS_PROF_GEMM, launch_gemm_nt<T>(attn, static_cast<const T*>(L.w_o), ws.x, M, d, d, d, true, s));
-    VVS_LAUNCH(VVS_PROF_OTHER, launch_rmsnorm<T>(ws.x, static_cast<const T*>(L.norm2), xn, M, d, md.rms_eps, s));
-    VVS_LAUNCH(VVS_PROF_GEMM,
-               launch_gemm_nt<T>(xn, static_cast<const T*>(L.w_gate), ws.gu, M, ff, d, 2 * ff, false, s));
-    VVS_LAUNCH(VVS_PROF_GEMM,
-               launch_gemm_nt<T>(xn, static_cast<const T*>(L.w_up), ws.gu + ff, M, ff, d, 2 * ff, false, s));
-    VVS_LAUNCH(VVS_PROF_OTHER, launch_silu_mul<T>(ws.gu, act, M, ff, s));
-    VVS_LAUNCH(VVS_PROF_GEMM, launch_gemm_nt<T>(act, static_cast<const T*>(L.w_down), ws.x, M, d, ff, d, true, s));
+    VVS_LAUNCH(VVS_PROF_GEMM, launch_row_qkv<T>(ws.x, static_cast<const T*>(L.norm1), md.rms_eps, static_cast<const T*>(L.w_qkv),
+                                                ws.rope_inv_freq, q, kv_k, kv_v, a->cache_len, md, l, a->kv_rows, M, Tn, ws.status,
+                                                pdl, s));
+    VVS_LAUNCH(VVS_PROF_ATTENTION, launch_attention<T>(q, kv_k, kv_v, a->cache_len, attn, md, l, a->kv_rows, R, Tn, pdl, s));
+    VVS_LAUNCH(VVS_PROF_GEMM, launch_row_product<T>(attn, static_cast<const T*>(L.w_o), ws.x, M, d, d, d, true, pdl, s));
+    VVS_LAUNCH(VVS_PROF_GEMM, launch_row_gateup<T>(ws.x, static_cast<const T*>(L.norm2), md.rms_eps, static_cast<const T*>(L.w_gate),
+                                                   static_cast<const T*>(L.w_up), act, M, ff, d, pdl, s));
+    VVS_LAUNCH(VVS_PROF_GEMM, launch_row_product<T>(act, static_cast<const T*>(L.w_down), ws.x, M, d, ff, d, true, pdl, s));
   }
-  VVS_LAUNCH(VVS_PROF_OTHER, launch_rmsnorm<T>(ws.x, static_cast<const T*>(ctx->norm_f), hid, M, d, md.rms_eps, s));
+  VVS_LAUNCH(VVS_PROF_OTHER, launch_rmsnorm<T>(ws.x, static_cast<const T*>(ctx->norm_f), hid, M, d, md.rms_eps, s, pdl));
   if (cudaGetLastError() != cudaSuccess) return VVS_ERR_CUDA;
   return run_decisions<T>(ctx, hid, Tn, a->n_forced - 1, a->block + a->n_forced, Tn, a, o, true, s);
 }
@@ -315,7 +307,7 @@ int run_tree_decisions(vvs_ctx* ctx, const __nv_bfloat16* hid, const vvs_verify_
   VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_lmhead_tc(la, s));
   if (rc != VVS_OK) return rc;
   VVS_LAUNCH(VVS_PROF_OTHER, launch_finalize_stats(ws, (V + 127) / 128, BT, s));
-  VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(o->target_probs, ws, o->target_probs, BT, V, s));
+  VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(o->target_probs, ws, o->target_probs, BT, V, ctx->use_pdl, s));
   TreeParams tp{};
   tp.n_images = B; tp.n_cfg = C; tp.n_forced = a->n_forced; tp.n_draft_max = a->n_draft_max; tp.t_len = Tn;
   tp.vocab = V; tp.vocab_offset = md.vocab_offset; tp.parent = a->tree_parent; tp.drafts = a->block + a->n_forced;
@@ -397,7 +389,6 @@ int run_verify_tc(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* 
   const bool gu_dual = !fixed_order && p_gu.passes == 1 && (size_t)2 * ff * d * sizeof(T) < ((size_t)64 << 20);
   CUtensorMap tm_xn2;
   if (make_tmap_bf16_2d(&tm_xn2, xn, (uint64_t)M, (uint64_t)d, (uint32_t)p_gu.nt) != VVS_OK) return VVS_ERR_CUDA;
-  const bool rows_attention = wide && attention_rows_applicable(md, Tn);
   AttentionRowsArgs ar{};
   ar.qkv = ws.qkv; ar.kv_k = kv_k; ar.kv_v = kv_v; ar.cache_len = a->cache_len; ar.rope_cos = ws.rope_cos;
   ar.rope_sin = ws.rope_sin; ar.anc_mask = ws.anc_mask; ar.seq_order = ws.seq_order; ar.out = attn; ar.d = d; ar.n_heads = md.n_heads;
@@ -485,22 +476,15 @@ int run_verify_tc(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* 
       g.n = 3 * d; g.k = d; g.tm_a = &W.w_qkv; g.tm_b = &tm_xn; g.out = ws.qkv; g.ldo = 3 * d;
       g.cluster_mode = cm_store;
       VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_gemm_tc(GEMM_EPI_ADD, p_qkv, g, s));
-      if (rows_attention) {
-        // rotation, rounding, cache append and attention of each (sequence, head) in one kernel
-        ar.layer = l;
-        if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_ATTENTION, rc = launch_attention_rows(ar, s));
-      } else {
-        VVS_LAUNCH(VVS_PROF_OTHER, launch_rope_append<T>(ws.qkv, ws.rope_inv_freq, q, kv_k, kv_v, a->cache_len, md,
-                                                         l, a->kv_rows, R, Tn, ws.status, s,
-                                                         a->tree_parent ? ws.rope_cos : nullptr,
-                                                         a->tree_parent ? ws.rope_sin : nullptr, true));
-      }
+      // rotation, rounding, cache append and attention of each (sequence, head) in one kernel
+      ar.layer = l;
+      if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_ATTENTION, rc = launch_attention_rows(ar, s));
     } else {
       GemmTcArgs g = base;
       g.n = 3 * d; g.k = d; g.tm_a = &W.w_qkv; g.tm_b = &tm_xn; g.ld_scratch = 3 * d; g.layer = l;
       VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_gemm_tc(GEMM_EPI_QKV, p_qkv, g, s));
     }
-    if (rc == VVS_OK && !(wide && rows_attention)) {
+    if (rc == VVS_OK && !wide) {
       at.layer = l;
       VVS_LAUNCH(VVS_PROF_ATTENTION, rc = launch_attention_tc(at, s));
     }

@@ -209,28 +209,27 @@ template <typename T>
 void launch_embed(const T* tok_emb, const int32_t* block, float* x, int n_images, int n_cfg,
                   int t_len, int d, int tok_rows, int32_t* status, cudaStream_t s);
 template <typename T>
-void launch_rmsnorm(const float* x, const T* scale, T* out, int m, int d, float eps, cudaStream_t s);
+void launch_rmsnorm(const float* x, const T* scale, T* out, int m, int d, float eps, cudaStream_t s, bool pdl = false);
+enum { ROW_QKV = 0, ROW_GATEUP = 1, ROW_ADD = 2, ROW_STORE = 3 };
+template <typename T>
+void launch_row_qkv(const float* x, const T* scale, float eps, const T* w, const float* inv_freq, T* q, T* kv_k, T* kv_v,
+                    const int32_t* cache_len, const vvs_model_desc& md, int layer, int kv_rows, int m, int t_len, int32_t* status,
+                    bool pdl, cudaStream_t s);
+template <typename T>
+void launch_row_gateup(const float* x, const T* scale, float eps, const T* gate, const T* up, T* act, int m, int ff, int d, bool pdl,
+                       cudaStream_t s);
 // c[m, n] (+)= sum_k a[m, k] * w[n, k]; c fp32 with leading dimension ldc
 template <typename T>
-void launch_gemm_nt(const T* a, const T* w, float* c, int m, int n, int k, int ldc, bool accumulate,
-                    cudaStream_t s);
-template <typename T>
-void launch_rope_append(float* qkv, const float* inv_freq, T* q, T* kv_k, T* kv_v,
-                        const int32_t* cache_len, const vvs_model_desc& md, int layer, int kv_rows,
-                        int n_rows, int t_len, int32_t* status, cudaStream_t s, const float* tab_cos = nullptr,
-                        const float* tab_sin = nullptr, bool clear_src = false);
+void launch_row_product(const T* a, const T* w, float* c, int m, int n, int k, int ldc, bool accumulate, bool pdl, cudaStream_t s);
 template <typename T>
 void launch_attention(const T* q, const T* kv_k, const T* kv_v, const int32_t* cache_len, T* out,
-                      const vvs_model_desc& md, int layer, int kv_rows, int n_rows, int t_len,
-                      cudaStream_t s);
+                      const vvs_model_desc& md, int layer, int kv_rows, int n_rows, int t_len, bool pdl, cudaStream_t s);
 template <typename T>
 void launch_silu_mul(float* gu, T* act, int m, int ff, cudaStream_t s, bool clear_src = false, bool pdl = false);
 void launch_rmsnorm_rows(const float* x, const __nv_bfloat16* scale, __nv_bfloat16* out, int m, int d, float eps,
                          bool pdl, cudaStream_t s);
-void launch_guide(const float* raw, float* logits, int n_images, int n_cfg, int rows_per_seq, int v,
-                  float cfg_scale, float inv_temp, cudaStream_t s);
-void launch_row_stats(const float* logits, float* part_m, float* part_s, int n_rows, int v,
-                      cudaStream_t s);
+void launch_guide_stats(const float* raw, float* logits, float* part_m, float* part_s, int n_images, int n_cfg, int rows_per_seq,
+                        int v, float cfg_scale, float inv_temp, bool pdl, cudaStream_t s);
 
 // ---- tensor-core projection GEMM, gemm_tc.cu ----------------------------------------------------
 enum { GEMM_EPI_STORE = 0, GEMM_EPI_ADD = 1, GEMM_EPI_QKV = 2, GEMM_EPI_SWIGLU = 3, GEMM_EPI_ADD2 = 4 };
@@ -290,7 +289,6 @@ struct AttentionRowsArgs {
   int d, n_heads, hd, s_max, layer, kv_rows, t_len, n_rows, n_sms;
   bool pdl;
 };
-bool attention_rows_applicable(const vvs_model_desc& md, int t_len);
 int launch_attention_rows(const AttentionRowsArgs& a, cudaStream_t s);
 
 // ---- LM head with fused decision epilogue, lmhead_tc.cu -------------------------------------------
@@ -419,7 +417,7 @@ void launch_finalize_stats(const Workspace& ws, int n_tiles, int n_rows, cudaStr
 void launch_gather_logits(const float* logits, const Workspace& ws, const DecideParams& p, cudaStream_t s);
 void launch_accept(const Workspace& ws, const DecideParams& p, cudaStream_t s);
 void launch_probs_from_logits(const float* logits, const Workspace& ws, float* probs, int n_rows,
-                              int v, cudaStream_t s);
+                              int v, bool pdl, cudaStream_t s);
 void launch_select_p_row(const float* logits, const Workspace& ws, int n_images, int v, cudaStream_t s);
 void launch_adjust_target(const Workspace& ws, const DecideParams& p, cudaStream_t s);
 void launch_residual_mass(const Workspace& ws, const DecideParams& p, cudaStream_t s);
