@@ -56,12 +56,12 @@ __global__ void finalize_stats_kernel(const float* __restrict__ part_m, const fl
   int lane = threadIdx.x & 31;
   if (row >= n_rows) return;
   float mx = -CUDART_INF_F;
-  for (int t = lane; t < n_tiles; t += 32) mx = fmaxf(mx, part_m[(size_t)t * n_rows + row]);
+  for (int t = lane; t < n_tiles; t += 32) mx = fmaxf(mx, part_m[(size_t)row * n_tiles + t]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   float sum = 0.f;
   for (int t = lane; t < n_tiles; t += 32)
-    sum += part_s[(size_t)t * n_rows + row] * expf(part_m[(size_t)t * n_rows + row] - mx);
+    sum += part_s[(size_t)row * n_tiles + t] * expf(part_m[(size_t)row * n_tiles + t] - mx);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
   if (lane == 0) {
@@ -423,10 +423,10 @@ __device__ __forceinline__ double ld_cluster_f64(const double* local, uint32_t r
   return v;
 }
 
-// LOGITS: rows hold guided logits, statistics come from the [n_tiles, n_rows] softmax partials; else probabilities.
+// LOGITS: rows hold guided logits, statistics come from the [rows, n_tiles] softmax partials; else probabilities.
 template <bool LOGITS>
 __global__ void __launch_bounds__(kDecideThreads) decide_kernel(Workspace ws, DecideParams p, const float* __restrict__ rows,
-                                                                int n_tiles, int n_rows) {
+                                                                int n_tiles) {
   __shared__ float s_m[32], s_inv[32];
   __shared__ double s_ratio[32];
   __shared__ double s_w[2][kDecideWarps];            // masses of this CTA's warps: residual, target
@@ -444,11 +444,15 @@ __global__ void __launch_bounds__(kDecideThreads) decide_kernel(Workspace ws, De
     for (int r = warp; r < p.rows_per_seq; r += kDecideWarps) {
       const int row = b * p.rows_per_seq + r;
       float mx = -CUDART_INF_F;
-      for (int t = lane; t < n_tiles; t += 32) mx = fmaxf(mx, ws.part_m[(size_t)t * n_rows + row]);
+      const float* pm = ws.part_m + (size_t)row * n_tiles;
+      const float* ps = ws.part_s + (size_t)row * n_tiles;
+#pragma unroll 4
+      for (int t = lane; t < n_tiles; t += 32) mx = fmaxf(mx, pm[t]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       float sum = 0.f;
-      for (int t = lane; t < n_tiles; t += 32) sum += ws.part_s[(size_t)t * n_rows + row] * expf(ws.part_m[(size_t)t * n_rows + row] - mx);
+#pragma unroll 4
+      for (int t = lane; t < n_tiles; t += 32) sum += ps[t] * expf(pm[t] - mx);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
       if (lane == 0) {
@@ -484,15 +488,41 @@ __global__ void __launch_bounds__(kDecideThreads) decide_kernel(Workspace ws, De
         const int beg = p.row_ptr[x], len = p.row_ptr[x + 1] - beg;
         if (len < 1 && lane == 0) atomicOr(ws.status, VVS_DEV_BAD_NEIGHBOUR);
         const int kk = min(p.nbr_k, len);
-        int j_end;
-        mass += pooled_prefix(kk, (double)p.delta, lane, [&](int j) {
-          const int c = p.col[beg + j];
-          if (c < 0 || c >= V) {
-            atomicOr(ws.status, VVS_DEV_BAD_NEIGHBOUR);
-            return 0.0;
+        // entries 1 .. kk-1, 128 at a time: their columns, then their values in flight together; with an unlimited
+        // delta only the sum is wanted, else the longest prefix whose mass stays <= delta
+        constexpr int kBatch = 4;
+        const bool all = isinf(p.delta);
+        double cum = 0.0;
+        bool over = false;
+        for (int j0 = 1; j0 < kk && !over; j0 += 32 * kBatch) {
+          int c[kBatch];
+          float pn[kBatch];
+#pragma unroll
+          for (int e = 0; e < kBatch; ++e) c[e] = j0 + e * 32 + lane < kk ? p.col[beg + j0 + e * 32 + lane] : -2;
+#pragma unroll
+          for (int e = 0; e < kBatch; ++e) {
+            if (c[e] != -2 && (c[e] < 0 || c[e] >= V)) {
+              atomicOr(ws.status, VVS_DEV_BAD_NEIGHBOUR);
+              c[e] = -2;
+            }
+            pn[e] = c[e] >= 0 ? row[c[e]] : 0.f;
           }
-          return (double)(LOGITS ? prob_of(row[c], m, inv) : row[c]);
-        }, &j_end);
+#pragma unroll
+          for (int e = 0; e < kBatch; ++e) {
+            const double v = c[e] >= 0 ? (double)(LOGITS ? prob_of(pn[e], m, inv) : pn[e]) : 0.0;
+            if (all) {
+              cum += v;                               // this lane's share
+            } else if (!over) {
+              const double tot = cum + warp_incl_scan_d(v, lane);
+              const unsigned stop = __ballot_sync(0xffffffffu, j0 + e * 32 + lane < kk && tot > (double)p.delta);
+              const int last = stop ? __ffs(stop) - 2 : 31;        // last lane pooled
+              const double upto = __shfl_sync(0xffffffffu, tot, last < 0 ? 0 : last);
+              if (last >= 0) cum = upto;
+              over = stop != 0;
+            }
+          }
+        }
+        mass += all ? warp_sum_d(cum) : cum;
       }
       ratio = qx > 0.0 ? fmin(1.0, mass / qx) : (mass > 0.0 ? 1.0 : 0.0);
     }
@@ -530,18 +560,38 @@ __global__ void __launch_bounds__(kDecideThreads) decide_kernel(Workspace ws, De
   const float* p_row = rows + ((size_t)b * p.rows_per_seq + (has_row ? r_sel : 0)) * V;
   const float* q_row = p.draft_probs + ((size_t)b * K + (s_kind == 0 ? n : 0)) * V;
   const float m = LOGITS ? s_m[has_row ? r_sel : 0] : 0.f, inv = LOGITS ? s_inv[has_row ? r_sel : 0] : 1.f;
-  const int per = (V + S * kDecideWarps - 1) / (S * kDecideWarps), at = (rank * kDecideWarps + warp) * per;
-  const int v0 = min(V, at), v1 = min(V, at + per), kind = s_kind;
-  auto target = [&](int j) { return LOGITS ? prob_of(p_row[j], m, inv) : p_row[j]; };
+  // a contiguous range per warp and, inside it, per lane (whole 16-byte pieces), so that the sample is found by one
+  // scan of the lanes' sums and a walk of one lane's few codes
+  const int per_lane = ((V + S * kDecideThreads - 1) / (S * kDecideThreads) + 3) & ~3;
+  const int at = (rank * kDecideThreads + tid) * per_lane;
+  const int v0 = min(V, at), v1 = min(V, at + per_lane), kind = s_kind;
+  auto target = [&](float x) { return LOGITS ? prob_of(x, m, inv) : x; };
+  auto value = [&](float pr, float q, int how) { return (double)(how != 0 ? pr : fmaxf(0.f, pr - q)); };
+  const bool vec = (V & 3) == 0;                      // rows start on 16-byte boundaries
   double sr = 0.0, sp = 0.0;
   if (has_row) {
-#pragma unroll 8
-    for (int j = v0 + lane; j < v1; j += 32) {
-      const float pr = target(j);
-      sr += (double)(kind != 0 ? pr : fmaxf(0.f, pr - q_row[j]));
-      sp += (double)pr;
+    if (vec) {
+#pragma unroll 4
+      for (int j = v0; j < v1; j += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(p_row + j);
+        const float4 q = kind == 0 ? *reinterpret_cast<const float4*>(q_row + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float pr[4] = {target(x.x), target(x.y), target(x.z), target(x.w)}, qv[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          sr += value(pr[e], qv[e], kind);
+          sp += (double)pr[e];
+        }
+      }
+    } else {
+#pragma unroll 4
+      for (int j = v0; j < v1; ++j) {
+        const float pr = target(p_row[j]);
+        sr += value(pr, kind == 0 ? q_row[j] : 0.f, kind);
+        sp += (double)pr;
+      }
     }
   }
+  const double lane_mass[2] = {sr, sp};
   sr = warp_sum_d(sr);
   sp = warp_sum_d(sp);
   if (lane == 0) {
@@ -595,25 +645,34 @@ __global__ void __launch_bounds__(kDecideThreads) decide_kernel(Workspace ws, De
     }
     if (sel < 0) { sel = last_nz; sel_lo = nz_lo; }
     if (warp == sel) {
-      double run = sel_lo, pick_lo = 0.0, pick_hi = 0.0;
-      int pick = -1;
-      bool found = false;
-      for (int j0 = v0; j0 < v1 && !found; j0 += 32) {
-        const int j = j0 + lane;
-        const float pr = j < v1 ? target(j) : 0.f;
-        const double val = j < v1 ? (double)(eff != 0 ? pr : fmaxf(0.f, pr - q_row[j])) : 0.0;
-        const double inc = warp_incl_scan_d(val, lane), cdf = run + inc;
-        const unsigned over = __ballot_sync(0xffffffffu, j < v1 && cdf > s_t), nz = __ballot_sync(0xffffffffu, val > 0.0);
-        const int src = over ? __ffs(over) - 1 : nz ? 31 - __clz(nz) : -1;
-        if (src >= 0) {
-          pick = j0 + src;
-          pick_hi = __shfl_sync(0xffffffffu, cdf, src);
-          pick_lo = pick_hi - __shfl_sync(0xffffffffu, val, src);
+      const double mine = lane_mass[s_use_p], incl = warp_incl_scan_d(mine, lane);
+      const unsigned hit = __ballot_sync(0xffffffffu, sel_lo + incl > s_t), nz = __ballot_sync(0xffffffffu, mine > 0.0);
+      const int src = hit ? __ffs(hit) - 1 : nz ? 31 - __clz(nz) : 0;
+      if (lane == src) {
+        double run = sel_lo + (incl - mine), pick_lo = run, pick_hi = run;
+        int pick = -1;
+        for (int j0 = v0; j0 < v1; j0 += 4) {
+          float x[4], q[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int j = min(j0 + e, V - 1);
+            x[e] = p_row[j];
+            q[e] = eff == 0 ? q_row[j] : 0.f;
+          }
+          bool found = false;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const double val = j0 + e < v1 ? value(target(x[e]), q[e], eff) : 0.0;
+            if (!found && val > 0.0) {
+              pick = j0 + e;
+              pick_lo = run;
+              pick_hi = run + val;
+              found = pick_hi > s_t;
+            }
+            run += val;
+          }
+          if (found) break;
         }
-        found = over != 0;
-        run += __shfl_sync(0xffffffffu, inc, 31);
-      }
-      if (lane == 0) {
         p.next_token[b] = pick < 0 ? -1 : p.vocab_offset + pick;
         if (p.margins && pick >= 0)
           p.margins[(size_t)b * (K + 1) + K] = (float)(fmin(fabs(s_t - pick_lo), fabs(pick_hi - s_t)) / s_total);
@@ -627,7 +686,7 @@ __global__ void __launch_bounds__(kDecideThreads) decide_kernel(Workspace ws, De
 
 // Parts of a codebook: 2048 codes or more each, eight CTAs (the portable cluster) at most -- fewer where the images
 // alone fill the GPU.
-int launch_decide(const float* rows, bool logits, int n_tiles, int n_rows, const Workspace& ws, const DecideParams& p, bool pdl,
+int launch_decide(const float* rows, bool logits, int n_tiles, const Workspace& ws, const DecideParams& p, bool pdl,
                   cudaStream_t s) {
   int S = 1;
   while (S < 8 && p.vocab >= 2048 * 2 * S) S *= 2;
@@ -649,8 +708,8 @@ int launch_decide(const float* rows, bool logits, int n_tiles, int n_rows, const
   }
   cfg.attrs = attr;
   cfg.numAttrs = na;
-  const cudaError_t e = logits ? cudaLaunchKernelEx(&cfg, decide_kernel<true>, ws, p, rows, n_tiles, n_rows)
-                               : cudaLaunchKernelEx(&cfg, decide_kernel<false>, ws, p, rows, n_tiles, n_rows);
+  const cudaError_t e = logits ? cudaLaunchKernelEx(&cfg, decide_kernel<true>, ws, p, rows, n_tiles)
+                               : cudaLaunchKernelEx(&cfg, decide_kernel<false>, ws, p, rows, n_tiles);
   return e == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
 }
 

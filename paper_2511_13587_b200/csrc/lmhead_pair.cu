@@ -1,0 +1,331 @@
+// LM head of larger calls on CTA pairs (bf16): guided logits written out, softmax partials per 128 codes.
+//
+// A pair of SMs works on one 256-code x 256-column tile (tcgen05.mma.cta_group::2, M = 256): each CTA stages its own 128
+// codebook rows and HALF of the feature columns, and keeps the accumulators of its 128 codes.  With guidance the
+// columns are up to 128 decision rows, conditional (staged by rank 0) then unconditional (rank 1); without, up to 256
+// decision rows.  What bounds a one-CTA tile of this shape is the fill of shared memory from L2 (48 KB per k-block
+// for 128 codes, against ~60 B per clock and SM); the pair needs 32 KB, 64 B per clock at the full tensor rate.  The
+// accumulators are double-buffered (2 x 256 TMEM columns), so the epilogue of a tile runs under the next tile's MMAs.
+// Pairs stay resident and walk (tile, pass) units, passes first: the pairs that share codebook rows read them at
+// the same time and all but one find them in L2.
+// Roles: warp 0 loads (both CTAs; bytes are counted on rank 0's barriers), warp 1 of rank 0 issues the MMAs, warps 4-7
+// turn their 32 lanes' accumulators into logits and partials.
+#include <math_constants.h>
+
+#include "tc_common.cuh"
+#include "vvs_internal.cuh"
+
+namespace vvs {
+
+using namespace tc;
+
+namespace {
+
+constexpr int kThreads = 256;
+constexpr int kMaxStages = 6;
+constexpr int kChunk = 64;            // decision rows per epilogue step
+constexpr int kLd = 129;              // padded row of the logit tile
+constexpr uint32_t kBlockK = 64;
+constexpr uint32_t kABytes = 128 * kBlockK * 2;
+// k-blocks per pipeline stage: the issuing thread pays a wait and a commit (~270 cycles) per stage against 64 cycles
+// per MMA, and a k-block's four MMAs run 512 cycles at full width
+constexpr uint32_t kSub = 2;
+
+struct Params {
+  int v, bt, n_cfg, nd, passes, units, kb_total, stages /* of kSub k-blocks */, n_tiles;    // nd: decision rows per pass (padded)
+  uint32_t b_rows;                    // feature rows staged by a CTA
+  float cfg_scale, inv_temp;
+  float* part_m; float* part_s;       // [bt][n_tiles], tiles of 128 codes
+  float* logits;                      // [bt][v]
+  int32_t* status;
+};
+
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// load into this CTA, bytes counted on a barrier of the pair (cluster address)
+__device__ __forceinline__ void tma_load_pair(void* dst, const CUtensorMap* m, uint32_t bar, int x, int y) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void mma_pair_k64(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
+#pragma unroll
+  for (uint32_t k = 0; k < 4; ++k) {
+    const uint64_t ad = ((uint64_t)kDescHiSw128 << 32) | (a_lo + 2 * k), bd = ((uint64_t)kDescHiSw128 << 32) | (b_lo + 2 * k);
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(tmem_d), "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate | k) : "memory");
+  }
+}
+// arrive on the same barrier of both CTAs once the MMAs issued so far have completed
+__device__ __forceinline__ void commit_pair(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+               ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+}
+__device__ __forceinline__ void arrive_remote(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool try_wait_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+  return ok != 0;
+}
+// bounded wait; gives up when another role of the CTA already did
+__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* status) {
+  for (uint32_t i = 0; i < kSpinLimit; ++i) {
+    if (try_wait_cluster(bar, parity)) return true;
+    if ((i & 1023u) == 1023u && *abort_flag) return false;
+  }
+  *abort_flag = 1;
+  atomicOr(status, VVS_DEV_TIMEOUT);
+  return false;
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], acc_full[2], acc_empty[2];
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int s_abort;
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = (int)(blockIdx.x & 1), pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
+  const uint32_t b_bytes = p.b_rows * kBlockK * 2u, stage_bytes = kSub * (kABytes + b_bytes);
+  float* sL = reinterpret_cast<float*>(smem + (size_t)p.stages * stage_bytes);      // [kChunk][kLd]
+
+  if (tid == 0) {
+    for (int i = 0; i < p.stages; ++i) {
+      mbar_init(&full_bar[i], 1);
+      mbar_init(&empty_bar[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&acc_full[i], 1);
+      mbar_init(&acc_empty[i], 8);                // four epilogue warps of each CTA
+    }
+    s_abort = 0;
+    fence_barrier_init();
+    tma_prefetch_desc(&tm_a);
+    tma_prefetch_desc(&tm_b);
+  }
+  if (warp == 2) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&tmem_slot)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  cluster_sync_all();                             // both CTAs' barriers are ready
+  const uint32_t tmem = tmem_slot;
+  pdl_launch_dependents();
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---- TMA producer (codebook rows of the first stages may be requested before the features exist) -------------
+      uint32_t stage = 0, par = 1, bar0[kMaxStages];
+      for (int i = 0; i < kMaxStages; ++i) bar0[i] = mapa(smem_u32(&full_bar[i]), 0);
+      int issued = 0;
+      bool ok = true, waited = false;
+      auto load_a = [&](uint8_t* st, int i, int kb, int y) {
+#pragma unroll
+        for (uint32_t h = 0; h < kSub; ++h) tma_load_pair(st + h * kABytes, &tm_a, bar0[i], (kb * (int)kSub + (int)h) * (int)kBlockK, y);
+      };
+      auto load_b = [&](uint8_t* st, int i, int kb, int y) {
+#pragma unroll
+        for (uint32_t h = 0; h < kSub; ++h)
+          tma_load_pair(st + kSub * kABytes + h * b_bytes, &tm_b, bar0[i], (kb * (int)kSub + (int)h) * (int)kBlockK, y);
+      };
+      for (int u = pair; u < p.units && ok; u += n_pairs) {
+        const int tile = u / p.passes, row0 = (u - tile * p.passes) * p.nd;
+        const int ya = tile * 256 + rank * 128;
+        const int yb = p.n_cfg == 2 ? rank * p.bt + row0 : row0 + rank * (int)p.b_rows;
+        if (!waited) {
+          const int n_pre = p.kb_total < p.stages ? p.kb_total : p.stages;
+          for (int i = 0; i < n_pre; ++i) {
+            if (rank == 0) mbar_expect_tx(&full_bar[i], 2 * stage_bytes);
+            load_a(smem + (size_t)i * stage_bytes, i, i, ya);
+          }
+          pdl_wait();
+          waited = true;
+          for (int kb = 0; kb < p.kb_total; ++kb) {
+            uint8_t* st = smem + (size_t)stage * stage_bytes;
+            if (kb >= n_pre) {
+              if (!(ok = wait_or_abort(&empty_bar[stage], par, &s_abort, p.status))) break;
+              if (rank == 0) mbar_expect_tx(&full_bar[stage], 2 * stage_bytes);
+              load_a(st, stage, kb, ya);
+            }
+            load_b(st, stage, kb, yb);
+            ++issued;
+            if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1u; }
+          }
+          continue;
+        }
+        for (int kb = 0; kb < p.kb_total; ++kb) {
+          if (!(ok = wait_or_abort(&empty_bar[stage], par, &s_abort, p.status))) break;
+          uint8_t* st = smem + (size_t)stage * stage_bytes;
+          if (rank == 0) mbar_expect_tx(&full_bar[stage], 2 * stage_bytes);
+          load_a(st, stage, kb, ya);
+          load_b(st, stage, kb, yb);
+          ++issued;
+          if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1u; }
+        }
+      }
+      if (!ok && rank == 0) {                     // gave up: nothing may be in flight when the pair leaves (bounded)
+        for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
+          for (uint32_t k = 0; k < kSpinLimit && !try_wait_cluster(&full_bar[i % p.stages], (i / p.stages) & 1); ++k) {}
+      }
+    }
+  } else if (warp == 1 && rank == 0) {
+    if (lane == 0) {
+      // ---- MMA issuer ------------------------------------------------------------------------------------------------
+      const uint32_t n_cols = p.n_cfg == 2 ? 2u * (uint32_t)p.nd : (uint32_t)p.nd;
+      const uint32_t idesc = idesc_bf16_f32(256, n_cols);
+      const uint32_t lo0 = desc_lo_sw128(smem_u32(smem)), stage_lo = stage_bytes >> 4;
+      uint32_t stage = 0, par = 0;
+      int it = 0;
+      bool ok = true;
+      for (int u = pair; u < p.units && ok; u += n_pairs, ++it) {
+        const uint32_t buf = it & 1, d = tmem + buf * 256u;
+        if (!(ok = wait_or_abort(&acc_empty[buf], ((it >> 1) & 1) ^ 1, &s_abort, p.status))) break;
+        tc_fence_after();
+        for (int kb = 0; kb < p.kb_total; ++kb) {
+          if (!(ok = wait_or_abort(&full_bar[stage], par, &s_abort, p.status))) break;
+          tc_fence_after();
+          const uint32_t a_lo = lo0 + stage * stage_lo;
+#pragma unroll
+          for (uint32_t h = 0; h < kSub; ++h)
+            mma_pair_k64(d, a_lo + h * (kABytes >> 4), a_lo + ((kSub * kABytes + h * b_bytes) >> 4), idesc, kb > 0 || h > 0);
+          commit_pair(&empty_bar[stage]);
+          if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1u; }
+        }
+        commit_pair(&acc_full[buf]);
+      }
+    }
+  } else if (warp >= 4) {
+    // ---- epilogue: thread = one code; logits out, then partials from a shared tile, two threads per decision row ------
+    const int e = tid - 128, q = warp - 4;
+    const uint32_t t_lane = (uint32_t)(q * 32) << 16;
+    const uint32_t empty0 = mapa(smem_u32(&acc_empty[0]), 0), empty1 = mapa(smem_u32(&acc_empty[1]), 0);
+    int it = 0;
+    pdl_wait();
+    for (int u = pair; u < p.units; u += n_pairs, ++it) {
+      const int tile = u / p.passes, row0 = (u - tile * p.passes) * p.nd, buf = it & 1;
+      const int nd = min(p.nd, p.bt - row0);
+      const int n = tile * 256 + rank * 128 + e, t128 = tile * 2 + rank;
+      const bool n_ok = n < p.v;
+      if (!wait_or_abort(&acc_full[buf], (it >> 1) & 1, &s_abort, p.status)) break;
+      tc_fence_after();
+      const uint32_t t_row = tmem + (uint32_t)buf * 256u + t_lane;
+      float* dst = p.logits + (size_t)row0 * p.v + n;
+      for (int c0 = 0; c0 < nd; c0 += kChunk) {
+        const int rows = min(kChunk, nd - c0);
+        for (int c = 0; c < rows; c += 16) {
+          float lc[16], lu[16];
+          tmem_ld16(t_row + c0 + c, lc);
+          if (p.n_cfg == 2) tmem_ld16(t_row + (uint32_t)p.nd + c0 + c, lu);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            if (c + j < rows) {
+              float l = lc[j];
+              if (p.n_cfg == 2) l = lu[j] + p.cfg_scale * (l - lu[j]);
+              l *= p.inv_temp;
+              sL[(c + j) * kLd + e] = n_ok ? l : -CUDART_INF_F;
+              if (n_ok) dst[(size_t)(c0 + c + j) * p.v] = l;
+            }
+          }
+        }
+        if (c0 + kChunk >= nd) {                  // the accumulator has been read: the next unit but one may have it
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) arrive_remote(buf ? empty1 : empty0);
+        }
+        named_bar_sync(1, 128);
+        if (t128 < p.n_tiles && (e >> 1) < rows) {
+          const float* row = sL + (e >> 1) * kLd + (e & 1) * 64;
+          float m0 = -CUDART_INF_F, m1 = m0, m2 = m0, m3 = m0;
+#pragma unroll 4
+          for (int i = 0; i < 64; i += 4) {
+            m0 = fmaxf(m0, row[i]); m1 = fmaxf(m1, row[i + 1]); m2 = fmaxf(m2, row[i + 2]); m3 = fmaxf(m3, row[i + 3]);
+          }
+          float mx = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
+          const unsigned mate = 3u << (lane & ~1);
+          mx = fmaxf(mx, __shfl_xor_sync(mate, mx, 1));
+          float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+          if (mx > -CUDART_INF_F) {
+#pragma unroll 4
+            for (int i = 0; i < 64; i += 4) {
+              s0 += expf(row[i] - mx); s1 += expf(row[i + 1] - mx); s2 += expf(row[i + 2] - mx); s3 += expf(row[i + 3] - mx);
+            }
+          }
+          float sum = (s0 + s1) + (s2 + s3);
+          sum += __shfl_xor_sync(mate, sum, 1);
+          if ((e & 1) == 0) {
+            const size_t at = (size_t)(row0 + c0 + (e >> 1)) * p.n_tiles + t128;
+            p.part_m[at] = mx;
+            p.part_s[at] = sum;
+          }
+        }
+        named_bar_sync(1, 128);                   // the tile is written again
+      }
+    }
+  }
+  __syncwarp();
+  pdl_wait();
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();                             // no CTA leaves while the pair's MMAs or signals may still reach it
+  tc_fence_after();
+  if (warp == 2) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+}
+
+int pass_rows(int bt, int n_cfg, int* passes) {
+  const int most = n_cfg == 2 ? 128 : 256, step = n_cfg == 2 ? 16 : 32;
+  const int n = (bt + most - 1) / most, per = (bt + n - 1) / n;
+  const int nd = (per + step - 1) / step * step;
+  *passes = (bt + nd - 1) / nd;
+  return nd;
+}
+
+}  // namespace
+
+bool lmhead_pair_applicable(const LmHeadArgs& a) {
+  return !a.row_mode && a.n_draft_max == 0 && a.logits_out && a.bt * a.n_cfg > 96;
+}
+
+int lmhead_pair_box_rows(int bt, int n_cfg) {
+  int passes;
+  const int nd = pass_rows(bt, n_cfg, &passes);
+  return n_cfg == 2 ? nd : nd / 2;
+}
+
+int launch_lmhead_pair(const LmHeadArgs& a, cudaStream_t s) {
+  Params p{};
+  p.v = a.v; p.bt = a.bt; p.n_cfg = a.n_cfg; p.nd = pass_rows(a.bt, a.n_cfg, &p.passes);
+  p.n_tiles = (a.v + 127) / 128;
+  p.units = (a.v + 255) / 256 * p.passes;
+  p.kb_total = (a.k + (int)(kSub * kBlockK) - 1) / (int)(kSub * kBlockK);
+  p.b_rows = (uint32_t)lmhead_pair_box_rows(a.bt, a.n_cfg);
+  p.cfg_scale = a.cfg_scale; p.inv_temp = a.inv_temp; p.part_m = a.part_m; p.part_s = a.part_s; p.logits = a.logits_out;
+  p.status = a.status;
+  const int stage_bytes = (int)(kSub * (kABytes + p.b_rows * kBlockK * 2)), tile_bytes = kChunk * kLd * 4;
+  p.stages = (224 * 1024 - tile_bytes) / stage_bytes;
+  if (p.stages > kMaxStages) p.stages = kMaxStages;
+  if (ensure_dynamic_smem(reinterpret_cast<const void*>(lmhead_pair_kernel), 225 * 1024) != cudaSuccess) return VVS_ERR_CUDA;
+  int pairs = a.n_sms / 2;
+  if (pairs > p.units) pairs = p.units;
+  return launch_kernel(lmhead_pair_kernel, dim3(2 * pairs), dim3(kThreads), (size_t)(p.stages * stage_bytes + tile_bytes + 1024), a.pdl,
+                       s, p, *a.tm_a, *a.tm_b) == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
+}
+
+}  // namespace vvs

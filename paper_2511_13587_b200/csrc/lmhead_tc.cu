@@ -38,7 +38,7 @@ struct LmParams {
   int n_cfg, nd_pad, passes, kb_total, stages;
   uint32_t tmem_cols;
   float cfg_scale, inv_temp;
-  float* part_m; float* part_s;     // [n_tiles, bt]
+  float* part_m; float* part_s; int n_tiles;   // [bt, n_tiles]
   float* logits_out;                // optional [bt, v]
   int32_t* status;
   // gathers
@@ -227,8 +227,8 @@ lmhead_tc_kernel(const LmParams p, const __grid_constant__ CUtensorMap tm_a, con
         float sum = 0.f;
         if (mx > -CUDART_INF_F)
           for (int i = 0; i < 128; ++i) sum += expf(row[i] - mx);
-        p.part_m[(size_t)tile * p.bt + row0 + tid] = mx;
-        p.part_s[(size_t)tile * p.bt + row0 + tid] = sum;
+        p.part_m[(size_t)(row0 + tid) * p.n_tiles + tile] = mx;
+        p.part_s[(size_t)(row0 + tid) * p.n_tiles + tile] = sum;
       }
       // ---- 3. logits of the drafted tokens and of their neighbours that live in this tile --------
       // One warp per (image, draft) pair of the pass; its lanes walk the draft's neighbour row (one
@@ -288,6 +288,7 @@ int launch_lmhead_tc(const LmHeadArgs& a, cudaStream_t s) {
   p.passes = (a.bt + 127) / 128;
   p.kb_total = (a.k + (int)kBlockK - 1) / (int)kBlockK;
   p.cfg_scale = a.cfg_scale; p.inv_temp = a.inv_temp;
+  p.n_tiles = (a.v + 127) / 128;
   p.part_m = a.part_m; p.part_s = a.part_s; p.logits_out = a.logits_out; p.status = a.status;
   p.rows_per_seq = a.rows_per_seq; p.first_row = a.first_row; p.n_draft_max = a.n_draft_max;
   p.vocab_offset = a.vocab_offset; p.relaxed = a.relaxed; p.nbr_k = a.nbr_k; p.kmax = a.kmax;

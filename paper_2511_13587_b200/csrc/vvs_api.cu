@@ -163,6 +163,16 @@ DecideParams decide_params(const vvs_ctx* ctx, int rows_per_seq, int first_row, 
   return p;
 }
 
+// The LM head kernel of a call: CTA pairs where they apply, else one CTA per codebook tile.  Encodes the descriptor of
+// the `m` feature rows into *tm.
+int launch_lmhead(LmHeadArgs& la, const void* hid, int m, CUtensorMap* tm, cudaStream_t s) {
+  const bool pair = lmhead_pair_applicable(la);
+  const int box = pair ? lmhead_pair_box_rows(la.bt, la.n_cfg) : lmhead_box_rows(la.bt);
+  if (make_tmap_bf16_2d(tm, hid, (uint64_t)m, (uint64_t)la.k, (uint32_t)box) != VVS_OK) return VVS_ERR_CUDA;
+  la.tm_b = tm;
+  return pair ? launch_lmhead_pair(la, s) : launch_lmhead_tc(la, s);
+}
+
 // LM head over the codebook rows, guidance, softmax statistics, decisions.  Generic path: the
 // per-sequence logits and the guided logits live in scratch.
 template <typename T>
@@ -181,11 +191,10 @@ int run_decisions(vvs_ctx* ctx, const T* hid, int rows_per_seq, int first_row, c
   if (ctx->tensor_core_path) {
     // LM head with guidance, softmax partials and gathers fused into its epilogue
     CUtensorMap tm_hid, tm_sel;
-    if (make_tmap_bf16_2d(&tm_hid, hid, (uint64_t)M, (uint64_t)md.d_model, (uint32_t)lmhead_box_rows(BT)) != VVS_OK ||
-        make_tmap_bf16_2d(&tm_sel, ws.sel_hid, (uint64_t)R, (uint64_t)md.d_model, (uint32_t)lmhead_box_rows(B)) != VVS_OK)
+    if (make_tmap_bf16_2d(&tm_sel, ws.sel_hid, (uint64_t)R, (uint64_t)md.d_model, (uint32_t)lmhead_box_rows(B)) != VVS_OK)
       return VVS_ERR_CUDA;
     LmHeadArgs la{};
-    la.v = V; la.k = md.d_model; la.bt = BT; la.n_cfg = C; la.tm_a = &ctx->lm_map; la.tm_b = &tm_hid;
+    la.v = V; la.k = md.d_model; la.bt = BT; la.n_cfg = C; la.tm_a = &ctx->lm_map;
     la.pdl = ctx->use_pdl; la.n_sms = ctx->n_sms; la.cfg_scale = a->cfg_scale; la.inv_temp = 1.f / a->temperature;
     // The guided logits are written out (they mostly stay in L2: 0.6 MB at 9 rows, 19 MB at 288 rows of 16384 codes) and
     // the decision kernel gathers and samples from them.  Only calls too large for the buffer recompute the sampled
@@ -199,10 +208,10 @@ int run_decisions(vvs_ctx* ctx, const T* hid, int rows_per_seq, int first_row, c
     la.nbr_k = p.nbr_k; la.kmax = p.kmax; la.drafts_ld = drafts_ld; la.drafts = drafts;
     la.row_ptr = p.row_ptr; la.col = p.col; la.l_tok = ws.l_tok; la.l_nbr = ws.l_nbr;
     int rc = VVS_OK;
-    VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_lmhead_tc(la, s));
+    VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_lmhead(la, hid, M, &tm_hid, s));
     if (rc != VVS_OK) return rc;
     if (fused) {
-      VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(lbuf, true, (V + 127) / 128, BT, ws, p, ctx->use_pdl, s));
+      VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(lbuf, true, (V + 127) / 128, ws, p, ctx->use_pdl, s));
       if (rc == VVS_OK && o->target_probs)
         VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(o->target_probs, ws, o->target_probs, BT, V, ctx->use_pdl, s));
       return rc != VVS_OK ? rc : cudaGetLastError() == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
@@ -235,7 +244,7 @@ int run_decisions(vvs_ctx* ctx, const T* hid, int rows_per_seq, int first_row, c
                                                 1.f / a->temperature, ctx->use_pdl, s));
   if (!p.adjusted) {
     int rc = VVS_OK;
-    VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(ws.logits, true, 1, BT, ws, p, ctx->use_pdl, s));
+    VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(ws.logits, true, 1, ws, p, ctx->use_pdl, s));
     if (rc == VVS_OK && o->target_probs)
       VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(ws.logits, ws, o->target_probs, BT, V, ctx->use_pdl, s));
     return rc != VVS_OK ? rc : cudaGetLastError() == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
@@ -293,10 +302,8 @@ int run_tree_decisions(vvs_ctx* ctx, const __nv_bfloat16* hid, const vvs_verify_
   const int B = a->n_images, C = a->n_cfg, R = B * C, Tn = a->n_forced + a->n_draft_max;
   const int M = R * Tn, V = md.vocab, BT = B * Tn;
   CUtensorMap tm_hid;
-  if (make_tmap_bf16_2d(&tm_hid, hid, (uint64_t)M, (uint64_t)md.d_model, (uint32_t)lmhead_box_rows(BT)) != VVS_OK)
-    return VVS_ERR_CUDA;
   LmHeadArgs la{};
-  la.v = V; la.k = md.d_model; la.bt = BT; la.n_cfg = C; la.tm_a = &ctx->lm_map; la.tm_b = &tm_hid;
+  la.v = V; la.k = md.d_model; la.bt = BT; la.n_cfg = C; la.tm_a = &ctx->lm_map;
   la.pdl = ctx->use_pdl; la.n_sms = ctx->n_sms; la.cfg_scale = a->cfg_scale; la.inv_temp = 1.f / a->temperature;
   la.part_m = ws.part_m; la.part_s = ws.part_s; la.logits_out = o->target_probs; la.status = ws.status;
   la.rows_per_seq = Tn; la.first_row = a->n_forced - 1; la.n_draft_max = 0;
@@ -304,7 +311,7 @@ int run_tree_decisions(vvs_ctx* ctx, const __nv_bfloat16* hid, const vvs_verify_
   la.drafts = a->block + a->n_forced; la.row_ptr = ctx->nbr_row_ptr; la.col = ctx->nbr_col;
   la.l_tok = ws.l_tok; la.l_nbr = ws.l_nbr;
   int rc = VVS_OK;
-  VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_lmhead_tc(la, s));
+  VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_lmhead(la, hid, M, &tm_hid, s));
   if (rc != VVS_OK) return rc;
   VVS_LAUNCH(VVS_PROF_OTHER, launch_finalize_stats(ws, (V + 127) / 128, BT, s));
   VVS_LAUNCH(VVS_PROF_OTHER, launch_probs_from_logits(o->target_probs, ws, o->target_probs, BT, V, ctx->use_pdl, s));
@@ -894,7 +901,7 @@ int vvs_decide(vvs_ctx* ctx, const float* target_probs, int32_t n_rows_per_seq, 
   DecideParams p = decide_params(ctx, n_rows_per_seq, first_row, drafts, a->n_draft_max, a, o, false);
   p.direct_probs = target_probs;
   if (!p.adjusted) {
-    VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(target_probs, false, 0, 0, ws, p, ctx->use_pdl, s));
+    VVS_LAUNCH(VVS_PROF_OTHER, rc = launch_decide(target_probs, false, 0, ws, p, ctx->use_pdl, s));
     return rc;
   }
   if (p.n_draft_max > 0) VVS_LAUNCH(VVS_PROF_OTHER, launch_gather_logits(target_probs, ws, p, s));

@@ -70,8 +70,8 @@ struct Workspace {
   void* hid = nullptr;       // [M, d]   T features when the caller does not ask for them
   float* logits_raw = nullptr;  // [M, V] fp32 per-sequence logits (generic path)
   float* logits = nullptr;      // [B*T, V] fp32 guided logits / temperature (generic path)
-  float* part_m = nullptr;   // [n_tiles, B*T] per-tile running max
-  float* part_s = nullptr;   // [n_tiles, B*T] per-tile sum of exp(l - max)
+  float* part_m = nullptr;   // [B*T, n_tiles] per-tile running max
+  float* part_s = nullptr;   // [B*T, n_tiles] per-tile sum of exp(l - max)
   float* stat_m = nullptr;   // [B*T] row max
   float* stat_inv = nullptr; // [B*T] 1 / sum exp(l - max)
   float* l_tok = nullptr;    // [B, K] guided logit of each drafted token
@@ -299,7 +299,7 @@ struct LmHeadArgs {
   bool pdl;
   int n_sms;                     // SMs of the device (0: 148)
   float cfg_scale, inv_temp;
-  float* part_m; float* part_s;  // [n_tiles, bt] softmax partials per 128-code tile
+  float* part_m; float* part_s;  // [bt, n_tiles] softmax partials per 128-code tile
   float* logits_out;             // optional [bt, v] guided logits
   int32_t* status;
   int rows_per_seq, first_row, n_draft_max, vocab_offset, relaxed, nbr_k, kmax, drafts_ld;
@@ -309,6 +309,10 @@ struct LmHeadArgs {
   const int32_t* sel_row; const float* stat_m; const float* stat_inv; float* p_row;
 };
 int lmhead_box_rows(int bt);
+// the same for larger calls on CTA pairs, lmhead_pair.cu (logits written out, no gathers)
+bool lmhead_pair_applicable(const LmHeadArgs& a);
+int lmhead_pair_box_rows(int bt, int n_cfg);       // box rows of tm_b
+int launch_lmhead_pair(const LmHeadArgs& a, cudaStream_t s);
 int launch_lmhead_tc(const LmHeadArgs& a, cudaStream_t s);
 void launch_gather_sel_rows(const void* hid, const int32_t* sel_row, void* out, int n_images, int n_cfg, int bt,
                             int d, cudaStream_t s);
@@ -421,7 +425,7 @@ void launch_probs_from_logits(const float* logits, const Workspace& ws, float* p
 void launch_select_p_row(const float* logits, const Workspace& ws, int n_images, int v, cudaStream_t s);
 void launch_adjust_target(const Workspace& ws, const DecideParams& p, cudaStream_t s);
 void launch_residual_mass(const Workspace& ws, const DecideParams& p, cudaStream_t s);
-int launch_decide(const float* rows, bool logits, int n_tiles, int n_rows, const Workspace& ws, const DecideParams& p, bool pdl,
+int launch_decide(const float* rows, bool logits, int n_tiles, const Workspace& ws, const DecideParams& p, bool pdl,
                   cudaStream_t s);
 void launch_sample(const Workspace& ws, const DecideParams& p, cudaStream_t s);
 

@@ -89,5 +89,5 @@ extern "C" int vvs_decide_noalloc(const float* target_probs, int32_t vocab, int3
   p.accept_len = o->accept_len; p.next_token = o->next_token;
   p.accept_mask = o->accept_mask; p.margins = o->margins;
 
-  return launch_decide(target_probs, false, 0, 0, ws, p, true, static_cast<cudaStream_t>(stream));
+  return launch_decide(target_probs, false, 0, ws, p, true, static_cast<cudaStream_t>(stream));
 }
