@@ -388,50 +388,35 @@ gemm_tc_kernel(const KernelParams p, const __grid_constant__ CUtensorMap tm_a,
 }
 
 // ---------------------------------------------------------------------------------------------
-// positions, validity, visibility and rotation tables of the block rows: the same for every
-// layer of a call.  Chain: row t sits at position fill + t and sees block rows 0..t.  Tree
-// (tree_parent given): row t sits at fill + depth(t) and sees its ancestors and itself; its K/V
-// still go to cache slot fill + t.
-__global__ void rope_table_kernel(const int32_t* __restrict__ cache_len, const float* __restrict__ inv_freq,
-                                  const int32_t* __restrict__ tree_parent, int n_images, int n_forced,
-                                  int32_t* __restrict__ slot_pos, int32_t* __restrict__ seq_order,
-                                  uint32_t* __restrict__ anc_mask,
-                                  float* __restrict__ rope_cos, float* __restrict__ rope_sin, int t_len, int hd,
-                                  int s_max, int rope_mode, int grid_w, int n_prefix, int32_t* status,
-                                  unsigned* clear_words, int n_clear) {
+// positions, validity, visibility and rotation tables of block row m: the same for every layer of a
+// call.  Chain: row t sits at position fill + t and sees block rows 0..t.  Tree (tree_parent given):
+// row t sits at fill + depth(t) and sees its ancestors and itself; its K/V still go to cache slot
+// fill + t.  One CTA per row.
+struct RopeTableParams {
+  const int32_t* cache_len; const float* inv_freq; const int32_t* tree_parent;
+  int n_images, n_forced;
+  int32_t* slot_pos; int32_t* seq_order; uint32_t* anc_mask; float* rope_cos; float* rope_sin;
+  int t_len, hd, s_max, rope_mode, grid_w, n_prefix;
+  int32_t* status;
+};
+__device__ __forceinline__ void rope_table_row(const RopeTableParams& p, int m) {
   __shared__ int s_depth;
-  const int m = blockIdx.x, r = m / t_len, t = m % t_len;
-  // the stage counters of the chain kernel that follows in the stream start from zero
-  if (blockIdx.x == 0) {
-    for (int i = threadIdx.x; i < n_clear; i += blockDim.x) clear_words[i] = 0u;
-    // sequences by descending fill level (ties by index): the row-batched attention starts its longest
-    // (sequence, head) items first, so that the short ones fill the tail of the grid
-    const int n_rows = gridDim.x / t_len;
-    for (int i = threadIdx.x; i < n_rows; i += blockDim.x) {
-      const int fi = cache_len[i];
-      int rank = 0;
-      for (int j = 0; j < n_rows; ++j) {
-        const int fj = cache_len[j];
-        rank += (fj > fi || (fj == fi && j < i)) ? 1 : 0;
-      }
-      seq_order[rank] = i;
-    }
-  }
-  const int fill = cache_len[r];
-  const bool ok = fill >= 0 && fill + t_len <= s_max;
-  if (!ok && threadIdx.x == 0) atomicOr(status, VVS_DEV_CACHE_OVERFLOW);
+  const int t_len = p.t_len, r = m / t_len, t = m % t_len;
+  const int fill = p.cache_len[r];
+  const bool ok = fill >= 0 && fill + t_len <= p.s_max;
+  if (!ok && threadIdx.x == 0) atomicOr(p.status, VVS_DEV_CACHE_OVERFLOW);
   if (threadIdx.x == 0) {
     int depth = t;
     uint32_t mask = t >= 31 ? 0xffffffffu : ((2u << t) - 1u);
-    if (tree_parent) {
-      const int32_t* par = tree_parent + (size_t)(r % n_images) * t_len;
+    if (p.tree_parent) {
+      const int32_t* par = p.tree_parent + (size_t)(r % p.n_images) * t_len;
       bool bad = false;
       depth = 0;
       mask = 1u << t;
       for (int c = t, steps = 0; c > 0 && steps < 32; ++steps) {
         const int q = par[c];
         // forced rows form a chain; a draft node hangs below the last forced row or a draft node
-        if (q < 0 || q >= c || (c < n_forced && q != c - 1) || (c >= n_forced && q < n_forced - 1)) {
+        if (q < 0 || q >= c || (c < p.n_forced && q != c - 1) || (c >= p.n_forced && q < p.n_forced - 1)) {
           bad = true;
           break;
         }
@@ -441,32 +426,103 @@ __global__ void rope_table_kernel(const int32_t* __restrict__ cache_len, const f
       }
       if (par[0] != -1) bad = true;
       if (bad) {
-        atomicOr(status, VVS_DEV_BAD_ARG);
+        atomicOr(p.status, VVS_DEV_BAD_ARG);
         depth = t;
         mask = t >= 31 ? 0xffffffffu : ((2u << t) - 1u);
       }
     }
     s_depth = depth;
-    slot_pos[m] = ok ? fill + t : -1;
-    anc_mask[m] = mask;
+    p.slot_pos[m] = ok ? fill + t : -1;
+    p.anc_mask[m] = mask;
   }
   __syncthreads();
   const int pos = fill + s_depth;
   float c_lo = 0.f, c_hi = 0.f;
-  if (rope_mode == VVS_ROPE_1D) {
+  if (p.rope_mode == VVS_ROPE_1D) {
     c_lo = c_hi = (float)pos;
-  } else if (rope_mode == VVS_ROPE_2D_GRID && pos >= n_prefix) {
-    const int n = pos - n_prefix;
-    c_lo = (float)(n / grid_w);
-    c_hi = (float)(n % grid_w);
+  } else if (p.rope_mode == VVS_ROPE_2D_GRID && pos >= p.n_prefix) {
+    const int n = pos - p.n_prefix;
+    c_lo = (float)(n / p.grid_w);
+    c_hi = (float)(n % p.grid_w);
   }
-  const int half = hd / 2;
+  const int half = p.hd / 2;
   for (int i = threadIdx.x; i < half; i += blockDim.x) {
     float sn, cs;
-    sincosf(((i < half / 2) ? c_lo : c_hi) * inv_freq[i], &sn, &cs);
-    rope_cos[(size_t)m * half + i] = cs;
-    rope_sin[(size_t)m * half + i] = sn;
+    sincosf(((i < half / 2) ? c_lo : c_hi) * p.inv_freq[i], &sn, &cs);
+    p.rope_cos[(size_t)m * half + i] = cs;
+    p.rope_sin[(size_t)m * half + i] = sn;
   }
+}
+// sequences by descending fill level (ties by index): the row-batched attention starts its longest
+// (sequence, head) items first, so that the short ones fill the tail of the grid
+__device__ __forceinline__ void rank_sequences(const RopeTableParams& p, int n_rows) {
+  for (int i = threadIdx.x; i < n_rows; i += blockDim.x) {
+    const int fi = p.cache_len[i];
+    int rank = 0;
+    for (int j = 0; j < n_rows; ++j) {
+      const int fj = p.cache_len[j];
+      rank += (fj > fi || (fj == fi && j < i)) ? 1 : 0;
+    }
+    p.seq_order[rank] = i;
+  }
+}
+
+__global__ void rope_table_kernel(const RopeTableParams p, unsigned* clear_words, int n_clear) {
+  if (blockIdx.x == 0) {
+    // the stage counters of the chain kernel that follows in the stream start from zero
+    for (int i = threadIdx.x; i < n_clear; i += blockDim.x) clear_words[i] = 0u;
+    rank_sequences(p, gridDim.x / p.t_len);
+  }
+  rope_table_row(p, blockIdx.x);
+}
+
+// Start of a step of the folded-epilogue path, one CTA per block row: tables; embedding row x, the first projection's
+// operand bf16(x * scale) and the row's sum of squares (RMSNorm is applied to the projections' sums).  Two dependent
+// round trips (token id, embedding row); everything it writes stays in L2.
+constexpr int kBeginThreads = 160;
+__global__ void __launch_bounds__(kBeginThreads) step_begin_kernel(const RopeTableParams p, int n_rows,
+                                                                   const __nv_bfloat16* __restrict__ tok_emb,
+                                                                   const int32_t* __restrict__ block,
+                                                                   const __nv_bfloat16* __restrict__ scale, float* __restrict__ x,
+                                                                   __nv_bfloat16* __restrict__ xg, float* __restrict__ ss, int d,
+                                                                   int tok_rows) {
+  __shared__ float red[kBeginThreads / 32];
+  const int m = blockIdx.x, t_len = p.t_len, r = m / t_len, t = m % t_len;
+  const int tok = block[(r % p.n_images) * t_len + t];
+  const bool ok = tok >= 0 && tok < tok_rows;
+  if (!ok && threadIdx.x == 0) atomicOr(p.status, VVS_DEV_BAD_TOKEN);
+  const uint4* src = reinterpret_cast<const uint4*>(tok_emb + (size_t)(ok ? tok : 0) * d);
+  float sq = 0.f;
+  for (int i = threadIdx.x; i < d / 8; i += kBeginThreads) {
+    const uint4 e = ok ? src[i] : make_uint4(0, 0, 0, 0), g = reinterpret_cast<const uint4*>(scale)[i];
+    const uint32_t ew[4] = {e.x, e.y, e.z, e.w}, gw[4] = {g.x, g.y, g.z, g.w};
+    float v[8];
+    uint32_t ow[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      v[2 * j] = __uint_as_float(ew[j] << 16);
+      v[2 * j + 1] = __uint_as_float(ew[j] & 0xffff0000u);
+      sq += v[2 * j] * v[2 * j] + v[2 * j + 1] * v[2 * j + 1];
+      const __nv_bfloat162 pk = __floats2bfloat162_rn(v[2 * j] * __uint_as_float(gw[j] << 16),
+                                                      v[2 * j + 1] * __uint_as_float(gw[j] & 0xffff0000u));
+      ow[j] = *reinterpret_cast<const uint32_t*>(&pk);
+    }
+    float4* xd = reinterpret_cast<float4*>(x + (size_t)m * d + i * 8);
+    xd[0] = make_float4(v[0], v[1], v[2], v[3]);
+    xd[1] = make_float4(v[4], v[5], v[6], v[7]);
+    reinterpret_cast<uint4*>(xg + (size_t)m * d)[i] = make_uint4(ow[0], ow[1], ow[2], ow[3]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float s = 0.f;
+    for (int w = 0; w < kBeginThreads / 32; ++w) s += red[w];
+    reinterpret_cast<float4*>(ss)[m] = make_float4(s, 0.f, 0.f, 0.f);
+  }
+  if (m == 0) rank_sequences(p, n_rows);
+  rope_table_row(p, m);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -623,13 +679,26 @@ int launch_gemm_tc(int epi, const GemmTcPlan& plan, const GemmTcArgs& g, cudaStr
   return e == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
 }
 
+static RopeTableParams rope_params(const int32_t* cache_len, const int32_t* tree_parent, int n_images, int n_forced,
+                                   const Workspace& ws, const vvs_model_desc& md, int t_len) {
+  return RopeTableParams{cache_len, ws.rope_inv_freq, tree_parent, n_images, n_forced, ws.slot_pos, ws.seq_order,
+                         ws.anc_mask, ws.rope_cos, ws.rope_sin, t_len, md.head_dim, md.s_max, md.rope_mode, md.rope_grid_w,
+                         md.n_prefix, ws.status};
+}
+
 void launch_rope_table(const int32_t* cache_len, const int32_t* tree_parent, int n_images, int n_forced,
                        const Workspace& ws, const vvs_model_desc& md, int n_rows, int t_len, cudaStream_t s,
                        unsigned* clear_words, int n_clear) {
-  rope_table_kernel<<<n_rows * t_len, 64, 0, s>>>(cache_len, ws.rope_inv_freq, tree_parent, n_images, n_forced,
-                                                  ws.slot_pos, ws.seq_order, ws.anc_mask, ws.rope_cos, ws.rope_sin, t_len,
-                                                  md.head_dim, md.s_max, md.rope_mode, md.rope_grid_w, md.n_prefix,
-                                                  ws.status, clear_words, n_clear);
+  rope_table_kernel<<<n_rows * t_len, 64, 0, s>>>(rope_params(cache_len, tree_parent, n_images, n_forced, ws, md, t_len),
+                                                  clear_words, n_clear);
+}
+
+void launch_step_begin(const int32_t* cache_len, const int32_t* tree_parent, const int32_t* block, int n_images, int n_forced,
+                       const __nv_bfloat16* tok_emb, const __nv_bfloat16* scale, const Workspace& ws,
+                       const vvs_model_desc& md, int n_rows, int t_len, cudaStream_t s) {
+  step_begin_kernel<<<n_rows * t_len, kBeginThreads, 0, s>>>(
+      rope_params(cache_len, tree_parent, n_images, n_forced, ws, md, t_len), n_rows, tok_emb, block, scale, ws.x,
+      static_cast<__nv_bfloat16*>(ws.xn), ws.ss_part, md.d_model, md.tok_rows);
 }
 
 }  // namespace vvs

@@ -322,9 +322,11 @@ int launch_lmhead_pair(const LmHeadArgs& a, cudaStream_t s) {
   p.stages = (224 * 1024 - tile_bytes) / stage_bytes;
   if (p.stages > kMaxStages) p.stages = kMaxStages;
   if (ensure_dynamic_smem(reinterpret_cast<const void*>(lmhead_pair_kernel), 225 * 1024) != cudaSuccess) return VVS_ERR_CUDA;
+  // (all of the SM's shared memory: the two CTAs of a pair wait for each other, so neither may find its tensor memory
+  // held by a CTA of another stream's kernel that waits in the same way)
   int pairs = a.n_sms / 2;
   if (pairs > p.units) pairs = p.units;
-  return launch_kernel(lmhead_pair_kernel, dim3(2 * pairs), dim3(kThreads), (size_t)(p.stages * stage_bytes + tile_bytes + 1024), a.pdl,
+  return launch_kernel(lmhead_pair_kernel, dim3(2 * pairs), dim3(kThreads), (size_t)225 * 1024, a.pdl,
                        s, p, *a.tm_a, *a.tm_b) == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
 }
 

@@ -47,6 +47,7 @@ size_t layout(const vvs_model_desc& d, Workspace& ws, char* base) {
       const size_t wide = 3 * dm > 2 * ff ? 3 * dm : 2 * ff;
       const size_t tiles = (wide + 127) / 128, passes = (M + 255) / 256;
       c.take(ws.slot_pos, M * 4);
+      c.take(ws.ss_part, (dm + 127) / 128 * 8 * M * 4);
       c.take(ws.seq_order, (size_t)d.max_rows * 4);
       c.take(ws.rope_cos, M * (size_t)(d.head_dim / 2) * 4);
       c.take(ws.rope_sin, M * (size_t)(d.head_dim / 2) * 4);
@@ -333,6 +334,89 @@ int run_tree_decisions(vvs_ctx* ctx, const __nv_bfloat16* hid, const vvs_verify_
   return cudaGetLastError() == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
 }
 
+// Final norm (= the features), then the decisions, of a bf16 step.
+int finish_verify_tc(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* o, __nv_bfloat16* hid, cudaStream_t s) {
+  const vvs_model_desc& md = ctx->desc;
+  const int Tn = a->n_forced + a->n_draft_max, M = a->n_images * a->n_cfg * Tn;
+  VVS_LAUNCH(VVS_PROF_OTHER, launch_rmsnorm_rows(ctx->ws.x, static_cast<const __nv_bfloat16*>(ctx->norm_f), hid, M,
+                                                 md.d_model, md.rms_eps, ctx->use_pdl, s));
+  if (cudaGetLastError() != cudaSuccess) return VVS_ERR_CUDA;
+  if (a->tree_parent) return run_tree_decisions(ctx, hid, a, o, s);
+  return run_decisions<__nv_bfloat16>(ctx, hid, Tn, a->n_forced - 1, a->block + a->n_forced, Tn, a, o, true, s);
+}
+
+// The folded projections pay from d_model 1024 on; below that a step is a few kernels of a few CTAs either way, and the
+// per-projection path has them measured and tested.
+bool folded_applicable(const vvs_ctx* ctx) { return !ctx->use_chain_kernels && ctx->desc.d_model >= 1024; }
+
+// bf16 contexts of wide models: five kernels per layer (proj_tc.cu, attention_block.cu), each a programmatic dependent of
+// the one before.  Every sum is taken in a fixed order, so a call repeats bit for bit.
+int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* o, cudaStream_t s) {
+  using T = __nv_bfloat16;
+  const vvs_model_desc& md = ctx->desc;
+  Workspace& ws = ctx->ws;
+  const int B = a->n_images, R = B * a->n_cfg, Tn = a->n_forced + a->n_draft_max;
+  const int M = R * Tn, d = md.d_model, ff = md.d_ff;
+  T* xn = static_cast<T*>(ws.xn);
+  T* attn = static_cast<T*>(ws.attn);
+  T* act = static_cast<T*>(ws.act);
+  const ProjPlan p_qkv = plan_proj(M, 3 * d, d, false, ctx->n_sms), p_o = plan_proj(M, d, d, false, ctx->n_sms);
+  const ProjPlan p_gu = plan_proj(M, ff, d, true, ctx->n_sms), p_down = plan_proj(M, d, ff, false, ctx->n_sms);
+  CUtensorMap tm_xq, tm_xg, tm_attn, tm_act;
+  if (make_tmap_bf16_2d(&tm_xq, xn, (uint64_t)M, (uint64_t)d, (uint32_t)p_qkv.nt) != VVS_OK ||
+      make_tmap_bf16_2d(&tm_xg, xn, (uint64_t)M, (uint64_t)d, (uint32_t)p_gu.nt) != VVS_OK ||
+      make_tmap_bf16_2d(&tm_attn, attn, (uint64_t)M, (uint64_t)d, (uint32_t)p_o.nt) != VVS_OK ||
+      make_tmap_bf16_2d(&tm_act, act, (uint64_t)M, (uint64_t)ff, (uint32_t)p_down.nt) != VVS_OK)
+    return VVS_ERR_CUDA;
+  ProjArgs g{};
+  g.m = M; g.status = ws.status; g.ss_in = g.ss_out = ws.ss_part; g.eps = md.rms_eps; g.x = ws.x; g.xg = xn;
+  g.d = d; g.q = static_cast<T*>(ws.q); g.kv_k = static_cast<T*>(a->kv_k); g.kv_v = static_cast<T*>(a->kv_v);
+  g.slot_pos = ws.slot_pos; g.rope_cos = ws.rope_cos; g.rope_sin = ws.rope_sin; g.n_heads = md.n_heads; g.hd = md.head_dim;
+  g.s_max = md.s_max; g.kv_rows = a->kv_rows; g.t_len = Tn; g.act = act; g.ff = ff;
+  AttentionBlockArgs at{};
+  at.q = g.q; at.kv_k = g.kv_k; at.kv_v = g.kv_v; at.cache_len = a->cache_len; at.anc_mask = ws.anc_mask;
+  at.seq_order = ws.seq_order; at.out = attn; at.status = ws.status; at.d = d; at.n_heads = md.n_heads; at.hd = md.head_dim;
+  at.s_max = md.s_max; at.kv_rows = a->kv_rows; at.t_len = Tn; at.n_rows = R; at.n_sms = ctx->n_sms; at.pdl = ctx->use_pdl;
+
+  VVS_LAUNCH(VVS_PROF_OTHER, launch_step_begin(a->cache_len, a->tree_parent, a->block, B, a->n_forced,
+                                               static_cast<const T*>(ctx->tok_emb), static_cast<const T*>(ctx->layers[0].norm1),
+                                               ws, md, R, Tn, s));
+  int rc = VVS_OK;
+  // Weights of the projection after next are requested into L2 when three layers fit there (XL shape, 39 MB per layer:
+  // 989 -> 977 us at 18 tokens, 1263 -> 1235 at 54); larger ones push each other out (101 MB: 1005 -> 1110 us; 405 MB:
+  // 3.11 -> 4.26 ms)
+  const size_t layer_bytes = ((size_t)4 * d + (size_t)3 * ff) * d * sizeof(T);
+  const bool prefetch = 3 * layer_bytes <= (size_t)ctx->l2_bytes;
+  for (int l = 0; l < md.n_layers && rc == VVS_OK; ++l) {
+    const LayerMaps& W = ctx->layer_maps[l];
+    const Layer& L = ctx->layers[l];
+    const Layer* next = l + 1 < md.n_layers ? &ctx->layers[l + 1] : nullptr;
+    auto ahead = [&](const void* w0, const void* w1, size_t rows, size_t cols) {
+      g.ahead[0] = prefetch ? w0 : nullptr; g.ahead[1] = prefetch ? w1 : nullptr; g.ahead_bytes = (uint32_t)(rows * cols * sizeof(T));
+    };
+    // (the first projection is an ordinary successor of the kernel that wrote the step's tables: the kernels behind it
+    // read those before their own waits)
+    g.n = 3 * d; g.tm_a = &W.w_qkv; g.tm_b = &tm_xq; g.layer = at.layer = l; g.ss_parts = l > 0 ? proj_ss_parts(p_down) : 4;
+    g.pdl = ctx->use_pdl && l > 0;
+    ahead(L.w_gate, L.w_up, ff, d);
+    VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_proj(PROJ_QKV, p_qkv, g, s));
+    g.pdl = ctx->use_pdl;
+    if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_ATTENTION, rc = launch_attention_block(at, s));
+    g.n = d; g.tm_a = &W.w_o; g.tm_b = &tm_attn; g.scale = static_cast<const T*>(ctx->layers[l].norm2);
+    ahead(L.w_down, nullptr, d, ff);
+    if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_proj(PROJ_ADD, p_o, g, s));
+    g.n = ff; g.tm_a = &W.w_gate; g.tm_a2 = &W.w_up; g.tm_b = &tm_xg; g.ss_parts = proj_ss_parts(p_o);
+    ahead(next ? next->w_qkv : nullptr, nullptr, 3 * d, d);
+    if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_proj(PROJ_GATEUP, p_gu, g, s));
+    g.n = d; g.tm_a = &W.w_down; g.tm_a2 = nullptr; g.tm_b = &tm_act;
+    g.scale = static_cast<const T*>(l + 1 < md.n_layers ? ctx->layers[l + 1].norm1 : ctx->norm_f);
+    ahead(next ? next->w_o : nullptr, nullptr, d, d);
+    if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_proj(PROJ_ADD, p_down, g, s));
+  }
+  if (rc != VVS_OK) return rc;
+  return finish_verify_tc(ctx, a, o, o->hidden ? static_cast<T*>(o->hidden) : static_cast<T*>(ws.hid), s);
+}
+
 // bf16 contexts: projections on the tensor cores (gemm_tc.cu), everything else as above.
 int run_verify_tc(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* o, cudaStream_t s) {
   using T = __nv_bfloat16;
@@ -541,7 +625,9 @@ int run_verify_tc(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* 
 }
 
 int enqueue_verify(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* o, cudaStream_t s) {
-  if (ctx->tensor_core_path) return run_verify_tc(ctx, a, o, s);
+  if (ctx->tensor_core_path) {
+    return folded_applicable(ctx) ? run_verify_folded(ctx, a, o, s) : run_verify_tc(ctx, a, o, s);
+  }
   return ctx->desc.dtype == VVS_DTYPE_BF16 ? run_verify<__nv_bfloat16>(ctx, a, o, s)
                                            : run_verify<float>(ctx, a, o, s);
 }
@@ -698,6 +784,7 @@ int vvs_create(const vvs_model_desc* desc, vvs_ctx** out) {
   if (cudaDeviceGetAttribute(&ctx->n_sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess ||
       ctx->n_sms < 1)
     ctx->n_sms = 148;
+  if (cudaDeviceGetAttribute(&ctx->l2_bytes, cudaDevAttrL2CacheSize, ctx->device) != cudaSuccess) ctx->l2_bytes = 0;
   if (ctx->tensor_core_path && desc->n_layers > 0 && chain_stream_configure() != VVS_OK) {
     cudaGetLastError();
     ctx->use_chain_kernels = false;

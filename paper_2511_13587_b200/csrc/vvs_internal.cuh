@@ -87,6 +87,7 @@ struct Workspace {
   float* rope_inv_freq = nullptr;  // [head_dim/2] angle per unit coordinate of each pair
   // tensor-core path
   int32_t* slot_pos = nullptr;   // [M] cache slot of each block row, -1 if its sequence overflows
+  float* ss_part = nullptr;      // [M][d / 16] partial sums of squares of the residual rows
   int32_t* seq_order = nullptr;  // [R] sequences by descending fill level (longest attention items first)
   uint32_t* anc_mask = nullptr;  // [M] bit j set: block row j of the same sequence is visible (ancestor or self)
   double* tree_res = nullptr;    // [2][max_rows, V] residuals of the tree walk (ping-pong)
@@ -177,6 +178,7 @@ struct vvs_ctx {
   vvs::ChainCtaPlan* cs_d_plan = nullptr;  // device copy of cs_plan.cta
   CUtensorMap lm_map;
   int n_sms = 148;
+  int l2_bytes = 0;
   // CUDA-graph replay of vvs_verify (one graph per distinct argument set, small LRU cache)
   bool use_graph = true;
   cudaStream_t capture_stream = nullptr;
@@ -260,6 +262,55 @@ int launch_gemm_tc(int epi, const GemmTcPlan& plan, const GemmTcArgs& g, cudaStr
 void launch_rope_table(const int32_t* cache_len, const int32_t* tree_parent, int n_images, int n_forced,
                        const Workspace& ws, const vvs_model_desc& md, int n_rows,
                        int t_len, cudaStream_t s, unsigned* clear_words = nullptr, int n_clear = 0);
+
+// Start of a step of the folded-epilogue path (one kernel): tables, longest-first order, embedding rows x,
+// xn = bf16(x * scale), sums of squares.
+void launch_step_begin(const int32_t* cache_len, const int32_t* tree_parent, const int32_t* block, int n_images, int n_forced,
+                       const __nv_bfloat16* tok_emb, const __nv_bfloat16* scale, const Workspace& ws,
+                       const vvs_model_desc& md, int n_rows, int t_len, cudaStream_t s);
+
+// ---- projections with folded epilogues, proj_tc.cu -----------------------------------------------
+enum { PROJ_QKV = 0, PROJ_ADD = 1, PROJ_GATEUP = 2 };
+struct ProjPlan {
+  int nt, passes, tiles, kb_total, splits, stages, alias, recv_off, smem_bytes, tmem_cols;
+};
+struct ProjArgs {
+  int m, n;                    // tokens, weight rows (per matrix)
+  const CUtensorMap* tm_a;     // weights [n, k]
+  const CUtensorMap* tm_a2;    // GATEUP: up
+  const CUtensorMap* tm_b;     // activations [m, k], box rows = plan.nt
+  bool pdl;
+  int32_t* status;
+  const float* ss_in;          // QKV, GATEUP: [m][ss_parts] partial sums of squares of the residual rows
+  int ss_parts;
+  float eps;
+  float* x;                    // ADD: residual [m, d], updated; xg = bf16(x * scale), ss_out [m][proj_ss_parts]
+  __nv_bfloat16* xg; const __nv_bfloat16* scale; float* ss_out;
+  int d;
+  __nv_bfloat16* q; __nv_bfloat16* kv_k; __nv_bfloat16* kv_v;   // QKV
+  const int32_t* slot_pos; const float* rope_cos; const float* rope_sin;
+  int n_heads, hd, s_max, layer, kv_rows, t_len;
+  __nv_bfloat16* act; int ff;  // GATEUP
+  const void* ahead[2]; uint32_t ahead_bytes;   // matrices of the projection after next (same size; null: none)
+};
+ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms);
+int proj_ss_parts(const ProjPlan& plan);     // partial sums per token an ADD projection writes (at most d / 16 rounded up to tiles)
+int launch_proj(int epi, const ProjPlan& plan, const ProjArgs& g, cudaStream_t s);
+
+// ---- block-vs-cache attention on rotated queries and appended keys, attention_block.cu ------------------
+struct AttentionBlockArgs {
+  const __nv_bfloat16* q;      // [M, d] rotated queries
+  const __nv_bfloat16* kv_k;   // cache [layers][kv_rows][heads][s_max][hd], the block's own rows appended
+  const __nv_bfloat16* kv_v;
+  const int32_t* cache_len;    // [R]
+  const uint32_t* anc_mask;    // [M] visible block rows per block row
+  const int32_t* seq_order;    // [R] the sequence CTA row y works on: longest caches first
+  __nv_bfloat16* out;          // [M, d]
+  int32_t* status;
+  int d, n_heads, hd, s_max, layer, kv_rows, t_len, n_rows, n_sms;
+  bool pdl;
+};
+int launch_attention_block(const AttentionBlockArgs& a, cudaStream_t s);
 
 // ---- tensor-core attention, attention_tc.cu ----------------------------------------------------------
 struct AttentionTcArgs {
