@@ -1,5 +1,6 @@
-// LM head with the decision epilogue fused in (bf16, tensor cores): logits over the codebook are
-// never written to global memory unless the caller asked for target_probs.
+// LM head with the decision's gathers fused in (bf16, tensor cores): for calls that want adjusted probabilities and for
+// those whose guided logits would not fit the workspace's buffer -- logits over the codebook are then written to global
+// memory only when the caller asked for target_probs.  Other calls take lmhead_few.cu or lmhead_pair.cu.
 //
 // Roles as in the projection GEMM: the 128 codebook rows of a tile sit on the MMA's M side, the
 // feature rows on N.  One pass covers up to 128 DECISION rows (image, block position); with

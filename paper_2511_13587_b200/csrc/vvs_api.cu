@@ -164,14 +164,14 @@ DecideParams decide_params(const vvs_ctx* ctx, int rows_per_seq, int first_row, 
   return p;
 }
 
-// The LM head kernel of a call: CTA pairs where they apply, else one CTA per codebook tile.  Encodes the descriptor of
-// the `m` feature rows into *tm.
+// The LM head kernel of a call that has its logits written out: one CTA per codebook tile for few feature rows, CTA pairs
+// for more; of any other call lmhead_tc.cu.  Encodes the descriptor of the `m` feature rows into *tm.
 int launch_lmhead(LmHeadArgs& la, const void* hid, int m, CUtensorMap* tm, cudaStream_t s) {
-  const bool pair = lmhead_pair_applicable(la);
+  const bool few = lmhead_few_applicable(la), pair = !few && lmhead_pair_applicable(la);
   const int box = pair ? lmhead_pair_box_rows(la.bt, la.n_cfg) : lmhead_box_rows(la.bt);
   if (make_tmap_bf16_2d(tm, hid, (uint64_t)m, (uint64_t)la.k, (uint32_t)box) != VVS_OK) return VVS_ERR_CUDA;
   la.tm_b = tm;
-  return pair ? launch_lmhead_pair(la, s) : launch_lmhead_tc(la, s);
+  return few ? launch_lmhead_few(la, s) : pair ? launch_lmhead_pair(la, s) : launch_lmhead_tc(la, s);
 }
 
 // LM head over the codebook rows, guidance, softmax statistics, decisions.  Generic path: the
@@ -200,7 +200,7 @@ int run_decisions(vvs_ctx* ctx, const T* hid, int rows_per_seq, int first_row, c
     // The guided logits are written out (they mostly stay in L2: 0.6 MB at 9 rows, 19 MB at 288 rows of 16384 codes) and
     // the decision kernel gathers and samples from them.  Only calls too large for the buffer recompute the sampled
     // rows by a second pass over the head and pick the gathered logits in its epilogue (which at 576 feature rows of
-    // a 4096-wide, 16384-code head with 64 neighbours took 278 us per call against X with the logits written).
+    // a 4096-wide, 16384-code head with 64 neighbours took 278 us per call against 154 with the logits written).
     float* lbuf = o->target_probs ? o->target_probs : (BT <= ws.logit_rows ? ws.logits_small : nullptr);
     const bool fused = lbuf && !p.adjusted;
     la.part_m = ws.part_m; la.part_s = ws.part_s; la.logits_out = lbuf; la.status = ws.status;

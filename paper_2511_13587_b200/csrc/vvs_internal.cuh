@@ -360,6 +360,9 @@ struct LmHeadArgs {
   const int32_t* sel_row; const float* stat_m; const float* stat_inv; float* p_row;
 };
 int lmhead_box_rows(int bt);
+// the same for few feature rows, lmhead_few.cu (logits written out, no gathers; tm_b box rows = lmhead_box_rows(bt))
+bool lmhead_few_applicable(const LmHeadArgs& a);
+int launch_lmhead_few(const LmHeadArgs& a, cudaStream_t s);
 // the same for larger calls on CTA pairs, lmhead_pair.cu (logits written out, no gathers)
 bool lmhead_pair_applicable(const LmHeadArgs& a);
 int lmhead_pair_box_rows(int bt, int n_cfg);       // box rows of tm_b
