@@ -30,7 +30,7 @@ using namespace tc;
 namespace {
 
 constexpr int kMaxStages = 12;
-constexpr int kThreads = 256;
+constexpr int kMaxThreads = 512;
 constexpr int kMaxTok = 128;              // tokens per pass
 constexpr uint32_t kTileRows = 128;       // weight rows per tile = MMA M
 constexpr uint32_t kBlockK = 64;          // bf16 elements per smem row = one 128-byte swizzle row
@@ -85,7 +85,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 }
 
 template <int EPI, bool SPLIT>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kMaxThreads)
 proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_a2,
                const __grid_constant__ CUtensorMap tm_b) {
   constexpr bool DUAL = EPI == PROJ_GATEUP;
@@ -100,7 +100,7 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
   __shared__ float s_rs[EPI == PROJ_ADD ? 1 : kMaxTok];            // 1/rms of the pass's tokens
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, n_threads = (int)blockDim.x;
   const int tile = blockIdx.x, rank = SPLIT ? (int)blockIdx.y : 0, S = SPLIT ? p.splits : 1;
   const int tok0 = (int)blockIdx.z * p.nt, ntok = min(p.nt, p.m - tok0), nq = (ntok + 3) >> 2;
   const int kb0 = (int)(((long long)rank * p.kb_total) / S);
@@ -135,9 +135,11 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
   pdl_launch_dependents();  // after this CTA holds its TMEM: a dependent grid cannot take it first
   if (SPLIT) cluster_arrive();              // this rank's barrier is ready for its peers' pushes
 
-  if (warp == 3 && p.ahead_bytes > 0) {
+  if (warp == n_threads / 32 - 1 && p.ahead_bytes > 0) {
     // This CTA's share of a later projection's weights, HBM -> L2: a ring a few stages deep covers the latency of L2, not
-    // that of HBM, and with some hundred tokens a tile's weights are read by several CTAs at once.
+    // that of HBM, and with some hundred tokens a tile's weights are read by several CTAs at once.  4 KB per request: the
+    // unit that moves them takes ~50 cycles for each (1 KB pieces: 961 -> 1055 us per step of the XL shape, 16 KB: 972); by
+    // the last warp, which has no token's 1/rms to find at up to 32 tokens (by the first of those that have: 967).
     const uint32_t n_cta = gridDim.x * gridDim.y * gridDim.z, cta = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     const uint32_t share = ((p.ahead_bytes + n_cta - 1) / n_cta + 4095u) & ~4095u, end = min((cta + 1) * share, p.ahead_bytes);
 #pragma unroll
@@ -201,7 +203,7 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
   // ---- 1/rms of the pass's tokens, while the MMAs run: a warp per token, eight tokens' loads in flight ---------------
   if (EPI != PROJ_ADD && warp >= 3) {
     const int n4 = p.ss_parts >> 2;
-    for (int t0 = (warp - 3) * 8; t0 < ntok; t0 += 40) {
+    for (int t0 = (warp - 3) * 8; t0 < ntok; t0 += 8 * (n_threads / 32 - 3)) {
       float ss[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       for (int i = lane; i < n4; i += 32) {
         float4 v[8];
@@ -238,7 +240,7 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
     for (int j = 0; j < 4; ++j) xo[j] = n < p.n && t + j < p.m ? p.x[(size_t)(t + j) * p.d + n] : 0.f;
   };
   if (SPLIT && EPI == PROJ_ADD && tid < items) {
-    load_x(tid);                                                   // (kThreads is a multiple of rpr: the row stays)
+    load_x(tid);                                                   // (n_threads is a multiple of rpr: the row stays)
     const int n = n0 + (tid & (rpr - 1));
     if (n < p.n) gsc = __bfloat162float(p.scale[n]);
   }
@@ -295,7 +297,7 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
     __syncthreads();                          // s_rs; every warp has passed the accumulator's barrier
     const bool odd = lane & 1;
 #pragma unroll 1
-    for (int c0 = (warp >> 2) * 16; c0 < ntok; c0 += 32) {
+    for (int c0 = (warp >> 2) * 16; c0 < ntok; c0 += n_threads / 8) {
       float y[16], z[16];
       tmem_ld16(t_row + (uint32_t)c0, y);
       if (DUAL || two) tmem_ld16(t_row + (uint32_t)(p.nt + c0), z);
@@ -348,7 +350,7 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
         }
         *reinterpret_cast<uint32_t*>(out + j * kOutLd) = pack_bf16(a, b);
       }
-      if (c0 + 32 < ntok) operands(c0 + 32);
+      if (c0 + n_threads / 8 < ntok) operands(c0 + n_threads / 8);
     }
     tc_fence_before();
     __syncthreads();
@@ -374,7 +376,7 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
     }
     const float inv_tl = EPI == PROJ_QKV ? 1.f / (float)p.t_len : 0.f;
 #pragma unroll 4
-    for (int t = tid >> 4; t < ntok; t += kThreads / 16) {
+    for (int t = tid >> 4; t < ntok; t += n_threads / 16) {
       const uint4 v = *reinterpret_cast<const uint4*>(smem + (size_t)t * kOutLd + c8 * 16);
       const int tok = tok0 + t;
       if (EPI == PROJ_QKV && s8 > 0) {
@@ -392,7 +394,7 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
     const uint32_t at = (uint32_t)((rank << log_r) + (row_t & (rpr - 1))) * 16u;        // inside a quad's [S][rpr]
     const bool self = owner == rank;
     const uint32_t recv_dst = mapa(smem_u32(recv) + at, (uint32_t)owner), bar_dst = mapa(smem_u32(&recv_bar), (uint32_t)owner);
-    for (int c0 = (warp >> 2) * 4; c0 < nq; c0 += 8) {
+    for (int c0 = (warp >> 2) * 4; c0 < nq; c0 += n_threads / 32) {
 #pragma unroll
       for (int a = 0; a < NACC; ++a) {
         float v[16], w[16];
@@ -437,7 +439,7 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
   const size_t kv_row = (size_t)p.n_heads * p.s_max;               // cache rows per sequence
   const size_t kv_base = EPI == PROJ_QKV ? (((size_t)p.layer * p.kv_rows * p.n_heads + h) * p.s_max) * p.hd + i2 : 0;
   const int items_up = (items + 31) & ~31;                         // whole warps: the shuffles below need their lanes
-  for (int idx = tid; idx < items_up; idx += kThreads) {
+  for (int idx = tid; idx < items_up; idx += n_threads) {
     const int quad = idx >> log_r, t_first = tok0 + quad * 4;
     const bool live = idx < items;
     float acc[NACC][4];
@@ -459,7 +461,7 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
         xn[j] = xo[j] + acc[0][j];
         sq[j] = live && n_ok && t_first + j < p.m ? xn[j] * xn[j] : 0.f;
       }
-      if (idx + kThreads < items) load_x(idx + kThreads);          // the next item's residual travels under this one
+      if (idx + n_threads < items) load_x(idx + n_threads);          // the next item's residual travels under this one
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int tok = t_first + j;
@@ -527,7 +529,7 @@ cudaError_t launch_epi(const ProjPlan& pl, const Params& kp, const ProjArgs& g, 
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(pl.tiles, pl.splits, pl.passes);
-  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.blockDim = dim3(pl.threads, 1, 1);
   cfg.dynamicSmemBytes = pl.smem_bytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
@@ -585,7 +587,7 @@ ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
       const int waves = (ctas + n_sms * per_sm - 1) / (n_sms * per_sm);
       const double fill = (kATileBytes * nacc + 2.0 * kBlockK * (nt < 32 ? 32 : nt)) / 55.0, issue = 280.0 * nacc;
       double t = kb * (fill > issue ? fill : issue);
-      t += sp > 1 ? 2000.0 + 60.0 * tok * nacc + 400.0 * ((tok + 3) / 4 * ((int)kTileRows / sp) / kThreads + 1) : 47.0 * tok;
+      t += sp > 1 ? 2000.0 + 60.0 * tok * nacc + 400.0 * ((tok + 3) / 4 * ((int)kTileRows / sp) / 256 + 1) : 47.0 * tok;
       t = t * waves + 1500.0 * (waves - 1);
       if (best < 0.0 || t < best) {
         best = t;
@@ -610,6 +612,10 @@ ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
   // lap ahead would find the other's unfinished phase
   if (!dual && stages < per_cta) stages = stages < 2 ? 2 : stages & ~1;
   if (alias && stages * stage_bytes + recv <= budget) alias = 0;
+  // Eight warps are two per scheduler, and an epilogue item (a row's four tokens: ~250 dependent instructions) then takes
+  // 0.9 us: from two items per thread on there are sixteen (XL shape, 288 tokens 2015 -> 1970 us per step, 54 tokens 1243
+  // -> 1224; 7B shape 3172 -> 3134).  With fewer, starting eight more warps only costs (18 tokens 958 -> 976).
+  pl.threads = (S > 1 ? pl.nt / 4 * (int)kTileRows / S : pl.nt * 8) > 256 ? kMaxThreads : 256;
   pl.stages = stages;
   pl.alias = alias;
   pl.recv_off = alias ? 0 : stages * stage_bytes;

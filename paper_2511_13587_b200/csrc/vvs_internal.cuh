@@ -272,7 +272,7 @@ void launch_step_begin(const int32_t* cache_len, const int32_t* tree_parent, con
 // ---- projections with folded epilogues, proj_tc.cu -----------------------------------------------
 enum { PROJ_QKV = 0, PROJ_ADD = 1, PROJ_GATEUP = 2 };
 struct ProjPlan {
-  int nt, passes, tiles, kb_total, splits, stages, alias, recv_off, smem_bytes, tmem_cols;
+  int nt, passes, tiles, kb_total, splits, stages, alias, recv_off, smem_bytes, tmem_cols, threads;
 };
 struct ProjArgs {
   int m, n;                    // tokens, weight rows (per matrix)
