@@ -67,21 +67,12 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
   constexpr int NC = HD / 64, NJ = HD / 8;
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ __align__(8) uint64_t x_bar;
-  const int h = blockIdx.x, r = a.seq_order[blockIdx.y];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, c = lane & 3;
   const int T = a.t_len, S = (int)gridDim.z, rank = (int)blockIdx.z;
-  const int fill = a.cache_len[r];
-  const bool ok = fill >= 0 && fill + T <= a.s_max;
-  const size_t row_base = ((size_t)(a.layer * a.kv_rows + r) * a.n_heads + h) * a.s_max;
-  const bf16* kp = a.kv_k + row_base * HD;
-  const bf16* vp = a.kv_v + row_base * HD;
   // warps are dealt to the m-tiles in groups when a warp holds one m-tile and the block has two
   const int groups = (NMT == 1 && T > 16) ? 2 : 1;
   const int wpg = W / groups, grp = warp / wpg, wg = warp - grp * wpg;
   const int first = rank * wpg + wg, stride = S * wpg;
-  const int n_keys = ok ? fill + T : 0;
-  const int n_old = ok ? fill >> 4 : 0;                       // slices that hold old keys only
-  const int n_slices = (n_keys + 15) >> 4;
   const uint32_t ring = tc::smem_u32(smem) + (uint32_t)(warp * D) * L::kSlice;
 
   if (S > 1) {
@@ -93,174 +84,193 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   }
-  auto request = [&](int i) {                                 // slice i of this warp into its ring slot
-    const int s = first + i * stride;
-    const uint32_t dst0 = ring + (uint32_t)(i % D) * L::kSlice;
-    const int rows = min(16, n_keys - s * 16);
-    constexpr int per_row = HD / 8;                           // 16-byte pieces
-#pragma unroll
-    for (int u = 0; u < 2 * 16 * per_row / 32; ++u) {
-      const int idx = lane + u * 32, which = idx / (16 * per_row), rem = idx - which * 16 * per_row;
-      const int key = rem / per_row, ch = rem - key * per_row;
-      if (key < rows)
-        cp_async16(dst0 + (uint32_t)(which * NC + (ch >> 3)) * 2048u + key * 128 + (((ch & 7) ^ (key & 7)) << 4),
-                   (which ? vp : kp) + (size_t)(s * 16 + key) * HD + ch * 8);
-    }
-  };
-#pragma unroll
-  for (int i = 0; i < D; ++i) {
-    if (first + i * stride < n_old) request(i);
-    cp_async_commit();
-  }
-  tc::pdl_launch_dependents();      // the projection after this kernel may start fetching its weights
-  uint32_t anc[NMT][2];
-#pragma unroll
-  for (int mi = 0; mi < NMT; ++mi)
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int t = (grp + mi) * 16 + g + 8 * i;
-      anc[mi][i] = t < T ? a.anc_mask[r * T + t] : 0u;
-    }
-  tc::pdl_wait();
-#pragma unroll
-  for (int i = 0; i < D; ++i) {
-    const int s = first + i * stride;
-    if (s >= n_old && s < n_slices) request(i);
-  }
-  cp_async_commit();
-  uint32_t qa[NMT][HD / 16][4];
-#pragma unroll
-  for (int mi = 0; mi < NMT; ++mi) {
-    const int t0 = (grp + mi) * 16 + g, t1 = t0 + 8;
-    const bf16* q0 = a.q + (size_t)(r * T + t0) * a.d + h * HD + 2 * c;
-    const bf16* q1 = q0 + (size_t)8 * a.d;
-#pragma unroll
-    for (int kk = 0; kk < HD / 16; ++kk) {
-      qa[mi][kk][0] = t0 < T ? __ldcg(reinterpret_cast<const unsigned*>(q0 + 16 * kk)) : 0u;
-      qa[mi][kk][1] = t1 < T ? __ldcg(reinterpret_cast<const unsigned*>(q1 + 16 * kk)) : 0u;
-      qa[mi][kk][2] = t0 < T ? __ldcg(reinterpret_cast<const unsigned*>(q0 + 16 * kk + 8)) : 0u;
-      qa[mi][kk][3] = t1 < T ? __ldcg(reinterpret_cast<const unsigned*>(q1 + 16 * kk + 8)) : 0u;
-    }
-  }
-  AttState<HD> st[NMT];
-#pragma unroll
-  for (int mi = 0; mi < NMT; ++mi) {
-    st[mi].m[0] = st[mi].m[1] = -CUDART_INF_F;
-    st[mi].l[0] = st[mi].l[1] = 0.f;
-#pragma unroll
-    for (int j = 0; j < NJ; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) st[mi].o[j][e] = 0.f;
-  }
-  const float sl2 = rsqrtf((float)HD) * 1.4426950408889634f;
-
+  const int n_items = a.n_heads * a.n_rows, G = (int)gridDim.x;
+  // More items than the GPU holds CTAs: the grid is one wave, and its CTAs walk the list forth and back (longest first).
 #pragma unroll 1
-  for (int i = 0; first + i * stride < n_slices; ++i) {
-    const int s = first + i * stride;
-    // groups so far: D before the wait, one after it, one per iteration; slice i is in one of the oldest i + 2 of them
-    // unless it was requested after the wait
-    if (s >= n_old) cp_async_wait<0>(); else cp_async_wait<D - 1>();
-    __syncwarp();
-    const uint32_t k_base = ring + (uint32_t)(i % D) * L::kSlice, v_base = k_base + NC * 2048u;
-    const int left = n_keys - s * 16, old = fill - s * 16;    // valid keys of the slice; old ones among them
-    const uint32_t vmem = left >= 16 ? 0xffffu : ((1u << left) - 1u);
-    const uint32_t vold = old >= 16 ? 0xffffu : old > 0 ? ((1u << old) - 1u) : 0u;
+  for (int k = 0;; ++k) {
+    const int item = k * G + ((k & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
+    if (item >= n_items) break;
+    const int h = item % a.n_heads, r = a.seq_order[item / a.n_heads];
+    const int fill = a.cache_len[r];
+    const bool ok = fill >= 0 && fill + T <= a.s_max;
+    const size_t row_base = ((size_t)(a.layer * a.kv_rows + r) * a.n_heads + h) * a.s_max;
+    const bf16* kp = a.kv_k + row_base * HD;
+    const bf16* vp = a.kv_v + row_base * HD;
+    const int n_keys = ok ? fill + T : 0;
+    const int n_old = ok ? fill >> 4 : 0;                       // slices that hold old keys only
+    const int n_slices = (n_keys + 15) >> 4;
+    if (k > 0) __syncthreads();                                 // the merge of the item before is done with the rings
+    auto request = [&](int i) {                                 // slice i of this warp into its ring slot
+      const int s = first + i * stride;
+      const uint32_t dst0 = ring + (uint32_t)(i % D) * L::kSlice;
+      const int rows = min(16, n_keys - s * 16);
+      constexpr int per_row = HD / 8;                           // 16-byte pieces
+#pragma unroll
+      for (int u = 0; u < 2 * 16 * per_row / 32; ++u) {
+        const int idx = lane + u * 32, which = idx / (16 * per_row), rem = idx - which * 16 * per_row;
+        const int key = rem / per_row, ch = rem - key * per_row;
+        if (key < rows)
+          cp_async16(dst0 + (uint32_t)(which * NC + (ch >> 3)) * 2048u + key * 128 + (((ch & 7) ^ (key & 7)) << 4),
+                     (which ? vp : kp) + (size_t)(s * 16 + key) * HD + ch * 8);
+      }
+    };
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      if (first + i * stride < n_old) request(i);
+      cp_async_commit();
+    }
+    if (k == 0) tc::pdl_launch_dependents();      // the projection after this kernel may start fetching its weights
+    uint32_t anc[NMT][2];
+#pragma unroll
+    for (int mi = 0; mi < NMT; ++mi)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int t = (grp + mi) * 16 + g + 8 * i;
+        anc[mi][i] = t < T ? a.anc_mask[r * T + t] : 0u;
+      }
+    if (k == 0) tc::pdl_wait();
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      const int s = first + i * stride;
+      if (s >= n_old && s < n_slices) request(i);
+    }
+    cp_async_commit();
+    uint32_t qa[NMT][HD / 16][4];
 #pragma unroll
     for (int mi = 0; mi < NMT; ++mi) {
-      uint32_t vis[2];
+      const int t0 = (grp + mi) * 16 + g, t1 = t0 + 8;
+      const bf16* q0 = a.q + (size_t)(r * T + t0) * a.d + h * HD + 2 * c;
+      const bf16* q1 = q0 + (size_t)8 * a.d;
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const uint32_t own = old >= 16 ? 0u : old >= 0 ? anc[mi][e] << old : anc[mi][e] >> (-old);
-        vis[e] = (vold | own) & vmem;
+      for (int kk = 0; kk < HD / 16; ++kk) {
+        qa[mi][kk][0] = t0 < T ? __ldcg(reinterpret_cast<const unsigned*>(q0 + 16 * kk)) : 0u;
+        qa[mi][kk][1] = t1 < T ? __ldcg(reinterpret_cast<const unsigned*>(q1 + 16 * kk)) : 0u;
+        qa[mi][kk][2] = t0 < T ? __ldcg(reinterpret_cast<const unsigned*>(q0 + 16 * kk + 8)) : 0u;
+        qa[mi][kk][3] = t1 < T ? __ldcg(reinterpret_cast<const unsigned*>(q1 + 16 * kk + 8)) : 0u;
       }
-      att_slice<HD>(st[mi], qa[mi], k_base, v_base, 2048u, 0, lane, sl2, vis, vmem);
     }
-    __syncwarp();                                             // every lane is done with the ring slot
-    if (first + (i + D) * stride < n_slices) request(i + D);
-    cp_async_commit();
-  }
-  cp_async_wait<0>();
-  // ---- merge: every warp leaves (max, normaliser, output) of its rows, the CTA folds them in warp order --
-  __syncthreads();                                            // the rings have drained everywhere
-  float* s_o = reinterpret_cast<float*>(smem);                // [W][NMT * 16][kLd]
-  float* s_ml = s_o + W * NMT * 16 * L::kLd;                  // [W][NMT * 16][2]
+    AttState<HD> st[NMT];
 #pragma unroll
-  for (int mi = 0; mi < NMT; ++mi)
+    for (int mi = 0; mi < NMT; ++mi) {
+      st[mi].m[0] = st[mi].m[1] = -CUDART_INF_F;
+      st[mi].l[0] = st[mi].l[1] = 0.f;
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int row = mi * 16 + g + 8 * i;
-      float l = st[mi].l[i];
-      l += __shfl_xor_sync(0xffffffffu, l, 1);
-      l += __shfl_xor_sync(0xffffffffu, l, 2);
-      if ((grp + mi) * 16 + g + 8 * i < T) {
-        float* dst = s_o + (size_t)(warp * NMT * 16 + row) * L::kLd + 2 * c;
+      for (int j = 0; j < NJ; ++j)
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) *reinterpret_cast<float2*>(dst + 8 * j) = make_float2(st[mi].o[j][2 * i], st[mi].o[j][2 * i + 1]);
-        if (c == 0) {
-          s_ml[(warp * NMT * 16 + row) * 2] = st[mi].m[i];
-          s_ml[(warp * NMT * 16 + row) * 2 + 1] = l;
+        for (int e = 0; e < 4; ++e) st[mi].o[j][e] = 0.f;
+    }
+    const float sl2 = rsqrtf((float)HD) * 1.4426950408889634f;
+
+#pragma unroll 1
+    for (int i = 0; first + i * stride < n_slices; ++i) {
+      const int s = first + i * stride;
+      // groups so far: D before the wait, one after it, one per iteration; slice i is in one of the oldest i + 2 of them
+      // unless it was requested after the wait
+      if (s >= n_old) cp_async_wait<0>(); else cp_async_wait<D - 1>();
+      __syncwarp();
+      const uint32_t k_base = ring + (uint32_t)(i % D) * L::kSlice, v_base = k_base + NC * 2048u;
+      const int left = n_keys - s * 16, old = fill - s * 16;    // valid keys of the slice; old ones among them
+      const uint32_t vmem = left >= 16 ? 0xffffu : ((1u << left) - 1u);
+      const uint32_t vold = old >= 16 ? 0xffffu : old > 0 ? ((1u << old) - 1u) : 0u;
+#pragma unroll
+      for (int mi = 0; mi < NMT; ++mi) {
+        uint32_t vis[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const uint32_t own = old >= 16 ? 0u : old >= 0 ? anc[mi][e] << old : anc[mi][e] >> (-old);
+          vis[e] = (vold | own) & vmem;
+        }
+        att_slice<HD>(st[mi], qa[mi], k_base, v_base, 2048u, 0, lane, sl2, vis, vmem);
+      }
+      __syncwarp();                                             // every lane is done with the ring slot
+      if (first + (i + D) * stride < n_slices) request(i + D);
+      cp_async_commit();
+    }
+    cp_async_wait<0>();
+    // ---- merge: every warp leaves (max, normaliser, output) of its rows, the CTA folds them in warp order --
+    __syncthreads();                                            // the rings have drained everywhere
+    float* s_o = reinterpret_cast<float*>(smem);                // [W][NMT * 16][kLd]
+    float* s_ml = s_o + W * NMT * 16 * L::kLd;                  // [W][NMT * 16][2]
+#pragma unroll
+    for (int mi = 0; mi < NMT; ++mi)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int row = mi * 16 + g + 8 * i;
+        float l = st[mi].l[i];
+        l += __shfl_xor_sync(0xffffffffu, l, 1);
+        l += __shfl_xor_sync(0xffffffffu, l, 2);
+        if ((grp + mi) * 16 + g + 8 * i < T) {
+          float* dst = s_o + (size_t)(warp * NMT * 16 + row) * L::kLd + 2 * c;
+#pragma unroll
+          for (int j = 0; j < NJ; ++j) *reinterpret_cast<float2*>(dst + 8 * j) = make_float2(st[mi].o[j][2 * i], st[mi].o[j][2 * i + 1]);
+          if (c == 0) {
+            s_ml[(warp * NMT * 16 + row) * 2] = st[mi].m[i];
+            s_ml[(warp * NMT * 16 + row) * 2 + 1] = l;
+          }
         }
       }
-    }
-  __syncthreads();
-  if (S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // rank 0's barrier is ready
-  float* xbuf = reinterpret_cast<float*>(smem + L::kMain);    // [S - 1][T][HD + 2]
-  const uint32_t x_bar0 = S > 1 ? mapa0(tc::smem_u32(&x_bar)) : 0u;
-  const uint32_t xbuf0 = S > 1 ? mapa0(tc::smem_u32(xbuf)) : 0u;
-  bool waited = S == 1;
-  for (int idx = tid; idx < T * (HD / 2); idx += 32 * W) {
-    const int t = idx / (HD / 2), cp = idx - t * (HD / 2);
-    const int grp_t = groups == 2 ? t >> 4 : 0, row = groups == 2 ? t & 15 : t;
-    const float* o_src = s_o + (size_t)(grp_t * wpg * NMT * 16 + row) * L::kLd + 2 * cp;
-    const float* ml = s_ml + (grp_t * wpg * NMT * 16 + row) * 2;
-    float m = -CUDART_INF_F;
+    __syncthreads();
+    if (S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // rank 0's barrier is ready
+    float* xbuf = reinterpret_cast<float*>(smem + L::kMain);    // [S - 1][T][HD + 2]
+    const uint32_t x_bar0 = S > 1 ? mapa0(tc::smem_u32(&x_bar)) : 0u;
+    const uint32_t xbuf0 = S > 1 ? mapa0(tc::smem_u32(xbuf)) : 0u;
+    bool waited = S == 1;
+    for (int idx = tid; idx < T * (HD / 2); idx += 32 * W) {
+      const int t = idx / (HD / 2), cp = idx - t * (HD / 2);
+      const int grp_t = groups == 2 ? t >> 4 : 0, row = groups == 2 ? t & 15 : t;
+      const float* o_src = s_o + (size_t)(grp_t * wpg * NMT * 16 + row) * L::kLd + 2 * cp;
+      const float* ml = s_ml + (grp_t * wpg * NMT * 16 + row) * 2;
+      float m = -CUDART_INF_F;
 #pragma unroll 4
-    for (int w = 0; w < wpg; ++w) m = fmaxf(m, ml[w * NMT * 32]);
-    const float m_safe = m == -CUDART_INF_F ? 0.f : m;
-    float l = 0.f, o0 = 0.f, o1 = 0.f;
+      for (int w = 0; w < wpg; ++w) m = fmaxf(m, ml[w * NMT * 32]);
+      const float m_safe = m == -CUDART_INF_F ? 0.f : m;
+      float l = 0.f, o0 = 0.f, o1 = 0.f;
 #pragma unroll 4
-    for (int w = 0; w < wpg; ++w) {
-      const float f = ex2(ml[w * NMT * 32] - m_safe);
-      const float2 v = *reinterpret_cast<const float2*>(o_src + (size_t)w * NMT * 16 * L::kLd);
-      l += ml[w * NMT * 32 + 1] * f;
-      o0 += v.x * f;
-      o1 += v.y * f;
+      for (int w = 0; w < wpg; ++w) {
+        const float f = ex2(ml[w * NMT * 32] - m_safe);
+        const float2 v = *reinterpret_cast<const float2*>(o_src + (size_t)w * NMT * 16 * L::kLd);
+        l += ml[w * NMT * 32 + 1] * f;
+        o0 += v.x * f;
+        o1 += v.y * f;
+      }
+      if (rank > 0) {
+        const uint32_t dst = xbuf0 + (uint32_t)(((rank - 1) * T + t) * (HD + 2)) * 4u;
+        st_async2(dst + (uint32_t)cp * 8u, x_bar0, o0, o1);
+        if (cp == 0) st_async2(dst + HD * 4u, x_bar0, m, l);
+        continue;
+      }
+      if (!waited) {
+        // the peers' loops hold no unbounded wait; the limit only guards against a CTA that never runs
+        bool got = false;
+        for (uint32_t i = 0; i < 4u * tc::kSpinLimit && !got; ++i) got = try_wait_cluster(&x_bar);
+        if (!got) atomicOr(a.status, VVS_DEV_TIMEOUT);
+        waited = true;
+      }
+      for (int q = 0; q < S - 1; ++q) {
+        const float* x = xbuf + (size_t)(q * T + t) * (HD + 2);
+        const float mo = x[HD], lo = x[HD + 1];
+        const float m_new = fmaxf(m, mo), ms = m_new == -CUDART_INF_F ? 0.f : m_new;
+        const float aa = ex2(m - ms), bb = ex2(mo - ms);
+        m = m_new;
+        l = l * aa + lo * bb;
+        o0 = o0 * aa + x[2 * cp] * bb;
+        o1 = o1 * aa + x[2 * cp + 1] * bb;
+      }
+      const float inv = l > 0.f ? 1.f / l : 0.f;                // a sequence that failed its cache check gives zeros
+      *reinterpret_cast<uint32_t*>(a.out + (size_t)(r * T + t) * a.d + h * HD + 2 * cp) = pack2(o0 * inv, o1 * inv);
     }
-    if (rank > 0) {
-      const uint32_t dst = xbuf0 + (uint32_t)(((rank - 1) * T + t) * (HD + 2)) * 4u;
-      st_async2(dst + (uint32_t)cp * 8u, x_bar0, o0, o1);
-      if (cp == 0) st_async2(dst + HD * 4u, x_bar0, m, l);
-      continue;
-    }
-    if (!waited) {
-      // the peers' loops hold no unbounded wait; the limit only guards against a CTA that never runs
-      bool got = false;
-      for (uint32_t i = 0; i < 4u * tc::kSpinLimit && !got; ++i) got = try_wait_cluster(&x_bar);
-      if (!got) atomicOr(a.status, VVS_DEV_TIMEOUT);
-      waited = true;
-    }
-    for (int q = 0; q < S - 1; ++q) {
-      const float* x = xbuf + (size_t)(q * T + t) * (HD + 2);
-      const float mo = x[HD], lo = x[HD + 1];
-      const float m_new = fmaxf(m, mo), ms = m_new == -CUDART_INF_F ? 0.f : m_new;
-      const float aa = ex2(m - ms), bb = ex2(mo - ms);
-      m = m_new;
-      l = l * aa + lo * bb;
-      o0 = o0 * aa + x[2 * cp] * bb;
-      o1 = o1 * aa + x[2 * cp + 1] * bb;
-    }
-    const float inv = l > 0.f ? 1.f / l : 0.f;                // a sequence that failed its cache check gives zeros
-    *reinterpret_cast<uint32_t*>(a.out + (size_t)(r * T + t) * a.d + h * HD + 2 * cp) = pack2(o0 * inv, o1 * inv);
   }
 }
 
 template <int HD, int NMT, int W, int D>
-int launch_variant(const AttentionBlockArgs& a, int split, cudaStream_t s) {
+int launch_variant(const AttentionBlockArgs& a, int split, int per_sm, cudaStream_t s) {
   using L = Smem<HD, NMT, W, D>;
   const void* fn = reinterpret_cast<const void*>(attention_block_kernel<HD, NMT, W, D>);
   if (ensure_dynamic_smem(fn, L::bytes(kMaxT, split)) != cudaSuccess) return VVS_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.n_heads, a.n_rows, split);
+  int ctas = a.n_heads * a.n_rows;
+  if (split == 1 && ctas > per_sm * a.n_sms) ctas = per_sm * a.n_sms;
+  cfg.gridDim = dim3(ctas, 1, split);
   cfg.blockDim = dim3(32 * W, 1, 1);
   cfg.dynamicSmemBytes = L::bytes(a.t_len, split);
   cfg.stream = s;
@@ -283,6 +293,11 @@ int launch_variant(const AttentionBlockArgs& a, int split, cudaStream_t s) {
 
 }  // namespace
 
+// Warps per item by how many items there are: with few, one item's slices over many warps (XL shape, step of 18 tokens
+// with 16, 8 and 4 warps 962, 1004 and 1013 us; 54 tokens, two row groups of 8 warps 1184, of 4 warps 1286, four warps
+// with two m-tiles each 1272); with many, small CTAs (288 tokens, 640 items: 4 warps, three CTAs per SM 1.88 ms, 8 warps
+// 2.07 ms).  The item loop let the compiler keep addresses in registers: 160 instead of 128 a thread, three CTAs per SM
+// instead of four, and all the same 1.97 -> 1.88 ms (7B shape 3.13 -> 3.08 ms).
 int launch_attention_block(const AttentionBlockArgs& a, cudaStream_t s) {
   if (a.t_len > kMaxT) return VVS_ERR_SHAPE;
   const long long items = (long long)a.n_heads * a.n_rows;
@@ -290,12 +305,11 @@ int launch_attention_block(const AttentionBlockArgs& a, cudaStream_t s) {
   int split = 1;
   if (a.hd == 128) while (split < 4 && items * split * 2 <= a.n_sms && a.s_max >= 512 * split) split *= 2;
   if (a.hd == 64) {
-    if (a.t_len <= 16)
-      return few ? launch_variant<64, 1, 16, 2>(a, split, s) : some ? launch_variant<64, 1, 8, 3>(a, split, s)
-                                                                    : launch_variant<64, 1, 4, 3>(a, split, s);
-    return few ? launch_variant<64, 2, 8, 3>(a, split, s) : launch_variant<64, 2, 4, 3>(a, split, s);
+    if (few) return launch_variant<64, 1, 16, 2>(a, split, 1, s);
+    if (a.t_len > 16) return launch_variant<64, 2, 4, 3>(a, split, 2, s);
+    return some ? launch_variant<64, 1, 8, 3>(a, split, 2, s) : launch_variant<64, 1, 4, 3>(a, split, 3, s);
   }
-  if (a.hd == 128) return some ? launch_variant<128, 1, 8, 2>(a, split, s) : launch_variant<128, 1, 4, 3>(a, split, s);
+  if (a.hd == 128) return some ? launch_variant<128, 1, 8, 2>(a, split, 1, s) : launch_variant<128, 1, 4, 3>(a, split, 2, s);
   return VVS_ERR_SHAPE;
 }
 

@@ -25,7 +25,9 @@ WIDE128 = replace(B7, name="wide128", n_layers=2, d_model=1024, n_heads=8, d_ff=
     (WIDE64, 3, 2, 2, 15, [0, 47, 150]),                  # 102 tokens, 17 rows per sequence, an empty cache
     (WIDE64, 16, 2, 1, 9, list(range(3, 195, 12))),       # 320 tokens: several passes
     (WIDE128, 1, 2, 1, 4, [513]),                         # keys of a head over a cluster
-    (WIDE128, 5, 1, 3, 20, [5, 160, 333, 64, 677])])      # 115 tokens, 23 rows per sequence
+    (WIDE128, 5, 1, 3, 20, [5, 160, 333, 64, 677]),       # 115 tokens, 23 rows per sequence
+    (WIDE64, 7, 2, 2, 15, [3, 20, 37, 90, 111, 144, 170]),   # more (sequence, head) items than CTAs, 17 rows per sequence
+    (WIDE128, 19, 2, 1, 2, list(range(1, 96, 5)))])       # the same, heads of 128
 def test_folded_step(ms, n_images, n_cfg, n_forced, k, fills):
     case = H.build_case_independent(ms, 1700 + k, n_images, n_cfg, n_forced, k, fills, logit_std=0.6)
     run = H.GpuRunner(ms, case["w"], n_images * n_cfg, n_forced + k)
