@@ -560,35 +560,67 @@ int proj_ss_parts(const ProjPlan& pl) {
 //
 // Up to 20 MB of weights (a step's layers then fit in L2 together, see the prefetch) a projection is bound by the chain
 // of one CTA, one CTA per SM: k-blocks x the slower of filling shared memory (55 bytes per clock and SM, measured from
-// L2) and issuing (280 cycles per issuer and k-block), then the exchange (a fixed 2000 cycles, 60 per token and
-// accumulator) or, unsplit, the epilogue (47 per token); 1500 cycles per further wave.  The cheapest of all pass counts
-// and splits is taken.  At the XL shape (d 1280): 18 tokens 1 pass x 4 (QKV, gate/up) or 8 (O, down) slices, 972 us per
-// step against 1054 with as many small slices as make two CTAs per SM; 288 tokens unsplit passes of 64-80 tokens for QKV
-// and gate/up, 1.95 ms against 3.01 ms with the same rule; the estimate finds a combination within 1 % of the best of a
-// sweep at 18, 28, 54 and 288 tokens.
+// L2) and issuing (280 cycles per issuer and k-block), then the exchange (a fixed 2000 cycles, 25 per token, three times
+// that with two accumulators, 1500 for the barrier of one that lies over the stages, 400 per epilogue item) or, unsplit,
+// the epilogue (47 per token); 1500 cycles per further wave.  The cheapest of all pass counts and splits is taken.  At the
+// XL shape (d 1280): 18 tokens 1 pass x 4 (QKV, gate/up) or 8 (O, down) slices, 972 us per step against 1054 with as many
+// small slices as make two CTAs per SM; 288 tokens unsplit passes of 64-80 tokens for QKV and gate/up, 1.95 ms against
+// 3.01 ms with the same rule.  (With eight warps an exchanged token cost 60 cycles; 25 chooses a split QKV at 54 tokens,
+// 1183 -> 1152 us, and split O at 108 and 180, 1452 -> 1415 and 1615 -> 1551 us.)
 // A larger one is bound by HBM: two CTAs per SM keep more of the stream in flight (7B shape, d 4096, 18 tokens: 3.13 ms
 // per step against 3.29 with one), and a split deals the rows out evenly over the SMs.
+// Where several passes of 32 tokens or more give nearly every SM one CTA with 32 k-blocks or more to stream, a deep ring
+// for each does better still (d 2048, 72 tokens 1415 -> 1383 us per step, 126 tokens 1667 -> 1525).  Beyond 64 MB more
+// than the fewest passes would stream the weights from HBM again.
+// A cluster needs its CTAs' room inside one GPC: of 148 SMs 132 take clusters of four and 120 clusters of eight at one
+// CTA per SM, 284 and 264 of 296 at two.
 ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
   ProjPlan pl{};
   const int nacc = dual ? 2 : 1;
   pl.tiles = (n + (int)kTileRows - 1) / (int)kTileRows;
   pl.kb_total = (k + (int)kBlockK - 1) / (int)kBlockK;
-  const bool large = (size_t)n * k * 2 * nacc > ((size_t)20 << 20);
-  const int per_sm = large ? 2 : 1;
-  const int most = large ? 64 : kMaxTok;      // (64: two CTAs' accumulators and their shared memory, below, fit on an SM)
+  const size_t bytes = (size_t)n * k * 2 * nacc;
+  const bool large = bytes > ((size_t)20 << 20), huge = bytes > ((size_t)64 << 20);
+  const int most = large && !huge ? 64 : kMaxTok;      // (64: two CTAs' accumulators and their shared memory, below, fit on an SM)
+  auto room = [&](int sp, int per_sm) {
+    return per_sm == 1 ? (sp == 8 ? n_sms * 30 / 37 : sp == 4 ? n_sms * 33 / 37 : n_sms)
+                       : (sp == 8 ? n_sms * 66 / 37 : sp == 4 ? n_sms * 71 / 37 : 2 * n_sms);
+  };
+  auto ring = [&](int passes, int nt, int sp, int* alias) {
+    const int stage_bytes = (int)kATileBytes * nacc + nt * (int)kBlockK * 2, per_cta = (pl.kb_total + sp - 1) / sp;
+    const int recv = sp > 1 ? nacc * (nt / 4) * (int)kTileRows * 16 : 0;
+    // one CTA per SM: as deep as it gets if nothing is exchanged (XL shape, 288 tokens: 160 KB 1851, 200 KB 1839 us per step)
+    // or HBM is the bound, else 160 KB, which leave room for the attention kernel's first CTAs beside it; two: 108 KB
+    const int kb = pl.tiles * passes * sp > room(sp, 1) ? 108 : sp == 1 || large ? 200 : 160, budget = kb * 1024 - 1024;
+    *alias = recv > 24 * 1024 ? 1 : 0;        // the exchange over the drained stages (costs a cluster barrier)
+    int stages = (budget - (*alias ? 0 : recv)) / stage_bytes;
+    if (stages > kMaxStages) stages = kMaxStages;
+    if (stages > per_cta) stages = per_cta;
+    if (stages < 1) stages = 1;
+    // a ring that is used again: every stage must always belong to the same issuer (they take turns), or one that is a
+    // lap ahead would find the other's unfinished phase
+    if (!dual && stages < per_cta) stages = stages < 2 ? 2 : stages & ~1;
+    if (*alias && stages * stage_bytes + recv <= budget) *alias = 0;
+    return stages;
+  };
   double best = -1.0;
   int S = 1;
   for (int passes = (m + most - 1) / most; passes <= (m + 15) / 16; ++passes) {
     const int nt = ((m + passes - 1) / passes + 15) / 16 * 16;
     if (nt > most || (m + nt - 1) / nt != passes) continue;
+    if (huge && pl.passes > 0) break;         // (the weights do not stay in L2 from one pass to the next)
     const int tok = nt < m ? nt : m;
     for (int sp = 1; sp <= 8 && sp <= pl.kb_total; sp *= 2) {
-      const int ctas = pl.tiles * passes * sp, kb = (pl.kb_total + sp - 1) / sp;
-      const int waves = (ctas + n_sms * per_sm - 1) / (n_sms * per_sm);
+      const int ctas = pl.tiles * passes * sp, kb = (pl.kb_total + sp - 1) / sp, fit = room(sp, large && nt <= 64 ? 2 : 1);
+      const int waves = (ctas + fit - 1) / fit;
+      int alias;
+      ring(passes, nt, sp, &alias);
       const double fill = (kATileBytes * nacc + 2.0 * kBlockK * (nt < 32 ? 32 : nt)) / 55.0, issue = 280.0 * nacc;
       double t = kb * (fill > issue ? fill : issue);
-      t += sp > 1 ? 2000.0 + 60.0 * tok * nacc + 400.0 * ((tok + 3) / 4 * ((int)kTileRows / sp) / 256 + 1) : 47.0 * tok;
+      t += sp > 1 ? 2000.0 + 25.0 * tok * (dual ? 3 : 1) + 1500.0 * alias + 400.0 * ((tok + 3) / 4 * ((int)kTileRows / sp) / 256 + 1)
+                  : 47.0 * tok;
       t = t * waves + 1500.0 * (waves - 1);
+      if (large && !huge && kb >= 32 && nt >= 32 && ctas <= room(sp, 1) && ctas * 20 >= n_sms * 17) t = 0.0;
       if (best < 0.0 || t < best) {
         best = t;
         pl.passes = passes;
@@ -598,20 +630,10 @@ ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
     }
   }
   pl.splits = S;
+  int alias;
+  const int stages = ring(pl.passes, pl.nt, S, &alias);
   const int stage_bytes = (int)kATileBytes * nacc + pl.nt * (int)kBlockK * 2;
-  const int per_cta = (pl.kb_total + S - 1) / S;
   const int recv = S > 1 ? nacc * (pl.nt / 4) * (int)kTileRows * 16 : 0;
-  // one CTA per SM: 160 KB leave room for the attention kernel's first CTAs beside it; else two of 108 KB
-  const int budget = (pl.tiles * pl.passes * S <= n_sms ? 160 : 108) * 1024 - 1024;
-  int alias = recv > 24 * 1024 ? 1 : 0;       // the exchange over the drained stages (costs a cluster barrier)
-  int stages = (budget - (alias ? 0 : recv)) / stage_bytes;
-  if (stages > kMaxStages) stages = kMaxStages;
-  if (stages > per_cta) stages = per_cta;
-  if (stages < 1) stages = 1;
-  // a ring that is used again: every stage must always belong to the same issuer (they take turns), or one that is a
-  // lap ahead would find the other's unfinished phase
-  if (!dual && stages < per_cta) stages = stages < 2 ? 2 : stages & ~1;
-  if (alias && stages * stage_bytes + recv <= budget) alias = 0;
   // Eight warps are two per scheduler, and an epilogue item (a row's four tokens: ~250 dependent instructions) then takes
   // 0.9 us: from two items per thread on there are sixteen (XL shape, 288 tokens 2015 -> 1970 us per step, 54 tokens 1243
   // -> 1224; 7B shape 3172 -> 3134).  With fewer, starting eight more warps only costs (18 tokens 958 -> 976).
