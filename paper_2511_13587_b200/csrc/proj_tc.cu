@@ -592,15 +592,23 @@ ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
     // one CTA per SM: as deep as it gets if nothing is exchanged (XL shape, 288 tokens: 160 KB 1851, 200 KB 1839 us per step)
     // or HBM is the bound, else 160 KB, which leave room for the attention kernel's first CTAs beside it; two: 108 KB
     const int kb = pl.tiles * passes * sp > room(sp, 1) ? 108 : sp == 1 || large ? 200 : 160, budget = kb * 1024 - 1024;
-    *alias = recv > 24 * 1024 ? 1 : 0;        // the exchange over the drained stages (costs a cluster barrier)
-    int stages = (budget - (*alias ? 0 : recv)) / stage_bytes;
-    if (stages > kMaxStages) stages = kMaxStages;
-    if (stages > per_cta) stages = per_cta;
-    if (stages < 1) stages = 1;
     // a ring that is used again: every stage must always belong to the same issuer (they take turns), or one that is a
     // lap ahead would find the other's unfinished phase
-    if (!dual && stages < per_cta) stages = stages < 2 ? 2 : stages & ~1;
+    auto usable = [&](int room_for) {
+      int st = room_for < kMaxStages ? room_for : kMaxStages;
+      if (st < per_cta && !dual) st &= ~1;
+      return st < per_cta ? st : per_cta;
+    };
+    int stages = usable((budget - recv) / stage_bytes);
+    // too shallow beside the exchange's buffer: the exchange lies over the drained stages (costs a cluster barrier: XL shape,
+    // 54 tokens, down projection with 4 stages or with 6 and the barrier 1128, 1152 us per step)
+    *alias = stages < per_cta && stages < (dual ? 2 : 4);
+    if (*alias) stages = usable(budget / stage_bytes);
+    if (stages < 2 && per_cta > 1) stages = 2;
     if (*alias && stages * stage_bytes + recv <= budget) *alias = 0;
+    // one stage fewer than k-blocks where that is even: the next kernel's first CTAs then fit beside more of this one's
+    // (18 tokens 958 -> 940 us, 28 tokens 1004 -> 988; with 16 or 64 tokens a pass they do not, and it costs 1 %)
+    if (!dual && sp > 1 && nt == 32 && stages == per_cta && per_cta >= 5 && (per_cta & 1)) stages = per_cta - 1;
     return stages;
   };
   double best = -1.0;
