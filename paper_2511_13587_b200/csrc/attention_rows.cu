@@ -1,4 +1,4 @@
-// Block-vs-cache attention of the per-projection path (calls of more than 32 block tokens), with the
+// Block-vs-cache attention of the per-projection path (bf16 models of d_model below 1024), with the
 // rotation of q / k and the cache append of the block's own K / V rows folded in (Alg. 2 line 9: the
 // target forward over the block; Sec. 4.1: the call restores the block's KV entries).
 //

@@ -1,4 +1,5 @@
-// Weight-streaming projection GEMM for small token counts on the 5th-generation tensor cores.
+// Weight-streaming projection GEMM for small token counts on the 5th-generation tensor cores (bf16 models of d_model below
+// 1024 and the debug-switch paths; wider models take proj_tc.cu), and the kernels that begin a step.
 //
 //   out[tok, n] = sum_k act[tok, k] * w[n, k]          (w is [out_features, in_features])
 //
@@ -9,7 +10,7 @@
 // activation tiles are staged by TMA into 128-byte-swizzled shared memory, one elected thread
 // issues the MMAs, accumulators live in TMEM, and the four warps read them back (tcgen05.ld) for
 // a fused epilogue:
-//   ADD     out[tok, n] += acc                     (every projection of the default path: fp32 sums that
+//   ADD     out[tok, n] += acc                     (every projection but the debug-switch ones: fp32 sums that
 //                                                   the next kernel rotates / gates / normalises)
 //   ADD2    the same for two weight matrices sharing the activation tile (gate and up as one launch)
 //   QKV     rotate q, k pairs, write q and append k, v to the KV cache      (debug-switch path, 33-64 tokens)

@@ -243,28 +243,50 @@ void launch_rmsnorm_rows(const float* x, const __nv_bfloat16* scale, __nv_bfloat
 //   GATEUP  a = norm(x) * scale; silu(gate) * up
 //   ADD     residual x += acc
 //   STORE   plain product
+//   NORM_STORE  a = norm(x) * scale, which is also written out; plain product (the LM head after the last layer)
 // A small model's step is a chain of dependent kernels of a few microseconds each, so what counts is their number
 // (five per layer instead of ten) and the loads in a row inside one: weights are requested before
-// griddepcontrol.wait, the activation rows of all their pieces together.  (Tiny float32 step of 5 rows: 128 -> 66 us.)
+// griddepcontrol.wait, the activations of all rows of a piece together and a piece ahead (one row after the other they
+// were as many round trips to L2: 8-10 us a kernel).  In float32 1/rms multiplies the finished sums, so no pass over the
+// rows comes first, and the final norm is part of the LM head.  (Tiny float32 step of 5 rows: 128 -> 66 -> 49 us.)
 template <typename T>
 struct RowGemm {
   int m, n, k;                 // n: warps' worth of columns (pairs for QKV)
   const T* a;                  // ADD, STORE: activations [m, k]
-  const float* x_in;           // QKV, GATEUP: residual rows [m, k]
+  const float* x_in;           // QKV, GATEUP, NORM_STORE: residual rows [m, k]
   const T* scale; float eps;
   const T* w; const T* w2;     // GATEUP: gate, up
   float* c; int ldc;           // ADD, STORE
-  T* act;                      // GATEUP [m, n]
+  T* act;                      // GATEUP [m, n]; NORM_STORE: the normalised rows [m, k]
   T* q; T* kv_k; T* kv_v;      // QKV
   const float* inv_freq; const int32_t* cache_len; int32_t* status;
   int d, n_heads, hd, s_max, rope_mode, grid_w, n_prefix, layer, kv_rows, t_len;
 };
 
+// Sums of eight values over the warp: the lanes trade half of what they hold three times (9 shuffles instead of 40); lanes
+// 4 i .. 4 i + 3 get the sum of value i.
+__device__ __forceinline__ float sum_rows(float (&v)[8], int lane) {
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    const int o = 16 >> s, half = 4 >> s;
+    const bool up = lane & o;
+#pragma unroll
+    for (int j = 0; j < half; ++j) {
+      const float mine = up ? v[half + j] : v[j], theirs = up ? v[j] : v[half + j];
+      v[j] = mine + __shfl_xor_sync(0xffffffffu, theirs, o);
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  return v[0];
+}
+
 template <typename T, int EPI>
 __global__ void __launch_bounds__(128) row_gemm_kernel(const RowGemm<T> p) {
   constexpr int VEC = VecOf<T>::n, MT = 8;
-  constexpr bool NORM = EPI == ROW_QKV || EPI == ROW_GATEUP;
-  constexpr int NW = NORM ? 2 : 1, PF = NORM ? 4 : 8;           // weight rows per warp, pieces of them in flight
+  constexpr bool NORM = EPI == ROW_QKV || EPI == ROW_GATEUP || EPI == ROW_NORM_STORE;
+  constexpr int NW = EPI == ROW_QKV || EPI == ROW_GATEUP ? 2 : 1, PF = NORM ? 4 : 8;           // weight rows per warp, pieces of them in flight
+  constexpr bool FOLD = NORM && sizeof(T) == 4;                 // 1/rms multiplies the sums; nothing is rounded before them
   __shared__ float s_rs[MT];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int col = blockIdx.x * 4 + warp, m0 = blockIdx.y * MT, k = p.k;
@@ -285,7 +307,7 @@ __global__ void __launch_bounds__(128) row_gemm_kernel(const RowGemm<T> p) {
   fetch(0);
   grid_dep_launch();
   grid_dep_wait();
-  if (NORM) {
+  if (NORM && !FOLD) {
     for (int i = warp; i < MT; i += 4) {
       float ss = 0.f;
       if (m0 + i < p.m) {
@@ -301,58 +323,83 @@ __global__ void __launch_bounds__(128) row_gemm_kernel(const RowGemm<T> p) {
     }
     __syncthreads();
   }
-  if (!live) return;
-  float acc[NW][MT];
+  if (!live && EPI != ROW_NORM_STORE) return;
+  float acc[NW][MT], ss[MT];
 #pragma unroll
-  for (int r = 0; r < NW; ++r)
+  for (int i = 0; i < MT; ++i) {
+    ss[i] = 0.f;
 #pragma unroll
-    for (int i = 0; i < MT; ++i) acc[r][i] = 0.f;
+    for (int r = 0; r < NW; ++r) acc[r][i] = 0.f;
+  }
+  // A piece's activations of all rows are requested before the first is used, the next piece's with them (rows and columns
+  // past the end repeat the last ones; their weights are zero, their sums are not stored).
+  const int last_m = p.m - 1 - m0, last_k = k - VEC;
+  const T* a0 = NORM ? nullptr : p.a + (size_t)m0 * k;
+  const float* x0 = NORM ? p.x_in + (size_t)m0 * k : nullptr;
+  constexpr int AV = NORM ? VEC / 4 : 1;                        // 16-byte pieces of a row's activations
+  uint4 av4[2][MT][AV];
+  auto request = [&](int slot, int k0) {
+    const int kc = min(k0, last_k);
+#pragma unroll
+    for (int i = 0; i < MT; ++i)
+#pragma unroll
+      for (int q = 0; q < AV; ++q)
+        av4[slot][i][q] = NORM ? *reinterpret_cast<const uint4*>(x0 + (size_t)min(i, last_m) * k + kc + 4 * q)
+                               : *reinterpret_cast<const uint4*>(a0 + (size_t)min(i, last_m) * k + kc);
+  };
+  request(0, lane * VEC);
   for (int base = 0; base < k; base += PF * 32 * VEC) {
     if (base > 0) fetch(base);
 #pragma unroll
     for (int j = 0; j < PF; ++j) {
       const int k0 = base + (j * 32 + lane) * VEC;
-      if (k0 >= k) break;
+      if (base + j * 32 * VEC >= k) break;
+      request((j + 1) & 1, k0 + 32 * VEC);
       float wf[NW][VEC], sc[VEC];
 #pragma unroll
       for (int r = 0; r < NW; ++r) load_vec(reinterpret_cast<const T*>(&wv[r][j]), wf[r]);
-      if (NORM) load_vec(p.scale + k0, sc);
+      if (NORM) load_vec(p.scale + min(k0, last_k), sc);
 #pragma unroll
       for (int i = 0; i < MT; ++i) {
-        if (m0 + i < p.m) {
-          float av[VEC];
-          if (NORM) {
-            const float rs = s_rs[i];
+        float av[VEC];
+        if (NORM) {
+          const float rs = FOLD ? 1.f : s_rs[i];
 #pragma unroll
-            for (int e = 0; e < VEC; e += 4) load_vec(p.x_in + (size_t)(m0 + i) * k + k0 + e, av + e);
+          for (int q = 0; q < AV; ++q) load_vec(reinterpret_cast<const float*>(&av4[j & 1][i][q]), av + 4 * q);
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) av[e] = to_f(from_f<T>(av[e] * rs * sc[e]));
-          } else {
-            load_vec(p.a + (size_t)(m0 + i) * k + k0, av);
+          for (int e = 0; e < VEC; ++e) {
+            if (FOLD) ss[i] = k0 < k ? fmaf(av[e], av[e], ss[i]) : ss[i];
+            av[e] = FOLD ? av[e] * sc[e] : to_f(from_f<T>(av[e] * rs * sc[e]));
           }
-#pragma unroll
-          for (int r = 0; r < NW; ++r)
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) acc[r][i] = fmaf(av[e], wf[r][e], acc[r][i]);
+        } else {
+          load_vec(reinterpret_cast<const T*>(&av4[j & 1][i][0]), av);
         }
+#pragma unroll
+        for (int r = 0; r < NW; ++r)
+#pragma unroll
+          for (int e = 0; e < VEC; ++e) acc[r][i] = fmaf(av[e], wf[r][e], acc[r][i]);
       }
     }
   }
-  float v[NW];                                   // lane i keeps row m0 + i
+  float v[NW];                                   // lanes 4 i .. 4 i + 3 keep row m0 + i
 #pragma unroll
-  for (int r = 0; r < NW; ++r) {
-    v[r] = 0.f;
+  for (int r = 0; r < NW; ++r) v[r] = sum_rows(acc[r], lane);
+  const int row = m0 + (lane >> 2);
+  if (FOLD) {
+    const float rs = rsqrtf(sum_rows(ss, lane) / (float)k + p.eps);
 #pragma unroll
-    for (int i = 0; i < MT; ++i) {
-      const float s = warp_sum(acc[r][i]);
-      if (lane == i) v[r] = s;
+    for (int r = 0; r < NW; ++r) v[r] *= rs;
+    if (EPI == ROW_NORM_STORE && blockIdx.x == 0) {               // the normalised rows themselves, two per warp
+      for (int i = warp; i < MT && m0 + i < p.m; i += 4) {
+        const float rs_i = __shfl_sync(0xffffffffu, rs, 4 * i);
+        for (int j = lane; j < k; j += 32) p.act[(size_t)(m0 + i) * k + j] = from_f<T>(p.x_in[(size_t)(m0 + i) * k + j] * rs_i * to_f(p.scale[j]));
+      }
     }
   }
-  const int row = m0 + lane;
-  if (lane >= MT || row >= p.m) return;
+  if ((lane & 3) || row >= p.m || !live) return;
   if constexpr (EPI == ROW_ADD) {
     p.c[(size_t)row * p.ldc + col] += v[0];
-  } else if constexpr (EPI == ROW_STORE) {
+  } else if constexpr (EPI == ROW_STORE || EPI == ROW_NORM_STORE) {
     p.c[(size_t)row * p.ldc + col] = v[0];
   } else if constexpr (EPI == ROW_GATEUP) {
     p.act[(size_t)row * p.n + col] = from_f<T>(v[0] / (1.f + expf(-v[0])) * v[NW - 1]);
@@ -406,6 +453,13 @@ void launch_row_qkv(const float* x, const T* scale, float eps, const T* w, const
   p.layer = layer; p.kv_rows = kv_rows; p.t_len = t_len;
   launch_row_gemm<T>(ROW_QKV, p, pdl, s);
 }
+// hid = norm(x) * scale, c[m, n] = hid . w[n] (float32: bf16 contexts round hid before the product, see rmsnorm_kernel)
+void launch_row_norm_product(const float* x, const float* scale, float eps, const float* w, float* hid, float* c, int m, int n, int k,
+                             bool pdl, cudaStream_t s) {
+  RowGemm<float> p{};
+  p.m = m; p.n = n; p.k = k; p.x_in = x; p.scale = scale; p.eps = eps; p.w = w; p.act = hid; p.c = c; p.ldc = n;
+  launch_kernel(row_gemm_kernel<float, ROW_NORM_STORE>, dim3((n + 3) / 4, (m + 7) / 8), dim3(128), 0, pdl, s, p);
+}
 template <typename T>
 void launch_row_gateup(const float* x, const T* scale, float eps, const T* gate, const T* up, T* act, int m, int ff, int d, bool pdl,
                        cudaStream_t s) {
@@ -438,14 +492,25 @@ __global__ void __launch_bounds__(128) attention_kernel(const T* __restrict__ q,
   __shared__ float red[32];
   const int h = blockIdx.x, r = blockIdx.y, t = blockIdx.z, tid = threadIdx.x;
   grid_dep_launch();
-  grid_dep_wait();
   const int fill = cache_len[r];
   const size_t o = ((size_t)r * t_len + t) * d + (size_t)h * HD;
-  if (fill < 0 || fill + t_len > s_max) {
+  const size_t base = (((size_t)layer * kv_rows + r) * n_heads + h) * (size_t)s_max * HD;
+  const bool ok = fill >= 0 && fill + t_len <= s_max;
+  if (ok && ((reinterpret_cast<uintptr_t>(kv_k) | reinterpret_cast<uintptr_t>(kv_v)) & 127) == 0) {
+    // the cached rows into L1 while the projection before this kernel is still running (it writes slots fill .. only, and
+    // a row is whole lines)
+    constexpr int kLines = HD * (int)sizeof(T) / 128;
+    for (int i = tid; i < fill * kLines && i < 512; i += 128) {
+      const size_t at = base + (size_t)i * (128 / sizeof(T));
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(kv_k + at));
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(kv_v + at));
+    }
+  }
+  grid_dep_wait();
+  if (!ok) {
     for (int i = tid; i < HD; i += 128) out[o + i] = from_f<T>(0.f);
     return;
   }
-  const size_t base = (((size_t)layer * kv_rows + r) * n_heads + h) * (size_t)s_max * HD;
   const int nk = fill + t + 1;
   const float scale = rsqrtf((float)HD);
   // ---- scores: group g takes keys g, g + kGroups, ..; lane c of it columns [c VEC, ..) and the same in the second half

@@ -1,6 +1,7 @@
 // C ABI of the verify-step library: argument checks, scratch layout, launch sequences.
 #include <cmath>
 #include <cstdlib>
+#include <type_traits>
 #include <cstring>
 #include <new>
 
@@ -179,7 +180,7 @@ int launch_lmhead(LmHeadArgs& la, const void* hid, int m, CUtensorMap* tm, cudaS
 template <typename T>
 int run_decisions(vvs_ctx* ctx, const T* hid, int rows_per_seq, int first_row, const int32_t* drafts,
                   int drafts_ld, const vvs_verify_args* a, const vvs_verify_out* o, bool with_cache,
-                  cudaStream_t s) {
+                  cudaStream_t s, T* norm_to = nullptr) {
   const vvs_model_desc& md = ctx->desc;
   Workspace& ws = ctx->ws;
   const int B = a->n_images, C = a->n_cfg, R = B * C;
@@ -240,7 +241,12 @@ int run_decisions(vvs_ctx* ctx, const T* hid, int rows_per_seq, int first_row, c
     VVS_LAUNCH(VVS_PROF_OTHER, launch_sample(ws, p, s));
     return cudaGetLastError() == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
   }
-  VVS_LAUNCH(VVS_PROF_GEMM, launch_row_product<T>(hid, w_lm, ws.logits_raw, M, V, md.d_model, V, false, ctx->use_pdl, s));
+  if constexpr (std::is_same_v<T, float>) {
+    if (norm_to)
+      VVS_LAUNCH(VVS_PROF_GEMM, launch_row_norm_product(ws.x, static_cast<const T*>(ctx->norm_f), md.rms_eps, w_lm, norm_to, ws.logits_raw,
+                                                        M, V, md.d_model, ctx->use_pdl, s));
+  }
+  if (!norm_to) VVS_LAUNCH(VVS_PROF_GEMM, launch_row_product<T>(hid, w_lm, ws.logits_raw, M, V, md.d_model, V, false, ctx->use_pdl, s));
   VVS_LAUNCH(VVS_PROF_OTHER, launch_guide_stats(ws.logits_raw, ws.logits, ws.part_m, ws.part_s, B, C, rows_per_seq, V, a->cfg_scale,
                                                 1.f / a->temperature, ctx->use_pdl, s));
   if (!p.adjusted) {
@@ -289,9 +295,12 @@ int run_verify(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* o, 
                                                    static_cast<const T*>(L.w_up), act, M, ff, d, pdl, s));
     VVS_LAUNCH(VVS_PROF_GEMM, launch_row_product<T>(act, static_cast<const T*>(L.w_down), ws.x, M, d, ff, d, true, pdl, s));
   }
-  VVS_LAUNCH(VVS_PROF_OTHER, launch_rmsnorm<T>(ws.x, static_cast<const T*>(ctx->norm_f), hid, M, d, md.rms_eps, s, pdl));
+  // (float32: the final norm is part of the LM head)
+  if (!std::is_same_v<T, float>)
+    VVS_LAUNCH(VVS_PROF_OTHER, launch_rmsnorm<T>(ws.x, static_cast<const T*>(ctx->norm_f), hid, M, d, md.rms_eps, s, pdl));
   if (cudaGetLastError() != cudaSuccess) return VVS_ERR_CUDA;
-  return run_decisions<T>(ctx, hid, Tn, a->n_forced - 1, a->block + a->n_forced, Tn, a, o, true, s);
+  return run_decisions<T>(ctx, hid, Tn, a->n_forced - 1, a->block + a->n_forced, Tn, a, o, true, s,
+                          std::is_same_v<T, float> ? hid : nullptr);
 }
 
 // Tree calls: LM head with guidance over all block rows, probabilities written out, walk of the

@@ -212,7 +212,9 @@ void launch_embed(const T* tok_emb, const int32_t* block, float* x, int n_images
                   int t_len, int d, int tok_rows, int32_t* status, cudaStream_t s);
 template <typename T>
 void launch_rmsnorm(const float* x, const T* scale, T* out, int m, int d, float eps, cudaStream_t s, bool pdl = false);
-enum { ROW_QKV = 0, ROW_GATEUP = 1, ROW_ADD = 2, ROW_STORE = 3 };
+enum { ROW_QKV = 0, ROW_GATEUP = 1, ROW_ADD = 2, ROW_STORE = 3, ROW_NORM_STORE = 4 };
+void launch_row_norm_product(const float* x, const float* scale, float eps, const float* w, float* hid, float* c, int m, int n, int k,
+                             bool pdl, cudaStream_t s);
 template <typename T>
 void launch_row_qkv(const float* x, const T* scale, float eps, const T* w, const float* inv_freq, T* q, T* kv_k, T* kv_v,
                     const int32_t* cache_len, const vvs_model_desc& md, int layer, int kv_rows, int m, int t_len, int32_t* status,
