@@ -32,7 +32,8 @@ from vvs_synth.configs import CONFIGS, MODE_RELAXED  # noqa: E402
 # ncu capture summarised under profiles/.  Keyed by (workload, fixed-order sums); each entry names the
 # kernel sources the step runs and the first 16 hex digits of the SHA-256 over their concatenation when
 # the counters were taken: the line reports null, and says why, once any of them has changed.
-STEP_SOURCES = ("gemm_tc.cu", "attention_rows.cu", "kernels_generic.cu", "lmhead_tc.cu", "kernels_decide.cu")
+STEP_SOURCES = ("proj_tc.cu", "attention_block.cu", "gemm_tc.cu", "lmhead_few.cu", "lmhead_pair.cu", "kernels_generic.cu",
+                "kernels_decide.cu")
 NCU_CAPTURES = {
     (1, False): ("1748279beacd934c", 1.5709e+09, "profiles/verify_step_configs1_per_projection_launch_list_and_counters.txt"),
     (1, True): ("1748279beacd934c", 1.5459e+09, "profiles/verify_step_configs1_per_projection_launch_list_and_counters.txt"),
@@ -522,7 +523,7 @@ def run_ours(args) -> None:
                    "trials": len(S.trials), "draft": S.drafter,
                    "sums": "fixed order (bitwise repeatable)" if args.deterministic else "arrival order (split-K adds in L2)",
                    "kernels": "whole-chain kernels (previous generation, debug switch)" if args.chain_kernels
-                              else "per-projection kernels",
+                              else "five kernels per layer, epilogues folded in",
                    "timing": "median over `repeats` regions of `steps` steps each, every region bracketed by barrier + synchronize",
                    "l2": f"weights streamed per step ({alg['weights'] / 1e9:.2f} GB) exceed the 126 MB L2; no flush needed"
                          if alg["weights"] > 126e6 else "weights fit in L2: a latency case, not a bandwidth case",

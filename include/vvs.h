@@ -105,10 +105,11 @@ typedef struct vvs_model_desc {
                                 K / V rows and hence next_token): the K splits of a projection tile
                                 form a thread-block cluster that adds its partial tiles in rank order
                                 through distributed shared memory, each output written by one thread;
-                            0 = split-K partial sums are added in L2 in arrival order: faster (a
-                                quarter to a third per step; measured numbers in the repository's
-                                notes), the last bits of the logits differ from run to run, and a
-                                residual sample over many nearly equally likely codes need not repeat.
+                            0 = split-K partial sums may be added in L2 in arrival order; the last bits of
+                                the logits can then differ from run to run, and a residual sample over
+                                many nearly equally likely codes need not repeat.  Only models of d_model
+                                below 1024 are faster for it (by a quarter to a third per step); wider
+                                ones add in rank order either way.
                             float32 contexts are always repeatable. */
 } vvs_model_desc;
 
