@@ -9,9 +9,11 @@
 // (the chain's relaxed rule with p_res in the place of p); with the adjusted-residual flag a
 // rejection subtracts q from p_res after the pooled neighbours' mass has been moved onto x.
 //
-// One CTA per image; the walk is sequential over tree depth and siblings, each residual update
-// and the final inverse-CDF draw are block-wide passes over the V codes.  Sums run in a fixed
-// order, so a call repeats bit for bit on the same probabilities.
+// A cluster of S CTAs per image, each with a contiguous part of the codes; the walk is sequential over tree depth and
+// siblings and every CTA takes it, each residual update and the final inverse-CDF draw are passes over the parts whose
+// sums are exchanged through distributed shared memory and added in rank order, so a call repeats bit for bit on the same
+// probabilities.  What bounds it: the chain of tests and passes; one SM's float64 units and loads were what a pass of
+// 16384 codes took before (4 images, 26 nodes: 47 -> 25 us per call; 8 images of 32768 codes, relaxed: 60 -> 31).
 #include <math_constants.h>
 
 #include "vvs_internal.cuh"
@@ -72,17 +74,53 @@ __device__ double tw_block_sum(double v, double* s_warp) {
   return tot;
 }
 
+__device__ __forceinline__ void tw_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t tw_remote(const void* local, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(local)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ double tw_load_f64(const double* local, uint32_t rank) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(tw_remote(local, rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ int tw_load_s32(const int* local, uint32_t rank) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(tw_remote(local, rank)) : "memory");
+  return v;
+}
+// The CTAs' values at *slot: their sum and the sum of those before `rank`, in rank order.  Consecutive calls take two slots
+// in turn: a CTA that writes a slot again has met every reader of it at the barrier of the call between.  The barrier also
+// publishes what the CTAs have written to global memory.
+__device__ __forceinline__ double tw_exchange(double v, double* slot, int S, int rank, double* before) {
+  if (threadIdx.x == 0) *slot = v;
+  tw_cluster_sync();
+  double tot = 0.0;
+  for (int r = 0; r < S; ++r) {
+    if (r == rank) *before = tot;
+    tot += tw_load_f64(slot, (uint32_t)r);
+  }
+  return tot;
+}
+
 __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
-  __shared__ double s_warp[kTreeThreads / 32];
+  __shared__ double s_warp[kTreeThreads / 32], s_slot[2];
   __shared__ int s_child[32];
   __shared__ int s_n, s_pass, s_first, s_last, s_jend;
   __shared__ double s_mass;
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.y, S = (int)gridDim.x, rank = (int)blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int F = p.n_forced, K = p.n_draft_max, T = p.t_len, V = p.vocab;
   const int32_t* par = p.parent + (size_t)b * T;
   double* buf[2] = {p.res + (size_t)b * V, p.res + ((size_t)p.n_images + b) * V};
 
-  if (tid == 0) {
+  const int part = (V + S - 1) / S, r0 = min(V, rank * part), r1 = min(V, r0 + part);   // this CTA's codes
+  int turn = 0;
+  double before_part = 0.0;
+  if (rank == 0 && tid == 0) {
     for (int i = 0; i <= K; ++i)
       if (p.margins) p.margins[(size_t)b * (K + 1) + i] = CUDART_INF_F;
     for (int i = 0; i < K; ++i) {
@@ -121,7 +159,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
         if (!x_ok) {
           if (lane == 0) atomicOr(p.status, VVS_DEV_BAD_TOKEN);
         } else {
-          double px = first_round ? (double)prow[x] : buf[src][x] / z;
+          double px = first_round ? (double)prow[x] : __ldcg(buf[src] + x) / z;   // (another CTA's part, maybe)
           int j_end = 1;
           if (p.relaxed) {
             const int beg = p.row_ptr[x], len = p.row_ptr[x + 1] - beg;
@@ -131,12 +169,12 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
             px += tw_pooled_prefix(kk, (double)p.delta, lane, [&](int j) {
               const int cc = p.col[beg + j];
               if (cc < 0 || cc >= V) return 0.0;
-              return cur_res ? cur_res[cc] / z : (double)prow[cc]; }, &j_end);
+              return cur_res ? __ldcg(cur_res + cc) / z : (double)prow[cc]; }, &j_end);
           }
           const double qx = (double)qrow[x];
           const double ratio = qx > 0.0 ? fmin(1.0, px / qx) : (px > 0.0 ? 1.0 : 0.0);
           const double u = (double)p.uniforms[(size_t)b * (K + 1) + i];
-          if (lane == 0 && p.margins) p.margins[(size_t)b * (K + 1) + i] = (float)fabs(u - ratio);
+          if (rank == 0 && lane == 0 && p.margins) p.margins[(size_t)b * (K + 1) + i] = (float)fabs(u - ratio);
           pass = u < ratio ? 1 : 0;
           if (lane == 0) {
             s_mass = px;
@@ -147,7 +185,8 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
       }
       __syncthreads();
       const int pass = s_pass;
-      __syncthreads();
+      if (src >= 0) tw_cluster_sync();            // everyone has read the residual: it may be overwritten from here on
+      else __syncthreads();
       if (pass) {
         accepted = c;
         break;
@@ -157,14 +196,14 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
       double* dst = buf[src < 0 ? 0 : (src ^ 1)];
       double local = 0.0;
       if (first_round) {
-        for (int v = tid; v < V; v += kTreeThreads) {
+        for (int v = r0 + tid; v < r1; v += kTreeThreads) {
           const double r = (double)fmaxf(0.f, __fsub_rn(prow[v], qrow[v]));
           dst[v] = r;
           local += r;
         }
       } else {
         const double* cur_res = buf[src];
-        for (int v = tid; v < V; v += kTreeThreads) {
+        for (int v = r0 + tid; v < r1; v += kTreeThreads) {
           const double r = fmax(0.0, __dsub_rn(cur_res[v] / z, (double)qrow[v]));
           dst[v] = r;
           local += r;
@@ -178,17 +217,18 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
         const int j_end = s_jend;
         for (int j = 1 + tid; j < j_end; j += kTreeThreads) {
           const int cc = p.col[beg + j];
-          if (cc >= 0 && cc < V) dst[cc] = 0.0;
+          if (cc >= r0 && cc < r1) dst[cc] = 0.0;
         }
         __syncthreads();
-        if (tid == 0)
+        if (tid == 0 && x >= r0 && x < r1)
           dst[x] = first_round ? (double)fmaxf(0.f, __fsub_rn((float)s_mass, qrow[x]))
                                : fmax(0.0, __dsub_rn(s_mass, (double)qrow[x]));
         __syncthreads();
         local = 0.0;
-        for (int v = tid; v < V; v += kTreeThreads) local += dst[v];
+        for (int v = r0 + tid; v < r1; v += kTreeThreads) local += dst[v];
       }
-      const double z_new = tw_block_sum(local, s_warp);
+      const double z_new = tw_exchange(tw_block_sum(local, s_warp), &s_slot[turn], S, rank, &before_part);
+      turn ^= 1;
       if (z_new > 0.0) {                          // else p_res == q numerically: keep p_res
         src = src < 0 ? 0 : (src ^ 1);
         z = z_new;
@@ -196,7 +236,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
       }
     }
     if (accepted < 0) break;
-    if (tid == 0) {
+    if (rank == 0 && tid == 0) {
       p.accept_path[(size_t)b * K + n_acc] = accepted;
       if (p.accept_mask) p.accept_mask[(size_t)b * K + (accepted - F)] = 1;
     }
@@ -206,8 +246,8 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
   __syncthreads();
 
   // ---- inverse-CDF draw from the un-normalised source, ascending index ----
-  const int seg = (V + kTreeThreads - 1) / kTreeThreads;
-  const int v0 = tid * seg, v1 = min(V, v0 + seg);
+  const int seg = (part + kTreeThreads - 1) / kTreeThreads;
+  const int v0 = min(r1, r0 + tid * seg), v1 = min(r1, v0 + seg);
   const double* dsrc = src < 0 ? nullptr : buf[src];
   double local = 0.0;
   for (int v = v0; v < v1; ++v) local += dsrc ? dsrc[v] : (double)prow[v];
@@ -224,6 +264,8 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
     if (w < warp) before += t;
     total += t;
   }
+  total = tw_exchange(total, &s_slot[turn], S, rank, &before_part);
+  before += before_part;
   const double excl = before + incl - local;
   const double target = (double)p.uniforms[(size_t)b * (K + 1) + K] * total;
   {
@@ -239,7 +281,13 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
     if (last >= 0) atomicMax(&s_last, last);
   }
   __syncthreads();
-  const int pick = s_first != 0x7fffffff ? s_first : s_last;
+  tw_cluster_sync();
+  int first = 0x7fffffff, last = -1;
+  for (int r = 0; r < S; ++r) {
+    first = min(first, tw_load_s32(&s_first, (uint32_t)r));
+    last = max(last, tw_load_s32(&s_last, (uint32_t)r));
+  }
+  const int pick = first != 0x7fffffff ? first : last;
   if (pick >= v0 && pick < v1) {
     double c = excl;
     for (int v = v0; v < pick; ++v) c += dsrc ? dsrc[v] : (double)prow[v];
@@ -247,7 +295,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
     p.next_token[b] = p.vocab_offset + pick;
     if (p.margins) p.margins[(size_t)b * (K + 1) + K] = (float)(fmin(fabs(target - c), fabs(hi - target)) / total);
   }
-  if (tid == 0) {
+  if (rank == 0 && tid == 0) {
     if (pick < 0) {                               // an all-zero source: no token can be drawn
       p.next_token[b] = -1;
       atomicOr(p.status, VVS_DEV_BAD_ARG);
@@ -259,6 +307,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
       if (p.n_commit) p.n_commit[r] = F + n_acc;
     }
   }
+  tw_cluster_sync();                              // nobody leaves while its shared memory may be read
 }
 
 // K/V of the accepted nodes move from their block slots fill + node to fill + F + i (i-th
@@ -288,8 +337,22 @@ __global__ void tree_commit_kernel(T* __restrict__ kv_k, T* __restrict__ kv_v, c
 
 }  // namespace
 
+// Parts of 2048 codes or more, eight CTAs (the portable cluster) at most.
 void launch_tree_walk(const TreeParams& p, cudaStream_t s) {
-  tree_walk_kernel<<<p.n_images, kTreeThreads, 0, s>>>(p);
+  int S = 1;
+  while (S < 8 && p.vocab >= 2048 * 2 * S) S *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(S, p.n_images, 1);
+  cfg.blockDim = dim3(kTreeThreads, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = S;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, tree_walk_kernel, p);   // (the caller reads cudaGetLastError)
 }
 
 void launch_tree_commit(void* kv_k, void* kv_v, const int32_t* cache_len, const int32_t* accept_len,
