@@ -570,8 +570,8 @@ int proj_ss_parts(const ProjPlan& pl) {
 // A larger one is bound by HBM: two CTAs per SM keep more of the stream in flight (7B shape, d 4096, 18 tokens: 3.13 ms
 // per step against 3.29 with one), and a split deals the rows out evenly over the SMs.
 // Where several passes of 32 tokens or more give nearly every SM one CTA with 32 k-blocks or more to stream, a deep ring
-// for each does better still (d 2048, 72 tokens 1415 -> 1383 us per step, 126 tokens 1667 -> 1525).  Beyond 64 MB more
-// than the fewest passes would stream the weights from HBM again.
+// for each does better still (d 2048, 72 tokens 1415 -> 1383 us per step, 126 tokens 1667 -> 1525; 7B down projection,
+// 32 tiles x 4, 3049 -> 3028).  Beyond 64 MB more than the fewest passes would stream the weights from HBM again.
 // A cluster needs its CTAs' room inside one GPC: of 148 SMs 132 take clusters of four and 120 clusters of eight at one
 // CTA per SM, 284 and 264 of 296 at two.
 ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
@@ -628,7 +628,7 @@ ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
       t += sp > 1 ? 2000.0 + 25.0 * tok * (dual ? 3 : 1) + 1500.0 * alias + 400.0 * ((tok + 3) / 4 * ((int)kTileRows / sp) / 256 + 1)
                   : 47.0 * tok;
       t = t * waves + 1500.0 * (waves - 1);
-      if (large && !huge && kb >= 32 && nt >= 32 && ctas <= room(sp, 1) && ctas * 20 >= n_sms * 17) t = 0.0;
+      if (large && kb >= 32 && (huge || nt >= 32) && ctas <= room(sp, 1) && ctas * 20 >= n_sms * 17) t = 0.0;
       if (best < 0.0 || t < best) {
         best = t;
         pl.passes = passes;
