@@ -26,15 +26,9 @@
 namespace vvs {
 
 using namespace tc;
+using namespace proj;
 
 namespace {
-
-constexpr int kMaxStages = 12;
-constexpr int kMaxThreads = 512;
-constexpr int kMaxTok = 128;              // tokens per pass
-constexpr uint32_t kTileRows = 128;       // weight rows per tile = MMA M
-constexpr uint32_t kBlockK = 64;          // bf16 elements per smem row = one 128-byte swizzle row
-constexpr uint32_t kATileBytes = kTileRows * kBlockK * 2;
 
 struct Params {
   int m, n, nt, kb_total, splits, log_s, stages, alias;
@@ -550,116 +544,6 @@ cudaError_t launch_epi(const ProjPlan& pl, const Params& kp, const ProjArgs& g, 
 }
 
 }  // namespace
-
-int proj_ss_parts(const ProjPlan& pl) {
-  const int rpr = (int)kTileRows / pl.splits;
-  return pl.tiles * (int)kTileRows / (rpr < 32 ? rpr : 32);
-}
-
-// Token passes, K splits and ring of one projection.
-//
-// Up to 20 MB of weights (a step's layers then fit in L2 together, see the prefetch) a projection is bound by the chain
-// of one CTA, one CTA per SM: k-blocks x the slower of filling shared memory (55 bytes per clock and SM, measured from
-// L2) and issuing (280 cycles per issuer and k-block), then the exchange (a fixed 2000 cycles, 25 per token, three times
-// that with two accumulators, 1500 for the barrier of one that lies over the stages, 400 per epilogue item) or, unsplit,
-// the epilogue (47 per token); 1500 cycles per further wave.  The cheapest of all pass counts and splits is taken.  At the
-// XL shape (d 1280): 18 tokens 1 pass x 4 (QKV, gate/up) or 8 (O, down) slices, 972 us per step against 1054 with as many
-// small slices as make two CTAs per SM; 288 tokens unsplit passes of 64-80 tokens for QKV and gate/up, 1.95 ms against
-// 3.01 ms with the same rule.  (With eight warps an exchanged token cost 60 cycles; 25 chooses a split QKV at 54 tokens,
-// 1183 -> 1152 us, and split O at 108 and 180, 1452 -> 1415 and 1615 -> 1551 us.)
-// A larger one is bound by HBM: two CTAs per SM keep more of the stream in flight (7B shape, d 4096, 18 tokens: 3.13 ms
-// per step against 3.29 with one), and a split deals the rows out evenly over the SMs.
-// Where several passes of 32 tokens or more give nearly every SM one CTA with 32 k-blocks or more to stream, a deep ring
-// for each does better still (d 2048, 72 tokens 1415 -> 1383 us per step, 126 tokens 1667 -> 1525; 7B down projection,
-// 32 tiles x 4, 3049 -> 3028).  Beyond 64 MB more than the fewest passes would stream the weights from HBM again.
-// A cluster needs its CTAs' room inside one GPC: of 148 SMs 132 take clusters of four and 120 clusters of eight at one
-// CTA per SM, 284 and 264 of 296 at two.
-ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
-  ProjPlan pl{};
-  const int nacc = dual ? 2 : 1;
-  pl.tiles = (n + (int)kTileRows - 1) / (int)kTileRows;
-  pl.kb_total = (k + (int)kBlockK - 1) / (int)kBlockK;
-  const size_t bytes = (size_t)n * k * 2 * nacc;
-  const bool large = bytes > ((size_t)20 << 20), huge = bytes > ((size_t)64 << 20);
-  const int most = large && !huge ? 64 : kMaxTok;      // (64: two CTAs' accumulators and their shared memory, below, fit on an SM)
-  auto room = [&](int sp, int per_sm) {
-    return per_sm == 1 ? (sp == 8 ? n_sms * 30 / 37 : sp == 4 ? n_sms * 33 / 37 : n_sms)
-                       : (sp == 8 ? n_sms * 66 / 37 : sp == 4 ? n_sms * 71 / 37 : 2 * n_sms);
-  };
-  auto ring = [&](int passes, int nt, int sp, int* alias) {
-    const int stage_bytes = (int)kATileBytes * nacc + nt * (int)kBlockK * 2, per_cta = (pl.kb_total + sp - 1) / sp;
-    const int recv = sp > 1 ? nacc * (nt / 4) * (int)kTileRows * 16 : 0;
-    // one CTA per SM: as deep as it gets if nothing is exchanged (XL shape, 288 tokens: 160 KB 1851, 200 KB 1839 us per step)
-    // or HBM is the bound, else 160 KB, which leave room for the attention kernel's first CTAs beside it; two: 108 KB
-    const int kb = pl.tiles * passes * sp > room(sp, 1) ? 108 : sp == 1 || large ? 200 : 160, budget = kb * 1024 - 1024;
-    // a ring that is used again: every stage must always belong to the same issuer (they take turns), or one that is a
-    // lap ahead would find the other's unfinished phase
-    auto usable = [&](int room_for) {
-      int st = room_for < kMaxStages ? room_for : kMaxStages;
-      if (st < per_cta && !dual) st &= ~1;
-      return st < per_cta ? st : per_cta;
-    };
-    int stages = usable((budget - recv) / stage_bytes);
-    // too shallow beside the exchange's buffer: the exchange lies over the drained stages (costs a cluster barrier: XL shape,
-    // 54 tokens, down projection with 4 stages or with 6 and the barrier 1128, 1152 us per step)
-    *alias = stages < per_cta && stages < (dual ? 2 : 4);
-    if (*alias) stages = usable(budget / stage_bytes);
-    if (stages < 2 && per_cta > 1) stages = 2;
-    if (*alias && stages * stage_bytes + recv <= budget) *alias = 0;
-    // one stage fewer than k-blocks where that is even: the next kernel's first CTAs then fit beside more of this one's
-    // (18 tokens 958 -> 940 us, 28 tokens 1004 -> 988; with 16 or 64 tokens a pass they do not, and it costs 1 %)
-    if (!dual && sp > 1 && nt == 32 && stages == per_cta && per_cta >= 5 && (per_cta & 1)) stages = per_cta - 1;
-    return stages;
-  };
-  double best = -1.0;
-  int S = 1;
-  for (int passes = (m + most - 1) / most; passes <= (m + 15) / 16; ++passes) {
-    const int nt = ((m + passes - 1) / passes + 15) / 16 * 16;
-    if (nt > most || (m + nt - 1) / nt != passes) continue;
-    if (huge && pl.passes > 0) break;         // (the weights do not stay in L2 from one pass to the next)
-    const int tok = nt < m ? nt : m;
-    for (int sp = 1; sp <= 8 && sp <= pl.kb_total; sp *= 2) {
-      const int ctas = pl.tiles * passes * sp, kb = (pl.kb_total + sp - 1) / sp, fit = room(sp, large && nt <= 64 ? 2 : 1);
-      const int waves = (ctas + fit - 1) / fit;
-      int alias;
-      ring(passes, nt, sp, &alias);
-      const double fill = (kATileBytes * nacc + 2.0 * kBlockK * (nt < 32 ? 32 : nt)) / 55.0, issue = 280.0 * nacc;
-      double t = kb * (fill > issue ? fill : issue);
-      t += sp > 1 ? 2000.0 + 25.0 * tok * (dual ? 3 : 1) + 1500.0 * alias + 400.0 * ((tok + 3) / 4 * ((int)kTileRows / sp) / 256 + 1)
-                  : 47.0 * tok;
-      t = t * waves + 1500.0 * (waves - 1);
-      if (large && kb >= 32 && (huge || nt >= 32) && ctas <= room(sp, 1) && ctas * 20 >= n_sms * 17) t = 0.0;
-      if (best < 0.0 || t < best) {
-        best = t;
-        pl.passes = passes;
-        pl.nt = nt;
-        S = sp;
-      }
-    }
-  }
-  pl.splits = S;
-  int alias;
-  const int stages = ring(pl.passes, pl.nt, S, &alias);
-  const int stage_bytes = (int)kATileBytes * nacc + pl.nt * (int)kBlockK * 2;
-  const int recv = S > 1 ? nacc * (pl.nt / 4) * (int)kTileRows * 16 : 0;
-  // Eight warps are two per scheduler, and an epilogue item (a row's four tokens: ~250 dependent instructions) then takes
-  // 0.9 us: from two items per thread on there are sixteen (XL shape, 288 tokens 2015 -> 1970 us per step, 54 tokens 1243
-  // -> 1224; 7B shape 3172 -> 3134).  With fewer, starting eight more warps only costs (18 tokens 958 -> 976).
-  pl.threads = (S > 1 ? pl.nt / 4 * (int)kTileRows / S : pl.nt * 8) > 256 ? kMaxThreads : 256;
-  pl.stages = stages;
-  pl.alias = alias;
-  pl.recv_off = alias ? 0 : stages * stage_bytes;
-  pl.smem_bytes = (alias ? (stages * stage_bytes > recv ? stages * stage_bytes : recv) : stages * stage_bytes + recv) + 1024;
-  if (S == 1 && pl.smem_bytes < pl.nt * 272 + 1024) pl.smem_bytes = pl.nt * 272 + 1024;   // the finished tile, token-major
-  int cols = 32;
-  while (cols < pl.nt * 2) cols <<= 1;        // two accumulators
-  pl.tmem_cols = cols;
-  // CTAs of a cluster wait for one another, so none may wait for tensor memory that a waiting one holds: each takes at
-  // least as large a share of an SM's shared memory as of its tensor memory, whatever shares the SM with it
-  const int share = (int)((228u * 1024u * (unsigned)cols + 511u) / 512u) - 1024;          // (1 KB per CTA is the system's)
-  if (pl.smem_bytes < share) pl.smem_bytes = share;
-  return pl;
-}
 
 int launch_proj(int epi, const ProjPlan& pl, const ProjArgs& g, cudaStream_t s) {
   Params kp{};

@@ -11,6 +11,7 @@
 #include <utility>
 #include <vector>
 
+#include "launch_plans.h"
 #include "vvs.h"
 
 #define VVS_CUDA_OK(expr)                         \
@@ -271,11 +272,8 @@ void launch_step_begin(const int32_t* cache_len, const int32_t* tree_parent, con
                        const __nv_bfloat16* tok_emb, const __nv_bfloat16* scale, const Workspace& ws,
                        const vvs_model_desc& md, int n_rows, int t_len, cudaStream_t s);
 
-// ---- projections with folded epilogues, proj_tc.cu -----------------------------------------------
+// ---- projections with folded epilogues, proj_tc.cu (their plans: launch_plans.h) -------------------
 enum { PROJ_QKV = 0, PROJ_ADD = 1, PROJ_GATEUP = 2 };
-struct ProjPlan {
-  int nt, passes, tiles, kb_total, splits, stages, alias, recv_off, smem_bytes, tmem_cols, threads;
-};
 struct ProjArgs {
   int m, n;                    // tokens, weight rows (per matrix)
   const CUtensorMap* tm_a;     // weights [n, k]
@@ -295,8 +293,6 @@ struct ProjArgs {
   __nv_bfloat16* act; int ff;  // GATEUP
   const void* ahead[2]; uint32_t ahead_bytes;   // matrices of the projection after next (same size; null: none)
 };
-ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms);
-int proj_ss_parts(const ProjPlan& plan);     // partial sums per token an ADD projection writes (at most d / 16 rounded up to tiles)
 int launch_proj(int epi, const ProjPlan& plan, const ProjArgs& g, cudaStream_t s);
 
 // ---- block-vs-cache attention on rotated queries and appended keys, attention_block.cu ------------------

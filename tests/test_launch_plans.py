@@ -1,0 +1,71 @@
+"""How a call is dealt to CTAs (csrc/launch_plans.h), checked over sizes on the host: the header holds no CUDA and is compiled
+with the host compiler."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2511_13587_b200", "csrc")
+N_SMS = 148
+FIELDS = ("nt", "passes", "tiles", "kb_total", "splits", "stages", "alias", "recv_off", "smem_bytes", "tmem_cols", "threads")
+SHIM = """
+#include "launch_plans.h"
+extern "C" void proj(int m, int n, int k, int dual, int n_sms, int* o) {
+  const vvs::ProjPlan p = vvs::plan_proj(m, n, k, dual != 0, n_sms);
+  const int v[] = {%s, vvs::proj_ss_parts(p)};
+  for (unsigned i = 0; i < sizeof(v) / sizeof(v[0]); ++i) o[i] = v[i];
+}
+""" % ", ".join("p." + f for f in FIELDS)
+
+# (d_model, d_ff): the benchmark shapes, one between them, one below and one above
+WIDTHS = [(1024, 2752), (1280, 3456), (1536, 2744), (2048, 5504), (4096, 11008), (8192, 22016)]
+
+
+@pytest.fixture(scope="module")
+def plans(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plans")
+    src, lib = str(d / "shim.cc"), str(d / "shim.so")
+    with open(src, "w") as f:
+        f.write(SHIM)
+    subprocess.run([os.environ.get("CXX", "g++"), "-std=c++17", "-O1", "-Wall", "-Werror", "-shared", "-fPIC", "-I", CSRC, src,
+                    "-o", lib], check=True)
+    return ctypes.CDLL(lib)
+
+
+def _proj(plans, m, n, k, dual):
+    out = (ctypes.c_int * (len(FIELDS) + 1))()
+    plans.proj(m, n, k, int(dual), N_SMS, out)
+    return dict(zip(FIELDS + ("ss_parts",), out))
+
+
+def _projections(d, ff):
+    return [(3 * d, d, False), (d, d, False), (ff, d, True), (d, ff, False)]
+
+
+@pytest.mark.parametrize("d,ff", WIDTHS)
+def test_projection_plans_fit_the_hardware(plans, d, ff):
+    for m in list(range(1, 130)) + list(range(130, 1537, 7)):
+        for n, k, dual in _projections(d, ff):
+            p = _proj(plans, m, n, k, dual)
+            at = (m, n, k, dual, p)
+            nacc, kb = 2 if dual else 1, -(-p["kb_total"] // p["splits"])
+            assert p["nt"] % 16 == 0 and 16 <= p["nt"] <= 128 and (p["passes"] - 1) * p["nt"] < m <= p["passes"] * p["nt"], at
+            assert p["tiles"] == -(-n // 128) and p["kb_total"] == -(-k // 64), at
+            assert p["splits"] in (1, 2, 4, 8) and p["splits"] <= p["kb_total"], at
+            # a ring that is used again belongs stage by stage to the same one of two issuers
+            assert 1 <= p["stages"] <= min(12, kb) and (p["stages"] == kb or p["stages"] >= 2), at
+            assert dual or p["stages"] == kb or p["stages"] % 2 == 0, at
+            stage = 128 * 64 * 2 * nacc + p["nt"] * 128
+            recv = nacc * p["nt"] // 4 * 128 * 16 if p["splits"] > 1 else 0
+            need = max(p["stages"] * stage, recv) if p["alias"] else p["stages"] * stage + recv
+            assert p["recv_off"] == (0 if p["alias"] else p["stages"] * stage), at
+            if p["splits"] == 1:
+                need = max(need, p["nt"] * 272)                     # the finished tile, token-major
+            assert need + 1024 <= p["smem_bytes"] <= 222 * 1024, at
+            # two accumulators; a CTA takes at least as large a share of shared memory as of tensor memory
+            assert 2 * p["nt"] <= p["tmem_cols"] <= 512 and p["tmem_cols"] in (32, 64, 128, 256, 512), at
+            assert (p["smem_bytes"] + 1024) * 512 >= p["tmem_cols"] * 228 * 1024 - 512, at
+            assert p["threads"] in (256, 512) and p["threads"] % (128 // p["splits"]) == 0, at
+            assert p["ss_parts"] % 4 == 0 and p["ss_parts"] <= p["tiles"] * 8, at
