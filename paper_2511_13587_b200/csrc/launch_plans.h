@@ -18,6 +18,7 @@ constexpr uint32_t kATileBytes = kTileRows * kBlockK * 2;
 
 struct ProjPlan {
   int nt, passes, tiles, kb_total, splits, stages, alias, recv_off, smem_bytes, tmem_cols, threads;
+  int tiles_on_z;              // grid (passes, slices, tiles) in the place of (tiles, slices, passes)
 };
 
 // partial sums of squares per token an ADD projection writes (at most d / 16 rounded up to tiles)
@@ -42,7 +43,12 @@ inline int proj_ss_parts(const ProjPlan& pl) {
 // per step against 3.29 with one), and a split deals the rows out evenly over the SMs.
 // Where several passes of 32 tokens or more give nearly every SM one CTA with 32 k-blocks or more to stream, a deep ring
 // for each does better still (d 2048, 72 tokens 1415 -> 1383 us per step, 126 tokens 1667 -> 1525; 7B down projection,
-// 32 tiles x 4, 3049 -> 3028).  Beyond 64 MB more than the fewest passes would stream the weights from HBM again.
+// 32 tiles x 4, 3049 -> 3028).
+// Beyond 64 MB the weights do not stay in L2 from one pass to the next.  Up to 128 tokens one pass streams them once (four
+// layers of the 7B shape, 128 tokens 514 us, two passes of 64 595).  More take passes of up to 64, as few as there can be, and
+// the passes of a tile run side by side, grid x, so that all but one of them find its weights in L2: 180 tokens 1084 us with
+// two passes of 96 one behind the other, 734 with three of 64, 730 with these side by side; 288 tokens 1455, 1191 and 1102;
+// 576 tokens 2602, 1981 and 1859.  (Smaller ones stay in L2 and lose by it: d 2048, 72 tokens 430 -> 435.)
 // A cluster needs its CTAs' room inside one GPC: of 148 SMs 132 take clusters of four and 120 clusters of eight at one
 // CTA per SM, 284 and 264 of 296 at two.
 inline ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
@@ -53,7 +59,8 @@ inline ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
   pl.kb_total = (k + (int)kBlockK - 1) / (int)kBlockK;
   const size_t bytes = (size_t)n * k * 2 * nacc;
   const bool large = bytes > ((size_t)20 << 20), huge = bytes > ((size_t)64 << 20);
-  const int most = large && !huge ? 64 : kMaxTok;      // (64: two CTAs' accumulators and their shared memory, below, fit on an SM)
+  // (64: two CTAs' accumulators and their shared memory, below, fit on an SM)
+  const int most = large && !(huge && m <= kMaxTok) ? 64 : kMaxTok;
   auto room = [&](int sp, int per_sm) {
     return per_sm == 1 ? (sp == 8 ? n_sms * 30 / 37 : sp == 4 ? n_sms * 33 / 37 : n_sms)
                        : (sp == 8 ? n_sms * 66 / 37 : sp == 4 ? n_sms * 71 / 37 : 2 * n_sms);
@@ -110,6 +117,7 @@ inline ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
     }
   }
   pl.splits = S;
+  pl.tiles_on_z = huge && pl.passes > 1;
   int alias;
   const int stages = ring(pl.passes, pl.nt, S, &alias);
   const int stage_bytes = (int)kATileBytes * nacc + pl.nt * (int)kBlockK * 2;

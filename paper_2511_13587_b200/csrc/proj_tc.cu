@@ -78,7 +78,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-template <int EPI, bool SPLIT>
+// SIDE: grid (passes, slices, tiles), the passes of a tile side by side, in the place of (tiles, slices, passes)
+template <int EPI, bool SPLIT, bool SIDE>
 __global__ void __launch_bounds__(kMaxThreads)
 proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_a2,
                const __grid_constant__ CUtensorMap tm_b) {
@@ -95,8 +96,9 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, n_threads = (int)blockDim.x;
-  const int tile = blockIdx.x, rank = SPLIT ? (int)blockIdx.y : 0, S = SPLIT ? p.splits : 1;
-  const int tok0 = (int)blockIdx.z * p.nt, ntok = min(p.nt, p.m - tok0), nq = (ntok + 3) >> 2;
+  const int tile = (int)(SIDE ? blockIdx.z : blockIdx.x), pass = (int)(SIDE ? blockIdx.x : blockIdx.z);
+  const int rank = SPLIT ? (int)blockIdx.y : 0, S = SPLIT ? p.splits : 1;
+  const int tok0 = pass * p.nt, ntok = min(p.nt, p.m - tok0), nq = (ntok + 3) >> 2;
   const int kb0 = (int)(((long long)rank * p.kb_total) / S);
   const int nkb = (int)(((long long)(rank + 1) * p.kb_total) / S) - kb0;
   constexpr uint32_t a_bytes = kATileBytes * NACC;
@@ -518,11 +520,12 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
 
 template <int EPI>
 cudaError_t launch_epi(const ProjPlan& pl, const Params& kp, const ProjArgs& g, cudaStream_t s) {
-  auto* fn = pl.splits > 1 ? proj_tc_kernel<EPI, true> : proj_tc_kernel<EPI, false>;
+  auto* fn = pl.splits > 1 ? (pl.tiles_on_z ? proj_tc_kernel<EPI, true, true> : proj_tc_kernel<EPI, true, false>)
+                           : (pl.tiles_on_z ? proj_tc_kernel<EPI, false, true> : proj_tc_kernel<EPI, false, false>);
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(fn), 222 * 1024);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(pl.tiles, pl.splits, pl.passes);
+  cfg.gridDim = pl.tiles_on_z ? dim3(pl.passes, pl.splits, pl.tiles) : dim3(pl.tiles, pl.splits, pl.passes);
   cfg.blockDim = dim3(pl.threads, 1, 1);
   cfg.dynamicSmemBytes = pl.smem_bytes;
   cfg.stream = s;

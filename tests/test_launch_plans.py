@@ -9,7 +9,8 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2511_13587_b200", "csrc")
 N_SMS = 148
-FIELDS = ("nt", "passes", "tiles", "kb_total", "splits", "stages", "alias", "recv_off", "smem_bytes", "tmem_cols", "threads")
+FIELDS = ("nt", "passes", "tiles", "kb_total", "splits", "stages", "alias", "recv_off", "smem_bytes", "tmem_cols", "threads",
+          "tiles_on_z")
 SHIM = """
 #include "launch_plans.h"
 extern "C" void proj(int m, int n, int k, int dual, int n_sms, int* o) {
@@ -69,3 +70,16 @@ def test_projection_plans_fit_the_hardware(plans, d, ff):
             assert (p["smem_bytes"] + 1024) * 512 >= p["tmem_cols"] * 228 * 1024 - 512, at
             assert p["threads"] in (256, 512) and p["threads"] % (128 // p["splits"]) == 0, at
             assert p["ss_parts"] % 4 == 0 and p["ss_parts"] <= p["tiles"] * 8, at
+
+
+def test_passes_over_weights_that_exceed_l2(plans):
+    """Up to 128 tokens stream such weights once; more take the fewest passes of up to 64, those of a tile side by side."""
+    for m in list(range(1, 260)) + [288, 504, 576, 1152]:
+        for n, k, dual in _projections(4096, 11008):
+            p = _proj(plans, m, n, k, dual)
+            if n * k * 2 * (2 if dual else 1) <= 64 << 20:
+                assert not p["tiles_on_z"], (m, n, k, p)
+            elif m <= 128:
+                assert p["passes"] == 1 and not p["tiles_on_z"], (m, n, k, p)
+            else:
+                assert p["passes"] == -(-m // 64) and p["nt"] <= 64 and p["tiles_on_z"], (m, n, k, p)
