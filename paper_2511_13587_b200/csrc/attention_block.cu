@@ -2,7 +2,8 @@
 // against the cached keys [0, fill) and, under the ancestor mask, the block's own keys, which the QKV projection has
 // just written to slots fill .. fill + T - 1.
 //
-// One CTA per (sequence, head) -- or a cluster of S CTAs when there are few of them and the cache is long.  Every warp
+// One CTA per (sequence, head) -- or a cluster of S CTAs when there are few of them and the cache may be long
+// (attention_split, launch_plans.h).  Every warp
 // owns the 16-key slices w, w + W, ... and streams them through a ring of its own (cp.async, 16-byte pieces, D
 // slices deep): no barrier inside the loop.  Slices of old keys are requested BEFORE griddepcontrol.wait, while the
 // QKV projection is still running; after the wait only q (registers) and the one to three slices that hold new keys
@@ -302,8 +303,7 @@ int launch_attention_block(const AttentionBlockArgs& a, cudaStream_t s) {
   if (a.t_len > kMaxT) return VVS_ERR_SHAPE;
   const long long items = (long long)a.n_heads * a.n_rows;
   const bool few = items <= a.n_sms, some = items <= 2LL * a.n_sms;
-  int split = 1;
-  if (a.hd == 128) while (split < 4 && items * split * 2 <= a.n_sms && a.s_max >= 512 * split) split *= 2;
+  const int split = attention_split(a.hd, items, a.s_max, a.n_sms);
   if (a.hd == 64) {
     if (few) return launch_variant<64, 1, 16, 2>(a, split, 1, s);
     if (a.t_len > 16) return launch_variant<64, 2, 4, 3>(a, split, 2, s);

@@ -141,4 +141,19 @@ inline ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
   return pl;
 }
 
+// ---- block-vs-cache attention, attention_block.cu -------------------------------------------------
+// CTAs (a cluster) per (sequence, head) item.  The keys of an item are split where the items leave SMs idle and the cache can
+// be long enough to pay for the exchange: by its capacity s_max, since the fill levels are known to the GPU only.  Heads of 64
+// keep 16 warps on an item, which take 256 keys a turn; of 128, 8 warps and 128 keys.  XL shape (40 items of 64-wide heads,
+// 18 layers, 18 tokens), one CTA an item / two: 592 slots, 300 filled 473 / 477 us; 2304 slots, 64 filled 462 / 472, 2200
+// filled 626 / 558; 4608 slots, 4500 filled 819 / 656.  20 items, 4608 slots, two / four: 100 filled 448 / 466, 2000 filled
+// 511 / 497, 4500 filled 612 / 560.  7B shape (64 items of 128-wide heads, 8 layers), one / two: 60 filled 735 / 735, 450
+// filled 762 / 749, 2300 filled 864 / 816; 32 items, 4500 filled, two / four 837 / 785.
+inline int attention_split(int hd, long long items, int s_max, int n_sms) {
+  const int slots = hd == 128 ? 512 : 1536;
+  int split = 1;
+  while (split < 4 && items * split * 2 <= n_sms && s_max >= slots * split) split *= 2;
+  return split;
+}
+
 }  // namespace vvs

@@ -18,6 +18,7 @@ extern "C" void proj(int m, int n, int k, int dual, int n_sms, int* o) {
   const int v[] = {%s, vvs::proj_ss_parts(p)};
   for (unsigned i = 0; i < sizeof(v) / sizeof(v[0]); ++i) o[i] = v[i];
 }
+extern "C" int att_split(int hd, int items, int s_max, int n_sms) { return vvs::attention_split(hd, items, s_max, n_sms); }
 """ % ", ".join("p." + f for f in FIELDS)
 
 # (d_model, d_ff): the benchmark shapes, one between them, one below and one above
@@ -83,3 +84,15 @@ def test_passes_over_weights_that_exceed_l2(plans):
                 assert p["passes"] == 1 and not p["tiles_on_z"], (m, n, k, p)
             else:
                 assert p["passes"] == -(-m // 64) and p["nt"] <= 64 and p["tiles_on_z"], (m, n, k, p)
+
+
+@pytest.mark.parametrize("hd", [64, 128])
+def test_attention_split(plans, hd):
+    for items in range(1, 400):
+        for s_max in (1, 511, 512, 592, 1023, 1024, 1535, 1536, 3071, 3072, 4608, 1 << 20):
+            s = plans.att_split(hd, items, s_max, N_SMS)
+            assert s in (1, 2, 4) and (s == 1 or items * s <= N_SMS), (items, s_max, s)
+    # one image of 20 heads, with and without guidance: idle SMs share a long cache, a short one is not split
+    assert [plans.att_split(64, 40, s, N_SMS) for s in (592, 1535, 1536, 4608)] == [1, 1, 2, 2]
+    assert [plans.att_split(64, 20, s, N_SMS) for s in (592, 1536, 4608)] == [1, 2, 4]
+    assert [plans.att_split(128, 64, s, N_SMS) for s in (511, 512, 2384)] == [1, 2, 2]
