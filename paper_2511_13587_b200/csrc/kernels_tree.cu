@@ -9,11 +9,13 @@
 // (the chain's relaxed rule with p_res in the place of p); with the adjusted-residual flag a
 // rejection subtracts q from p_res after the pooled neighbours' mass has been moved onto x.
 //
-// A cluster of S CTAs per image, each with a contiguous part of the codes; the walk is sequential over tree depth and
-// siblings and every CTA takes it, each residual update and the final inverse-CDF draw are passes over the parts whose
-// sums are exchanged through distributed shared memory and added in rank order, so a call repeats bit for bit on the same
-// probabilities.  What bounds it: the chain of tests and passes; one SM's float64 units and loads were what a pass of
-// 16384 codes took before (4 images, 26 nodes: 47 -> 25 us per call; 8 images of 32768 codes, relaxed: 60 -> 31).
+// One CTA per image, or a cluster of S for larger codebooks (tree_walk_parts, launch_plans.h), each with a contiguous part of
+// the codes; the walk is sequential over tree depth and siblings and every CTA takes it, each residual update and the final
+// inverse-CDF draw are passes over the parts whose sums are exchanged through distributed shared memory and added in rank
+// order, so a call repeats bit for bit on the same probabilities.  What bounds it: the chain of tests and passes; a cluster
+// pays one barrier per rejection and two for the draw, a pass of 16384 codes on one SM (float64 units and loads) 7 us.
+// 26 nodes, most rejected, before with one CTA each / now: 4 images x 4096 codes 23.8 / 23.1 us, x 16384 67.6 / 24.2, 8 images
+// x 32768 123 / 30; most accepted 11.3 / 11.2, 19.8 / 13.3, 45.2 / 13.8.
 #include <math_constants.h>
 
 #include "vvs_internal.cuh"
@@ -92,26 +94,25 @@ __device__ __forceinline__ int tw_load_s32(const int* local, uint32_t rank) {
   asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(tw_remote(local, rank)) : "memory");
   return v;
 }
-// The CTAs' values at *slot: their sum and the sum of those before `rank`, in rank order.  Consecutive calls take two slots
-// in turn: a CTA that writes a slot again has met every reader of it at the barrier of the call between.  The barrier also
-// publishes what the CTAs have written to global memory.
-__device__ __forceinline__ double tw_exchange(double v, double* slot, int S, int rank, double* before) {
+// The sum of the CTAs' values at *slot, in rank order.  Consecutive calls take two slots in turn: a CTA that writes a slot
+// again has met every reader of it at the barrier of the call between.  The barrier also publishes what the CTAs have
+// written to global memory.
+__device__ __forceinline__ double tw_exchange(double v, double* slot, int S) {
   if (threadIdx.x == 0) *slot = v;
   tw_cluster_sync();
   double tot = 0.0;
-  for (int r = 0; r < S; ++r) {
-    if (r == rank) *before = tot;
-    tot += tw_load_f64(slot, (uint32_t)r);
-  }
+  for (int r = 0; r < S; ++r) tot += tw_load_f64(slot, (uint32_t)r);
   return tot;
 }
 
+// CLUSTER: several CTAs per image; else one, which needs none of the barriers and exchanges between them.
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
   __shared__ double s_warp[kTreeThreads / 32], s_slot[2];
   __shared__ int s_child[32];
   __shared__ int s_n, s_pass, s_first, s_last, s_jend;
   __shared__ double s_mass;
-  const int b = blockIdx.y, S = (int)gridDim.x, rank = (int)blockIdx.x;
+  const int b = blockIdx.y, S = CLUSTER ? (int)gridDim.x : 1, rank = CLUSTER ? (int)blockIdx.x : 0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int F = p.n_forced, K = p.n_draft_max, T = p.t_len, V = p.vocab;
   const int32_t* par = p.parent + (size_t)b * T;
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
 
   const int part = (V + S - 1) / S, r0 = min(V, rank * part), r1 = min(V, r0 + part);   // this CTA's codes
   int turn = 0;
-  double before_part = 0.0;
+  auto residual_at = [](const double* r) { return CLUSTER ? __ldcg(r) : *r; };          // (another CTA's part, maybe)
   if (rank == 0 && tid == 0) {
     for (int i = 0; i <= K; ++i)
       if (p.margins) p.margins[(size_t)b * (K + 1) + i] = CUDART_INF_F;
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
         if (!x_ok) {
           if (lane == 0) atomicOr(p.status, VVS_DEV_BAD_TOKEN);
         } else {
-          double px = first_round ? (double)prow[x] : __ldcg(buf[src] + x) / z;   // (another CTA's part, maybe)
+          double px = first_round ? (double)prow[x] : residual_at(buf[src] + x) / z;
           int j_end = 1;
           if (p.relaxed) {
             const int beg = p.row_ptr[x], len = p.row_ptr[x + 1] - beg;
@@ -169,7 +170,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
             px += tw_pooled_prefix(kk, (double)p.delta, lane, [&](int j) {
               const int cc = p.col[beg + j];
               if (cc < 0 || cc >= V) return 0.0;
-              return cur_res ? __ldcg(cur_res + cc) / z : (double)prow[cc]; }, &j_end);
+              return cur_res ? residual_at(cur_res + cc) / z : (double)prow[cc]; }, &j_end);
           }
           const double qx = (double)qrow[x];
           const double ratio = qx > 0.0 ? fmin(1.0, px / qx) : (px > 0.0 ? 1.0 : 0.0);
@@ -184,14 +185,17 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
         if (lane == 0) s_pass = pass;
       }
       __syncthreads();
-      const int pass = s_pass;
-      if (src >= 0) tw_cluster_sync();            // everyone has read the residual: it may be overwritten from here on
-      else __syncthreads();
-      if (pass) {
+      if (s_pass) {
+        // the next level's first residual may go where a slower CTA is still reading this one's; a rejection writes the other
+        // buffer, whose readers have all met at the exchange before
+        if (CLUSTER && src >= 0) tw_cluster_sync();
         accepted = c;
         break;
       }
-      if (!x_ok) continue;
+      if (!x_ok) {
+        __syncthreads();                          // s_pass is written again
+        continue;
+      }
       // rejected: residual of this round
       double* dst = buf[src < 0 ? 0 : (src ^ 1)];
       double local = 0.0;
@@ -227,7 +231,8 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
         local = 0.0;
         for (int v = r0 + tid; v < r1; v += kTreeThreads) local += dst[v];
       }
-      const double z_new = tw_exchange(tw_block_sum(local, s_warp), &s_slot[turn], S, rank, &before_part);
+      double z_new = tw_block_sum(local, s_warp);
+      if (CLUSTER) z_new = tw_exchange(z_new, &s_slot[turn], S);
       turn ^= 1;
       if (z_new > 0.0) {                          // else p_res == q numerically: keep p_res
         src = src < 0 ? 0 : (src ^ 1);
@@ -249,46 +254,72 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
   const int seg = (part + kTreeThreads - 1) / kTreeThreads;
   const int v0 = min(r1, r0 + tid * seg), v1 = min(r1, v0 + seg);
   const double* dsrc = src < 0 ? nullptr : buf[src];
-  double local = 0.0;
-  for (int v = v0; v < v1; ++v) local += dsrc ? dsrc[v] : (double)prow[v];
-  double incl = tw_warp_scan(local, lane);
-  if (lane == 31) s_warp[warp] = incl;
   if (tid == 0) {
     s_first = 0x7fffffff;
     s_last = -1;
   }
+  double local = 0.0;
+  int nz = -1;                                    // last code of this thread that carries mass
+  for (int v = v0; v < v1; ++v) {
+    const double r = dsrc ? dsrc[v] : (double)prow[v];
+    local += r;
+    if (r > 0.0) nz = v;
+  }
+  double incl = tw_warp_scan(local, lane);
+  if (lane == 31) s_warp[warp] = incl;
   __syncthreads();
-  double before = 0.0, total = 0.0;
+  if (nz >= 0) atomicMax(&s_last, nz);
+  double before = 0.0, total = 0.0;               // mass ahead of this warp, in front of the CTA's part at first
   for (int w = 0; w < kTreeThreads / 32; ++w) {
     const double t = s_warp[w];
     if (w < warp) before += t;
     total += t;
   }
-  total = tw_exchange(total, &s_slot[turn], S, rank, &before_part);
-  before += before_part;
-  const double excl = before + incl - local;
-  const double target = (double)p.uniforms[(size_t)b * (K + 1) + K] * total;
-  {
-    double c = excl;
-    int first = 0x7fffffff, last = -1;
-    for (int v = v0; v < v1; ++v) {
-      const double r = dsrc ? dsrc[v] : (double)prow[v];
-      c += r;
-      if (r > 0.0) last = v;
-      if (first == 0x7fffffff && c > target) first = v;
+  // the part that holds the sample point, by the parts' sums in rank order: the first whose end lies beyond it
+  const double u = (double)p.uniforms[(size_t)b * (K + 1) + K];
+  double target = u * total;
+  int last, owner = 0;
+  if (CLUSTER) {
+    if (tid == 0) s_slot[turn] = total;
+    tw_cluster_sync();                            // s_last is complete too
+    double sum = 0.0, part_sum[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) part_sum[r] = r < S ? tw_load_f64(&s_slot[turn], (uint32_t)r) : 0.0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) sum += part_sum[r];
+    target = u * sum;
+    total = sum;
+    owner = -1;
+    last = -1;
+    double ahead = 0.0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      if (r == rank) before += ahead;
+      ahead += part_sum[r];
+      if (owner < 0 && ahead > target) owner = r;
     }
-    if (first != 0x7fffffff) atomicMin(&s_first, first);
-    if (last >= 0) atomicMax(&s_last, last);
+    if (owner < 0)                                // the point rounds to the end: the last code with mass, wherever it is
+      for (int r = 0; r < S; ++r) last = max(last, tw_load_s32(&s_last, (uint32_t)r));
+    else
+      last = s_last;
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");     // (waited for at the end)
   }
-  __syncthreads();
-  tw_cluster_sync();
-  int first = 0x7fffffff, last = -1;
-  for (int r = 0; r < S; ++r) {
-    first = min(first, tw_load_s32(&s_first, (uint32_t)r));
-    last = max(last, tw_load_s32(&s_last, (uint32_t)r));
+  const double excl = before + incl - local;
+  if (owner == rank) {
+    double c = excl;
+    for (int v = v0; v < v1; ++v) {
+      c += dsrc ? dsrc[v] : (double)prow[v];
+      if (c > target) {
+        atomicMin(&s_first, v);
+        break;
+      }
+    }
   }
-  const int pick = first != 0x7fffffff ? first : last;
-  if (pick >= v0 && pick < v1) {
+  __syncthreads();                                // s_first; s_last too where there is one CTA
+  if (!CLUSTER) last = s_last;
+  // (in the part that holds the point its own last code with mass, should the sums of its threads round to less)
+  const int pick = owner == rank && s_first != 0x7fffffff ? s_first : last;
+  if ((owner == rank || owner < 0) && pick >= v0 && pick < v1) {
     double c = excl;
     for (int v = v0; v < pick; ++v) c += dsrc ? dsrc[v] : (double)prow[v];
     const double hi = c + (dsrc ? dsrc[pick] : (double)prow[pick]);
@@ -296,7 +327,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
     if (p.margins) p.margins[(size_t)b * (K + 1) + K] = (float)(fmin(fabs(target - c), fabs(hi - target)) / total);
   }
   if (rank == 0 && tid == 0) {
-    if (pick < 0) {                               // an all-zero source: no token can be drawn
+    if (owner == rank ? pick < 0 : owner < 0 && last < 0) {     // an all-zero source: no token can be drawn
       p.next_token[b] = -1;
       atomicOr(p.status, VVS_DEV_BAD_ARG);
     }
@@ -307,7 +338,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
       if (p.n_commit) p.n_commit[r] = F + n_acc;
     }
   }
-  tw_cluster_sync();                              // nobody leaves while its shared memory may be read
+  if (CLUSTER) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // nobody leaves while it may be read
 }
 
 // K/V of the accepted nodes move from their block slots fill + node to fill + F + i (i-th
@@ -337,10 +368,12 @@ __global__ void tree_commit_kernel(T* __restrict__ kv_k, T* __restrict__ kv_v, c
 
 }  // namespace
 
-// Parts of 2048 codes or more, eight CTAs (the portable cluster) at most.
-void launch_tree_walk(const TreeParams& p, cudaStream_t s) {
-  int S = 1;
-  while (S < 8 && p.vocab >= 2048 * 2 * S) S *= 2;
+void launch_tree_walk(const TreeParams& p, int n_sms, cudaStream_t s) {
+  const int S = tree_walk_parts(p.vocab, p.n_images, n_sms);
+  if (S == 1) {
+    tree_walk_kernel<false><<<dim3(1, p.n_images), kTreeThreads, 0, s>>>(p);
+    return;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(S, p.n_images, 1);
   cfg.blockDim = dim3(kTreeThreads, 1, 1);
@@ -352,7 +385,7 @@ void launch_tree_walk(const TreeParams& p, cudaStream_t s) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, tree_walk_kernel, p);   // (the caller reads cudaGetLastError)
+  cudaLaunchKernelEx(&cfg, tree_walk_kernel<true>, p);   // (the caller reads cudaGetLastError)
 }
 
 void launch_tree_commit(void* kv_k, void* kv_v, const int32_t* cache_len, const int32_t* accept_len,

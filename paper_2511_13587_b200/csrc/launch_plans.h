@@ -156,4 +156,17 @@ inline int attention_split(int hd, long long items, int s_max, int n_sms) {
   return split;
 }
 
+// ---- walk of a candidate tree, kernels_tree.cu ---------------------------------------------------
+// CTAs (a cluster) per image, each with a part of the codes: what a part saves on each residual has to outweigh the cluster's
+// barriers, also where most drafts are accepted and there are few residuals.  26 nodes, one image, most accepted / most
+// rejected: 4096 codes 9.2 / 22.9 us with one CTA, 10.4 / 19.6 with four; 8192 codes 10.8 / 34.4, 10.8 / 23.0, eight 10.9 /
+// 21.2; 16384 codes, four images 17.4 / 65.6, 13.1 / 28.5, 13.3 / 24.2.  And all clusters run at once: of clusters of eight
+// (one CTA per SM) 15 fit, of four 33 (16 images x 16384 codes, most rejected: 39 us with eight each, 29 with four; 40
+// images, all accepted: 38 with eight, 24 with two).
+inline int tree_walk_parts(int vocab, int n_images, int n_sms) {
+  int S = vocab < 8192 ? 1 : vocab < 16384 ? 4 : 8;
+  while (S > 1 && (long long)n_images * S > (S == 8 ? n_sms * 30 / 37 : S == 4 ? n_sms * 33 / 37 : n_sms)) S /= 2;
+  return S;
+}
+
 }  // namespace vvs

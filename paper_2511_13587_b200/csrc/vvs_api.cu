@@ -336,7 +336,7 @@ int run_tree_decisions(vvs_ctx* ctx, const __nv_bfloat16* hid, const vvs_verify_
   tp.accept_path = o->accept_path ? o->accept_path : ws.tree_path;
   tp.next_token = o->next_token; tp.new_len = o->new_len; tp.n_commit = o->n_commit;
   tp.accept_mask = o->accept_mask; tp.margins = o->margins; tp.status = ws.status;
-  VVS_LAUNCH(VVS_PROF_OTHER, launch_tree_walk(tp, s));
+  VVS_LAUNCH(VVS_PROF_OTHER, launch_tree_walk(tp, ctx->n_sms, s));
   if (a->n_draft_max > 0)
     VVS_LAUNCH(VVS_PROF_OTHER, launch_tree_commit(a->kv_k, a->kv_v, a->cache_len, o->accept_len, tp.accept_path, md,
                                                   a->kv_rows, B, C, a->n_forced, a->n_draft_max, s));
@@ -991,7 +991,7 @@ int vvs_decide(vvs_ctx* ctx, const float* target_probs, int32_t n_rows_per_seq, 
     tp.adjusted = (tp.relaxed && a->adjusted_residual) ? 1 : 0; tp.row_ptr = ctx->nbr_row_ptr; tp.col = ctx->nbr_col;
     tp.accept_len = o->accept_len; tp.accept_path = o->accept_path ? o->accept_path : ws.tree_path;
     tp.next_token = o->next_token; tp.accept_mask = o->accept_mask; tp.margins = o->margins; tp.status = ws.status;
-    VVS_LAUNCH(VVS_PROF_OTHER, launch_tree_walk(tp, s));
+    VVS_LAUNCH(VVS_PROF_OTHER, launch_tree_walk(tp, ctx->n_sms, s));
     return cudaGetLastError() == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
   }
   DecideParams p = decide_params(ctx, n_rows_per_seq, first_row, drafts, a->n_draft_max, a, o, false);

@@ -405,7 +405,7 @@ struct TreeParams {
   uint8_t* accept_mask; float* margins;
   int32_t* status;
 };
-void launch_tree_walk(const TreeParams& p, cudaStream_t s);
+void launch_tree_walk(const TreeParams& p, int n_sms, cudaStream_t s);
 void launch_tree_commit(void* kv_k, void* kv_v, const int32_t* cache_len, const int32_t* accept_len,
                         const int32_t* accept_path, const vvs_model_desc& md, int kv_rows, int n_images, int n_cfg,
                         int n_forced, int n_draft_max, cudaStream_t s);

@@ -18,6 +18,7 @@ extern "C" void proj(int m, int n, int k, int dual, int n_sms, int* o) {
   const int v[] = {%s, vvs::proj_ss_parts(p)};
   for (unsigned i = 0; i < sizeof(v) / sizeof(v[0]); ++i) o[i] = v[i];
 }
+extern "C" int tree_parts(int vocab, int n_images, int n_sms) { return vvs::tree_walk_parts(vocab, n_images, n_sms); }
 extern "C" int att_split(int hd, int items, int s_max, int n_sms) { return vvs::attention_split(hd, items, s_max, n_sms); }
 """ % ", ".join("p." + f for f in FIELDS)
 
@@ -96,3 +97,13 @@ def test_attention_split(plans, hd):
     assert [plans.att_split(64, 40, s, N_SMS) for s in (592, 1535, 1536, 4608)] == [1, 1, 2, 2]
     assert [plans.att_split(64, 20, s, N_SMS) for s in (592, 1536, 4608)] == [1, 2, 4]
     assert [plans.att_split(128, 64, s, N_SMS) for s in (511, 512, 2384)] == [1, 2, 2]
+
+
+def test_tree_walk_parts(plans):
+    for vocab in (1, 64, 2048, 4096, 8191, 8192, 10000, 16383, 16384, 65536, 1 << 23):
+        for n_images in (1, 2, 4, 8, 15, 16, 33, 34, 40, 74, 75, 500):
+            s = plans.tree_parts(vocab, n_images, N_SMS)
+            # small codebooks stay with one CTA; otherwise all clusters find room at once (15 of eight CTAs, 33 of four)
+            assert s == 1 if vocab < 8192 else s in (1, 2, 4, 8), (vocab, n_images, s)
+            assert n_images <= {1: n_images, 2: 74, 4: 33, 8: 15}[s], (vocab, n_images, s)
+    assert [plans.tree_parts(16384, b, N_SMS) for b in (1, 15, 16, 33, 34, 75)] == [8, 8, 4, 4, 2, 1]
