@@ -91,6 +91,7 @@ inline ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
     return stages;
   };
   double best = -1.0;
+  bool deep = false;                          // the plan taken is one of the deep rings described above
   int S = 1;
   for (int passes = (m + most - 1) / most; passes <= (m + 15) / 16; ++passes) {
     const int nt = ((m + passes - 1) / passes + 15) / 16 * 16;
@@ -107,8 +108,10 @@ inline ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
       t += sp > 1 ? 2000.0 + 25.0 * tok * (dual ? 3 : 1) + 1500.0 * alias + 400.0 * ((tok + 3) / 4 * ((int)kTileRows / sp) / 256 + 1)
                   : 47.0 * tok;
       t = t * waves + 1500.0 * (waves - 1);
-      if (large && kb >= 32 && (huge || nt >= 32) && ctas <= room(sp, 1) && ctas * 20 >= n_sms * 17) t = 0.0;
-      if (best < 0.0 || t < best) {
+      // (of several such the one of the fewest passes and slices, i.e. the longest streams: the estimate knows no HBM)
+      const bool d = large && kb >= 32 && (huge || nt >= 32) && ctas <= room(sp, 1) && ctas * 20 >= n_sms * 17;
+      if (!deep && (d || best < 0.0 || t < best)) {
+        deep = d;
         best = t;
         pl.passes = passes;
         pl.nt = nt;
