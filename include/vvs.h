@@ -136,10 +136,13 @@ typedef struct vvs_weights {
 } vvs_weights;
 
 /* Create a context on the current CUDA device and allocate its scratch memory (sized from
- * max_rows, max_block, max_nbr_k; see vvs_workspace_bytes).  *out is NULL on failure. */
+ * max_rows, max_block, max_nbr_k; see vvs_workspace_bytes).  *out is NULL on failure.
+ * The largest part in bf16 contexts are the guided logits of a call, float32 [decision rows, vocab], up to 1 GB and
+ * sized for calls without guidance (n_cfg = 1; guided calls use half).  Where that much is not free the context is
+ * created with room for 64 decision rows: calls of more then leave no logits in memory and take longer. */
 int vvs_create(const vvs_model_desc* desc, vvs_ctx** out);
 int vvs_destroy(vvs_ctx* ctx);
-/* Scratch bytes vvs_create will allocate for this description (host computation only). */
+/* Scratch bytes vvs_create asks for for this description (host computation only). */
 int vvs_workspace_bytes(const vvs_model_desc* desc, size_t* out_bytes);
 
 /* Bind caller-owned weights.  Checks non-NULL and 16-byte alignment (VVS_ERR_ALIGN).  Nothing is

@@ -14,7 +14,14 @@ namespace {
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline size_t elem_bytes(const vvs_model_desc& d) { return d.dtype == VVS_DTYPE_BF16 ? 2 : 4; }
 
-// Carves the scratch arena; with base == nullptr only the total size is computed.
+// Guided logits of a call (tensor-core path): 64 decision rows always, more as long as the buffer stays under a gigabyte; all
+// that max_rows and max_block allow without guidance, since a context does not know whether its calls use it.
+int logit_rows_of(const vvs_model_desc& d, bool few) {
+  const size_t rows = (size_t)d.max_rows * d.max_block, cap = few ? 64 : ((size_t)1 << 30) / ((size_t)d.vocab * 4);
+  return (int)(rows < 64 ? rows : cap < 64 ? 64 : rows < cap ? rows : cap);
+}
+
+// Carves the scratch arena; with base == nullptr only the total size is computed.  few_logits: see vvs_create.
 struct Carver {
   char* base;
   size_t off = 0;
@@ -26,7 +33,7 @@ struct Carver {
   }
 };
 
-size_t layout(const vvs_model_desc& d, Workspace& ws, char* base) {
+size_t layout(const vvs_model_desc& d, Workspace& ws, char* base, bool few_logits = false) {
   Carver c{base};
   const size_t es = elem_bytes(d);
   const size_t M = (size_t)d.max_rows * d.max_block;  // activation rows; also bounds B*T
@@ -92,13 +99,19 @@ size_t layout(const vvs_model_desc& d, Workspace& ws, char* base) {
   c.take(ws.r_part, (size_t)d.max_rows * n_chunks * 8);
   c.take(ws.p_part, (size_t)d.max_rows * n_chunks * 8);
   if (d.dtype == VVS_DTYPE_BF16 && d.n_layers > 0) c.take(ws.anc_mask, M * 4);
-  c.take(ws.tree_res, (size_t)2 * d.max_rows * V * 8);
   c.take(ws.tree_path, (size_t)d.max_rows * 32 * 4);
+  // last, because they need no clearing: the guided logits and the residuals of a tree walk, which lie in the same place (a
+  // tree call's logits are in the caller's target_probs)
+  c.off = (c.off + 255) & ~size_t(255);
+  ws.cleared_bytes = c.off;
+  const size_t res_bytes = (size_t)2 * d.max_rows * V * 8;
   if (d.dtype == VVS_DTYPE_BF16 && !std::getenv("VVS_DEBUG_GENERIC")) {
-    // guided logits of a call: 64 decision rows always, more as long as the buffer stays under a gigabyte
-    const size_t cap = ((size_t)1 << 30) / (V * 4);
-    ws.logit_rows = (int)(M < 64 ? M : cap < 64 ? 64 : M < cap ? M : cap);
-    c.take(ws.logits_small, (size_t)ws.logit_rows * V * 4);
+    ws.logit_rows = logit_rows_of(d, few_logits);
+    const size_t bytes = (size_t)ws.logit_rows * V * 4;
+    c.take(ws.logits_small, bytes > res_bytes ? bytes : res_bytes);
+    ws.tree_res = reinterpret_cast<double*>(ws.logits_small);
+  } else {
+    c.take(ws.tree_res, res_bytes);
   }
   return (c.off + 255) & ~size_t(255);
 }
@@ -749,13 +762,19 @@ int vvs_create(const vvs_model_desc* desc, vvs_ctx** out) {
   if (cudaGetDevice(&ctx->device) != cudaSuccess) { delete ctx; return VVS_ERR_CUDA; }
   Workspace tmp;
   ctx->arena_bytes = layout(*desc, tmp, nullptr);
-  if (cudaMalloc(&ctx->arena, ctx->arena_bytes) != cudaSuccess) {
+  // Where there is no room for the logits of the largest call, for those of 64 decision rows: larger calls then pick what
+  // they need in the LM head's epilogue and compute the sampled rows a second time
+  bool few = false;
+  while (cudaMalloc(&ctx->arena, ctx->arena_bytes) != cudaSuccess) {
     cudaGetLastError();
-    delete ctx;
-    return VVS_ERR_NOMEM;
+    ctx->arena = nullptr;
+    const size_t less = layout(*desc, tmp, nullptr, true);
+    if (few || less >= ctx->arena_bytes) { delete ctx; return VVS_ERR_NOMEM; }
+    few = true;
+    ctx->arena_bytes = less;
   }
-  layout(*desc, ctx->ws, static_cast<char*>(ctx->arena));
-  if (cudaMemset(ctx->arena, 0, ctx->arena_bytes) != cudaSuccess) { vvs_destroy(ctx); return VVS_ERR_CUDA; }
+  layout(*desc, ctx->ws, static_cast<char*>(ctx->arena), few);
+  if (cudaMemset(ctx->arena, 0, ctx->ws.cleared_bytes) != cudaSuccess) { vvs_destroy(ctx); return VVS_ERR_CUDA; }
   // rotation angle per unit coordinate of each consecutive pair
   const int half = desc->head_dim / 2;
   if (half > 0) {

@@ -91,7 +91,7 @@ struct Workspace {
   float* ss_part = nullptr;      // [M][d / 16] partial sums of squares of the residual rows
   int32_t* seq_order = nullptr;  // [R] sequences by descending fill level (longest attention items first)
   uint32_t* anc_mask = nullptr;  // [M] bit j set: block row j of the same sequence is visible (ancestor or self)
-  double* tree_res = nullptr;    // [2][max_rows, V] residuals of the tree walk (ping-pong)
+  double* tree_res = nullptr;    // [2][max_rows, V] residuals of the tree walk (ping-pong); over logits_small where there is one
   int32_t* tree_path = nullptr;  // [max_rows, 32] accepted nodes when the caller does not ask for them
   float* rope_cos = nullptr;     // [M, head_dim/2]
   float* rope_sin = nullptr;     // [M, head_dim/2]
@@ -116,6 +116,7 @@ struct Workspace {
   float* cs_ss2 = nullptr;
   unsigned* cs_flags = nullptr;  // [n_layers * 5 + 2] stage arrival counters, embedding counter, abort word
   int32_t* status = nullptr; // device status word
+  size_t cleared_bytes = 0;  // what vvs_create clears: all but logits_small and tree_res
 };
 
 struct Layer {
