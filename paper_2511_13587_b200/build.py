@@ -1,5 +1,5 @@
 """Builds the CUDA library (sm_100a) in-tree with nvcc: csrc/*.cu -> lib/libvvs.so, and the CPython
-entry points that marshal its calls: csrc/binding_native.c -> _native.so.
+entry points that marshal its calls: csrc/binding_native.c -> _native.<ABI of this interpreter>.so.
 
 nvcc cross-compiles without a GPU.  Objects go to _build/ (not committed); the shared library
 stays inside the package so that it travels with the source tree."""
@@ -18,7 +18,9 @@ LIB_DIR = os.path.join(PKG, "lib")
 LIB = os.path.join(LIB_DIR, "libvvs.so")
 OBJ_DIR = os.path.join(PKG, "_build")
 NATIVE_SRC = os.path.join(CSRC, "binding_native.c")
-NATIVE = os.path.join(PKG, "_native.so")
+# named for this interpreter: another version does not take it for its own, neither to load nor as built already
+NATIVE = os.path.join(PKG, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
+NATIVE_UNTAGGED = os.path.join(PKG, "_native.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -87,6 +89,8 @@ def build_native(force: bool = False) -> str:
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"gcc failed for {NATIVE_SRC}:\n{r.stdout}\n{r.stderr}")
+    if os.path.exists(NATIVE_UNTAGGED):       # of an earlier build: any interpreter without one of its own would load it
+        os.remove(NATIVE_UNTAGGED)
     return NATIVE
 
 
