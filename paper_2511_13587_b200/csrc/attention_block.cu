@@ -25,29 +25,9 @@ namespace {
 using bf16 = __nv_bfloat16;
 constexpr int kMaxT = 32;      // block rows per sequence
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ uint32_t mapa0(uint32_t addr) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
-  return r;
-}
 __device__ __forceinline__ void st_async2(uint32_t addr, uint32_t bar, float a, float b) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
                ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
-}
-__device__ __forceinline__ bool try_wait_cluster(uint64_t* bar) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(tc::smem_u32(bar)) : "memory");
-  return ok != 0;
 }
 
 // shared memory: rings of the W warps, over which the merge buffers lie afterwards; then, in a cluster, the states of
@@ -83,7 +63,7 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
       tc::mbar_expect_tx(&x_bar, rank == 0 ? (uint32_t)((S - 1) * T * (HD + 2) * 4) : 0u);
     }
     __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    tc::cluster_arrive();
   }
   const int n_items = a.n_heads * a.n_rows, G = (int)gridDim.x;
   // More items than the GPU holds CTAs: the grid is one wave, and its CTAs walk the list forth and back (longest first).
@@ -111,14 +91,14 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
         const int idx = lane + u * 32, which = idx / (16 * per_row), rem = idx - which * 16 * per_row;
         const int key = rem / per_row, ch = rem - key * per_row;
         if (key < rows)
-          cp_async16(dst0 + (uint32_t)(which * NC + (ch >> 3)) * 2048u + key * 128 + (((ch & 7) ^ (key & 7)) << 4),
+          tc::cp_async16(dst0 + (uint32_t)(which * NC + (ch >> 3)) * 2048u + key * 128 + (((ch & 7) ^ (key & 7)) << 4),
                      (which ? vp : kp) + (size_t)(s * 16 + key) * HD + ch * 8);
       }
     };
 #pragma unroll
     for (int i = 0; i < D; ++i) {
       if (first + i * stride < n_old) request(i);
-      cp_async_commit();
+      tc::cp_async_commit();
     }
     if (k == 0) tc::pdl_launch_dependents();      // the projection after this kernel may start fetching its weights
     uint32_t anc[NMT][2];
@@ -135,7 +115,7 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
       const int s = first + i * stride;
       if (s >= n_old && s < n_slices) request(i);
     }
-    cp_async_commit();
+    tc::cp_async_commit();
     uint32_t qa[NMT][HD / 16][4];
 #pragma unroll
     for (int mi = 0; mi < NMT; ++mi) {
@@ -167,7 +147,7 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
       const int s = first + i * stride;
       // groups so far: D before the wait, one after it, one per iteration; slice i is in one of the oldest i + 2 of them
       // unless it was requested after the wait
-      if (s >= n_old) cp_async_wait<0>(); else cp_async_wait<D - 1>();
+      if (s >= n_old) tc::cp_async_wait<0>(); else tc::cp_async_wait<D - 1>();
       __syncwarp();
       const uint32_t k_base = ring + (uint32_t)(i % D) * L::kSlice, v_base = k_base + NC * 2048u;
       const int left = n_keys - s * 16, old = fill - s * 16;    // valid keys of the slice; old ones among them
@@ -185,9 +165,9 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
       }
       __syncwarp();                                             // every lane is done with the ring slot
       if (first + (i + D) * stride < n_slices) request(i + D);
-      cp_async_commit();
+      tc::cp_async_commit();
     }
-    cp_async_wait<0>();
+    tc::cp_async_wait<0>();
     // ---- merge: every warp leaves (max, normaliser, output) of its rows, the CTA folds them in warp order --
     __syncthreads();                                            // the rings have drained everywhere
     float* s_o = reinterpret_cast<float*>(smem);                // [W][NMT * 16][kLd]
@@ -211,10 +191,10 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
         }
       }
     __syncthreads();
-    if (S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // rank 0's barrier is ready
+    if (S > 1) tc::cluster_wait();   // rank 0's barrier is ready
     float* xbuf = reinterpret_cast<float*>(smem + L::kMain);    // [S - 1][T][HD + 2]
-    const uint32_t x_bar0 = S > 1 ? mapa0(tc::smem_u32(&x_bar)) : 0u;
-    const uint32_t xbuf0 = S > 1 ? mapa0(tc::smem_u32(xbuf)) : 0u;
+    const uint32_t x_bar0 = S > 1 ? tc::mapa(tc::smem_u32(&x_bar), 0) : 0u;
+    const uint32_t xbuf0 = S > 1 ? tc::mapa(tc::smem_u32(xbuf), 0) : 0u;
     bool waited = S == 1;
     for (int idx = tid; idx < T * (HD / 2); idx += 32 * W) {
       const int t = idx / (HD / 2), cp = idx - t * (HD / 2);
@@ -243,7 +223,7 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
       if (!waited) {
         // the peers' loops hold no unbounded wait; the limit only guards against a CTA that never runs
         bool got = false;
-        for (uint32_t i = 0; i < 4u * tc::kSpinLimit && !got; ++i) got = try_wait_cluster(&x_bar);
+        for (uint32_t i = 0; i < 4u * tc::kSpinLimit && !got; ++i) got = tc::mbar_try_wait_cluster(&x_bar, 0);
         if (!got) atomicOr(a.status, VVS_DEV_TIMEOUT);
         waited = true;
       }

@@ -51,23 +51,6 @@ struct Layout {
   static_assert((kWarps / 2 + 2) * kRegs * 32 * 4 <= kStages * kStage, "merge buffers must fit in the ring");
 };
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ float ld_cluster_f32(uint32_t local_addr, uint32_t rank) {
-  uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local_addr), "r"(rank));
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
-  return v;
-}
-
 template <int HD>
 __global__ void __launch_bounds__(kThreads) attention_rows_kernel(AttentionRowsArgs a) {
   using L = Layout<HD>;
@@ -103,10 +86,10 @@ __global__ void __launch_bounds__(kThreads) attention_rows_kernel(AttentionRowsA
         const int rem = idx - which * n, key = rem / per_row, ch = rem - key * per_row;
         const uint32_t dst = stage + (uint32_t)(which * NC + (ch >> 3)) * L::kTile + key * 128 +
                              (((ch & 7) ^ (key & 7)) << 4);
-        cp_async16(dst, (which ? v_src : k_src) + (size_t)key * HD + ch * 8);
+        tc::cp_async16(dst, (which ? v_src : k_src) + (size_t)key * HD + ch * 8);
       }
     }
-    cp_async_commit();
+    tc::cp_async_commit();
   };
   for (int s = 0; s < kStages - 1; ++s) request(s);
   tc::pdl_launch_dependents();      // the projection after this kernel may start fetching its weights
@@ -201,7 +184,7 @@ __global__ void __launch_bounds__(kThreads) attention_rows_kernel(AttentionRowsA
   for (int j = 0; j < nb; ++j) {
     const int blk = rank + j * S;
     request(j + kStages - 1);
-    cp_async_wait<kStages - 1>();
+    tc::cp_async_wait<kStages - 1>();
     __syncthreads();
     const uint32_t k_base = s_base + (uint32_t)(j % kStages) * L::kStage;
     const uint32_t v_base = k_base + NC * L::kTile;
@@ -217,7 +200,7 @@ __global__ void __launch_bounds__(kThreads) attention_rows_kernel(AttentionRowsA
     }
     __syncthreads();                              // the slot is requested again two iterations on
   }
-  cp_async_wait<0>();
+  tc::cp_async_wait<0>();
   // ---- the block's own keys: ancestors and the row itself, by the last warp of each m-tile ----------
   if (ok && own_keys && kg == wpm - 1) {
     const uint32_t k_base = tc::smem_u32(s_new), v_base = k_base + NC * L::kNewTile;
@@ -283,7 +266,7 @@ __global__ void __launch_bounds__(kThreads) attention_rows_kernel(AttentionRowsA
       xslot[(NJ * 4 + 2) * 32 + lane] = st.l[0];
       xslot[(NJ * 4 + 3) * 32 + lane] = st.l[1];
     }
-    cluster_sync_all();
+    tc::cluster_sync();
     if (rank == 0) {
       // every rank has read its q / k / v sums long ago: clear them for the next layer
       for (int idx = tid; idx < T * HALF; idx += kThreads) {
@@ -300,8 +283,8 @@ __global__ void __launch_bounds__(kThreads) attention_rows_kernel(AttentionRowsA
         for (int q = 1; q < S; ++q) {
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
-            const float mo = ld_cluster_f32(xaddr + (uint32_t)((NJ * 4 + i) * 32 + lane) * 4u, (uint32_t)q);
-            const float lo = ld_cluster_f32(xaddr + (uint32_t)((NJ * 4 + 2 + i) * 32 + lane) * 4u, (uint32_t)q);
+            const float mo = tc::ld_cluster_f32(xaddr + (uint32_t)((NJ * 4 + i) * 32 + lane) * 4u, (uint32_t)q);
+            const float lo = tc::ld_cluster_f32(xaddr + (uint32_t)((NJ * 4 + 2 + i) * 32 + lane) * 4u, (uint32_t)q);
             const float m_new = fmaxf(st.m[i], mo);
             const float m_safe = m_new == -CUDART_INF_F ? 0.f : m_new;
             const float aa = ex2(st.m[i] - m_safe), bb = ex2(mo - m_safe);
@@ -309,8 +292,8 @@ __global__ void __launch_bounds__(kThreads) attention_rows_kernel(AttentionRowsA
             st.l[i] = st.l[i] * aa + lo * bb;
 #pragma unroll
             for (int j = 0; j < NJ; ++j) {
-              const float o0 = ld_cluster_f32(xaddr + (uint32_t)((j * 4 + 2 * i) * 32 + lane) * 4u, (uint32_t)q);
-              const float o1 = ld_cluster_f32(xaddr + (uint32_t)((j * 4 + 2 * i + 1) * 32 + lane) * 4u, (uint32_t)q);
+              const float o0 = tc::ld_cluster_f32(xaddr + (uint32_t)((j * 4 + 2 * i) * 32 + lane) * 4u, (uint32_t)q);
+              const float o1 = tc::ld_cluster_f32(xaddr + (uint32_t)((j * 4 + 2 * i + 1) * 32 + lane) * 4u, (uint32_t)q);
               st.o[j][2 * i] = st.o[j][2 * i] * aa + o0 * bb;
               st.o[j][2 * i + 1] = st.o[j][2 * i + 1] * aa + o1 * bb;
             }
@@ -332,7 +315,7 @@ __global__ void __launch_bounds__(kThreads) attention_rows_kernel(AttentionRowsA
       }
     }
   }
-  if (S > 1) cluster_sync_all();      // no rank leaves while rank 0 may still read its state
+  if (S > 1) tc::cluster_sync();      // no rank leaves while rank 0 may still read its state
 }
 
 template <int HD>

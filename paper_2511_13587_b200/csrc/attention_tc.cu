@@ -45,16 +45,6 @@ struct AttnParams {
 
 __device__ __forceinline__ bool wait_bounded(uint64_t* bar, uint32_t parity) { return mbar_wait(bar, parity); }
 
-__device__ __forceinline__ float warp_max_f(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ float warp_sum_f(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
 template <int HD>
 __global__ void __launch_bounds__(128)

@@ -76,7 +76,6 @@ constexpr int kCT = kCW * 32;
 constexpr int kThreads = kCT + 128;         // + one warp group: weight producer warp, sequencer warp, two idle
 constexpr int kTP = 4;                      // weight tiles per sub-panel (accumulators held at once)
 constexpr int kGroupSpans = 20;             // 32-wide k spans per k group (one ring slot per tile and group)
-constexpr int kMaxSpw = (kGroupSpans + kCW - 1) / kCW;   // spans of a group per warp
 constexpr int kSlotBytes = kGroupSpans * 1024;
 constexpr int kMaxSlots = 8;
 constexpr int kActSlots = 2;                  // (the sequencer toggles between exactly two)
@@ -90,7 +89,6 @@ constexpr int kMaxBlocks = 1024;             // ring blocks of one layer of one 
 constexpr int kMaxOwn = 2;                   // 16-column tiles of the residual stream a CTA may own
 constexpr uint32_t kParkNs = 4000;
 constexpr uint32_t kParkedPolls = 1u << 19;   // ~2 s
-constexpr uint32_t kSpinPolls = 1u << 24;
 constexpr uint32_t kFlagPolls = 1u << 22;
 enum { ST_QKV = 0, ST_ATT = 1, ST_O = 2, ST_GU = 3, ST_DOWN = 4, N_ST = 5 };
 enum { G_QKV = 0, G_O = 1, G_GU = 2, G_DOWN = 3 };

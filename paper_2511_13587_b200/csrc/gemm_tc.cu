@@ -63,14 +63,6 @@ struct KernelParams {
   int ff;
 };
 
-// bounded wait that also gives up when another role of the CTA already did
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  for (uint32_t i = 0; i < kSpinLimit; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((i & 1023u) == 1023u && *abort_flag) return false;
-  }
-  return false;
-}
 
 template <int EPI>
 __device__ __forceinline__ void final_chunk(const KernelParams& p, int n, int tok_base, const float* v,
@@ -122,17 +114,6 @@ __device__ __forceinline__ void final_chunk(const KernelParams& p, int n, int to
   }
 }
 
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ float4 ld_cluster_f4(uint32_t local_addr, uint32_t rank) {
-  uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local_addr), "r"(rank));
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(remote) : "memory");
-  return v;
-}
 
 template <int EPI>
 __global__ void __launch_bounds__(128, 1)
@@ -251,8 +232,8 @@ gemm_tc_kernel(const KernelParams p, const __grid_constant__ CUtensorMap tm_a,
     if (__syncthreads_or(got ? 0 : 1)) {
       if (threadIdx.x == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
       if (EPI == GEMM_EPI_ADD && p.cluster_mode) {   // the other CTAs of the cluster wait on these two barriers
-        cluster_sync_all();
-        cluster_sync_all();
+        cluster_sync();
+        cluster_sync();
       }
       alive = false;
       break;
@@ -309,7 +290,7 @@ gemm_tc_kernel(const KernelParams p, const __grid_constant__ CUtensorMap tm_a,
         // The K splits of this (tile, token pass) are the CTAs of one cluster (cluster rank = split).
         // Rank r sums token rows r, r + splits, ... over all ranks' staged tiles in rank order and is
         // the only writer of those outputs.
-        cluster_sync_all();
+        cluster_sync();
         const uint32_t rank = (uint32_t)split, nrank = (uint32_t)p.splits;
         const int mine = ntok > (int)rank ? (ntok - (int)rank + (int)nrank - 1) / (int)nrank : 0;
         const uint32_t sT_addr = smem_u32(sT);
@@ -336,7 +317,7 @@ gemm_tc_kernel(const KernelParams p, const __grid_constant__ CUtensorMap tm_a,
               if (n_base + g4 + e < p.n) dst[e] = (p.cluster_mode == 2 ? dst[e] : 0.f) + a4[e];
           }
         }
-        cluster_sync_all();      // nobody leaves while its tile may still be read
+        cluster_sync();      // nobody leaves while its tile may still be read
       } else
       for (int idx = threadIdx.x; idx < ntok * (int)(kTileRows / 4); idx += blockDim.x) {
         const int tk = idx >> 5, g4 = (idx & 31) * 4;

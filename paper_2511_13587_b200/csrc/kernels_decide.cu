@@ -4,6 +4,7 @@
 // (logits never written out).
 #include <math_constants.h>
 
+#include "tc_common.cuh"
 #include "vvs_internal.cuh"
 
 namespace vvs {
@@ -417,13 +418,6 @@ namespace {
 
 constexpr int kDecideThreads = 512, kDecideWarps = kDecideThreads / 32;
 
-__device__ __forceinline__ double ld_cluster_f64(const double* local, uint32_t rank) {
-  uint32_t a = (uint32_t)__cvta_generic_to_shared(local), r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  double v;
-  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
-  return v;
-}
 
 // LOGITS: rows hold guided logits, statistics come from the [rows, n_tiles] softmax partials; else probabilities.
 template <bool LOGITS>
@@ -641,13 +635,13 @@ __global__ void __launch_bounds__(kDecideThreads) decide_kernel(Workspace ws, De
     for (int w = 0; w < kDecideWarps; ++w) s += s_w[tid][w];
     s_seg[tid] = s;
   }
-  if (S > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (S > 1) tc::cluster_sync();
   else __syncthreads();
   if (warp == 0) {
     double seg[2] = {0.0, 0.0};
     if (lane < S) {
-      seg[0] = S > 1 ? ld_cluster_f64(&s_seg[0], lane) : s_seg[0];
-      seg[1] = S > 1 ? ld_cluster_f64(&s_seg[1], lane) : s_seg[1];
+      seg[0] = S > 1 ? tc::ld_cluster_f64(&s_seg[0], lane) : s_seg[0];
+      seg[1] = S > 1 ? tc::ld_cluster_f64(&s_seg[1], lane) : s_seg[1];
     }
     const double total_r = warp_sum_d(seg[0]), total_p = warp_sum_d(seg[1]);
     const int use_p = total_r > 0.0 ? 0 : 1;          // p == q numerically: fall back to the target row itself
@@ -662,7 +656,7 @@ __global__ void __launch_bounds__(kDecideThreads) decide_kernel(Workspace ws, De
       s_part = has_row && total > 0.0 ? part : -1;
     }
   }
-  if (S > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // (waited for at the end)
+  if (S > 1) tc::cluster_arrive();   // (waited for at the end)
   __syncthreads();
   // ---- the sample point: smallest index whose cumulative mass exceeds t, in the part that holds it -----------------
   if (s_part < 0) {
@@ -716,7 +710,7 @@ __global__ void __launch_bounds__(kDecideThreads) decide_kernel(Workspace ws, De
       }
     }
   }
-  if (S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // nobody leaves while its sums may be read
+  if (S > 1) tc::cluster_wait();      // nobody leaves while its sums may be read
 }
 
 }  // namespace

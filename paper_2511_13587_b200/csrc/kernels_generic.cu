@@ -4,6 +4,7 @@
 // in-library cross-check of the bf16 tensor-core kernels.
 #include <math_constants.h>
 
+#include "tc_common.cuh"
 #include "vvs_internal.cuh"
 
 namespace vvs {
@@ -263,24 +264,6 @@ struct RowGemm {
   int d, n_heads, hd, s_max, rope_mode, grid_w, n_prefix, layer, kv_rows, t_len;
 };
 
-// Sums of eight values over the warp: the lanes trade half of what they hold three times (9 shuffles instead of 40); lanes
-// 4 i .. 4 i + 3 get the sum of value i.
-__device__ __forceinline__ float sum_rows(float (&v)[8], int lane) {
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    const int o = 16 >> s, half = 4 >> s;
-    const bool up = lane & o;
-#pragma unroll
-    for (int j = 0; j < half; ++j) {
-      const float mine = up ? v[half + j] : v[j], theirs = up ? v[j] : v[half + j];
-      v[j] = mine + __shfl_xor_sync(0xffffffffu, theirs, o);
-    }
-  }
-  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
-  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-  return v[0];
-}
-
 template <typename T, int EPI>
 __global__ void __launch_bounds__(128) row_gemm_kernel(const RowGemm<T> p) {
   constexpr int VEC = VecOf<T>::n, MT = 8;
@@ -383,10 +366,10 @@ __global__ void __launch_bounds__(128) row_gemm_kernel(const RowGemm<T> p) {
   }
   float v[NW];                                   // lanes 4 i .. 4 i + 3 keep row m0 + i
 #pragma unroll
-  for (int r = 0; r < NW; ++r) v[r] = sum_rows(acc[r], lane);
+  for (int r = 0; r < NW; ++r) v[r] = tc::warp_sums(acc[r], lane);
   const int row = m0 + (lane >> 2);
   if (FOLD) {
-    const float rs = rsqrtf(sum_rows(ss, lane) / (float)k + p.eps);
+    const float rs = rsqrtf(tc::warp_sums(ss, lane) / (float)k + p.eps);
 #pragma unroll
     for (int r = 0; r < NW; ++r) v[r] *= rs;
     if (EPI == ROW_NORM_STORE && blockIdx.x == 0) {               // the normalised rows themselves, two per warp

@@ -18,6 +18,7 @@
 // x 32768 123 / 30; most accepted 11.3 / 11.2, 19.8 / 13.3, 45.2 / 13.8.
 #include <math_constants.h>
 
+#include "tc_common.cuh"
 #include "vvs_internal.cuh"
 
 namespace vvs {
@@ -76,32 +77,14 @@ __device__ double tw_block_sum(double v, double* s_warp) {
   return tot;
 }
 
-__device__ __forceinline__ void tw_cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t tw_remote(const void* local, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(local)), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ double tw_load_f64(const double* local, uint32_t rank) {
-  double v;
-  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(tw_remote(local, rank)) : "memory");
-  return v;
-}
-__device__ __forceinline__ int tw_load_s32(const int* local, uint32_t rank) {
-  int v;
-  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(tw_remote(local, rank)) : "memory");
-  return v;
-}
 // The sum of the CTAs' values at *slot, in rank order.  Consecutive calls take two slots in turn: a CTA that writes a slot
 // again has met every reader of it at the barrier of the call between.  The barrier also publishes what the CTAs have
 // written to global memory.
 __device__ __forceinline__ double tw_exchange(double v, double* slot, int S) {
   if (threadIdx.x == 0) *slot = v;
-  tw_cluster_sync();
+  tc::cluster_sync();
   double tot = 0.0;
-  for (int r = 0; r < S; ++r) tot += tw_load_f64(slot, (uint32_t)r);
+  for (int r = 0; r < S; ++r) tot += tc::ld_cluster_f64(slot, (uint32_t)r);
   return tot;
 }
 
@@ -188,7 +171,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
       if (s_pass) {
         // the next level's first residual may go where a slower CTA is still reading this one's; a rejection writes the other
         // buffer, whose readers have all met at the exchange before
-        if (CLUSTER && src >= 0) tw_cluster_sync();
+        if (CLUSTER && src >= 0) tc::cluster_sync();
         accepted = c;
         break;
       }
@@ -281,10 +264,10 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
   int last, owner = 0;
   if (CLUSTER) {
     if (tid == 0) s_slot[turn] = total;
-    tw_cluster_sync();                            // s_last is complete too
+    tc::cluster_sync();                            // s_last is complete too
     double sum = 0.0, part_sum[8];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) part_sum[r] = r < S ? tw_load_f64(&s_slot[turn], (uint32_t)r) : 0.0;
+    for (int r = 0; r < 8; ++r) part_sum[r] = r < S ? tc::ld_cluster_f64(&s_slot[turn], (uint32_t)r) : 0.0;
 #pragma unroll
     for (int r = 0; r < 8; ++r) sum += part_sum[r];
     target = u * sum;
@@ -299,10 +282,10 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
       if (owner < 0 && ahead > target) owner = r;
     }
     if (owner < 0)                                // the point rounds to the end: the last code with mass, wherever it is
-      for (int r = 0; r < S; ++r) last = max(last, tw_load_s32(&s_last, (uint32_t)r));
+      for (int r = 0; r < S; ++r) last = max(last, tc::ld_cluster_s32(&s_last, (uint32_t)r));
     else
       last = s_last;
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");     // (waited for at the end)
+    tc::cluster_arrive();     // (waited for at the end)
   }
   const double excl = before + incl - local;
   if (owner == rank) {
@@ -338,7 +321,7 @@ __global__ void __launch_bounds__(kTreeThreads) tree_walk_kernel(TreeParams p) {
       if (p.n_commit) p.n_commit[r] = F + n_acc;
     }
   }
-  if (CLUSTER) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // nobody leaves while it may be read
+  if (CLUSTER) tc::cluster_wait();   // nobody leaves while it may be read
 }
 
 // K/V of the accepted nodes move from their block slots fill + node to fill + F + i (i-th

@@ -36,13 +36,6 @@ struct Params {
   int32_t* status;
 };
 
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  for (uint32_t i = 0; i < kSpinLimit; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((i & 1023u) == 1023u && *abort_flag) return false;
-  }
-  return false;
-}
 
 __global__ void __launch_bounds__(kThreads, 2)
 lmhead_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b) {
@@ -176,19 +169,8 @@ lmhead_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, cons
       }
 #pragma unroll
       for (int j = 0; j < 16; ++j) l[j] = mx[j] > -CUDART_INF_F ? expf(l[j] - mx[j]) : 0.f;
-      // sixteen sums over 32 lanes: halve the rows a lane keeps four times
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int o = 16 >> k, half = 8 >> k;
-        const bool up = lane & o;
-#pragma unroll
-        for (int j = 0; j < half; ++j) {
-          const float mine = up ? l[half + j] : l[j], theirs = up ? l[j] : l[half + j];
-          l[j] = mine + __shfl_xor_sync(0xffffffffu, theirs, o);
-        }
-      }
-      l[0] += __shfl_xor_sync(0xffffffffu, l[0], 1);
-      const int j0 = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
+      warp_sums(l, lane);
+      const int j0 = warp_sums_index<16>(lane);
       float m0 = mx[0];
 #pragma unroll
       for (int j = 1; j < 16; ++j) m0 = j == j0 ? mx[j] : m0;

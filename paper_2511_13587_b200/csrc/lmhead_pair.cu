@@ -40,14 +40,6 @@ struct Params {
   int32_t* status;
 };
 
-__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // load into this CTA, bytes counted on a barrier of the pair (cluster address)
 __device__ __forceinline__ void tma_load_pair(void* dst, const CUtensorMap* m, uint32_t bar, int x, int y) {
   asm volatile(
@@ -73,19 +65,10 @@ __device__ __forceinline__ void commit_pair(uint64_t* bar) {
 __device__ __forceinline__ void arrive_remote(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ bool try_wait_cluster(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-  return ok != 0;
-}
 // bounded wait; gives up when another role of the CTA already did
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* status) {
   for (uint32_t i = 0; i < kSpinLimit; ++i) {
-    if (try_wait_cluster(bar, parity)) return true;
+    if (mbar_try_wait_cluster(bar, parity)) return true;
     if ((i & 1023u) == 1023u && *abort_flag) return false;
   }
   *abort_flag = 1;
@@ -126,7 +109,7 @@ lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, con
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  cluster_sync_all();                             // both CTAs' barriers are ready
+  cluster_sync();                             // both CTAs' barriers are ready
   const uint32_t tmem = tmem_slot;
   pdl_launch_dependents();
 
@@ -183,7 +166,7 @@ lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, con
       }
       if (!ok && rank == 0) {                     // gave up: nothing may be in flight when the pair leaves (bounded)
         for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
-          for (uint32_t k = 0; k < kSpinLimit && !try_wait_cluster(&full_bar[i % p.stages], (i / p.stages) & 1); ++k) {}
+          for (uint32_t k = 0; k < kSpinLimit && !mbar_try_wait_cluster(&full_bar[i % p.stages], (i / p.stages) & 1); ++k) {}
       }
     }
   } else if (warp == 1 && rank == 0) {
@@ -284,7 +267,7 @@ lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, con
   pdl_wait();
   tc_fence_before();
   __syncthreads();
-  cluster_sync_all();                             // no CTA leaves while the pair's MMAs or signals may still reach it
+  cluster_sync();                             // no CTA leaves while the pair's MMAs or signals may still reach it
   tc_fence_after();
   if (warp == 2) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }

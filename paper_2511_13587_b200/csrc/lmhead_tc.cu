@@ -51,13 +51,6 @@ struct LmParams {
   const int32_t* sel_row; const float* stat_m; const float* stat_inv; float* p_row;
 };
 
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  for (uint32_t i = 0; i < kSpinLimit; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((i & 1023u) == 1023u && *abort_flag) return false;
-  }
-  return false;
-}
 
 // NM = codebook tiles of 128 rows per CTA.  With NM = 2 the feature tile of a k-block is read from L2
 // once for 256 codes (two MMAs on one B operand, two accumulators side by side in TMEM): half the

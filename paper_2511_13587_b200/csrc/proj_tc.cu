@@ -42,33 +42,9 @@ struct Params {
   const uint8_t* ahead[2]; uint32_t ahead_bytes;      // weights of the projection after next, to be brought into L2
 };
 
-// bounded wait that also gives up when another role of the CTA already did
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  for (uint32_t i = 0; i < kSpinLimit; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((i & 1023u) == 1023u && *abort_flag) return false;
-  }
-  return false;
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
 __device__ __forceinline__ void st_async4(uint32_t addr, uint32_t bar, const float* v) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
                ::"r"(addr), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(bar) : "memory");
-}
-__device__ __forceinline__ bool try_wait_cluster(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-  return ok != 0;
 }
 __device__ __forceinline__ void prefetch_l2(const void* ptr, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(ptr), "r"(bytes) : "memory");
@@ -209,20 +185,8 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
 #pragma unroll
         for (int j = 0; j < 8; ++j) ss[j] += (v[j].x + v[j].y) + (v[j].z + v[j].w);
       }
-      // eight sums over 32 lanes: halve the tokens a lane keeps three times, then add what is left
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const int o = 16 >> k, half = 4 >> k;
-        const bool up = lane & o;
-#pragma unroll
-        for (int j = 0; j < half; ++j) {
-          const float mine = up ? ss[half + j] : ss[j], theirs = up ? ss[j] : ss[half + j];
-          ss[j] = mine + __shfl_xor_sync(0xffffffffu, theirs, o);
-        }
-      }
-      ss[0] += __shfl_xor_sync(0xffffffffu, ss[0], 2);
-      ss[0] += __shfl_xor_sync(0xffffffffu, ss[0], 1);
-      const int j = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+      warp_sums(ss, lane);
+      const int j = warp_sums_index<8>(lane);
       if ((lane & 3) == 0 && t0 + j < kMaxTok) s_rs[t0 + j] = rsqrtf(ss[0] * p.inv_d + p.eps);
     }
   }
@@ -311,19 +275,8 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
           y[j] = xn * gsc1;
           sq[j] = ok ? xn * xn : 0.f;
         }
-        // sixteen sums over 32 lanes: halve the tokens a lane keeps four times
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int o = 16 >> k, half = 8 >> k;
-          const bool up = lane & o;
-#pragma unroll
-          for (int j = 0; j < half; ++j) {
-            const float mine = up ? sq[half + j] : sq[j], theirs = up ? sq[j] : sq[half + j];
-            sq[j] = mine + __shfl_xor_sync(0xffffffffu, theirs, o);
-          }
-        }
-        sq[0] += __shfl_xor_sync(0xffffffffu, sq[0], 1);
-        const int j = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
+        warp_sums(sq, lane);
+        const int j = warp_sums_index<16>(lane);
         if (!odd && c0 + j < ntok) p.ss_out[(size_t)(tok0 + c0 + j) * p.ss_out_parts + tile * 4 + (warp & 3)] = sq[0];
       } else {
 #pragma unroll
@@ -417,7 +370,7 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
   {
     // peers push after waits of at most kSpinLimit polls each, so this longer wait ends after their pushes
     bool got = false;
-    for (uint32_t i = 0; i < 16u * kSpinLimit && !got; ++i) got = try_wait_cluster(&recv_bar, 0);
+    for (uint32_t i = 0; i < 16u * kSpinLimit && !got; ++i) got = mbar_try_wait_cluster(&recv_bar, 0);
     if (!got && lane == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
   }
 

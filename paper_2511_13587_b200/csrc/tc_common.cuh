@@ -77,6 +77,24 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) { retu
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// Bounded wait that also gives up when another role of the CTA already did.
+__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  for (uint32_t i = 0; i < kSpinLimit; ++i) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((i & 1023u) == 1023u && *abort_flag) return false;
+  }
+  return false;
+}
+// The same test for a barrier that other CTAs of the cluster arrive on or write behind.
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+  return ok != 0;
+}
 // Named barrier among `n_threads` threads of the CTA (n_threads a multiple of 32).
 __device__ __forceinline__ void named_bar_sync(int id, int n_threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n_threads) : "memory");
@@ -86,6 +104,76 @@ __device__ __forceinline__ void fence_barrier_init() {
 }
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
+// ---- thread-block cluster ----------------------------------------------------------------------------
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() {
+  cluster_arrive();
+  cluster_wait();
+}
+// address of this CTA's shared location in the CTA of the given rank
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float ld_cluster_f32(uint32_t local_addr, uint32_t rank) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(mapa(local_addr, rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t local_addr, uint32_t rank) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(mapa(local_addr, rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ double ld_cluster_f64(const double* local, uint32_t rank) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(mapa(smem_u32(local), rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ int ld_cluster_s32(const int* local, uint32_t rank) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(mapa(smem_u32(local), rank)) : "memory");
+  return v;
+}
+
+// ---- 16-byte asynchronous copies of a thread -----------------------------------------------------------
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// ---- sums over a warp ------------------------------------------------------------------------------------
+// N sums of 32 lanes each: the lanes trade half of what they hold, log2(N) times, then add what is left (N = 16: 16 shuffles in
+// the place of 80).  Returned, and in v[0], is the sum of value warp_sums_index<N>(lane).
+template <int N>
+__device__ __forceinline__ float warp_sums(float (&v)[N], int lane) {
+  constexpr int kSteps = N == 16 ? 4 : 3;
+  static_assert(N == 16 || N == 8, "eight or sixteen sums");
+#pragma unroll
+  for (int k = 0; k < kSteps; ++k) {
+    const int o = 16 >> k, half = (N / 2) >> k;
+    const bool up = lane & o;
+#pragma unroll
+    for (int j = 0; j < half; ++j) {
+      const float mine = up ? v[half + j] : v[j], theirs = up ? v[j] : v[half + j];
+      v[j] = mine + __shfl_xor_sync(0xffffffffu, theirs, o);
+    }
+  }
+#pragma unroll
+  for (int o = 16 >> kSteps; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+template <int N>
+__device__ __forceinline__ int warp_sums_index(int lane) {
+  const int j = ((lane >> 4) & 1) * (N / 2) + ((lane >> 3) & 1) * (N / 4) + ((lane >> 2) & 1) * (N / 8);
+  return N == 16 ? j + ((lane >> 1) & 1) : j;
 }
 
 // ---- TMA -----------------------------------------------------------------------------------------
