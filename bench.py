@@ -26,22 +26,39 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 from vvs_synth import gen, philox  # noqa: E402
-from vvs_synth.configs import CONFIGS, MODE_RELAXED  # noqa: E402
+from vvs_synth.configs import CONFIGS, DTYPE_FP32, MODE_RELAXED  # noqa: E402
 
 # dram__bytes_read.sum + dram__bytes_write.sum of ONE STEP (all launches of a verify call), summed over an
 # ncu capture summarised under profiles/.  Keyed by (workload, fixed-order sums); each entry names the
 # kernel sources the step runs and the first 16 hex digits of the SHA-256 over their concatenation when
 # the counters were taken: the line reports null, and says why, once any of them has changed.
 STEP_SOURCES = ("proj_tc.cu", "attention_block.cu", "gemm_tc.cu", "lmhead_few.cu", "lmhead_pair.cu", "kernels_generic.cu",
-                "kernels_decide.cu")
-NCU_CAPTURES = {
-    (1, False): ("1748279beacd934c", 1.5709e+09, "profiles/verify_step_configs1_per_projection_launch_list_and_counters.txt"),
-    (1, True): ("1748279beacd934c", 1.5459e+09, "profiles/verify_step_configs1_per_projection_launch_list_and_counters.txt"),
-    (2, False): ("1748279beacd934c", 4.4629e+09, "profiles/verify_step_configs2_launch_list_and_counters.txt"),
-    (2, True): ("1748279beacd934c", 4.0170e+09, "profiles/verify_step_configs2_launch_list_and_counters.txt"),
+                "kernels_decide.cu", "launch_plans.h", "tc_common.cuh", "att_mma.cuh")
+NCU_CAPTURES = {       # (both settings of deterministic run the same kernels here)
+    (1, False): ("f8515c40e0eb62c2", 1.588e+09, "profiles/folded_step_launches.txt"),
+    (1, True): ("f8515c40e0eb62c2", 1.588e+09, "profiles/folded_step_launches.txt"),
+    (2, False): ("f8515c40e0eb62c2", 3.788e+09, "profiles/folded_step_launches.txt"),
+    (2, True): ("f8515c40e0eb62c2", 3.788e+09, "profiles/folded_step_launches.txt"),
 }
 N_TRIALS = 32           # distinct (fill, block, draft) inputs cycled through the steps
 DRAFT_LOGIT_STD = 1.0   # target-independent drafter: q = softmax(N(0, std^2))
+
+
+def sums_name(ms, deterministic: bool, chain_kernels: bool = False) -> str:
+    """In which order a step of this model takes its split sums."""
+    if ms.dtype == DTYPE_FP32:
+        return "fixed order (float32 contexts know no other)"
+    if ms.d_model >= 1024 and not chain_kernels:
+        return "rank order inside a cluster, bitwise repeatable (the same kernels for either value of deterministic)"
+    return "fixed order (bitwise repeatable)" if deterministic else "arrival order (split-K adds in L2)"
+
+
+def kernels_name(ms, chain_kernels: bool = False) -> str:
+    if chain_kernels:
+        return "whole-chain kernels (previous generation, debug switch)"
+    if ms.dtype == DTYPE_FP32:
+        return "five float32 kernels per layer, norms and epilogues folded in"
+    return "five kernels per layer, epilogues folded in" if ms.d_model >= 1024 else "nine kernels per layer"
 
 
 def metric_name(wl) -> str:
@@ -386,7 +403,7 @@ class VerifyBench:
             # dependents: no single kernel dominates, so the object describes the whole step (all launches
             # of one verify call).  The class times below are taken with events BETWEEN the launches, which
             # removes that overlap: they add up to more than the step and only rank the classes.
-            name = "whole step (per-projection GEMM, attention and element-wise launches together)"
+            name = "whole step (projection, attention, LM head and decision launches together)"
             dom_ms, dom_bytes, dom_launches = ms_step, alg["total"], sum(cls_n) / n_prof
         achieved = dom_bytes / (dom_ms * 1e-3) / 1e9 if dom_ms > 0 else 0.0
         return {"kernel": name, "bound": "hbm", "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s",
@@ -521,9 +538,8 @@ def run_ours(args) -> None:
         "config": {"workload": f"configs[{args.workload}] {wl.name}", "n_images": b, "n_cfg": cfg,
                    "n_draft": k, "block_rows": t_len, "fill": f"U[{wl.fill_lo},{wl.fill_hi}] per trial",
                    "trials": len(S.trials), "draft": S.drafter,
-                   "sums": "fixed order (bitwise repeatable)" if args.deterministic else "arrival order (split-K adds in L2)",
-                   "kernels": "whole-chain kernels (previous generation, debug switch)" if args.chain_kernels
-                              else "five kernels per layer, epilogues folded in",
+                   "sums": sums_name(wl.shape, bool(args.deterministic), args.chain_kernels),
+                   "kernels": kernels_name(wl.shape, args.chain_kernels),
                    "timing": "median over `repeats` regions of `steps` steps each, every region bracketed by barrier + synchronize",
                    "l2": f"weights streamed per step ({alg['weights'] / 1e9:.2f} GB) exceed the 126 MB L2; no flush needed"
                          if alg["weights"] > 126e6 else "weights fit in L2: a latency case, not a bandwidth case",
@@ -567,8 +583,8 @@ def quick_measure(index: int, deterministic: bool, steps: int, pk: dict, min_ms:
     alg = algorithmic_bytes(S.wl, S.trials)
     res = {"workload": f"configs[{index}] {S.wl.name}", "ms_per_step": ms_step, "steps": steps, "repeats": len(regions),
            "drafts_per_s": S.drafts_per_step(steps) / (ms_step * 1e-3), "launches_per_step": launches,
-           "sums": "fixed order" if deterministic else "arrival order",
-           "kernels": "whole-chain (previous generation)" if chain_kernels else "per-projection",
+           "sums": sums_name(S.wl.shape, deterministic, chain_kernels),
+           "kernels": kernels_name(S.wl.shape, chain_kernels),
            "algorithmic_bytes": alg["total"], "step_frac_of_measured_hbm": alg["total"] / (ms_step * 1e-3) / 1e9 / pk["hbm_gbs"],
            "roofline": {n: roof[n] for n in ("kernel", "achieved", "frac", "ms_per_launch", "class_ms_per_step")},
            "acceptance": S.acceptance(), "device_status": S.vb.vvs_device_status(S.ctx)}
@@ -935,10 +951,11 @@ def main() -> None:
     ap.add_argument("--sweep-point", type=int, default=None, choices=range(len(SWEEP_POINTS)),
                     help="with --workload 4: run this one point of the sweep only")
     ap.add_argument("--deterministic", type=int, default=0, choices=[0, 1],
-                    help="1: fixed-order sums (bitwise repeatable), 0: arrival-order split-K sums (faster)")
+                    help="1: fixed-order sums (bitwise repeatable), 0: split-K sums may arrive in any order (only models narrower "
+                         "than 1024 use it, and are faster for it)")
     ap.add_argument("--chain-kernels", action="store_true",
                     help="time the persistent whole-chain kernels of the previous generation (calls of at most 32 "
-                         "tokens) instead of the per-projection kernels")
+                         "tokens) instead of the folded step")
     ap.add_argument("--cpu-steps", type=int, default=2)   # 5-16 s of host time at configs[1], depending on the host
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--min-ms", type=float, default=500.0,

@@ -108,8 +108,9 @@ typedef struct vvs_model_desc {
                             0 = split-K partial sums may be added in L2 in arrival order; the last bits of
                                 the logits can then differ from run to run, and a residual sample over
                                 many nearly equally likely codes need not repeat.  Only models of d_model
-                                below 1024 are faster for it (by a quarter to a third per step); wider
-                                ones add in rank order either way.
+                                below 1024 are faster for it (24 layers of 512 or 768 columns, 18 to 288
+                                tokens: 17 to 30 % less time per step); wider ones add in rank order
+                                either way.
                             float32 contexts are always repeatable. */
 } vvs_model_desc;
 

@@ -274,7 +274,7 @@ int launch_variant(const AttentionBlockArgs& a, int split, int per_sm, cudaStrea
 
 }  // namespace
 
-// Warps per item by how many items there are: with few, one item's slices over many warps (XL shape, step of 18 tokens
+// CTAs per item: attention_split (launch_plans.h).  Warps per item by how many items there are: with few, one item's slices over many warps (XL shape, step of 18 tokens
 // with 16, 8 and 4 warps 962, 1004 and 1013 us; 54 tokens, two row groups of 8 warps 1184, of 4 warps 1286, four warps
 // with two m-tiles each 1272); with many, small CTAs (288 tokens, 640 items: 4 warps, three CTAs per SM 1.88 ms, 8 warps
 // 2.07 ms).  The item loop let the compiler keep addresses in registers: 160 instead of 128 a thread, three CTAs per SM

@@ -715,8 +715,10 @@ __global__ void __launch_bounds__(kDecideThreads) decide_kernel(Workspace ws, De
 
 }  // namespace
 
-// Parts of a codebook: 2048 codes or more each, eight CTAs (the portable cluster) at most -- fewer where the images
-// alone fill the GPU.
+// Parts of a codebook: 2048 codes or more each, eight CTAs (the portable cluster) at most, whatever the number of images.
+// One / two / four / eight CTAs, strict, 16 images: 4096 codes 4.8 / 5.4 / 5.4 / 5.7 us, 8192 codes 6.0 / 5.7 / 5.5 / 5.7,
+// 16384 codes 9.8 / 7.0 / 5.9 / 5.7, 32768 codes 15.3 / 10.9 / 7.7 / 6.2 (one image: 4.4 / 5.0, 5.3 / 5.4 / 5.2, 8.7 / 6.7 /
+// 5.6 / 5.2, 12.4 / 9.2 / 6.2 / 5.3).  At 4096 codes the line is half a microsecond early.
 int launch_decide(const float* rows, bool logits, int n_tiles, const Workspace& ws, const DecideParams& p, bool pdl,
                   cudaStream_t s) {
   int S = 1;

@@ -18,8 +18,8 @@
 // kernels still run (programmatic dependent launch) -- as long as there is room for this kernel's CTAs beside
 // theirs, which is why a CTA stays small; at some hundred tokens the fill of shared memory from L2.
 // Step of the XL shape (36 layers, five kernels each, against ten with separate norm, rotation, cache append, gate and
-// residual): 18 tokens 1012 -> 973 us (1535 in fixed-order contexts), 28 tokens 1721 -> 1016, 288 tokens 2605 -> 1980;
-// 7B shape, 18 tokens: 3406 -> 3183 us (4.6 TB/s over the whole step).
+// residual): 18 tokens 1012 -> 921 us (1535 in fixed-order contexts), 28 tokens 1720 -> 970, 288 tokens 2600 -> 1900;
+// 7B shape, 18 tokens: 3410 -> 3020 us (4.9 TB/s over the whole step).
 #include "tc_common.cuh"
 #include "vvs_internal.cuh"
 

@@ -367,8 +367,9 @@ int finish_verify_tc(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_ou
   return run_decisions<__nv_bfloat16>(ctx, hid, Tn, a->n_forced - 1, a->block + a->n_forced, Tn, a, o, true, s);
 }
 
-// The folded projections pay from d_model 1024 on; below that a step is a few kernels of a few CTAs either way, and the
-// per-projection path has them measured and tested.
+// Wide models take the folded projections: 24 layers of d_model 1024, 18 / 288 tokens, 579 / 1128 us a step against 743 / 1651
+// with the per-projection kernels (1023 / 2096 in rank order).  Where the line lies is history, not a crossing: at 768 columns
+// the folded step was measured at 527 / 919 us against 582 / 1471, at 512 at 538 / 723 against 700 / 1341.
 bool folded_applicable(const vvs_ctx* ctx) { return !ctx->use_chain_kernels && ctx->desc.d_model >= 1024; }
 
 // bf16 contexts of wide models: five kernels per layer (proj_tc.cu, attention_block.cu), each a programmatic dependent of
