@@ -2,9 +2,9 @@
 // rows, every feature row on the MMA's N side, guided logits written out and the tile's softmax partial (max, sum exp) of
 // every decision row taken from registers.
 //
-// What bounds it: the stream of codebook rows, if nothing else gets in its way.  One thread reaches an MMA k-block every
-// ~600 cycles (wait, four MMAs, commit), which is slower than the stream fills a stage, so two threads take every other
-// k-block, each with an accumulator of its own; the pipeline is as deep as shared memory allows and its weights are
+// What bounds it: the stream of codebook rows, if nothing else gets in its way.  Two warps issue, every other k-block each with
+// an accumulator of its own (one issuing lane in a branch of its own reached a k-block every ~600 cycles, which is slower than
+// the stream fills a stage; issued by converged warps 14.4 -> 14.0 us a call of one image and 16384 codes); the pipeline is as deep as shared memory allows and its weights are
 // requested before griddepcontrol.wait.  Up to one tile per SM a CTA takes the whole SM's shared memory; with more, two
 // CTAs share an SM so that one's epilogue runs under the other's stream.  With one issuer and a thread per decision row
 // summing 128 values from shared memory (2.1 us) a call of one image and 16384 codes took 21.8 us, decision included; 15.3
@@ -105,16 +105,16 @@ lmhead_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, cons
       pdl_wait();
       for (int i = 0; i < n_pre; ++i) load_b(i, i, 1);
     }
-  } else if ((warp == 1 || warp == 2) && lane == 0) {
+  } else if (warp == 1 || warp == 2) {
     // ---- MMA issuers: every other k-block each; the number of stages is even, or they are all used once, so that a
     // stage always belongs to the same one ---------------------------------------------------------------------
-    const int me = warp - 1;
+    const int me = __shfl_sync(0xffffffffu, warp, 0) - 1;
     const uint32_t idesc = idesc_bf16_f32(kTileRows, (uint32_t)nt), d = tmem + (uint32_t)(me * nt);
     const uint32_t lo0 = desc_lo_sw128(smem_u32(smem)), stage_lo = stage_bytes >> 4;
     uint32_t stage = (uint32_t)me, par = 0, add = 0;
     for (int i = me; i < p.kb_total; i += 2) {
-      if (!wait_or_abort(&full_bar[stage], par, &s_abort)) {
-        atomicOr(p.status, VVS_DEV_TIMEOUT);
+      if (!__all_sync(0xffffffffu, wait_or_abort(&full_bar[stage], par, &s_abort))) {
+        if (lane == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
         s_abort = 1;
         break;
       }
@@ -122,11 +122,11 @@ lmhead_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, cons
       const uint32_t a_lo = lo0 + stage * stage_lo;
       mma_bf16_k64(d, a_lo, a_lo + (kATileBytes >> 4), idesc, add);
       add = 1;
-      if (i + p.stages < p.kb_total) mma_commit(&empty_bar[stage]);
+      if (i + p.stages < p.kb_total) mma_commit_elect(&empty_bar[stage]);
       stage += 2;
       if (stage >= (uint32_t)p.stages) { stage -= p.stages; par ^= 1; }
     }
-    mma_commit(&acc_bar);
+    mma_commit_elect(&acc_bar);
   }
   __syncwarp();
   pdl_wait();

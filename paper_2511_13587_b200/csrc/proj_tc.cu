@@ -18,8 +18,9 @@
 // kernels still run (programmatic dependent launch) -- as long as there is room for this kernel's CTAs beside
 // theirs, which is why a CTA stays small; at some hundred tokens the fill of shared memory from L2.
 // Step of the XL shape (36 layers, five kernels each, against ten with separate norm, rotation, cache append, gate and
-// residual): 18 tokens 1012 -> 921 us (1535 in fixed-order contexts), 28 tokens 1720 -> 970, 288 tokens 2600 -> 1900;
-// 7B shape, 18 tokens: 3410 -> 3020 us (4.9 TB/s over the whole step).
+// residual): 18 tokens 1012 -> 921 us (1535 in fixed-order contexts), 28 tokens 1720 -> 970, 288 tokens 2600 -> 1930;
+// 7B shape, 18 tokens: 3410 -> 3025 us (4.9 TB/s over the whole step).  MMAs and loads issued by a converged warp in the place of a
+// lone lane: 876, 920, 1821 and 2967 us (54 tokens, a tree: 1107 -> 1061).
 #include "tc_common.cuh"
 #include "vvs_internal.cuh"
 
@@ -119,43 +120,45 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
       if (p.ahead[m])
         for (uint32_t at = cta * share + lane * 4096u; at < end; at += 32 * 4096u) prefetch_l2(p.ahead[m] + at, min(4096u, end - at));
   }
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---- TMA producer: all stages are free, so the weights go out before the wait -----------------
+    auto load_w = [&](int i, uint32_t stage) {
+      if (elect_one()) {
+        uint8_t* st = smem + (size_t)stage * stage_bytes;
+        mbar_expect_tx(&full_bar[stage], stage_bytes);
+        tma_load_2d(st, &tm_a, &full_bar[stage], (kb0 + i) * (int)kBlockK, tile * (int)kTileRows);
+        if (DUAL) tma_load_2d(st + kATileBytes, &tm_a2, &full_bar[stage], (kb0 + i) * (int)kBlockK, tile * (int)kTileRows);
+      }
+    };
     const int n_pre = nkb < p.stages ? nkb : p.stages;
-    for (int i = 0; i < n_pre; ++i) {
-      uint8_t* st = smem + (size_t)i * stage_bytes;
-      mbar_expect_tx(&full_bar[i], stage_bytes);
-      tma_load_2d(st, &tm_a, &full_bar[i], (kb0 + i) * (int)kBlockK, tile * (int)kTileRows);
-      if (DUAL) tma_load_2d(st + kATileBytes, &tm_a2, &full_bar[i], (kb0 + i) * (int)kBlockK, tile * (int)kTileRows);
-    }
+    for (int i = 0; i < n_pre; ++i) load_w(i, i);
+    auto load_act = [&](int i, uint32_t stage) {
+      if (elect_one()) tma_load_2d(smem + (size_t)stage * stage_bytes + a_bytes, &tm_b, &full_bar[stage], (kb0 + i) * (int)kBlockK, tok0);
+    };
     pdl_wait();  // activations come from the previous kernel
-    for (int i = 0; i < n_pre; ++i)
-      tma_load_2d(smem + (size_t)i * stage_bytes + a_bytes, &tm_b, &full_bar[i], (kb0 + i) * (int)kBlockK, tok0);
+    for (int i = 0; i < n_pre; ++i) load_act(i, i);
     uint32_t stage = 0, par = 0;                  // stage of block i, parity of its previous release
     for (int i = n_pre; i < nkb; ++i) {
-      if (!wait_or_abort(&empty_bar[stage], par, &s_abort)) {
-        atomicOr(p.status, VVS_DEV_TIMEOUT);
+      if (!__all_sync(0xffffffffu, wait_or_abort(&empty_bar[stage], par, &s_abort))) {
+        if (lane == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
         s_abort = 1;
         break;
       }
-      uint8_t* st = smem + (size_t)stage * stage_bytes;
-      mbar_expect_tx(&full_bar[stage], stage_bytes);
-      tma_load_2d(st, &tm_a, &full_bar[stage], (kb0 + i) * (int)kBlockK, tile * (int)kTileRows);
-      if (DUAL) tma_load_2d(st + kATileBytes, &tm_a2, &full_bar[stage], (kb0 + i) * (int)kBlockK, tile * (int)kTileRows);
-      tma_load_2d(st + a_bytes, &tm_b, &full_bar[stage], (kb0 + i) * (int)kBlockK, tok0);
+      load_w(i, stage);
+      load_act(i, stage);
       if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1; }
     }
-  } else if ((warp == 1 || warp == 2) && lane == 0) {
-    // ---- MMA issuers: one thread reaches an MMA per 64 cycles and pays ~270 for a wait and a commit, so two share the
-    // work, each with accumulators of its own: gate and up, or every other k-block of a single matrix (added below)
-    const int me = warp - 1;
+  } else if (warp == 1 || warp == 2) {
+    // ---- MMA issuers: one lane of the warp issues, all of it runs the loop (mma_bf16_k64).  Two warps share the work, each with
+    // accumulators of its own: gate and up, or every other k-block of a single matrix (added below)
+    const int me = __shfl_sync(0xffffffffu, warp, 0) - 1;
     const uint32_t idesc = idesc_bf16_f32(kTileRows, (uint32_t)p.nt), d = tmem_base + (uint32_t)(me * p.nt);
     const uint32_t lo0 = desc_lo_sw128(smem_u32(smem)), stage_lo = stage_bytes >> 4;
     uint32_t stage = DUAL ? 0 : me, par = 0, add = 0;
     if (stage >= (uint32_t)p.stages) { stage -= p.stages; par = 1; }
     for (int i = DUAL ? 0 : me; i < nkb; i += DUAL ? 1 : 2) {
-      if (!wait_or_abort(&full_bar[stage], par, &s_abort)) {
-        atomicOr(p.status, VVS_DEV_TIMEOUT);
+      if (!__all_sync(0xffffffffu, wait_or_abort(&full_bar[stage], par, &s_abort))) {
+        if (lane == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
         s_abort = 1;
         break;
       }
@@ -163,11 +166,11 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
       const uint32_t a_lo = lo0 + stage * stage_lo;
       mma_bf16_k64(d, a_lo + (DUAL ? me * (kATileBytes >> 4) : 0u), a_lo + (a_bytes >> 4), idesc, add);
       add = 1;
-      if (i + p.stages < nkb) mma_commit(&empty_bar[stage]);  // a block is still to come into this stage
+      if (i + p.stages < nkb) mma_commit_elect(&empty_bar[stage]);  // a block is still to come into this stage
       stage += DUAL ? 1 : 2;
       while (stage >= (uint32_t)p.stages) { stage -= p.stages; par ^= 1; }
     }
-    mma_commit(&acc_bar);
+    mma_commit_elect(&acc_bar);
   }
   __syncwarp();
   pdl_wait();
