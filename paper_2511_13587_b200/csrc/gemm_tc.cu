@@ -572,6 +572,21 @@ int make_tmap_bf16_2d(CUtensorMap* out, const void* base, uint64_t rows, uint64_
   return r == CUDA_SUCCESS ? VVS_OK : VVS_ERR_CUDA;
 }
 
+// [rows, cols] seen as cols / 64 blocks of 64 columns, cols a multiple of 64: a box is `box_rows` rows of `box_blocks` blocks, each
+// block a 128-byte swizzled tile of its own.
+int make_tmap_bf16_blocks(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_blocks) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return VVS_ERR_CUDA;
+  cuuint64_t dims[3] = {kBlockK, rows, cols / kBlockK};
+  cuuint64_t strides[2] = {cols * 2, kBlockK * 2};
+  cuuint32_t box[3] = {kBlockK, box_rows, box_blocks};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? VVS_OK : VVS_ERR_CUDA;
+}
+
 int make_weight_tmap(CUtensorMap* out, const void* w, int rows, int cols) {
   return make_tmap_bf16_2d(out, w, (uint64_t)rows, (uint64_t)cols, kTileRows);
 }

@@ -14,6 +14,9 @@ constexpr int kMaxTok = 128;              // tokens per pass
 constexpr uint32_t kTileRows = 128;       // weight rows per tile = MMA M
 constexpr uint32_t kBlockK = 64;          // bf16 elements per smem row = one 128-byte swizzle row
 constexpr uint32_t kATileBytes = kTileRows * kBlockK * 2;
+constexpr int kFewTok = 96;               // proj_few.cu: tokens of a call,
+constexpr int kFewStages = 12;            // stages of a ring,
+constexpr int kFewSmem = 226 * 1024;      // dynamic shared memory of a CTA
 }  // namespace proj
 
 struct ProjPlan {
@@ -140,6 +143,46 @@ inline ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
   // CTAs of a cluster wait for one another, so none may wait for tensor memory that a waiting one holds: each takes at
   // least as large a share of an SM's shared memory as of its tensor memory, whatever shares the SM with it
   const int share = (int)((228u * 1024u * (unsigned)cols + 511u) / 512u) - 1024;          // (1 KB per CTA is the system's)
+  if (pl.smem_bytes < share) pl.smem_bytes = share;
+  return pl;
+}
+
+// ---- the same for few tokens, proj_few.cu ----------------------------------------------------------
+struct ProjFewPlan {
+  int nt, tiles, kb_total, splits, group, stages, ring, recv_off, smem_bytes, tmem_cols;    // stages of `group` k-blocks
+};
+
+// partial sums of squares per token an ADD projection writes: one per tile and slice, rounded up to whole float4
+inline int proj_ss_parts(const ProjFewPlan& pl) { return (pl.tiles * pl.splits + 3) & ~3; }
+
+// One pass of at most kFewTok tokens, k a multiple of 64, for models whose weights are requested into L2 ahead.  K slices: proj_few.cu
+// has the measurements; fewer than eight k-blocks are not worth an exchange.
+inline ProjFewPlan plan_proj_few(int m, int n, int k, bool dual, bool add) {
+  using namespace proj;
+  ProjFewPlan pl{};
+  pl.nt = (m + 7) / 8 * 8;
+  pl.tiles = (n + (dual ? 31 : 63)) / (dual ? 32 : 64);
+  pl.kb_total = k / (int)kBlockK;
+  pl.splits = dual || pl.kb_total < 8 ? 1 : add ? 4 : 2;
+  const int kb_bytes = 64 * (int)kBlockK * 2 + pl.nt * (int)kBlockK * 2, per_cta = (pl.kb_total + pl.splits - 1) / pl.splits;
+  // the tile's rows on their way to the epilogue: unsplit they lie over the drained stages
+  const int recv = (m + 3) / 4 * 64 * 16, beside = pl.splits > 1 ? recv : 0, room = kFewSmem - 1024 - beside;
+  // All k-blocks at once where they fit, in stages of four, five or seven: as few blocks beyond the range as there can be, then as
+  // few stages.  A ring has stages of four.
+  auto fit = [&](int g) { return (per_cta + g - 1) / g * g * kb_bytes <= room; };
+  pl.group = 4;
+  for (int g = 5; g <= 7; g += 2)
+    if (fit(g) && (per_cta + g - 1) / g * g <= (per_cta + pl.group - 1) / pl.group * pl.group) pl.group = g;
+  const int stage_bytes = pl.group * kb_bytes, groups = (per_cta + pl.group - 1) / pl.group;
+  pl.stages = room / stage_bytes;
+  if (pl.stages > kFewStages) pl.stages = kFewStages;
+  if (pl.stages > groups) pl.stages = groups;
+  pl.ring = pl.stages < groups;
+  pl.recv_off = beside ? pl.stages * stage_bytes : 0;
+  pl.smem_bytes = pl.stages * stage_bytes + beside + 1024;
+  if (pl.smem_bytes < recv + 1024) pl.smem_bytes = recv + 1024;
+  pl.tmem_cols = pl.nt <= 32 ? 32 : pl.nt <= 64 ? 64 : 128;
+  const int share = (int)((228u * 1024u * (unsigned)pl.tmem_cols + 511u) / 512u) - 1024;   // as in plan_proj
   if (pl.smem_bytes < share) pl.smem_bytes = share;
   return pl;
 }

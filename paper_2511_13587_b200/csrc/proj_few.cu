@@ -1,0 +1,447 @@
+// Weight-streaming projections of calls with few tokens (bf16 contexts of wide models whose matrices stay in L2): the same
+// operations as proj_tc.cu on tiles of 64 weight rows.
+//
+// What bounds such a projection is the chain of one CTA: wait for the kernel before, activations from L2, MMAs, exchange, epilogue.
+// - An MMA of 64 rows reads half the shared memory of one of 128 and takes 24 cycles in the place of 40 (N = 24 or 32), so a CTA
+//   can hold more of the K range: gate/up all of it, QKV half, output and down projection a quarter (a cluster of S CTAs then
+//   exchanges partial sums, each pushing 64 rows in the place of 128: a CTA pushes some 32 bytes a cycle into its cluster).
+// - A stage is several k-blocks, loaded by one request and waited for once.
+// - All stages' weights are requested before tensor memory and the CTA's barrier, then whatever the epilogue needs besides
+//   the sums (rows, places in the cache, rotation) is found, all before griddepcontrol.wait.
+//   QKV, ADD  64 rows of one matrix;  GATEUP  32 rows of gate, then the same 32 of up
+// An accumulator of M = 64 lies in lanes 0-15 of the four lane quarters; its rows go to shared memory as [token quad][rank][row]
+// float4 (split: with st.async to the rank that owns the row, counted on its mbarrier), and the epilogue takes a pair of rows and
+// two tokens per thread (four where 64 rows are finished at once), partial sums in rank order.
+//
+// Step of the XL shape against 128-row tiles: 18 tokens 876 -> 709 us, 28 tokens 920 -> 766, 54 tokens (a tree) 1061 -> 881; 18
+// layers of it, 72 tokens 615 -> 538, 90 tokens 657 -> 585, 108 tokens 635 -> 641; of d_model 1024, 72 tokens 515 -> 473, 90
+// tokens 540 -> 544, 108 tokens 556 -> 569: calls of up to 96 tokens come here.  K slices at 18 tokens: QKV 1 736 us, 2 709, 4 722;
+// output projection 1 794, 2 733, 4 725; down projection 2 788, 4 733.
+#include "tc_common.cuh"
+#include "vvs_internal.cuh"
+
+namespace vvs {
+
+using namespace tc;
+using namespace proj;
+
+namespace {
+
+constexpr int kThreads = 256;
+constexpr uint32_t kRows = 64;
+constexpr uint32_t kABytes = kRows * kBlockK * 2;
+
+struct Params {
+  int m, n, nt, kb_total, stages;
+  uint32_t tmem_cols, recv_off;
+  int32_t* status;
+  const float* ss_in; int ss_parts; float inv_d, eps;                  // QKV, GATEUP: [token][ss_parts], a multiple of 4
+  float* x; __nv_bfloat16* xg; const __nv_bfloat16* scale; float* ss_out; int ss_out_parts; int d;   // ADD
+  __nv_bfloat16* q; __nv_bfloat16* kv_k; __nv_bfloat16* kv_v; const int32_t* slot_pos;               // QKV
+  const float* rope_cos; const float* rope_sin; int n_heads, hd, s_max, layer, kv_rows, t_len;
+  __nv_bfloat16* act; int ff;                                                                      // GATEUP
+  const uint8_t* ahead[2]; uint32_t ahead_bytes;      // weights of the projection after next, to be brought into L2
+};
+
+// LOG_S: log2 of the slices of K; G: k-blocks per stage; RING: stages are filled again.
+// The issuing warp is alone in its loop, where every wait, vote and branch shows: 80 MMAs of 64 x 24 x 16 take 27.8 cycles each with
+// ten k-blocks per wait, 31 with four, 47 with one, and 41 with four where a ring's bookkeeping and a test for a partial
+// stage are in the loop.
+template <int EPI, int LOG_S, int G, bool RING>
+__global__ void __launch_bounds__(kThreads)
+proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_a2,
+                const __grid_constant__ CUtensorMap tm_b) {
+  constexpr bool DUAL = EPI == PROJ_GATEUP;
+  constexpr int NACC = DUAL ? 2 : 1;
+  constexpr bool SPLIT = LOG_S > 0;
+  constexpr int S = 1 << LOG_S;
+  constexpr int TPI = DUAL || SPLIT ? 2 : 4;           // tokens per item of the epilogue
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t full_bar[kFewStages];
+  __shared__ __align__(8) uint64_t empty_bar[kFewStages];
+  __shared__ __align__(8) uint64_t acc_bar;
+  __shared__ __align__(8) uint64_t recv_bar;
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int s_abort;
+  __shared__ float s_rs[EPI == PROJ_ADD ? 1 : kFewTok];            // 1/rms of the tokens
+
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int tile = (int)blockIdx.x, rank = SPLIT ? (int)blockIdx.y : 0;
+  const int nq = (p.m + 3) >> 2;
+  const int kb0 = (rank * p.kb_total) >> LOG_S, nkb = (((rank + 1) * p.kb_total) >> LOG_S) - kb0, ng = (nkb + G - 1) / G;
+  const uint32_t b_bytes = (uint32_t)p.nt * kBlockK * 2u, stage_bytes = G * (kABytes + b_bytes);   // weights, then activations
+  uint8_t* recv = smem + p.recv_off;                               // [quad][source rank][row] float4
+
+  auto load_w = [&](int i, uint32_t stage) {         // k-blocks i * G ..; by a converged warp
+    uint8_t* st = smem + (size_t)stage * stage_bytes;
+    if (elect_one()) {
+      mbar_expect_tx(&full_bar[stage], stage_bytes);
+      if (DUAL) {                                    // (gate and up rows of a k-block have to lie together: boxes of one block)
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+          tma_load_3d(st + j * kABytes, &tm_a, &full_bar[stage], 0, tile * (int)(kRows / 2), kb0 + i * G + j);
+          tma_load_3d(st + j * kABytes + kABytes / 2, &tm_a2, &full_bar[stage], 0, tile * (int)(kRows / 2), kb0 + i * G + j);
+        }
+      } else {
+        tma_load_3d(st, &tm_a, &full_bar[stage], 0, tile * (int)kRows, kb0 + i * G);
+      }
+    }
+  };
+  const int n_pre = min(ng, p.stages);
+  if (warp == 0) {
+    if (lane == 0) {
+      tma_prefetch_desc(&tm_b);
+      for (int i = 0; i < p.stages; ++i) {
+        mbar_init(&full_bar[i], 1);
+        if (RING) mbar_init(&empty_bar[i], 1);
+      }
+      mbar_init(&acc_bar, 1);
+      mbar_init(&recv_bar, 1);
+      s_abort = 0;
+      fence_barrier_init();
+      fence_proxy_async();
+      if (SPLIT) mbar_expect_tx(&recv_bar, (uint32_t)nq * kRows * 16u);
+    }
+    __syncwarp();
+    // All stages are free, so the weights go out first of all: a CTA that could only start when the kernel before it drained has
+    // them sooner by what tensor memory and the barrier below take.
+    for (int i = 0; i < n_pre; ++i) load_w(i, i);
+  }
+  if (warp == 2) {
+    tmem_alloc(&tmem_slot, p.tmem_cols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_slot;
+  pdl_launch_dependents();  // after this CTA holds its TMEM: a dependent grid cannot take it first
+  if (SPLIT) cluster_arrive_relaxed();      // this rank's barrier is ready for its peers' pushes (fence_barrier_init above)
+
+  // ---- this thread's first item of the epilogue: a pair of rows and TPI tokens, the last warps first (the first ones have other
+  // work).  What does not depend on the kernel before is found here, under its tail; nothing waits for a load here.
+  constexpr int rpr = (int)kRows >> LOG_S, log_np = (DUAL ? 4 : 5) - LOG_S;     // rows of a rank, log2 of the pairs it finishes
+  const int eid = (kThreads / 32 - 1 - warp) * 32 + lane;
+  const int pair = (TPI == 2 ? eid >> 1 : eid) & ((1 << log_np) - 1), sub = TPI == 2 ? (eid & 1) * 2 : 0;
+  constexpr int log_sub = TPI == 2 ? 1 : 0;
+  const int items = nq << (log_np + log_sub);
+  const int row0 = DUAL ? tile * 32 : tile * (int)kRows + rank * rpr;       // first output row of this rank
+  const int n = row0 + 2 * pair;
+  const bool n_ok = n < p.n;
+  const int sec = EPI == PROJ_QKV ? (tile * (int)kRows) / p.d : 0;          // (a tile lies in one head: 64 divides both)
+  const int e = n - sec * p.d, h = EPI == PROJ_QKV ? e / p.hd : 0, i2 = e - h * p.hd;
+  const float inv_t = EPI == PROJ_QKV ? 1.f / (float)p.t_len : 0.f;
+  uint32_t scale2 = 0;                      // (converted where it is used: a conversion here would wait for it)
+  if (EPI == PROJ_ADD && n_ok) scale2 = __ldg(reinterpret_cast<const uint32_t*>(p.scale + n));
+  float cs[TPI], sn[TPI];
+  __nv_bfloat16* dst[TPI];                  // null: not to be stored
+  auto prepare = [&](int idx) {
+    const int t0 = (idx >> (log_np + log_sub)) * 4 + sub;
+#pragma unroll
+    for (int j = 0; j < TPI; ++j) {
+      const int tok = min(t0 + j, p.m - 1);
+      cs[j] = 1.f;
+      sn[j] = 0.f;
+      if (EPI == PROJ_GATEUP) dst[j] = p.act + (size_t)tok * p.ff + n;
+      if (EPI == PROJ_ADD) dst[j] = p.xg + (size_t)tok * p.d + n;
+      if (EPI == PROJ_QKV) {
+        if (sec < 2) {
+          cs[j] = __ldg(p.rope_cos + (size_t)tok * (p.hd / 2) + (i2 >> 1));
+          sn[j] = __ldg(p.rope_sin + (size_t)tok * (p.hd / 2) + (i2 >> 1));
+        }
+        if (sec == 0) {
+          dst[j] = p.q + (size_t)tok * p.d + e;
+        } else {
+          const int slot = __ldg(p.slot_pos + tok), r = (int)(((float)tok + 0.5f) * inv_t);   // tok / t_len (exact below 2^21)
+          const size_t row = (((size_t)p.layer * p.kv_rows + r) * p.n_heads + h) * p.s_max + slot;
+          dst[j] = slot < 0 ? nullptr : (sec == 1 ? p.kv_k : p.kv_v) + row * p.hd + i2;
+        }
+      }
+      if (idx >= items || !n_ok || t0 + j >= p.m) dst[j] = nullptr;
+    }
+  };
+  if (warp >= 2) prepare(eid);
+  if (warp == 2 && p.ahead_bytes > 0) {
+    // This CTA's share of a later projection's weights, HBM -> L2 (proj_tc.cu has the measurements)
+    const uint32_t n_cta = gridDim.x * gridDim.y, cta = blockIdx.y * gridDim.x + blockIdx.x;
+    const uint32_t share = ((p.ahead_bytes + n_cta - 1) / n_cta + 4095u) & ~4095u, end = min((cta + 1) * share, p.ahead_bytes);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (p.ahead[i])
+        for (uint32_t at = cta * share + lane * 4096u; at < end; at += 32 * 4096u) prefetch_l2(p.ahead[i] + at, min(4096u, end - at));
+  }
+  if (warp == 0) {
+    // ---- TMA producer: activations, then what the ring had no room for ---------------------------
+    auto load_act = [&](int i, uint32_t stage) {
+      if (elect_one()) tma_load_3d(smem + (size_t)stage * stage_bytes + G * kABytes, &tm_b, &full_bar[stage], 0, 0, kb0 + i * G);
+    };
+    pdl_wait();
+    for (int i = 0; i < n_pre; ++i) load_act(i, i);
+    if constexpr (RING) {
+      uint32_t stage = 0, par = 0;                  // stage of group i, parity of its previous release
+      for (int i = n_pre; i < ng; ++i) {
+        if (!__all_sync(0xffffffffu, wait_or_abort(&empty_bar[stage], par, &s_abort))) {
+          if (lane == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
+          s_abort = 1;
+          break;
+        }
+        load_w(i, stage);
+        load_act(i, stage);
+        if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1; }
+      }
+    }
+  } else if (warp == 1) {
+    // ---- MMA issuer -------------------------------------------------------------------------------
+    const uint32_t idesc = idesc_bf16_f32(kRows, (uint32_t)p.nt), lo0 = desc_lo_sw128(smem_u32(smem)), stage_lo = stage_bytes >> 4;
+    const uint32_t b_lo = b_bytes >> 4;
+    // (a wait that ran out is reported and the loop goes on over what is there: no lane leaves the warp)
+    auto wait_full = [&](uint32_t stage, uint32_t par) {
+      if (!wait_or_abort(&full_bar[stage], par, &s_abort)) {
+        atomicOr(p.status, VVS_DEV_TIMEOUT);
+        s_abort = 1;
+      }
+      tc_fence_after();
+    };
+    auto whole = [&](uint32_t a_lo, int i) {
+#pragma unroll
+      for (int j = 0; j < G; ++j)
+        mma_bf16_k64(tmem_base, a_lo + j * (kABytes >> 4), a_lo + G * (kABytes >> 4) + j * b_lo, idesc, j > 0 ? 1u : (uint32_t)i);
+    };
+    auto part = [&](uint32_t a_lo, int i) {
+#pragma unroll 1
+      for (int j = 0; j < nkb - i * G; ++j)
+        mma_bf16_k64(tmem_base, a_lo + j * (kABytes >> 4), a_lo + G * (kABytes >> 4) + j * b_lo, idesc, (uint32_t)(i + j));
+    };
+    pdl_wait();
+    if constexpr (RING) {
+      uint32_t stage = 0, par = 0;
+      for (int i = 0; i < ng; ++i) {
+        wait_full(stage, par);
+        const uint32_t a_lo = lo0 + stage * stage_lo;
+        if (nkb - i * G >= G) whole(a_lo, i);
+        else part(a_lo, i);
+        if (i + p.stages < ng) mma_commit_elect(&empty_bar[stage]);  // a group is still to come into this stage
+        if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1; }
+      }
+    } else {
+      const int n_whole = nkb / G;
+      for (int i = 0; i < n_whole; ++i) {
+        wait_full(i, 0);
+        whole(lo0 + i * stage_lo, i);
+      }
+      if (n_whole < ng) {
+        wait_full(n_whole, 0);
+        part(lo0 + n_whole * stage_lo, n_whole);
+      }
+    }
+    mma_commit_elect(&acc_bar);
+  }
+  __syncwarp();
+  if (warp >= 2) pdl_wait();
+  else if (eid < items) prepare(eid);
+  float2 xo[TPI];
+  auto load_x = [&](int idx) {
+    const int t0 = (idx >> (log_np + log_sub)) * 4 + sub;
+#pragma unroll
+    for (int j = 0; j < TPI; ++j)
+      xo[j] = *reinterpret_cast<const float2*>(p.x + (size_t)min(t0 + j, p.m - 1) * p.d + (n_ok ? n : 0));
+  };
+  if (EPI == PROJ_ADD && eid < items) load_x(eid);
+  // ---- 1/rms of the tokens, while the MMAs run: eight tokens' loads in flight per warp ------------------------------
+  if (EPI != PROJ_ADD && warp >= 3) {
+    const int n4 = p.ss_parts >> 2;
+    for (int t0 = (warp - 3) * 8; t0 < p.m; t0 += 8 * (kThreads / 32 - 3)) {
+      float ss[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      for (int i = lane; i < n4; i += 32) {
+        float4 v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          v[j] = __ldcg(reinterpret_cast<const float4*>(p.ss_in + (size_t)min(t0 + j, p.m - 1) * p.ss_parts) + i);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) ss[j] += (v[j].x + v[j].y) + (v[j].z + v[j].w);
+      }
+      warp_sums(ss, lane);
+      const int j = warp_sums_index<8>(lane);
+      if ((lane & 3) == 0 && t0 + j < kFewTok) s_rs[t0 + j] = rsqrtf(ss[0] * p.inv_d + p.eps);
+    }
+  }
+  if (SPLIT && EPI != PROJ_ADD) __syncthreads();    // s_rs
+  // A CTA that gave up pushes whatever its accumulator holds: its peers' waits must still end.
+  if (!wait_or_abort(&acc_bar, 0, &s_abort)) {
+    if (lane == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
+    s_abort = 1;
+  }
+  tc_fence_after();
+  if (SPLIT) cluster_wait();
+  // ---- rows to where the epilogue reads them ---------------------------------------------------------------------------
+  {
+    const int row_t = (warp & 3) * 16 + (lane & 15), owner = row_t >> (6 - LOG_S);
+    const uint32_t at = smem_u32(recv) + (uint32_t)(SPLIT ? rank * rpr + (row_t & (rpr - 1)) : row_t) * 16u;
+    const uint32_t recv_dst = SPLIT ? mapa(at, (uint32_t)owner) : at, bar_dst = SPLIT ? mapa(smem_u32(&recv_bar), (uint32_t)owner) : 0u;
+    const uint32_t t_row = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+    for (int c0 = (warp >> 2) * 2; c0 < nq; c0 += 4) {
+      float v[8];
+      tmem_ld8(t_row + (uint32_t)(c0 * 4), v);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        if (lane < 16 && c0 + j < nq) {
+          const uint32_t dst = recv_dst + (uint32_t)(c0 + j) * (kRows * 16u);
+          if (SPLIT) st_async4(dst, bar_dst, &v[4 * j]);
+          else st_shared4(dst, &v[4 * j]);
+        }
+      }
+    }
+  }
+  if (SPLIT) {
+    // peers push after waits of at most kSpinLimit polls each, so this longer wait ends after their pushes
+    bool got = false;
+    for (uint32_t i = 0; i < 16u * kSpinLimit && !got; ++i) got = mbar_try_wait_cluster(&recv_bar, 0);
+    if (!got && lane == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
+  } else {
+    tc_fence_before();
+    __syncthreads();                          // the tile, s_rs
+    if (warp == 2) tmem_dealloc(tmem_base, p.tmem_cols);
+  }
+
+  // ---- epilogue on finished sums ---------------------------------------------------------------------------------------
+  const uint32_t src_row = (uint32_t)(2 * pair) * 16u + (uint32_t)sub * 4u;
+  const int items_up = (items + 31) & ~31;                         // whole warps: the shuffles below need their lanes
+  for (int idx = eid; idx < items_up; idx += kThreads) {
+    const int quad = idx >> (log_np + log_sub), t0 = quad * 4 + sub;
+    float acc[NACC][2][TPI];                                       // [row][token]
+    const uint8_t* src = recv + (size_t)(idx < items ? quad : 0) * (kRows * 16u) + src_row;
+#pragma unroll
+    for (int a = 0; a < NACC; ++a)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const uint8_t* at = src + a * (kRows / 2 * 16u) + i * 16;
+        ld_shared_vec(at, acc[a][i]);
+#pragma unroll
+        for (int r = 1; r < S; ++r) {         // rank order
+          float v[TPI];
+          ld_shared_vec(at + r * rpr * 16, v);
+#pragma unroll
+          for (int j = 0; j < TPI; ++j) acc[a][i][j] += v[j];
+        }
+      }
+    if constexpr (EPI == PROJ_ADD) {
+      float sq[TPI];
+      const float2 gsc = make_float2(__uint_as_float(scale2 << 16), __uint_as_float(scale2 & 0xffff0000u));
+#pragma unroll
+      for (int j = 0; j < TPI; ++j) {
+        const float x0 = xo[j].x + acc[0][0][j], x1 = xo[j].y + acc[0][1][j];
+        sq[j] = dst[j] ? x0 * x0 + x1 * x1 : 0.f;
+        if (dst[j]) {
+          *reinterpret_cast<float2*>(p.x + (size_t)(t0 + j) * p.d + n) = make_float2(x0, x1);
+          *reinterpret_cast<uint32_t*>(dst[j]) = pack_bf16(x0 * gsc.x, x1 * gsc.y);
+        }
+      }
+      // sums of squares over the rank's rows; the row of parts is a multiple of four long, the last CTA fills it up
+      const int part = tile * S + rank, pad = p.ss_out_parts - (int)gridDim.x * S;
+      float* ss = p.ss_out + part;
+      if constexpr (TPI == 4) {
+        warp_sums(sq, lane);
+        const int j = warp_sums_index<4>(lane);
+        if ((lane & 7) == 0 && t0 + j < p.m) ss[(size_t)(t0 + j) * p.ss_out_parts] = sq[0];
+      } else {
+        for (int o = 1 << log_np; o > 1; o >>= 1)
+#pragma unroll
+          for (int j = 0; j < TPI; ++j) sq[j] += __shfl_xor_sync(0xffffffffu, sq[j], o);
+        if (idx < items && pair == 0)
+#pragma unroll
+          for (int j = 0; j < TPI; ++j)
+            if (t0 + j < p.m) ss[(size_t)(t0 + j) * p.ss_out_parts] = sq[j];
+      }
+      if (part + 1 == (int)gridDim.x * S && pad > 0 && pair == 0 && idx < items)
+        for (int j = 0; j < TPI; ++j)
+          for (int i = 1; i <= pad; ++i)
+            if (t0 + j < p.m) ss[(size_t)(t0 + j) * p.ss_out_parts + i] = 0.f;
+    } else {
+#pragma unroll
+      for (int j = 0; j < TPI; ++j) {
+        const float rs = s_rs[min(t0 + j, kFewTok - 1)];
+        float a = acc[0][0][j] * rs, b = acc[0][1][j] * rs;
+        if constexpr (DUAL) {
+          a = __fdividef(a, 1.f + expf(-a)) * (acc[1][0][j] * rs);
+          b = __fdividef(b, 1.f + expf(-b)) * (acc[1][1][j] * rs);
+        } else {
+          const float a0 = a;
+          a = a0 * cs[j] - b * sn[j];         // (1, 0 for values)
+          b = a0 * sn[j] + b * cs[j];
+        }
+        if (dst[j]) *reinterpret_cast<uint32_t*>(dst[j]) = pack_bf16(a, b);
+      }
+    }
+    if (idx + kThreads < items_up) {
+      prepare(idx + kThreads);
+      if (EPI == PROJ_ADD) load_x(idx + kThreads);
+    }
+  }
+  if (SPLIT) {
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 2) tmem_dealloc(tmem_base, p.tmem_cols);
+  }
+}
+
+template <int EPI, int LOG_S, int G, bool RING>
+cudaError_t launch_one(const ProjFewPlan& pl, const Params& kp, const ProjArgs& g, cudaStream_t s) {
+  auto* fn = proj_few_kernel<EPI, LOG_S, G, RING>;
+  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(fn), kFewSmem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(pl.tiles, pl.splits, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = pl.smem_bytes;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  int na = 0;
+  if (g.pdl) {
+    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[na++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (LOG_S > 0) {                           // the K slices of a tile: one cluster along grid y
+    attr[na].id = cudaLaunchAttributeClusterDimension;
+    attr[na].val.clusterDim.x = 1;
+    attr[na].val.clusterDim.y = (unsigned)pl.splits;
+    attr[na++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = na;
+  return cudaLaunchKernelEx(&cfg, fn, kp, *g.tm_a, g.tm_a2 ? *g.tm_a2 : *g.tm_a, *g.tm_b);
+}
+
+template <int EPI, int LOG_S>
+cudaError_t launch_epi(const ProjFewPlan& pl, const Params& kp, const ProjArgs& g, cudaStream_t s) {
+  if (pl.splits != 1 << LOG_S) return cudaErrorInvalidValue;
+  if (pl.ring) return launch_one<EPI, LOG_S, 4, true>(pl, kp, g, s);          // (a ring has stages of four)
+  if (pl.group == 4) return launch_one<EPI, LOG_S, 4, false>(pl, kp, g, s);
+  if (pl.group == 5) return launch_one<EPI, LOG_S, 5, false>(pl, kp, g, s);
+  return launch_one<EPI, LOG_S, 7, false>(pl, kp, g, s);
+}
+
+}  // namespace
+
+int launch_proj_few(int epi, const ProjFewPlan& pl, const ProjArgs& g, cudaStream_t s) {
+  Params kp{};
+  kp.m = g.m; kp.n = g.n; kp.nt = pl.nt; kp.kb_total = pl.kb_total; kp.stages = pl.stages;
+  kp.tmem_cols = (uint32_t)pl.tmem_cols; kp.recv_off = (uint32_t)pl.recv_off; kp.status = g.status;
+  kp.ss_in = g.ss_in; kp.ss_parts = g.ss_parts; kp.inv_d = 1.f / (float)g.d; kp.eps = g.eps;
+  kp.x = g.x; kp.xg = g.xg; kp.scale = g.scale; kp.ss_out = g.ss_out; kp.ss_out_parts = proj_ss_parts(pl); kp.d = g.d;
+  kp.q = g.q; kp.kv_k = g.kv_k; kp.kv_v = g.kv_v; kp.slot_pos = g.slot_pos; kp.rope_cos = g.rope_cos;
+  kp.rope_sin = g.rope_sin; kp.n_heads = g.n_heads; kp.hd = g.hd; kp.s_max = g.s_max; kp.layer = g.layer;
+  kp.kv_rows = g.kv_rows; kp.t_len = g.t_len; kp.act = g.act; kp.ff = g.ff;
+  kp.ahead[0] = static_cast<const uint8_t*>(g.ahead[0]); kp.ahead[1] = static_cast<const uint8_t*>(g.ahead[1]);
+  kp.ahead_bytes = g.ahead[0] ? g.ahead_bytes : 0;
+  cudaError_t e;
+  switch (epi) {
+    case PROJ_QKV: e = pl.splits == 2 ? launch_epi<PROJ_QKV, 1>(pl, kp, g, s) : launch_epi<PROJ_QKV, 0>(pl, kp, g, s); break;
+    case PROJ_ADD: e = pl.splits == 4 ? launch_epi<PROJ_ADD, 2>(pl, kp, g, s) : launch_epi<PROJ_ADD, 0>(pl, kp, g, s); break;
+    case PROJ_GATEUP: e = launch_epi<PROJ_GATEUP, 0>(pl, kp, g, s); break;
+    default: return VVS_ERR_INVALID_ARG;
+  }
+  return e == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
+}
+
+}  // namespace vvs

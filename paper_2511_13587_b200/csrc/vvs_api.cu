@@ -55,7 +55,7 @@ size_t layout(const vvs_model_desc& d, Workspace& ws, char* base, bool few_logit
       const size_t wide = 3 * dm > 2 * ff ? 3 * dm : 2 * ff;
       const size_t tiles = (wide + 127) / 128, passes = (M + 255) / 256;
       c.take(ws.slot_pos, M * 4);
-      c.take(ws.ss_part, (dm + 127) / 128 * 8 * M * 4);
+      c.take(ws.ss_part, (dm + 127) / 128 * 16 * M * 4);     // (proj_few.cu: eight slices of 64 rows)
       c.take(ws.seq_order, (size_t)d.max_rows * 4);
       c.take(ws.rope_cos, M * (size_t)(d.head_dim / 2) * 4);
       c.take(ws.rope_sin, M * (size_t)(d.head_dim / 2) * 4);
@@ -372,6 +372,27 @@ int finish_verify_tc(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_ou
 // the folded step was measured at 527 / 919 us against 582 / 1471, at 512 at 538 / 723 against 700 / 1341.
 bool folded_applicable(const vvs_ctx* ctx) { return !ctx->use_chain_kernels && ctx->desc.d_model >= 1024; }
 
+// FewMaps of a stage of `group` k-blocks
+inline int few_map(int group) { return group == 4 ? 0 : group == 5 ? 1 : 2; }
+
+// The kernel and plan of one projection.
+struct ProjPick {
+  bool few;
+  ProjPlan wide{};
+  ProjFewPlan small{};
+  ProjPick(int epi, int m, int n, int k, bool in_l2, int n_sms) : few(in_l2 && m <= proj::kFewTok) {      // (in_l2: see run_verify_folded)
+    const bool dual = epi == PROJ_GATEUP;
+    if (few) small = plan_proj_few(m, n, k, dual, epi == PROJ_ADD);
+    else wide = plan_proj(m, n, k, dual, n_sms);
+  }
+  int make_tmap(CUtensorMap* tm, const void* act, int m, int k) const {
+    return few ? make_tmap_bf16_blocks(tm, act, (uint64_t)m, (uint64_t)k, (uint32_t)small.nt, (uint32_t)small.group)
+               : make_tmap_bf16_2d(tm, act, (uint64_t)m, (uint64_t)k, (uint32_t)wide.nt);
+  }
+  int ss_parts() const { return few ? proj_ss_parts(small) : proj_ss_parts(wide); }
+  int launch(int epi, const ProjArgs& g, cudaStream_t s) const { return few ? launch_proj_few(epi, small, g, s) : launch_proj(epi, wide, g, s); }
+};
+
 // bf16 contexts of wide models: five kernels per layer (proj_tc.cu, attention_block.cu), each a programmatic dependent of
 // the one before.  Every sum is taken in a fixed order, so a call repeats bit for bit.
 int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* o, cudaStream_t s) {
@@ -383,13 +404,17 @@ int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_o
   T* xn = static_cast<T*>(ws.xn);
   T* attn = static_cast<T*>(ws.attn);
   T* act = static_cast<T*>(ws.act);
-  const ProjPlan p_qkv = plan_proj(M, 3 * d, d, false, ctx->n_sms), p_o = plan_proj(M, d, d, false, ctx->n_sms);
-  const ProjPlan p_gu = plan_proj(M, ff, d, true, ctx->n_sms), p_down = plan_proj(M, d, ff, false, ctx->n_sms);
+  // Weights of the projection after next are requested into L2 when three layers fit there (XL shape, 39 MB per layer:
+  // 989 -> 977 us at 18 tokens, 1263 -> 1235 at 54); larger ones push each other out (101 MB: 1005 -> 1110 us; 405 MB:
+  // 3.11 -> 4.26 ms)
+  const size_t layer_bytes = ((size_t)4 * d + (size_t)3 * ff) * d * sizeof(T);
+  const bool prefetch = 3 * layer_bytes <= (size_t)ctx->l2_bytes;
+  const bool few = prefetch && ff % 64 == 0;        // (proj_few.cu takes whole k-blocks)
+  const ProjPick p_qkv(PROJ_QKV, M, 3 * d, d, few, ctx->n_sms), p_o(PROJ_ADD, M, d, d, few, ctx->n_sms);
+  const ProjPick p_gu(PROJ_GATEUP, M, ff, d, few, ctx->n_sms), p_down(PROJ_ADD, M, d, ff, few, ctx->n_sms);
   CUtensorMap tm_xq, tm_xg, tm_attn, tm_act;
-  if (make_tmap_bf16_2d(&tm_xq, xn, (uint64_t)M, (uint64_t)d, (uint32_t)p_qkv.nt) != VVS_OK ||
-      make_tmap_bf16_2d(&tm_xg, xn, (uint64_t)M, (uint64_t)d, (uint32_t)p_gu.nt) != VVS_OK ||
-      make_tmap_bf16_2d(&tm_attn, attn, (uint64_t)M, (uint64_t)d, (uint32_t)p_o.nt) != VVS_OK ||
-      make_tmap_bf16_2d(&tm_act, act, (uint64_t)M, (uint64_t)ff, (uint32_t)p_down.nt) != VVS_OK)
+  if (p_qkv.make_tmap(&tm_xq, xn, M, d) != VVS_OK || p_gu.make_tmap(&tm_xg, xn, M, d) != VVS_OK ||
+      p_o.make_tmap(&tm_attn, attn, M, d) != VVS_OK || p_down.make_tmap(&tm_act, act, M, ff) != VVS_OK)
     return VVS_ERR_CUDA;
   ProjArgs g{};
   g.m = M; g.status = ws.status; g.ss_in = g.ss_out = ws.ss_part; g.eps = md.rms_eps; g.x = ws.x; g.xg = xn;
@@ -405,13 +430,9 @@ int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_o
                                                static_cast<const T*>(ctx->tok_emb), static_cast<const T*>(ctx->layers[0].norm1),
                                                ws, md, R, Tn, s));
   int rc = VVS_OK;
-  // Weights of the projection after next are requested into L2 when three layers fit there (XL shape, 39 MB per layer:
-  // 989 -> 977 us at 18 tokens, 1263 -> 1235 at 54); larger ones push each other out (101 MB: 1005 -> 1110 us; 405 MB:
-  // 3.11 -> 4.26 ms)
-  const size_t layer_bytes = ((size_t)4 * d + (size_t)3 * ff) * d * sizeof(T);
-  const bool prefetch = 3 * layer_bytes <= (size_t)ctx->l2_bytes;
   for (int l = 0; l < md.n_layers && rc == VVS_OK; ++l) {
     const LayerMaps& W = ctx->layer_maps[l];
+    const FewMaps& F = ctx->few_maps[l];
     const Layer& L = ctx->layers[l];
     const Layer* next = l + 1 < md.n_layers ? &ctx->layers[l + 1] : nullptr;
     auto ahead = [&](const void* w0, const void* w1, size_t rows, size_t cols) {
@@ -419,22 +440,22 @@ int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_o
     };
     // (the first projection is an ordinary successor of the kernel that wrote the step's tables: the kernels behind it
     // read those before their own waits)
-    g.n = 3 * d; g.tm_a = &W.w_qkv; g.tm_b = &tm_xq; g.layer = at.layer = l; g.ss_parts = l > 0 ? proj_ss_parts(p_down) : 4;
+    g.n = 3 * d; g.tm_a = p_qkv.few ? &F.w_qkv[few_map(p_qkv.small.group)] : &W.w_qkv; g.tm_b = &tm_xq; g.layer = at.layer = l; g.ss_parts = l > 0 ? p_down.ss_parts() : 4;
     g.pdl = ctx->use_pdl && l > 0;
     ahead(L.w_gate, L.w_up, ff, d);
-    VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_proj(PROJ_QKV, p_qkv, g, s));
+    VVS_LAUNCH(VVS_PROF_GEMM, rc = p_qkv.launch(PROJ_QKV, g, s));
     g.pdl = ctx->use_pdl;
     if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_ATTENTION, rc = launch_attention_block(at, s));
-    g.n = d; g.tm_a = &W.w_o; g.tm_b = &tm_attn; g.scale = static_cast<const T*>(ctx->layers[l].norm2);
+    g.n = d; g.tm_a = p_o.few ? &F.w_o[few_map(p_o.small.group)] : &W.w_o; g.tm_b = &tm_attn; g.scale = static_cast<const T*>(ctx->layers[l].norm2);
     ahead(L.w_down, nullptr, d, ff);
-    if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_proj(PROJ_ADD, p_o, g, s));
-    g.n = ff; g.tm_a = &W.w_gate; g.tm_a2 = &W.w_up; g.tm_b = &tm_xg; g.ss_parts = proj_ss_parts(p_o);
+    if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = p_o.launch(PROJ_ADD, g, s));
+    g.n = ff; g.tm_a = p_gu.few ? &F.w_gate : &W.w_gate; g.tm_a2 = p_gu.few ? &F.w_up : &W.w_up; g.tm_b = &tm_xg; g.ss_parts = p_o.ss_parts();
     ahead(next ? next->w_qkv : nullptr, nullptr, 3 * d, d);
-    if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_proj(PROJ_GATEUP, p_gu, g, s));
-    g.n = d; g.tm_a = &W.w_down; g.tm_a2 = nullptr; g.tm_b = &tm_act;
+    if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = p_gu.launch(PROJ_GATEUP, g, s));
+    g.n = d; g.tm_a = p_down.few ? &F.w_down[few_map(p_down.small.group)] : &W.w_down; g.tm_a2 = nullptr; g.tm_b = &tm_act;
     g.scale = static_cast<const T*>(l + 1 < md.n_layers ? ctx->layers[l + 1].norm1 : ctx->norm_f);
     ahead(next ? next->w_o : nullptr, nullptr, d, d);
-    if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_proj(PROJ_ADD, p_down, g, s));
+    if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = p_down.launch(PROJ_ADD, g, s));
   }
   if (rc != VVS_OK) return rc;
   return finish_verify_tc(ctx, a, o, o->hidden ? static_cast<T*>(o->hidden) : static_cast<T*>(ws.hid), s);
@@ -796,7 +817,8 @@ int vvs_create(const vvs_model_desc* desc, vvs_ctx** out) {
   if (desc->n_layers > 0) {
     ctx->layers = new (std::nothrow) Layer[desc->n_layers]();
     ctx->layer_maps = new (std::nothrow) LayerMaps[desc->n_layers]();
-    if (!ctx->layers || !ctx->layer_maps) { vvs_destroy(ctx); return VVS_ERR_NOMEM; }
+    ctx->few_maps = new (std::nothrow) FewMaps[desc->n_layers]();
+    if (!ctx->layers || !ctx->layer_maps || !ctx->few_maps) { vvs_destroy(ctx); return VVS_ERR_NOMEM; }
   }
   // Debug switches only: VVS_DEBUG_GENERIC runs bf16 contexts on the generic kernels,
   // VVS_DEBUG_NO_PDL launches the tensor-core GEMMs without programmatic dependent launch,
@@ -838,6 +860,7 @@ int vvs_destroy(vvs_ctx* ctx) {
   if (ctx->cs_d_plan) cudaFree(ctx->cs_d_plan);
   delete[] ctx->layers;
   delete[] ctx->layer_maps;
+  delete[] ctx->few_maps;
   delete ctx;
   return VVS_OK;
 }
@@ -875,6 +898,16 @@ int vvs_bind_weights(vvs_ctx* ctx, const vvs_weights* w) {
       if (rc == VVS_OK) rc = make_weight_tmap(&m.w_gate, s.w_gate, ff, d);
       if (rc == VVS_OK) rc = make_weight_tmap(&m.w_up, s.w_up, ff, d);
       if (rc == VVS_OK) rc = make_weight_tmap(&m.w_down, s.w_down, d, ff);
+      if (folded_applicable(ctx) && ff % 64 == 0) {
+        FewMaps& q = ctx->few_maps[l];
+        if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_gate, s.w_gate, ff, d, 32, 1);
+        if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_up, s.w_up, ff, d, 32, 1);
+        for (int g : {4, 5, 7}) {
+          if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_qkv[few_map(g)], s.w_qkv, 3 * (uint64_t)d, d, 64, g);
+          if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_o[few_map(g)], s.w_o, d, d, 64, g);
+          if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_down[few_map(g)], s.w_down, d, ff, 64, g);
+        }
+      }
     }
     if (rc == VVS_OK)
       rc = make_weight_tmap(&ctx->lm_map,

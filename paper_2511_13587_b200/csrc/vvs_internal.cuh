@@ -127,6 +127,10 @@ struct Layer {
 struct LayerMaps {
   CUtensorMap w_qkv, w_o, w_gate, w_up, w_down;
 };
+// the same matrices in the boxes of proj_few.cu: 64 rows (32 of gate and up) of one to several k-blocks
+struct FewMaps {
+  CUtensorMap w_gate, w_up, w_qkv[3], w_o[3], w_down[3];   // [stages of four, five, seven k-blocks]
+};
 
 }  // namespace vvs
 
@@ -174,6 +178,7 @@ struct vvs_ctx {
   bool use_pdl = true;               // programmatic dependent launch of the tensor-core GEMMs
   bool use_chain_kernels = false;  // debug: the persistent whole-chain kernels for calls of at most 32 tokens
   vvs::LayerMaps* layer_maps = nullptr;  // host array [n_layers]
+  vvs::FewMaps* few_maps = nullptr;      // host array [n_layers]
   std::vector<const __nv_bfloat16*> chain_norms;  // host [n_layers][2] norm-scale pointers
   vvs::ChainStreamPlan cs_plan;        // streaming chain kernel: split of the weights over the CTAs
   void* cs_packed = nullptr;           // device: private re-packed copy of the layer weights
@@ -259,6 +264,7 @@ struct GemmTcArgs {
   int d, n_heads, hd, s_max, layer, kv_rows, t_len;
   __nv_bfloat16* act; int ff;  // SWIGLU
 };
+int make_tmap_bf16_blocks(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_blocks);
 int make_tmap_bf16_2d(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 int make_weight_tmap(CUtensorMap* out, const void* w, int rows, int cols);
 GemmTcPlan plan_gemm_tc(int m, int n, int k, bool dual, bool allow_split, int n_sms, int split_cap = 32);
@@ -295,6 +301,7 @@ struct ProjArgs {
   const void* ahead[2]; uint32_t ahead_bytes;   // matrices of the projection after next (same size; null: none)
 };
 int launch_proj(int epi, const ProjPlan& plan, const ProjArgs& g, cudaStream_t s);
+int launch_proj_few(int epi, const ProjFewPlan& plan, const ProjArgs& g, cudaStream_t s);   // tensor maps: make_tmap_bf16_blocks, boxes of plan.group blocks; of b plan.nt rows
 
 // ---- block-vs-cache attention on rotated queries and appended keys, attention_block.cu ------------------
 struct AttentionBlockArgs {

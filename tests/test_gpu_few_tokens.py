@@ -1,0 +1,50 @@
+"""The folded step of few tokens (proj_few.cu) on two layers: token counts at the edges of MMA widths, quads and the range itself
+(97 tokens take proj_tc.cu), rings and stages that hold everything, K ranges that the slices and stages do not divide."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+
+import helpers as H
+from test_gpu_tree import _check_tree
+from test_gpu_verify import _check_end_to_end
+from vvs_synth.configs import B7, XL
+
+pytestmark = pytest.mark.gpu
+
+# 43 k-blocks of the down projection in four slices of 10 and 11; 86 tiles of gate and up
+FEW64 = replace(XL, name="few64", n_layers=2, d_model=1024, n_heads=16, d_ff=2752, vocab=1096, lm_rows=0, tok_rows=0, s_max=208)
+# heads of two tiles; 18 tiles: sums of squares in rows of 18 and 72 parts; a down projection of 5 k-blocks, unsplit
+FEW128 = replace(B7, name="few128", n_layers=2, d_model=1152, n_heads=9, d_ff=320, vocab=1096, vocab_offset=64, lm_rows=2048,
+                 tok_rows=0, s_max=700)
+
+
+@pytest.mark.parametrize("ms,n_images,n_cfg,n_forced,k,fills", [
+    (FEW64, 1, 1, 1, 0, [0]),                              # 1 token, no draft
+    (FEW64, 1, 2, 1, 3, [199]),                            # 8
+    (FEW64, 1, 1, 2, 7, [16]),                             # 9
+    (FEW64, 3, 1, 1, 10, [0, 47, 150]),                    # 33
+    (FEW64, 2, 2, 6, 10, [3, 190]),                        # 64
+    (FEW64, 5, 1, 3, 10, [3, 20, 37, 90, 190]),            # 65
+    (FEW64, 3, 2, 1, 15, [0, 47, 150]),                    # 96
+    (FEW64, 97, 1, 1, 0, list(range(97))),                 # 97
+    (FEW128, 1, 2, 1, 8, [513]),                           # 18
+    (FEW128, 3, 2, 1, 4, [5, 160, 677]),                   # 30
+    (FEW128, 4, 1, 3, 20, [5, 160, 333, 64])])             # 92
+def test_few_tokens(ms, n_images, n_cfg, n_forced, k, fills):
+    case = H.build_case_independent(ms, 1900 + k, n_images, n_cfg, n_forced, k, fills, logit_std=0.6)
+    run = H.GpuRunner(ms, case["w"], n_images * n_cfg, n_forced + k)
+    gpu = run.verify(case)
+    _check_end_to_end(case, gpu, H.run_oracle(case))
+    again = run.verify(case)
+    for key in ("accept_len", "next_token", "target_probs", "hidden", "kv_k", "kv_v"):
+        np.testing.assert_array_equal(gpu[key], again[key], err_msg=key)
+    run.close()
+
+
+def test_few_tokens_tree():
+    parent = [-1, 0, 0, 1, 1, 2, 3, 3, 6, 6, 4, 5, 9, 2, 7, 8, 8, 10, 11, 15, 1, 20]
+    case = H.build_tree_case(FEW64, 1950, 2, 2, 1, parent, [77, 0], q_noise=0.7)
+    run = H.GpuRunner(FEW64, case["w"], 4, len(parent))
+    _check_tree(case, H.run_tree_gpu(run, case), H.run_tree_oracle(case))
+    run.close()

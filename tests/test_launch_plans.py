@@ -11,6 +11,7 @@ CSRC = os.path.join(ROOT, "paper_2511_13587_b200", "csrc")
 N_SMS = 148
 FIELDS = ("nt", "passes", "tiles", "kb_total", "splits", "stages", "alias", "recv_off", "smem_bytes", "tmem_cols", "threads",
           "tiles_on_z")
+FEW_FIELDS = ("nt", "tiles", "kb_total", "splits", "group", "stages", "ring", "recv_off", "smem_bytes", "tmem_cols")
 SHIM = """
 #include "launch_plans.h"
 extern "C" void proj(int m, int n, int k, int dual, int n_sms, int* o) {
@@ -18,9 +19,14 @@ extern "C" void proj(int m, int n, int k, int dual, int n_sms, int* o) {
   const int v[] = {%s, vvs::proj_ss_parts(p)};
   for (unsigned i = 0; i < sizeof(v) / sizeof(v[0]); ++i) o[i] = v[i];
 }
+extern "C" void few(int m, int n, int k, int dual, int add, int* o) {
+  const vvs::ProjFewPlan p = vvs::plan_proj_few(m, n, k, dual != 0, add != 0);
+  const int v[] = {%s, vvs::proj_ss_parts(p)};
+  for (unsigned i = 0; i < sizeof(v) / sizeof(v[0]); ++i) o[i] = v[i];
+}
 extern "C" int tree_parts(int vocab, int n_images, int n_sms) { return vvs::tree_walk_parts(vocab, n_images, n_sms); }
 extern "C" int att_split(int hd, int items, int s_max, int n_sms) { return vvs::attention_split(hd, items, s_max, n_sms); }
-""" % ", ".join("p." + f for f in FIELDS)
+""" % (", ".join("p." + f for f in FIELDS), ", ".join("p." + f for f in FEW_FIELDS))
 
 # (d_model, d_ff): the benchmark shapes, one between them, one below and one above
 WIDTHS = [(1024, 2752), (1280, 3456), (1536, 2744), (2048, 5504), (4096, 11008), (8192, 22016)]
@@ -72,6 +78,34 @@ def test_projection_plans_fit_the_hardware(plans, d, ff):
             assert (p["smem_bytes"] + 1024) * 512 >= p["tmem_cols"] * 228 * 1024 - 512, at
             assert p["threads"] in (256, 512) and p["threads"] % (128 // p["splits"]) == 0, at
             assert p["ss_parts"] % 4 == 0 and p["ss_parts"] <= p["tiles"] * 8, at
+
+
+@pytest.mark.parametrize("d,ff", [(1024, 320), (1024, 2752), (1152, 3072), (1280, 3456), (1280, 64), (2048, 128)])
+def test_few_token_plans_fit_the_hardware(plans, d, ff):
+    for m in range(1, 97):
+        for n, k, dual, add in ((3 * d, d, 0, 0), (d, d, 0, 1), (ff, d, 1, 0), (d, ff, 0, 1)):
+            out = (ctypes.c_int * (len(FEW_FIELDS) + 1))()
+            plans.few(m, n, k, dual, add, out)
+            p = dict(zip(FEW_FIELDS + ("ss_parts",), out))
+            at = (m, n, k, dual, add, p)
+            assert p["nt"] % 8 == 0 and p["nt"] - 8 < m <= p["nt"], at
+            assert p["tiles"] == -(-n // (32 if dual else 64)) and p["kb_total"] == k // 64, at
+            # the kernels that exist: gate/up unsplit, QKV in one or two slices, the others in one or four; rings have stages of four
+            assert p["splits"] in ((1,) if dual else (1, 4) if add else (1, 2)) and p["splits"] <= p["kb_total"], at
+            per_cta = -(-p["kb_total"] // p["splits"])
+            groups = -(-per_cta // p["group"])
+            assert p["group"] in (4, 5, 7) and 1 <= p["stages"] <= min(12, groups) and p["ring"] == (p["stages"] < groups), at
+            assert not p["ring"] or (p["group"] == 4 and p["stages"] >= 2), at
+            # stages, and the tile's rows beside them (split) or over them
+            stage, recv = p["group"] * (64 + p["nt"]) * 128, -(-m // 4) * 1024
+            assert p["recv_off"] == (p["stages"] * stage if p["splits"] > 1 else 0), at
+            need = p["stages"] * stage + recv if p["splits"] > 1 else max(p["stages"] * stage, recv)
+            assert need + 1024 <= p["smem_bytes"] <= 226 * 1024, at
+            assert p["nt"] <= p["tmem_cols"] and p["tmem_cols"] in (32, 64, 128), at
+            assert (p["smem_bytes"] + 1024) * 512 >= p["tmem_cols"] * 228 * 1024 - 512, at
+            # the sums of squares: whole float4, room for d / 8 of them per token
+            assert p["ss_parts"] % 4 == 0 and p["tiles"] * p["splits"] <= p["ss_parts"] < p["tiles"] * p["splits"] + 4, at
+            assert not add or p["ss_parts"] <= (d + 127) // 128 * 16, at
 
 
 def test_passes_over_weights_that_exceed_l2(plans):
