@@ -155,29 +155,50 @@ struct ProjFewPlan {
 // partial sums of squares per token an ADD projection writes: one per tile and slice, rounded up to whole float4
 inline int proj_ss_parts(const ProjFewPlan& pl) { return (pl.tiles * pl.splits + 3) & ~3; }
 
-// One pass of at most kFewTok tokens, k a multiple of 64, for models whose weights are requested into L2 ahead.  K slices: proj_few.cu
-// has the measurements; fewer than eight k-blocks are not worth an exchange.
-inline ProjFewPlan plan_proj_few(int m, int n, int k, bool dual, bool add) {
+// One pass of at most kFewTok tokens, k a multiple of 64; no stages: proj_tc.cu has to take it.  K slices: proj_few.cu has the
+// measurements; fewer than eight k-blocks are not worth an exchange.
+// in_l2: the model's weights are requested into L2 ahead and a CTA takes as much shared memory as its K range fills.
+// Weights that come from HBM need all CTAs on the device at once, and those of the next projection beside them as they leave: one,
+// two or three CTAs per SM, as many as it takes, rings of stages of two k-blocks.  7B shape, 18 tokens, against proj_tc.cu on 128-row
+// tiles, 2967 us a step: QKV alone here (384 CTAs, three per SM) 2886, with 1 slice and two per SM 2894; output projection (256, two)
+// 2897; gate/up (344, three) 2875, with two per SM, i.e. two waves, 2998; down projection (256, two) 2941; all 2699.  d_model 2048, 24
+// layers, 18 tokens: 960 -> 803, with one CTA per SM and two waves 908, with two per SM everywhere 838; stages of four k-blocks
+// instead of two 858.  More tokens fill shared memory from L2 rather than from HBM: d_model 2048, 64 / 96 tokens 1193 -> 986 / 1166 ->
+// 1147; eight layers of 7B, 64 / 80 / 96 tokens 823 -> 792 / 851 -> 828 / 923 -> 915; of d_model 5120, 18 / 80 / 96 tokens 1019 -> 927 /
+// 1248 -> 1231 / 1502 -> 1524 (hence 80 for matrices beyond 64 MB).  Where even three CTAs per SM are not enough (d_model 8192) proj_tc.cu
+// is the better one, 18 / 48 tokens 1034 / 1080 us against 1033 / 1132 with fewer slices.
+inline ProjFewPlan plan_proj_few(int m, int n, int k, bool dual, bool add, bool in_l2, int n_sms) {
   using namespace proj;
   ProjFewPlan pl{};
   pl.nt = (m + 7) / 8 * 8;
   pl.tiles = (n + (dual ? 31 : 63)) / (dual ? 32 : 64);
   pl.kb_total = k / (int)kBlockK;
   pl.splits = dual || pl.kb_total < 8 ? 1 : add ? 4 : 2;
+  int q = 1;
+  if (!in_l2) {
+    const bool huge = (size_t)n * k * (dual ? 4 : 2) > (size_t)64 << 20;
+    if (!add && pl.tiles <= 2 * n_sms && pl.tiles * pl.splits > 3 * n_sms) pl.splits = 1;
+    const int ctas = pl.tiles * pl.splits, fit = pl.splits == 4 ? n_sms * 33 / 37 : n_sms;      // (clusters of four: as in plan_proj)
+    while (q < 3 && ctas > q * fit) ++q;
+    if (ctas > q * fit || (huge && m > 80)) return ProjFewPlan{};
+  }
   const int kb_bytes = 64 * (int)kBlockK * 2 + pl.nt * (int)kBlockK * 2, per_cta = (pl.kb_total + pl.splits - 1) / pl.splits;
   // the tile's rows on their way to the epilogue: unsplit they lie over the drained stages
-  const int recv = (m + 3) / 4 * 64 * 16, beside = pl.splits > 1 ? recv : 0, room = kFewSmem - 1024 - beside;
+  const int recv = (m + 3) / 4 * 64 * 16, beside = pl.splits > 1 ? recv : 0;
+  const int room = (q == 1 ? kFewSmem : 228 * 1024 / q - 2048) - 1024 - beside;      // for stages (a CTA's fixed part and the system's: 2 KB)
   // All k-blocks at once where they fit, in stages of four, five or seven: as few blocks beyond the range as there can be, then as
-  // few stages.  A ring has stages of four.
+  // few stages.
   auto fit = [&](int g) { return (per_cta + g - 1) / g * g * kb_bytes <= room; };
   pl.group = 4;
   for (int g = 5; g <= 7; g += 2)
     if (fit(g) && (per_cta + g - 1) / g * g <= (per_cta + pl.group - 1) / pl.group * pl.group) pl.group = g;
+  if (!in_l2 && !fit(pl.group)) pl.group = 2;
   const int stage_bytes = pl.group * kb_bytes, groups = (per_cta + pl.group - 1) / pl.group;
   pl.stages = room / stage_bytes;
   if (pl.stages > kFewStages) pl.stages = kFewStages;
   if (pl.stages > groups) pl.stages = groups;
   pl.ring = pl.stages < groups;
+  if (pl.ring && pl.stages < 2) return ProjFewPlan{};
   pl.recv_off = beside ? pl.stages * stage_bytes : 0;
   pl.smem_bytes = pl.stages * stage_bytes + beside + 1024;
   if (pl.smem_bytes < recv + 1024) pl.smem_bytes = recv + 1024;

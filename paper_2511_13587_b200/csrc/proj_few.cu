@@ -415,7 +415,8 @@ cudaError_t launch_one(const ProjFewPlan& pl, const Params& kp, const ProjArgs& 
 template <int EPI, int LOG_S>
 cudaError_t launch_epi(const ProjFewPlan& pl, const Params& kp, const ProjArgs& g, cudaStream_t s) {
   if (pl.splits != 1 << LOG_S) return cudaErrorInvalidValue;
-  if (pl.ring) return launch_one<EPI, LOG_S, 4, true>(pl, kp, g, s);          // (a ring has stages of four)
+  if (pl.ring) return pl.group == 2 ? launch_one<EPI, LOG_S, 2, true>(pl, kp, g, s) : launch_one<EPI, LOG_S, 4, true>(pl, kp, g, s);
+  if (pl.group == 2) return launch_one<EPI, LOG_S, 2, false>(pl, kp, g, s);
   if (pl.group == 4) return launch_one<EPI, LOG_S, 4, false>(pl, kp, g, s);
   if (pl.group == 5) return launch_one<EPI, LOG_S, 5, false>(pl, kp, g, s);
   return launch_one<EPI, LOG_S, 7, false>(pl, kp, g, s);
@@ -437,7 +438,7 @@ int launch_proj_few(int epi, const ProjFewPlan& pl, const ProjArgs& g, cudaStrea
   cudaError_t e;
   switch (epi) {
     case PROJ_QKV: e = pl.splits == 2 ? launch_epi<PROJ_QKV, 1>(pl, kp, g, s) : launch_epi<PROJ_QKV, 0>(pl, kp, g, s); break;
-    case PROJ_ADD: e = pl.splits == 4 ? launch_epi<PROJ_ADD, 2>(pl, kp, g, s) : launch_epi<PROJ_ADD, 0>(pl, kp, g, s); break;
+    case PROJ_ADD: e = pl.splits == 4 ? launch_epi<PROJ_ADD, 2>(pl, kp, g, s) : pl.splits == 2 ? launch_epi<PROJ_ADD, 1>(pl, kp, g, s) : launch_epi<PROJ_ADD, 0>(pl, kp, g, s); break;
     case PROJ_GATEUP: e = launch_epi<PROJ_GATEUP, 0>(pl, kp, g, s); break;
     default: return VVS_ERR_INVALID_ARG;
   }

@@ -373,17 +373,18 @@ int finish_verify_tc(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_ou
 bool folded_applicable(const vvs_ctx* ctx) { return !ctx->use_chain_kernels && ctx->desc.d_model >= 1024; }
 
 // FewMaps of a stage of `group` k-blocks
-inline int few_map(int group) { return group == 4 ? 0 : group == 5 ? 1 : 2; }
+inline int few_map(int group) { return group == 2 ? 0 : group == 4 ? 1 : group == 5 ? 2 : 3; }
 
 // The kernel and plan of one projection.
 struct ProjPick {
   bool few;
   ProjPlan wide{};
   ProjFewPlan small{};
-  ProjPick(int epi, int m, int n, int k, bool in_l2, int n_sms) : few(in_l2 && m <= proj::kFewTok) {      // (in_l2: see run_verify_folded)
+  ProjPick(int epi, int m, int n, int k, bool in_l2, bool whole, int n_sms) : few(whole && m <= proj::kFewTok) {
     const bool dual = epi == PROJ_GATEUP;
-    if (few) small = plan_proj_few(m, n, k, dual, epi == PROJ_ADD);
-    else wide = plan_proj(m, n, k, dual, n_sms);
+    if (few) small = plan_proj_few(m, n, k, dual, epi == PROJ_ADD, in_l2, n_sms);
+    few = small.stages > 0;
+    if (!few) wide = plan_proj(m, n, k, dual, n_sms);
   }
   int make_tmap(CUtensorMap* tm, const void* act, int m, int k) const {
     return few ? make_tmap_bf16_blocks(tm, act, (uint64_t)m, (uint64_t)k, (uint32_t)small.nt, (uint32_t)small.group)
@@ -409,9 +410,9 @@ int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_o
   // 3.11 -> 4.26 ms)
   const size_t layer_bytes = ((size_t)4 * d + (size_t)3 * ff) * d * sizeof(T);
   const bool prefetch = 3 * layer_bytes <= (size_t)ctx->l2_bytes;
-  const bool few = prefetch && ff % 64 == 0;        // (proj_few.cu takes whole k-blocks)
-  const ProjPick p_qkv(PROJ_QKV, M, 3 * d, d, few, ctx->n_sms), p_o(PROJ_ADD, M, d, d, few, ctx->n_sms);
-  const ProjPick p_gu(PROJ_GATEUP, M, ff, d, few, ctx->n_sms), p_down(PROJ_ADD, M, d, ff, few, ctx->n_sms);
+  const bool whole = ff % 64 == 0;                  // (proj_few.cu takes whole k-blocks)
+  const ProjPick p_qkv(PROJ_QKV, M, 3 * d, d, prefetch, whole, ctx->n_sms), p_o(PROJ_ADD, M, d, d, prefetch, whole, ctx->n_sms);
+  const ProjPick p_gu(PROJ_GATEUP, M, ff, d, prefetch, whole, ctx->n_sms), p_down(PROJ_ADD, M, d, ff, prefetch, whole, ctx->n_sms);
   CUtensorMap tm_xq, tm_xg, tm_attn, tm_act;
   if (p_qkv.make_tmap(&tm_xq, xn, M, d) != VVS_OK || p_gu.make_tmap(&tm_xg, xn, M, d) != VVS_OK ||
       p_o.make_tmap(&tm_attn, attn, M, d) != VVS_OK || p_down.make_tmap(&tm_act, act, M, ff) != VVS_OK)
@@ -902,7 +903,7 @@ int vvs_bind_weights(vvs_ctx* ctx, const vvs_weights* w) {
         FewMaps& q = ctx->few_maps[l];
         if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_gate, s.w_gate, ff, d, 32, 1);
         if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_up, s.w_up, ff, d, 32, 1);
-        for (int g : {4, 5, 7}) {
+        for (int g : {2, 4, 5, 7}) {
           if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_qkv[few_map(g)], s.w_qkv, 3 * (uint64_t)d, d, 64, g);
           if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_o[few_map(g)], s.w_o, d, d, 64, g);
           if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_down[few_map(g)], s.w_down, d, ff, 64, g);

@@ -129,7 +129,7 @@ struct LayerMaps {
 };
 // the same matrices in the boxes of proj_few.cu: 64 rows (32 of gate and up) of one to several k-blocks
 struct FewMaps {
-  CUtensorMap w_gate, w_up, w_qkv[3], w_o[3], w_down[3];   // [stages of four, five, seven k-blocks]
+  CUtensorMap w_gate, w_up, w_qkv[4], w_o[4], w_down[4];   // [stages of two, four, five, seven k-blocks]
 };
 
 }  // namespace vvs

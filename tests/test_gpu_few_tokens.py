@@ -17,6 +17,11 @@ FEW64 = replace(XL, name="few64", n_layers=2, d_model=1024, n_heads=16, d_ff=275
 # heads of two tiles; 18 tiles: sums of squares in rows of 18 and 72 parts; a down projection of 5 k-blocks, unsplit
 FEW128 = replace(B7, name="few128", n_layers=2, d_model=1152, n_heads=9, d_ff=320, vocab=1096, vocab_offset=64, lm_rows=2048,
                  tok_rows=0, s_max=700)
+# weights that do not stay in L2: rings of two k-blocks, one CTA per SM; 47 k-blocks in four slices
+STREAM1 = replace(XL, name="stream1", n_layers=1, d_model=1536, n_heads=24, d_ff=3008, vocab=1096, lm_rows=0, tok_rows=0, s_max=208)
+# the same with two CTAs per SM (QKV, 192) and three (gate and up, 298)
+STREAM3 = replace(B7, name="stream3", n_layers=1, d_model=2048, n_heads=16, d_ff=9536, vocab=1096, vocab_offset=64, lm_rows=2048,
+                  tok_rows=0, s_max=700)
 
 
 @pytest.mark.parametrize("ms,n_images,n_cfg,n_forced,k,fills", [
@@ -30,7 +35,13 @@ FEW128 = replace(B7, name="few128", n_layers=2, d_model=1152, n_heads=9, d_ff=32
     (FEW64, 97, 1, 1, 0, list(range(97))),                 # 97
     (FEW128, 1, 2, 1, 8, [513]),                           # 18
     (FEW128, 3, 2, 1, 4, [5, 160, 677]),                   # 30
-    (FEW128, 4, 1, 3, 20, [5, 160, 333, 64])])             # 92
+    (FEW128, 4, 1, 3, 20, [5, 160, 333, 64]),              # 92
+    (STREAM1, 1, 1, 1, 0, [0]),
+    (STREAM1, 1, 2, 1, 8, [199]),
+    (STREAM1, 3, 2, 1, 15, [0, 47, 150]),                  # 96
+    (STREAM3, 1, 2, 1, 8, [513]),
+    (STREAM3, 2, 2, 6, 10, [3, 677]),                      # 64
+    (STREAM3, 3, 1, 3, 24, [5, 160, 333])])                # 81: gate and up (78 MB) in proj_tc.cu, the others here
 def test_few_tokens(ms, n_images, n_cfg, n_forced, k, fills):
     case = H.build_case_independent(ms, 1900 + k, n_images, n_cfg, n_forced, k, fills, logit_std=0.6)
     run = H.GpuRunner(ms, case["w"], n_images * n_cfg, n_forced + k)

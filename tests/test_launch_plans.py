@@ -19,8 +19,8 @@ extern "C" void proj(int m, int n, int k, int dual, int n_sms, int* o) {
   const int v[] = {%s, vvs::proj_ss_parts(p)};
   for (unsigned i = 0; i < sizeof(v) / sizeof(v[0]); ++i) o[i] = v[i];
 }
-extern "C" void few(int m, int n, int k, int dual, int add, int* o) {
-  const vvs::ProjFewPlan p = vvs::plan_proj_few(m, n, k, dual != 0, add != 0);
+extern "C" void few(int m, int n, int k, int dual, int add, int in_l2, int n_sms, int* o) {
+  const vvs::ProjFewPlan p = vvs::plan_proj_few(m, n, k, dual != 0, add != 0, in_l2 != 0, n_sms);
   const int v[] = {%s, vvs::proj_ss_parts(p)};
   for (unsigned i = 0; i < sizeof(v) / sizeof(v[0]); ++i) o[i] = v[i];
 }
@@ -80,22 +80,28 @@ def test_projection_plans_fit_the_hardware(plans, d, ff):
             assert p["ss_parts"] % 4 == 0 and p["ss_parts"] <= p["tiles"] * 8, at
 
 
-@pytest.mark.parametrize("d,ff", [(1024, 320), (1024, 2752), (1152, 3072), (1280, 3456), (1280, 64), (2048, 128)])
-def test_few_token_plans_fit_the_hardware(plans, d, ff):
+@pytest.mark.parametrize("d,ff,in_l2", [(1024, 320, 1), (1024, 2752, 1), (1152, 3072, 1), (1280, 3456, 1), (1280, 64, 1), (2048, 128, 1),
+                                        (1536, 3008, 0), (2048, 5504, 0), (4096, 11008, 0), (5120, 13824, 0), (8192, 28672, 0),
+                                        (1024, 65536, 0), (16384, 64, 0)])
+def test_few_token_plans_fit_the_hardware(plans, d, ff, in_l2):
+    taken = 0
     for m in range(1, 97):
         for n, k, dual, add in ((3 * d, d, 0, 0), (d, d, 0, 1), (ff, d, 1, 0), (d, ff, 0, 1)):
             out = (ctypes.c_int * (len(FEW_FIELDS) + 1))()
-            plans.few(m, n, k, dual, add, out)
+            plans.few(m, n, k, dual, add, in_l2, N_SMS, out)
             p = dict(zip(FEW_FIELDS + ("ss_parts",), out))
             at = (m, n, k, dual, add, p)
+            if not in_l2 and p["stages"] == 0:
+                continue                                            # left to proj_tc.cu
+            taken += 1
             assert p["nt"] % 8 == 0 and p["nt"] - 8 < m <= p["nt"], at
             assert p["tiles"] == -(-n // (32 if dual else 64)) and p["kb_total"] == k // 64, at
-            # the kernels that exist: gate/up unsplit, QKV in one or two slices, the others in one or four; rings have stages of four
+            # the kernels that exist: gate/up unsplit, QKV in one or two slices, the others in one or four; rings have stages of two or four
             assert p["splits"] in ((1,) if dual else (1, 4) if add else (1, 2)) and p["splits"] <= p["kb_total"], at
             per_cta = -(-p["kb_total"] // p["splits"])
             groups = -(-per_cta // p["group"])
-            assert p["group"] in (4, 5, 7) and 1 <= p["stages"] <= min(12, groups) and p["ring"] == (p["stages"] < groups), at
-            assert not p["ring"] or (p["group"] == 4 and p["stages"] >= 2), at
+            assert p["group"] in (2, 4, 5, 7) and 1 <= p["stages"] <= min(12, groups) and p["ring"] == (p["stages"] < groups), at
+            assert not p["ring"] or (p["group"] == (4 if in_l2 else 2) and p["stages"] >= 2), at
             # stages, and the tile's rows beside them (split) or over them
             stage, recv = p["group"] * (64 + p["nt"]) * 128, -(-m // 4) * 1024
             assert p["recv_off"] == (p["stages"] * stage if p["splits"] > 1 else 0), at
@@ -106,6 +112,11 @@ def test_few_token_plans_fit_the_hardware(plans, d, ff):
             # the sums of squares: whole float4, room for d / 8 of them per token
             assert p["ss_parts"] % 4 == 0 and p["tiles"] * p["splits"] <= p["ss_parts"] < p["tiles"] * p["splits"] + 4, at
             assert not add or p["ss_parts"] <= (d + 127) // 128 * 16, at
+            if not in_l2:                                           # all CTAs at once, with 1 KB each for the system and what is static
+                per_sm = 228 * 1024 // (p["smem_bytes"] + 2048) if p["smem_bytes"] <= 112 * 1024 else 1
+                assert p["tiles"] * p["splits"] <= per_sm * N_SMS * (33 / 37 if p["splits"] == 4 else 1), at
+    assert taken == 4 * 96 if in_l2 else taken > 0 or d > 8000
+
 
 
 def test_passes_over_weights_that_exceed_l2(plans):
