@@ -4,14 +4,19 @@
 //
 // One CTA per (sequence, head) -- or a cluster of S CTAs when there are few of them and the cache may be long
 // (attention_split, launch_plans.h).  Every warp
-// owns the 16-key slices w, w + W, ... and streams them through a ring of its own (cp.async, 16-byte pieces, D
+// owns the slices w, w + W, ... of 16 or 32 keys and streams them through a ring of its own (cp.async, 16-byte pieces, D
 // slices deep): no barrier inside the loop.  Slices of old keys are requested BEFORE griddepcontrol.wait, while the
 // QKV projection is still running; after the wait only q (registers) and the one to three slices that hold new keys
 // travel.  Online softmax per warp, then one merge through shared memory in warp order (and rank order), so the
 // result does not depend on timing.
 //
 // What bounds it: with few items the dependency chain (wait, q from L2, two or three slices, merge), which is why an
-// item gets as many warps as it has slices to deal; with many items the K / V stream.
+// item gets as many warps as it has slices to deal; with many items the instructions a warp executes one after the other (7.4 cycles
+// each; half of them were per item, not per slice).  Hence no masks on slices of old keys only, scaling and subtraction as one
+// FMA, copies and merge with addresses of one add each, and the next item's first slices requested before the merge, whose
+// buffer lies over the last slot of the rings only.  XL shape, 16 images (288 tokens, 640 items) 1803 -> 1724 us a step, fills of 300 to 575
+// 1946 -> 1848; 8 images 1384 -> 1294, 4 images 1006 -> 958; 5 images of 27 rows each 1721 -> 1596; d_model 2048, 16 images of 4 rows
+// 1800 -> 1739; one image 708 -> 702 (a cache filled to 570: 756 -> 761), a tree of 27 rows 872 -> 865.
 #include "att_mma.cuh"
 #include "tc_common.cuh"
 #include "vvs_internal.cuh"
@@ -30,22 +35,103 @@ __device__ __forceinline__ void st_async2(uint32_t addr, uint32_t bar, float a, 
                ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
 }
 
-// shared memory: rings of the W warps, over which the merge buffers lie afterwards; then, in a cluster, the states of
-// ranks 1 .. S-1 (written by them into rank 0)
-template <int HD, int NMT, int W, int D>
+// Shared memory: the rings of the W warps, [slot][warp]; the merge buffer lies over the last slot of them; then, in a cluster,
+// the states of ranks 1 .. S-1 (written by them into rank 0).  A slice is 16 NS keys.
+template <int HD, int NMT, int W, int D, int NS, bool MANY>
 struct Smem {
-  static constexpr int kSlice = 64 * HD;                      // 16 keys, K and V
-  static constexpr int kRing = W * D * kSlice;
+  static constexpr int kSlice = 64 * HD * NS;                 // K, then V
   static constexpr int kLd = HD + 8;                          // padded row of the merge buffer
   static constexpr int kMerge = W * NMT * 16 * (kLd + 2) * 4;
-  static constexpr int kMain = kRing > kMerge ? kRing : kMerge;
+  static constexpr int kRing = D * W * kSlice, kMergeAt = MANY ? (D - 1) * W * kSlice : 0;
+  static constexpr int kMain = kRing > kMergeAt + kMerge ? kRing : kMergeAt + kMerge;
   static int bytes(int t_len, int s) { return kMain + (s - 1) * t_len * (HD + 2) * 4; }
 };
 
-template <int HD, int NMT, int W, int D>
+// The 16 NS keys of a slice against the 16 query rows of an m-tile.  MASKED: bit k of vis[i] = key k is visible to row g + 8 i, of
+// vmem = row k of the V tile holds data (others are zeroed before they are multiplied).  The running maximum is kept unscaled, so that
+// scaling and subtraction are one FMA.
+template <int HD, int NS, bool MASKED>
+__device__ __forceinline__ void att_keys(AttState<HD>& st, const uint32_t (&qa)[HD / 16][4], uint32_t k_base, uint32_t v_base, int lane,
+                                         float sl2, const uint32_t (&vis)[2], uint32_t vmem) {
+  constexpr uint32_t kChunk = NS * 2048u;                     // 64 columns of all keys
+  const int c = lane & 3, mi = lane >> 3, ri = lane & 7;
+  float s[2 * NS][4];
+#pragma unroll
+  for (int n = 0; n < 2 * NS; ++n)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) s[n][e] = 0.f;
+#pragma unroll
+  for (int kk = 0; kk < HD / 16; ++kk) {
+    const int cc = 2 * kk + (mi & 1);
+    const uint32_t at = k_base + (cc >> 3) * kChunk + (((mi >> 1) << 3) + ri) * 128 + (((cc & 7) ^ ri) << 4);
+#pragma unroll
+    for (int n = 0; n < NS; ++n) {
+      uint32_t r0, r1, r2, r3;
+      ldsm4(at + n * 2048, r0, r1, r2, r3);
+      mma16816(s[2 * n], qa[kk][0], qa[kk][1], qa[kk][2], qa[kk][3], r0, r1);
+      mma16816(s[2 * n + 1], qa[kk][0], qa[kk][1], qa[kk][2], qa[kk][3], r2, r3);
+    }
+  }
+  // online softmax for rows g (i = 0) and g + 8 (i = 1); this lane holds keys 8 n + 2c, 8 n + 2c + 1
+  uint32_t pa[NS][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    if (MASKED) {
+      const uint32_t vb = vis[i] >> (2 * c);
+#pragma unroll
+      for (int n = 0; n < 2 * NS; ++n)
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (!((vb >> (8 * n + e)) & 1u)) s[n][2 * i + e] = -CUDART_INF_F;
+    }
+    float mx = fmaxf(s[0][2 * i], s[0][2 * i + 1]);
+#pragma unroll
+    for (int n = 1; n < 2 * NS; ++n) mx = fmaxf(mx, fmaxf(s[n][2 * i], s[n][2 * i + 1]));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    const float m_new = fmaxf(st.m[i], mx);
+    const float m_scaled = m_new == -CUDART_INF_F ? 0.f : m_new * sl2;
+    const float alpha = ex2(fmaf(st.m[i], sl2, -m_scaled));
+    st.m[i] = m_new;
+    float sum = 0.f;
+#pragma unroll
+    for (int n = 0; n < 2 * NS; ++n) {
+      const float p0 = ex2(fmaf(s[n][2 * i], sl2, -m_scaled)), p1 = ex2(fmaf(s[n][2 * i + 1], sl2, -m_scaled));
+      sum += p0 + p1;
+      pa[n >> 1][i + 2 * (n & 1)] = pack2(p0, p1);
+    }
+    st.l[i] = fmaf(st.l[i], alpha, sum);
+#pragma unroll
+    for (int j = 0; j < HD / 8; ++j) {
+      st.o[j][2 * i] *= alpha;
+      st.o[j][2 * i + 1] *= alpha;
+    }
+  }
+  // O += P V
+#pragma unroll
+  for (int n = 0; n < NS; ++n) {
+    const uint32_t vm = vmem >> (16 * n + 2 * c);
+    const uint32_t vlo = (vm & 1u ? 0x0000ffffu : 0u) | (vm & 2u ? 0xffff0000u : 0u);
+    const uint32_t vhi = (vm & 0x100u ? 0x0000ffffu : 0u) | (vm & 0x200u ? 0xffff0000u : 0u);
+#pragma unroll
+    for (int jj = 0; jj < HD / 16; ++jj) {
+      const int cc = 2 * jj + (mi >> 1);
+      uint32_t r0, r1, r2, r3;
+      ldsm4t(v_base + (cc >> 3) * kChunk + n * 2048 + (((mi & 1) << 3) + ri) * 128 + (((cc & 7) ^ ri) << 4), r0, r1, r2, r3);
+      if (MASKED) {
+        r0 &= vlo; r1 &= vhi; r2 &= vlo; r3 &= vhi;
+      }
+      mma16816(st.o[2 * jj], pa[n][0], pa[n][1], pa[n][2], pa[n][3], r0, r1);
+      mma16816(st.o[2 * jj + 1], pa[n][0], pa[n][1], pa[n][2], pa[n][3], r2, r3);
+    }
+  }
+}
+
+template <int HD, int NMT, int W, int D, int NS, bool MANY>
 __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockArgs a) {
-  using L = Smem<HD, NMT, W, D>;
-  constexpr int NC = HD / 64, NJ = HD / 8;
+  using L = Smem<HD, NMT, W, D, NS, MANY>;
+  constexpr int NC = HD / 64, NJ = HD / 8, KS = 16 * NS;
+  constexpr uint32_t kChunk = NS * 2048u;
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ __align__(8) uint64_t x_bar;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, c = lane & 3;
@@ -54,7 +140,7 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
   const int groups = (NMT == 1 && T > 16) ? 2 : 1;
   const int wpg = W / groups, grp = warp / wpg, wg = warp - grp * wpg;
   const int first = rank * wpg + wg, stride = S * wpg;
-  const uint32_t ring = tc::smem_u32(smem) + (uint32_t)(warp * D) * L::kSlice;
+  const uint32_t ring = tc::smem_u32(smem) + (uint32_t)warp * L::kSlice;
 
   if (S > 1) {
     if (tid == 0) {
@@ -66,61 +152,58 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
     tc::cluster_arrive();
   }
   const int n_items = a.n_heads * a.n_rows, G = (int)gridDim.x;
+  // 16-byte pieces of a slice: this lane's first key and chunk; a step of kStep keys keeps the chunk and changes the swizzle by
+  // a constant
+  constexpr int kPer = HD / 8, kStep = 32 / kPer;
+  const int key0 = lane / kPer, ch = lane % kPer;
+  const uint32_t piece = (uint32_t)(ch >> 3) * kChunk + key0 * 128, swz = (uint32_t)((ch & 7) ^ key0) << 4;
+  struct Item {
+    int h, r, fill, n_keys, n_old, n_slices;                    // n_old: slices that hold old keys only
+    const bf16* kp; const bf16* vp;                             // this lane's pieces of the first keys
+  };
   // More items than the GPU holds CTAs: the grid is one wave, and its CTAs walk the list forth and back (longest first).
-#pragma unroll 1
-  for (int k = 0;; ++k) {
-    const int item = k * G + ((k & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
-    if (item >= n_items) break;
-    const int h = item % a.n_heads, r = a.seq_order[item / a.n_heads];
-    const int fill = a.cache_len[r];
-    const bool ok = fill >= 0 && fill + T <= a.s_max;
-    const size_t row_base = ((size_t)(a.layer * a.kv_rows + r) * a.n_heads + h) * a.s_max;
-    const bf16* kp = a.kv_k + row_base * HD;
-    const bf16* vp = a.kv_v + row_base * HD;
-    const int n_keys = ok ? fill + T : 0;
-    const int n_old = ok ? fill >> 4 : 0;                       // slices that hold old keys only
-    const int n_slices = (n_keys + 15) >> 4;
-    if (k > 0) __syncthreads();                                 // the merge of the item before is done with the rings
-    auto request = [&](int i) {                                 // slice i of this warp into its ring slot
-      const int s = first + i * stride;
-      const uint32_t dst0 = ring + (uint32_t)(i % D) * L::kSlice;
-      const int rows = min(16, n_keys - s * 16);
-      constexpr int per_row = HD / 8;                           // 16-byte pieces
+  auto item_of = [&](int k) { return k * G + ((k & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x); };
+  auto locate = [&](int item, Item& it) {
+    const int rk = item / a.n_heads;
+    it.h = item - rk * a.n_heads;
+    it.r = a.seq_order[rk];
+    it.fill = a.cache_len[it.r];
+    const bool ok = it.fill >= 0 && it.fill + T <= a.s_max;
+    const size_t at = (((size_t)(a.layer * a.kv_rows + it.r) * a.n_heads + it.h) * a.s_max + key0) * HD + ch * 8;
+    it.kp = a.kv_k + at;
+    it.vp = a.kv_v + at;
+    it.n_keys = ok ? it.fill + T : 0;
+    it.n_old = ok ? it.fill / KS : 0;
+    it.n_slices = (it.n_keys + KS - 1) / KS;
+  };
+  auto request = [&](const Item& it, int i) {                   // slice i of this warp into its ring slot
+    const int s = first + i * stride, rows = it.n_keys - s * KS - key0;
+    const uint32_t dst = ring + (uint32_t)(i % D) * (W * L::kSlice) + piece;
+    const bf16* ks = it.kp + (size_t)s * (KS * HD);
+    const bf16* vs = it.vp + (size_t)s * (KS * HD);
 #pragma unroll
-      for (int u = 0; u < 2 * 16 * per_row / 32; ++u) {
-        const int idx = lane + u * 32, which = idx / (16 * per_row), rem = idx - which * 16 * per_row;
-        const int key = rem / per_row, ch = rem - key * per_row;
-        if (key < rows)
-          tc::cp_async16(dst0 + (uint32_t)(which * NC + (ch >> 3)) * 2048u + key * 128 + (((ch & 7) ^ (key & 7)) << 4),
-                     (which ? vp : kp) + (size_t)(s * 16 + key) * HD + ch * 8);
+    for (int u = 0; u < KS / kStep; ++u)
+      if (u * kStep < rows) {
+        const uint32_t at = dst + u * kStep * 128 + (swz ^ (uint32_t)(((u * kStep) & 7) << 4));
+        tc::cp_async16(at, ks + u * kStep * HD);
+        tc::cp_async16(at + NC * kChunk, vs + u * kStep * HD);
       }
-    };
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      if (first + i * stride < n_old) request(i);
-      tc::cp_async_commit();
-    }
-    if (k == 0) tc::pdl_launch_dependents();      // the projection after this kernel may start fetching its weights
-    uint32_t anc[NMT][2];
+  };
+  uint32_t anc[NMT][2], qa[NMT][HD / 16][4];
+  auto load_anc = [&](const Item& it) {
 #pragma unroll
     for (int mi = 0; mi < NMT; ++mi)
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const int t = (grp + mi) * 16 + g + 8 * i;
-        anc[mi][i] = t < T ? a.anc_mask[r * T + t] : 0u;
+        anc[mi][i] = t < T ? a.anc_mask[it.r * T + t] : 0u;
       }
-    if (k == 0) tc::pdl_wait();
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      const int s = first + i * stride;
-      if (s >= n_old && s < n_slices) request(i);
-    }
-    tc::cp_async_commit();
-    uint32_t qa[NMT][HD / 16][4];
+  };
+  auto load_q = [&](const Item& it) {
 #pragma unroll
     for (int mi = 0; mi < NMT; ++mi) {
       const int t0 = (grp + mi) * 16 + g, t1 = t0 + 8;
-      const bf16* q0 = a.q + (size_t)(r * T + t0) * a.d + h * HD + 2 * c;
+      const bf16* q0 = a.q + (size_t)(it.r * T + t0) * a.d + it.h * HD + 2 * c;
       const bf16* q1 = q0 + (size_t)8 * a.d;
 #pragma unroll
       for (int kk = 0; kk < HD / 16; ++kk) {
@@ -130,6 +213,34 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
         qa[mi][kk][3] = t1 < T ? __ldcg(reinterpret_cast<const unsigned*>(q1 + 16 * kk + 8)) : 0u;
       }
     }
+  };
+  const float sl2 = rsqrtf((float)HD) * 1.4426950408889634f;
+
+  // ---- the first item: slices of old keys before the wait ---------------------------------------------------------------
+  Item it;
+  locate(item_of(0), it);                                       // (the grid has no more CTAs than items)
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    if (first + i * stride < it.n_old) request(it, i);
+    tc::cp_async_commit();
+  }
+  tc::pdl_launch_dependents();                  // the projection after this kernel may start fetching its weights
+  load_anc(it);
+  tc::pdl_wait();
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    const int s = first + i * stride;
+    if (s >= it.n_old && s < it.n_slices) request(it, i);
+  }
+  tc::cp_async_commit();
+  load_q(it);
+
+#pragma unroll 1
+  for (int k = 0;; ++k) {
+    const int next_item = item_of(k + 1);
+    const bool more = MANY && next_item < n_items;
+    Item nx;
+    if (more) locate(next_item, nx);
     AttState<HD> st[NMT];
 #pragma unroll
     for (int mi = 0; mi < NMT; ++mi) {
@@ -140,113 +251,157 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
 #pragma unroll
         for (int e = 0; e < 4; ++e) st[mi].o[j][e] = 0.f;
     }
-    const float sl2 = rsqrtf((float)HD) * 1.4426950408889634f;
-
 #pragma unroll 1
-    for (int i = 0; first + i * stride < n_slices; ++i) {
+    for (int i = 0; first + i * stride < it.n_slices; ++i) {
       const int s = first + i * stride;
-      // groups so far: D before the wait, one after it, one per iteration; slice i is in one of the oldest i + 2 of them
+      const uint32_t k_base = ring + (uint32_t)(i % D) * (W * L::kSlice), v_base = k_base + NC * kChunk;
+      // groups so far: D for the first slices, one more, one per iteration; slice i is in one of the oldest i + 2 of them
       // unless it was requested after the wait
-      if (s >= n_old) tc::cp_async_wait<0>(); else tc::cp_async_wait<D - 1>();
-      __syncwarp();
-      const uint32_t k_base = ring + (uint32_t)(i % D) * L::kSlice, v_base = k_base + NC * 2048u;
-      const int left = n_keys - s * 16, old = fill - s * 16;    // valid keys of the slice; old ones among them
-      const uint32_t vmem = left >= 16 ? 0xffffu : ((1u << left) - 1u);
-      const uint32_t vold = old >= 16 ? 0xffffu : old > 0 ? ((1u << old) - 1u) : 0u;
+      if (MANY && s < it.n_old) {
+        tc::cp_async_wait<D - 1>();
+        __syncwarp();
+        const uint32_t all[2] = {0u, 0u};
 #pragma unroll
-      for (int mi = 0; mi < NMT; ++mi) {
-        uint32_t vis[2];
+        for (int mi = 0; mi < NMT; ++mi) att_keys<HD, NS, false>(st[mi], qa[mi], k_base, v_base, lane, sl2, all, 0u);
+      } else {
+        if (MANY || s >= it.n_old) tc::cp_async_wait<0>(); else tc::cp_async_wait<D - 1>();
+        __syncwarp();
+        const int left = it.n_keys - s * KS, old = it.fill - s * KS;      // valid keys of the slice (at least one); old ones among them
+        const uint32_t vmem = 0xffffffffu >> (32 - min(left, KS)), vold = old > 0 ? 0xffffffffu >> (32 - min(old, KS)) : 0u;
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const uint32_t own = old >= 16 ? 0u : old >= 0 ? anc[mi][e] << old : anc[mi][e] >> (-old);
-          vis[e] = (vold | own) & vmem;
+        for (int mi = 0; mi < NMT; ++mi) {
+          uint32_t vis[2];
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const uint32_t own = old >= KS ? 0u : old >= 0 ? anc[mi][e] << old : anc[mi][e] >> (-old);
+            vis[e] = (vold | own) & vmem;
+          }
+          att_keys<HD, NS, true>(st[mi], qa[mi], k_base, v_base, lane, sl2, vis, vmem);
         }
-        att_slice<HD>(st[mi], qa[mi], k_base, v_base, 2048u, 0, lane, sl2, vis, vmem);
       }
       __syncwarp();                                             // every lane is done with the ring slot
-      if (first + (i + D) * stride < n_slices) request(i + D);
+      if (first + (i + D) * stride < it.n_slices) request(it, i + D);
       tc::cp_async_commit();
     }
-    tc::cp_async_wait<0>();
-    // ---- merge: every warp leaves (max, normaliser, output) of its rows, the CTA folds them in warp order --
-    __syncthreads();                                            // the rings have drained everywhere
-    float* s_o = reinterpret_cast<float*>(smem);                // [W][NMT * 16][kLd]
+    // ---- this warp's part of the next item: all slots but the last, over which the merge buffer lies --
+    if (more) {
+#pragma unroll
+      for (int i = 0; i < D - 1; ++i) {
+        if (first + i * stride < nx.n_slices) request(nx, i);
+        tc::cp_async_commit();
+      }
+    }
+    // ---- merge: every warp that had keys leaves (max, normaliser, output) of its rows, the CTA folds them in warp order --
+    const int busy = min(wpg, max(it.n_slices - rank * wpg, 0));
+    __syncthreads();                                            // the last slots have drained everywhere
+    float* s_o = reinterpret_cast<float*>(smem + L::kMergeAt);  // [W][NMT * 16][kLd]
     float* s_ml = s_o + W * NMT * 16 * L::kLd;                  // [W][NMT * 16][2]
+    if (wg < busy) {
 #pragma unroll
-    for (int mi = 0; mi < NMT; ++mi)
+      for (int mi = 0; mi < NMT; ++mi)
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int row = mi * 16 + g + 8 * i;
-        float l = st[mi].l[i];
-        l += __shfl_xor_sync(0xffffffffu, l, 1);
-        l += __shfl_xor_sync(0xffffffffu, l, 2);
-        if ((grp + mi) * 16 + g + 8 * i < T) {
-          float* dst = s_o + (size_t)(warp * NMT * 16 + row) * L::kLd + 2 * c;
+        for (int i = 0; i < 2; ++i) {
+          const int row = mi * 16 + g + 8 * i;
+          float l = st[mi].l[i];
+          l += __shfl_xor_sync(0xffffffffu, l, 1);
+          l += __shfl_xor_sync(0xffffffffu, l, 2);
+          if ((grp + mi) * 16 + g + 8 * i < T) {
+            float* dst = s_o + (size_t)(warp * NMT * 16 + row) * L::kLd + 2 * c;
 #pragma unroll
-          for (int j = 0; j < NJ; ++j) *reinterpret_cast<float2*>(dst + 8 * j) = make_float2(st[mi].o[j][2 * i], st[mi].o[j][2 * i + 1]);
-          if (c == 0) {
-            s_ml[(warp * NMT * 16 + row) * 2] = st[mi].m[i];
-            s_ml[(warp * NMT * 16 + row) * 2 + 1] = l;
+            for (int j = 0; j < NJ; ++j) *reinterpret_cast<float2*>(dst + 8 * j) = make_float2(st[mi].o[j][2 * i], st[mi].o[j][2 * i + 1]);
+            if (c == 0) *reinterpret_cast<float2*>(s_ml + (warp * NMT * 16 + row) * 2) = make_float2(st[mi].m[i] * sl2, l);
           }
         }
-      }
+    }
+    const int h = it.h, r = it.r;
+    if (more) {
+      it = nx;
+      load_anc(it);
+      load_q(it);
+    }
     __syncthreads();
     if (S > 1) tc::cluster_wait();   // rank 0's barrier is ready
     float* xbuf = reinterpret_cast<float*>(smem + L::kMain);    // [S - 1][T][HD + 2]
     const uint32_t x_bar0 = S > 1 ? tc::mapa(tc::smem_u32(&x_bar), 0) : 0u;
     const uint32_t xbuf0 = S > 1 ? tc::mapa(tc::smem_u32(xbuf), 0) : 0u;
     bool waited = S == 1;
-    for (int idx = tid; idx < T * (HD / 2); idx += 32 * W) {
-      const int t = idx / (HD / 2), cp = idx - t * (HD / 2);
+    constexpr int CP = W > 4 ? 2 : 8;                          // columns per item of the merge
+    for (int idx = tid; idx < T * (HD / CP); idx += 32 * W) {
+      const int t = idx / (HD / CP), cp = idx - t * (HD / CP);
       const int grp_t = groups == 2 ? t >> 4 : 0, row = groups == 2 ? t & 15 : t;
-      const float* o_src = s_o + (size_t)(grp_t * wpg * NMT * 16 + row) * L::kLd + 2 * cp;
-      const float* ml = s_ml + (grp_t * wpg * NMT * 16 + row) * 2;
+      const float* o_src = s_o + (size_t)(grp_t * wpg * NMT * 16 + row) * L::kLd + CP * cp;
+      const float2* ml = reinterpret_cast<const float2*>(s_ml) + (grp_t * wpg * NMT * 16 + row);
       float m = -CUDART_INF_F;
 #pragma unroll 4
-      for (int w = 0; w < wpg; ++w) m = fmaxf(m, ml[w * NMT * 32]);
+      for (int w = 0; w < busy; ++w) m = fmaxf(m, ml[w * NMT * 16].x);
       const float m_safe = m == -CUDART_INF_F ? 0.f : m;
-      float l = 0.f, o0 = 0.f, o1 = 0.f;
+      float l = 0.f, o[CP];
+#pragma unroll
+      for (int e = 0; e < CP; ++e) o[e] = 0.f;
 #pragma unroll 4
-      for (int w = 0; w < wpg; ++w) {
-        const float f = ex2(ml[w * NMT * 32] - m_safe);
-        const float2 v = *reinterpret_cast<const float2*>(o_src + (size_t)w * NMT * 16 * L::kLd);
-        l += ml[w * NMT * 32 + 1] * f;
-        o0 += v.x * f;
-        o1 += v.y * f;
+      for (int w = 0; w < busy; ++w) {
+        const float2 x = ml[w * NMT * 16];
+        const float f = ex2(x.x - m_safe);
+        l += x.y * f;
+        const float* v = o_src + (size_t)w * NMT * 16 * L::kLd;
+        if constexpr (CP == 2) {
+          const float2 y = *reinterpret_cast<const float2*>(v);
+          o[0] += y.x * f;
+          o[1] += y.y * f;
+        } else {
+#pragma unroll
+          for (int e = 0; e < CP; e += 4) {
+            const float4 y = *reinterpret_cast<const float4*>(v + e);
+            o[e] += y.x * f; o[e + 1] += y.y * f; o[e + 2] += y.z * f; o[e + 3] += y.w * f;
+          }
+        }
       }
-      if (rank > 0) {
-        const uint32_t dst = xbuf0 + (uint32_t)(((rank - 1) * T + t) * (HD + 2)) * 4u;
-        st_async2(dst + (uint32_t)cp * 8u, x_bar0, o0, o1);
-        if (cp == 0) st_async2(dst + HD * 4u, x_bar0, m, l);
-        continue;
-      }
-      if (!waited) {
-        // the peers' loops hold no unbounded wait; the limit only guards against a CTA that never runs
-        bool got = false;
-        for (uint32_t i = 0; i < 4u * tc::kSpinLimit && !got; ++i) got = tc::mbar_try_wait_cluster(&x_bar, 0);
-        if (!got) atomicOr(a.status, VVS_DEV_TIMEOUT);
-        waited = true;
-      }
-      for (int q = 0; q < S - 1; ++q) {
-        const float* x = xbuf + (size_t)(q * T + t) * (HD + 2);
-        const float mo = x[HD], lo = x[HD + 1];
-        const float m_new = fmaxf(m, mo), ms = m_new == -CUDART_INF_F ? 0.f : m_new;
-        const float aa = ex2(m - ms), bb = ex2(mo - ms);
-        m = m_new;
-        l = l * aa + lo * bb;
-        o0 = o0 * aa + x[2 * cp] * bb;
-        o1 = o1 * aa + x[2 * cp + 1] * bb;
+      bf16* out = a.out + (size_t)(r * T + t) * a.d + h * HD + CP * cp;
+      if constexpr (CP == 2) {
+        if (rank > 0) {
+          const uint32_t dst = xbuf0 + (uint32_t)(((rank - 1) * T + t) * (HD + 2)) * 4u;
+          st_async2(dst + (uint32_t)cp * 8u, x_bar0, o[0], o[1]);
+          if (cp == 0) st_async2(dst + HD * 4u, x_bar0, m, l);
+          continue;
+        }
+        if (!waited) {
+          // the peers' loops hold no unbounded wait; the limit only guards against a CTA that never runs
+          bool got = false;
+          for (uint32_t i = 0; i < 4u * tc::kSpinLimit && !got; ++i) got = tc::mbar_try_wait_cluster(&x_bar, 0);
+          if (!got) atomicOr(a.status, VVS_DEV_TIMEOUT);
+          waited = true;
+        }
+        for (int q = 0; q < S - 1; ++q) {
+          const float* x = xbuf + (size_t)(q * T + t) * (HD + 2);
+          const float mo = x[HD], lo = x[HD + 1];
+          const float m_new = fmaxf(m, mo), ms = m_new == -CUDART_INF_F ? 0.f : m_new;
+          const float aa = ex2(m - ms), bb = ex2(mo - ms);
+          m = m_new;
+          l = l * aa + lo * bb;
+          o[0] = o[0] * aa + x[2 * cp] * bb;
+          o[1] = o[1] * aa + x[2 * cp + 1] * bb;
+        }
       }
       const float inv = l > 0.f ? 1.f / l : 0.f;                // a sequence that failed its cache check gives zeros
-      *reinterpret_cast<uint32_t*>(a.out + (size_t)(r * T + t) * a.d + h * HD + 2 * cp) = pack2(o0 * inv, o1 * inv);
+      if constexpr (CP == 2) {
+        *reinterpret_cast<uint32_t*>(out) = pack2(o[0] * inv, o[1] * inv);
+      } else {
+        *reinterpret_cast<uint4*>(out) = make_uint4(pack2(o[0] * inv, o[1] * inv), pack2(o[2] * inv, o[3] * inv),
+                                                    pack2(o[4] * inv, o[5] * inv), pack2(o[6] * inv, o[7] * inv));
+      }
     }
+    if (!more) break;
+    __syncthreads();                                            // the merge is done with the last slots
+    if (first + (D - 1) * stride < it.n_slices) request(it, D - 1);
+    tc::cp_async_commit();
+    tc::cp_async_commit();                                      // (as many groups as the first item has)
   }
 }
 
-template <int HD, int NMT, int W, int D>
+template <int HD, int NMT, int W, int D, int NS, bool MANY>
 int launch_variant(const AttentionBlockArgs& a, int split, int per_sm, cudaStream_t s) {
-  using L = Smem<HD, NMT, W, D>;
-  const void* fn = reinterpret_cast<const void*>(attention_block_kernel<HD, NMT, W, D>);
+  using L = Smem<HD, NMT, W, D, NS, MANY>;
+  const void* fn = reinterpret_cast<const void*>(attention_block_kernel<HD, NMT, W, D, NS, MANY>);
   if (ensure_dynamic_smem(fn, L::bytes(kMaxT, split)) != cudaSuccess) return VVS_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   int ctas = a.n_heads * a.n_rows;
@@ -269,27 +424,27 @@ int launch_variant(const AttentionBlockArgs& a, int split, int per_sm, cudaStrea
   }
   cfg.attrs = attr;
   cfg.numAttrs = na;
-  return cudaLaunchKernelEx(&cfg, attention_block_kernel<HD, NMT, W, D>, a) == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
+  return cudaLaunchKernelEx(&cfg, attention_block_kernel<HD, NMT, W, D, NS, MANY>, a) == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
 }
 
 }  // namespace
 
-// CTAs per item: attention_split (launch_plans.h).  Warps per item by how many items there are: with few, one item's slices over many warps (XL shape, step of 18 tokens
-// with 16, 8 and 4 warps 962, 1004 and 1013 us; 54 tokens, two row groups of 8 warps 1184, of 4 warps 1286, four warps
-// with two m-tiles each 1272); with many, small CTAs (288 tokens, 640 items: 4 warps, three CTAs per SM 1.88 ms, 8 warps
-// 2.07 ms).  The item loop let the compiler keep addresses in registers: 160 instead of 128 a thread, three CTAs per SM
-// instead of four, and all the same 1.97 -> 1.88 ms (7B shape 3.13 -> 3.08 ms).
+// CTAs per item: attention_split (launch_plans.h).  Warps per item by how many items there are: with few, one item's slices over
+// many warps (XL shape, one image: 16 warps with a slot of 32 keys each 702 us a step, with two of 16 keys 721, 14 warps 698 but 886
+// where they are dealt to two row groups (16: 863), 8 warps with two slots 713); with many, small CTAs: four warps with three slots of 16 keys,
+// three CTAs per SM (16 images 1724, 8 images 1294, 4 images 958; four CTAs per SM with two slots 1716, 1329 and 1021; three with two slots
+// of 32 keys 1766, 1294 and 959), two m-tiles a warp beyond 16 rows (5 images of 27 rows, two slots of 32 keys 1596, three of 16 keys 1624).
+// Heads of 128: 224 items with four warps 1378, with eight 1398.
 int launch_attention_block(const AttentionBlockArgs& a, cudaStream_t s) {
   if (a.t_len > kMaxT) return VVS_ERR_SHAPE;
   const long long items = (long long)a.n_heads * a.n_rows;
-  const bool few = items <= a.n_sms, some = items <= 2LL * a.n_sms;
   const int split = attention_split(a.hd, items, a.s_max, a.n_sms);
   if (a.hd == 64) {
-    if (few) return launch_variant<64, 1, 16, 2>(a, split, 1, s);
-    if (a.t_len > 16) return launch_variant<64, 2, 4, 3>(a, split, 2, s);
-    return some ? launch_variant<64, 1, 8, 3>(a, split, 2, s) : launch_variant<64, 1, 4, 3>(a, split, 3, s);
+    if (items <= a.n_sms) return launch_variant<64, 1, 16, 1, 2, false>(a, split, 1, s);
+    return a.t_len > 16 ? launch_variant<64, 2, 4, 2, 2, true>(a, split, 2, s) : launch_variant<64, 1, 4, 3, 1, true>(a, split, 3, s);
   }
-  if (a.hd == 128) return some ? launch_variant<128, 1, 8, 2>(a, split, 1, s) : launch_variant<128, 1, 4, 3>(a, split, 2, s);
+  if (a.hd == 128)
+    return items <= a.n_sms ? launch_variant<128, 1, 8, 2, 1, true>(a, split, 1, s) : launch_variant<128, 1, 4, 3, 1, true>(a, split, 2, s);
   return VVS_ERR_SHAPE;
 }
 
