@@ -5,10 +5,11 @@
 // - An MMA of 64 rows reads half the shared memory of one of 128 and takes 24 cycles in the place of 40 (N = 24 or 32), so a CTA
 //   can hold more of the K range: gate/up all of it, QKV half, output and down projection a quarter (a cluster of S CTAs then
 //   exchanges partial sums, each pushing 64 rows in the place of 128: a CTA pushes some 32 bytes a cycle into its cluster).
-// - A stage is several k-blocks, loaded by one request and waited for once.
+// - A stage is several k-blocks, loaded by one request and waited for once.  Gate and up are one tensor of two matrices at the distance of
+//   their addresses: as two requests per k-block they took a late CTA 1 us (18 tokens 704 -> 697 us, a tree of 54 868 -> 862).
 // - All stages' weights are requested before tensor memory and the CTA's barrier, then whatever the epilogue needs besides
 //   the sums (rows, places in the cache, rotation) is found, all before griddepcontrol.wait.
-//   QKV, ADD  64 rows of one matrix;  GATEUP  32 rows of gate, then the same 32 of up
+//   QKV, ADD  64 rows of one matrix;  GATEUP  32 rows of gate, then the same 32 of up, in the order of their addresses
 // An accumulator of M = 64 lies in lanes 0-15 of the four lane quarters; its rows go to shared memory as [token quad][rank][row]
 // float4 (split: with st.async to the rank that owns the row, counted on its mbarrier), and the epilogue takes a pair of rows and
 // two tokens per thread (four where 64 rows are finished at once), partial sums in rank order.
@@ -39,7 +40,7 @@ struct Params {
   float* x; __nv_bfloat16* xg; const __nv_bfloat16* scale; float* ss_out; int ss_out_parts; int d;   // ADD
   __nv_bfloat16* q; __nv_bfloat16* kv_k; __nv_bfloat16* kv_v; const int32_t* slot_pos;               // QKV
   const float* rope_cos; const float* rope_sin; int n_heads, hd, s_max, layer, kv_rows, t_len;
-  __nv_bfloat16* act; int ff;                                                                      // GATEUP
+  __nv_bfloat16* act; int ff, up_first;                                                            // GATEUP
   const uint8_t* ahead[2]; uint32_t ahead_bytes;      // weights of the projection after next, to be brought into L2
 };
 
@@ -49,8 +50,7 @@ struct Params {
 // stage are in the loop.
 template <int EPI, int LOG_S, int G, bool RING>
 __global__ void __launch_bounds__(kThreads)
-proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_a2,
-                const __grid_constant__ CUtensorMap tm_b) {
+proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b) {
   constexpr bool DUAL = EPI == PROJ_GATEUP;
   constexpr int NACC = DUAL ? 2 : 1;
   constexpr bool SPLIT = LOG_S > 0;
@@ -77,12 +77,8 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
     uint8_t* st = smem + (size_t)stage * stage_bytes;
     if (elect_one()) {
       mbar_expect_tx(&full_bar[stage], stage_bytes);
-      if (DUAL) {                                    // (gate and up rows of a k-block have to lie together: boxes of one block)
-#pragma unroll
-        for (int j = 0; j < G; ++j) {
-          tma_load_3d(st + j * kABytes, &tm_a, &full_bar[stage], 0, tile * (int)(kRows / 2), kb0 + i * G + j);
-          tma_load_3d(st + j * kABytes + kABytes / 2, &tm_a2, &full_bar[stage], 0, tile * (int)(kRows / 2), kb0 + i * G + j);
-        }
+      if (DUAL) {
+        tma_load_4d(st, &tm_a, &full_bar[stage], 0, tile * (int)(kRows / 2), 0, kb0 + i * G);
       } else {
         tma_load_3d(st, &tm_a, &full_bar[stage], 0, tile * (int)kRows, kb0 + i * G);
       }
@@ -315,7 +311,7 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
     for (int a = 0; a < NACC; ++a)
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        const uint8_t* at = src + a * (kRows / 2 * 16u) + i * 16;
+        const uint8_t* at = src + (DUAL ? a ^ p.up_first : 0) * (kRows / 2 * 16u) + i * 16;
         ld_shared_vec(at, acc[a][i]);
 #pragma unroll
         for (int r = 1; r < S; ++r) {         // rank order
@@ -409,7 +405,7 @@ cudaError_t launch_one(const ProjFewPlan& pl, const Params& kp, const ProjArgs& 
   }
   cfg.attrs = attr;
   cfg.numAttrs = na;
-  return cudaLaunchKernelEx(&cfg, fn, kp, *g.tm_a, g.tm_a2 ? *g.tm_a2 : *g.tm_a, *g.tm_b);
+  return cudaLaunchKernelEx(&cfg, fn, kp, *g.tm_a, *g.tm_b);
 }
 
 template <int EPI, int LOG_S>
@@ -432,7 +428,7 @@ int launch_proj_few(int epi, const ProjFewPlan& pl, const ProjArgs& g, cudaStrea
   kp.x = g.x; kp.xg = g.xg; kp.scale = g.scale; kp.ss_out = g.ss_out; kp.ss_out_parts = proj_ss_parts(pl); kp.d = g.d;
   kp.q = g.q; kp.kv_k = g.kv_k; kp.kv_v = g.kv_v; kp.slot_pos = g.slot_pos; kp.rope_cos = g.rope_cos;
   kp.rope_sin = g.rope_sin; kp.n_heads = g.n_heads; kp.hd = g.hd; kp.s_max = g.s_max; kp.layer = g.layer;
-  kp.kv_rows = g.kv_rows; kp.t_len = g.t_len; kp.act = g.act; kp.ff = g.ff;
+  kp.kv_rows = g.kv_rows; kp.t_len = g.t_len; kp.act = g.act; kp.ff = g.ff; kp.up_first = g.up_first ? 1 : 0;
   kp.ahead[0] = static_cast<const uint8_t*>(g.ahead[0]); kp.ahead[1] = static_cast<const uint8_t*>(g.ahead[1]);
   kp.ahead_bytes = g.ahead[0] ? g.ahead_bytes : 0;
   cudaError_t e;

@@ -412,7 +412,7 @@ int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_o
   const bool prefetch = 3 * layer_bytes <= (size_t)ctx->l2_bytes;
   const bool whole = ff % 64 == 0;                  // (proj_few.cu takes whole k-blocks)
   const ProjPick p_qkv(PROJ_QKV, M, 3 * d, d, prefetch, whole, ctx->n_sms), p_o(PROJ_ADD, M, d, d, prefetch, whole, ctx->n_sms);
-  const ProjPick p_gu(PROJ_GATEUP, M, ff, d, prefetch, whole, ctx->n_sms), p_down(PROJ_ADD, M, d, ff, prefetch, whole, ctx->n_sms);
+  const ProjPick p_gu(PROJ_GATEUP, M, ff, d, prefetch, whole && ctx->few_pairs, ctx->n_sms), p_down(PROJ_ADD, M, d, ff, prefetch, whole, ctx->n_sms);
   CUtensorMap tm_xq, tm_xg, tm_attn, tm_act;
   if (p_qkv.make_tmap(&tm_xq, xn, M, d) != VVS_OK || p_gu.make_tmap(&tm_xg, xn, M, d) != VVS_OK ||
       p_o.make_tmap(&tm_attn, attn, M, d) != VVS_OK || p_down.make_tmap(&tm_act, act, M, ff) != VVS_OK)
@@ -450,7 +450,7 @@ int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_o
     g.n = d; g.tm_a = p_o.few ? &F.w_o[few_map(p_o.small.group)] : &W.w_o; g.tm_b = &tm_attn; g.scale = static_cast<const T*>(ctx->layers[l].norm2);
     ahead(L.w_down, nullptr, d, ff);
     if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = p_o.launch(PROJ_ADD, g, s));
-    g.n = ff; g.tm_a = p_gu.few ? &F.w_gate : &W.w_gate; g.tm_a2 = p_gu.few ? &F.w_up : &W.w_up; g.tm_b = &tm_xg; g.ss_parts = p_o.ss_parts();
+    g.n = ff; g.tm_a = p_gu.few ? &F.w_gateup[few_map(p_gu.small.group)] : &W.w_gate; g.tm_a2 = &W.w_up; g.up_first = L.w_up < L.w_gate; g.tm_b = &tm_xg; g.ss_parts = p_o.ss_parts();
     ahead(next ? next->w_qkv : nullptr, nullptr, 3 * d, d);
     if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = p_gu.launch(PROJ_GATEUP, g, s));
     g.n = d; g.tm_a = p_down.few ? &F.w_down[few_map(p_down.small.group)] : &W.w_down; g.tm_a2 = nullptr; g.tm_b = &tm_act;
@@ -891,6 +891,7 @@ int vvs_bind_weights(vvs_ctx* ctx, const vvs_weights* w) {
     const vvs_model_desc& md = ctx->desc;
     const int d = md.d_model, ff = md.d_ff;
     int rc = VVS_OK;
+    ctx->few_pairs = true;
     for (int l = 0; l < n && rc == VVS_OK; ++l) {
       const vvs_layer_weights& s = w->layers[l];
       LayerMaps& m = ctx->layer_maps[l];
@@ -901,12 +902,16 @@ int vvs_bind_weights(vvs_ctx* ctx, const vvs_weights* w) {
       if (rc == VVS_OK) rc = make_weight_tmap(&m.w_down, s.w_down, d, ff);
       if (folded_applicable(ctx) && ff % 64 == 0) {
         FewMaps& q = ctx->few_maps[l];
-        if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_gate, s.w_gate, ff, d, 32, 1);
-        if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_up, s.w_up, ff, d, 32, 1);
+        const bool up_first = s.w_up < s.w_gate;
+        const char *w0 = static_cast<const char*>(up_first ? s.w_up : s.w_gate), *w1 = static_cast<const char*>(up_first ? s.w_gate : s.w_up);
+        const uint64_t dist = (uint64_t)(w1 - w0);
+        const bool pair = dist > 0 && dist % 16 == 0 && dist < (uint64_t)1 << 40;         // (what a descriptor takes as a stride)
+        ctx->few_pairs = ctx->few_pairs && pair;
         for (int g : {2, 4, 5, 7}) {
           if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_qkv[few_map(g)], s.w_qkv, 3 * (uint64_t)d, d, 64, g);
           if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_o[few_map(g)], s.w_o, d, d, 64, g);
           if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_down[few_map(g)], s.w_down, d, ff, 64, g);
+          if (rc == VVS_OK && pair) rc = make_tmap_bf16_pair_blocks(&q.w_gateup[few_map(g)], w0, dist, ff, d, 32, g);
         }
       }
     }

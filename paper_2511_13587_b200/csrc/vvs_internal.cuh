@@ -129,7 +129,7 @@ struct LayerMaps {
 };
 // the same matrices in the boxes of proj_few.cu: 64 rows (32 of gate and up) of one to several k-blocks
 struct FewMaps {
-  CUtensorMap w_gate, w_up, w_qkv[4], w_o[4], w_down[4];   // [stages of two, four, five, seven k-blocks]
+  CUtensorMap w_qkv[4], w_o[4], w_gateup[4], w_down[4];   // [stages of two, four, five, seven k-blocks]
 };
 
 }  // namespace vvs
@@ -179,6 +179,7 @@ struct vvs_ctx {
   bool use_chain_kernels = false;  // debug: the persistent whole-chain kernels for calls of at most 32 tokens
   vvs::LayerMaps* layer_maps = nullptr;  // host array [n_layers]
   vvs::FewMaps* few_maps = nullptr;      // host array [n_layers]
+  bool few_pairs = false;                // gate and up of every layer can be loaded by one request
   std::vector<const __nv_bfloat16*> chain_norms;  // host [n_layers][2] norm-scale pointers
   vvs::ChainStreamPlan cs_plan;        // streaming chain kernel: split of the weights over the CTAs
   void* cs_packed = nullptr;           // device: private re-packed copy of the layer weights
@@ -265,6 +266,8 @@ struct GemmTcArgs {
   __nv_bfloat16* act; int ff;  // SWIGLU
 };
 int make_tmap_bf16_blocks(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_blocks);
+int make_tmap_bf16_pair_blocks(CUtensorMap* out, const void* base, uint64_t dist, uint64_t rows, uint64_t cols, uint32_t box_rows,
+                               uint32_t box_blocks);
 int make_tmap_bf16_2d(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 int make_weight_tmap(CUtensorMap* out, const void* w, int rows, int cols);
 GemmTcPlan plan_gemm_tc(int m, int n, int k, bool dual, bool allow_split, int n_sms, int split_cap = 32);
@@ -298,6 +301,7 @@ struct ProjArgs {
   const int32_t* slot_pos; const float* rope_cos; const float* rope_sin;
   int n_heads, hd, s_max, layer, kv_rows, t_len;
   __nv_bfloat16* act; int ff;  // GATEUP
+  bool up_first;               // GATEUP, few tokens: w_up lies before w_gate
   const void* ahead[2]; uint32_t ahead_bytes;   // matrices of the projection after next (same size; null: none)
 };
 int launch_proj(int epi, const ProjPlan& plan, const ProjArgs& g, cudaStream_t s);

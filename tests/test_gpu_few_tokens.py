@@ -59,3 +59,28 @@ def test_few_tokens_tree():
     run = H.GpuRunner(FEW64, case["w"], 4, len(parent))
     _check_tree(case, H.run_tree_gpu(run, case), H.run_tree_oracle(case))
     run.close()
+
+
+@pytest.mark.parametrize("ms", [FEW64, STREAM1])
+def test_gate_and_up_wherever_they_lie(ms):
+    """They are loaded as one tensor of two matrices: up before gate gives the same bits, one matrix as both takes the other kernel."""
+    import torch
+    case = H.build_case_independent(ms, 1970, 1, 2, 1, 8, [150], logit_std=0.6)
+    run = H.GpuRunner(ms, case["w"], 2, 9)
+    want = run.verify(case)
+    for layer in run.wd["layers"]:
+        both = torch.stack([layer["w_up"], layer["w_gate"]])
+        layer["w_up"], layer["w_gate"] = both[0], both[1]
+    run.vb.vvs_bind_weights(run.ctx, run.wd)
+    got = run.verify(case)
+    for key in ("accept_len", "next_token", "target_probs", "hidden", "kv_k", "kv_v"):
+        np.testing.assert_array_equal(want[key], got[key], err_msg=key)
+    for layer in run.wd["layers"]:
+        layer["w_up"] = layer["w_gate"].clone()
+    run.vb.vvs_bind_weights(run.ctx, run.wd)
+    want = run.verify(case)
+    for layer in run.wd["layers"]:
+        layer["w_up"] = layer["w_gate"]
+    run.vb.vvs_bind_weights(run.ctx, run.wd)
+    assert H.rel_err_rows(run.verify(case)["hidden"], want["hidden"]) < 1e-2      # (bf16 features, as against the oracle)
+    run.close()
