@@ -44,7 +44,8 @@ struct Smem {
   static constexpr int kMerge = W * NMT * 16 * (kLd + 2) * 4;
   static constexpr int kRing = D * W * kSlice, kMergeAt = MANY ? (D - 1) * W * kSlice : 0;
   static constexpr int kMain = kRing > kMergeAt + kMerge ? kRing : kMergeAt + kMerge;
-  static int bytes(int t_len, int s) { return kMain + (s - 1) * t_len * (HD + 2) * 4; }
+  static constexpr int kQ = 32 * HD * 2;                      // the item's q: 64-column tiles, 128-byte swizzled
+  static int bytes(int t_len, int s) { return kMain + kQ + (s - 1) * t_len * (HD + 2) * 4; }
 };
 
 // The 16 NS keys of a slice against the 16 query rows of an m-tile.  MASKED: bit k of vis[i] = key k is visible to row g + 8 i, of
@@ -199,20 +200,36 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
         anc[mi][i] = t < T ? a.anc_mask[it.r * T + t] : 0u;
       }
   };
+  // q goes through shared memory, each piece read from L2 by one thread: as fragments, by every warp for itself, it took 1.2 us
+  // of a CTA of 16 warps (one image 699 -> 687 us a step, a tree of 27 rows 863 -> 855, 5 images of 27 rows 1600 -> 1572, d_model 2048, 4
+  // images 1127 -> 1112).  (Rows past the block hold whatever lies there; their results are not stored.)
+  constexpr int kQP = (32 * kPer + 32 * W - 1) / (32 * W);      // pieces of a thread
+  const uint32_t q_smem = tc::smem_u32(smem) + L::kMain;
+  uint4 qv[kQP];
   auto load_q = [&](const Item& it) {
 #pragma unroll
-    for (int mi = 0; mi < NMT; ++mi) {
-      const int t0 = (grp + mi) * 16 + g, t1 = t0 + 8;
-      const bf16* q0 = a.q + (size_t)(it.r * T + t0) * a.d + it.h * HD + 2 * c;
-      const bf16* q1 = q0 + (size_t)8 * a.d;
+    for (int u = 0; u < kQP; ++u) {
+      const int t = (tid + u * 32 * W) / kPer;                  // (the chunk is the same every time)
+      if (t < T) qv[u] = __ldcg(reinterpret_cast<const uint4*>(a.q + (size_t)(it.r * T + t) * a.d + it.h * HD + ch * 8));
+    }
+  };
+  auto store_q = [&]() {
+#pragma unroll
+    for (int u = 0; u < kQP; ++u) {
+      const int t = (tid + u * 32 * W) / kPer;
+      if (t < T)
+        *reinterpret_cast<uint4*>(smem + L::kMain + (ch >> 3) * 4096 + t * 128 + (((ch & 7) ^ (t & 7)) << 4)) = qv[u];
+    }
+  };
+  auto take_q = [&]() {
+#pragma unroll
+    for (int mi = 0; mi < NMT; ++mi)
 #pragma unroll
       for (int kk = 0; kk < HD / 16; ++kk) {
-        qa[mi][kk][0] = t0 < T ? __ldcg(reinterpret_cast<const unsigned*>(q0 + 16 * kk)) : 0u;
-        qa[mi][kk][1] = t1 < T ? __ldcg(reinterpret_cast<const unsigned*>(q1 + 16 * kk)) : 0u;
-        qa[mi][kk][2] = t0 < T ? __ldcg(reinterpret_cast<const unsigned*>(q0 + 16 * kk + 8)) : 0u;
-        qa[mi][kk][3] = t1 < T ? __ldcg(reinterpret_cast<const unsigned*>(q1 + 16 * kk + 8)) : 0u;
+        const int row = (grp + mi) * 16 + (lane & 15), cc = 2 * kk + (lane >> 4);
+        ldsm4(q_smem + (cc >> 3) * 4096 + row * 128 + (((cc & 7) ^ (row & 7)) << 4), qa[mi][kk][0], qa[mi][kk][1], qa[mi][kk][2],
+              qa[mi][kk][3]);
       }
-    }
   };
   const float sl2 = rsqrtf((float)HD) * 1.4426950408889634f;
 
@@ -227,13 +244,15 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
   tc::pdl_launch_dependents();                  // the projection after this kernel may start fetching its weights
   load_anc(it);
   tc::pdl_wait();
+  load_q(it);
 #pragma unroll
   for (int i = 0; i < D; ++i) {
     const int s = first + i * stride;
     if (s >= it.n_old && s < it.n_slices) request(it, i);
   }
   tc::cp_async_commit();
-  load_q(it);
+  store_q();
+  __syncthreads();
 
 #pragma unroll 1
   for (int k = 0;; ++k) {
@@ -241,6 +260,7 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
     const bool more = MANY && next_item < n_items;
     Item nx;
     if (more) locate(next_item, nx);
+    take_q();
     AttState<HD> st[NMT];
 #pragma unroll
     for (int mi = 0; mi < NMT; ++mi) {
@@ -321,7 +341,7 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
     }
     __syncthreads();
     if (S > 1) tc::cluster_wait();   // rank 0's barrier is ready
-    float* xbuf = reinterpret_cast<float*>(smem + L::kMain);    // [S - 1][T][HD + 2]
+    float* xbuf = reinterpret_cast<float*>(smem + L::kMain + L::kQ);    // [S - 1][T][HD + 2]
     const uint32_t x_bar0 = S > 1 ? tc::mapa(tc::smem_u32(&x_bar), 0) : 0u;
     const uint32_t xbuf0 = S > 1 ? tc::mapa(tc::smem_u32(xbuf), 0) : 0u;
     bool waited = S == 1;
@@ -391,7 +411,8 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
       }
     }
     if (!more) break;
-    __syncthreads();                                            // the merge is done with the last slots
+    store_q();
+    __syncthreads();                                            // q; the merge is done with the last slots
     if (first + (D - 1) * stride < it.n_slices) request(it, D - 1);
     tc::cp_async_commit();
     tc::cp_async_commit();                                      // (as many groups as the first item has)
