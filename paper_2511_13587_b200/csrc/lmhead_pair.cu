@@ -8,8 +8,13 @@
 // accumulators are double-buffered (2 x 256 TMEM columns), so the epilogue of a tile runs under the next tile's MMAs.
 // Pairs stay resident and walk (tile, pass) units, passes first: the pairs that share codebook rows read them at
 // the same time and all but one find them in L2.
-// Roles: warp 0 loads (both CTAs; bytes are counted on rank 0's barriers), warp 1 of rank 0 issues the MMAs, warps 4-7
-// turn their 32 lanes' accumulators into logits and partials.
+// Roles: warp 0 loads (both CTAs; bytes are counted on rank 0's barriers), warp 1 of rank 0 issues the MMAs, warps 4-19
+// turn their 32 lanes' accumulators into logits and partials.  Four epilogue warps, one per scheduler, took 7 to 11 us a unit, more than
+// the MMAs of a unit of d = 1280 and all of it in the open behind the last one.  Sixteen, and loads and MMAs issued by converged
+// warps (a lone lane: 3 to 4 % more everywhere), epilogue and decisions, us: d 1280, 16384 codes, 16 images of 9 rows 35.1 -> 24.5; 20000
+// codes, 40 images of 6 rows without guidance 67.9 -> 41.1; 4096 codes, 64 images 42.5 -> 29.5; d 2048, 8192 codes, 20 images of 11 rows
+// 32.2 -> 26; 30000 codes, 12 images of 13 rows without guidance 58.3 -> 44; d 4096, 16384 codes, 32 images, 64 neighbours 87.6 -> 80.2; 65536
+// codes, 64 images of 17 rows 921 -> 833 (the groups' tiles leave room for a third stage of 256 columns).
 #include <math_constants.h>
 
 #include "tc_common.cuh"
@@ -21,10 +26,11 @@ using namespace tc;
 
 namespace {
 
-constexpr int kThreads = 256;
 constexpr int kMaxStages = 6;
-constexpr int kChunk = 64;            // decision rows per epilogue step
-constexpr int kLd = 129;              // padded row of the logit tile
+constexpr int kGroups = 4;            // of four epilogue warps, one per lane quarter of the tensor memory
+constexpr int kThreads = 128 + kGroups * 128;
+constexpr int kChunk = 16;            // decision rows per epilogue step of a group
+constexpr int kTileBytes = kGroups * kChunk * 128 * 4;     // the groups' logit tiles
 constexpr uint32_t kBlockK = 64;
 constexpr uint32_t kABytes = 128 * kBlockK * 2;
 // k-blocks per pipeline stage: the issuing thread pays a wait and a commit (~270 cycles) per stage against 64 cycles
@@ -46,21 +52,29 @@ __device__ __forceinline__ void tma_load_pair(void* dst, const CUtensorMap* m, u
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
       ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y) : "memory");
 }
+// mma_bf16_k64 and mma_commit_elect for a pair: called by a converged warp, of which one lane issues; the commit arrives on the same
+// barrier of both CTAs once the MMAs issued so far have completed
 __device__ __forceinline__ void mma_pair_k64(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
-#pragma unroll
-  for (uint32_t k = 0; k < 4; ++k) {
-    const uint64_t ad = ((uint64_t)kDescHiSw128 << 32) | (a_lo + 2 * k), bd = ((uint64_t)kDescHiSw128 << 32) | (b_lo + 2 * k);
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate | k) : "memory");
-  }
+  asm volatile(
+      "{\n\t.reg .pred e, p, q;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, %5, %5;\n\t"
+      "mov.b64 a, {%1, %5};\n\tmov.b64 b, {%2, %5};\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, p;\n\t"
+      "add.u32 x, %1, 2;\n\tadd.u32 y, %2, 2;\n\tmov.b64 a, {x, %5};\n\tmov.b64 b, {y, %5};\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, q;\n\t"
+      "add.u32 x, %1, 4;\n\tadd.u32 y, %2, 4;\n\tmov.b64 a, {x, %5};\n\tmov.b64 b, {y, %5};\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, q;\n\t"
+      "add.u32 x, %1, 6;\n\tadd.u32 y, %2, 6;\n\tmov.b64 a, {x, %5};\n\tmov.b64 b, {y, %5};\n\t"
+      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, q;\n\t}"
+      ::"r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHiSw128)
+      : "memory");
 }
-// arrive on the same barrier of both CTAs once the MMAs issued so far have completed
 __device__ __forceinline__ void commit_pair(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+  asm volatile(
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
+      ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
 }
 __device__ __forceinline__ void arrive_remote(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -83,10 +97,10 @@ lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, con
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_abort;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int rank = (int)(blockIdx.x & 1), pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
   const uint32_t b_bytes = p.b_rows * kBlockK * 2u, stage_bytes = kSub * (kABytes + b_bytes);
-  float* sL = reinterpret_cast<float*>(smem + (size_t)p.stages * stage_bytes);      // [kChunk][kLd]
+  float* sL = reinterpret_cast<float*>(smem + (size_t)p.stages * stage_bytes);      // [kGroups][kChunk][128]
 
   if (tid == 0) {
     for (int i = 0; i < p.stages; ++i) {
@@ -95,7 +109,7 @@ lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, con
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&acc_full[i], 1);
-      mbar_init(&acc_empty[i], 8);                // four epilogue warps of each CTA
+      mbar_init(&acc_empty[i], 8 * kGroups);      // the epilogue warps of both CTAs
     }
     s_abort = 0;
     fence_barrier_init();
@@ -114,92 +128,85 @@ lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, con
   pdl_launch_dependents();
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---- TMA producer (codebook rows of the first stages may be requested before the features exist) -------------
-      uint32_t stage = 0, par = 1, bar0[kMaxStages];
-      for (int i = 0; i < kMaxStages; ++i) bar0[i] = mapa(smem_u32(&full_bar[i]), 0);
-      int issued = 0;
-      bool ok = true, waited = false;
-      auto load_a = [&](uint8_t* st, int i, int kb, int y) {
+    // ---- TMA producer, a converged warp of which one lane issues (codebook rows of the first stages may be requested before the
+    // features exist) ---------------------------------------------------------------------------------------------------
+    uint32_t stage = 0, par = 1;
+    int issued = 0;
+    bool ok = true;
+    auto load_a = [&](uint32_t i, int kb, int y) {
+      if (elect_one()) {
+        const uint32_t bar0 = mapa(smem_u32(&full_bar[i]), 0);
+        uint8_t* st = smem + (size_t)i * stage_bytes;
+        if (rank == 0) mbar_expect_tx(&full_bar[i], 2 * stage_bytes);
 #pragma unroll
-        for (uint32_t h = 0; h < kSub; ++h) tma_load_pair(st + h * kABytes, &tm_a, bar0[i], (kb * (int)kSub + (int)h) * (int)kBlockK, y);
-      };
-      auto load_b = [&](uint8_t* st, int i, int kb, int y) {
+        for (uint32_t h = 0; h < kSub; ++h) tma_load_pair(st + h * kABytes, &tm_a, bar0, (kb * (int)kSub + (int)h) * (int)kBlockK, y);
+      }
+    };
+    auto load_b = [&](uint32_t i, int kb, int y) {
+      if (elect_one()) {
+        const uint32_t bar0 = mapa(smem_u32(&full_bar[i]), 0);
+        uint8_t* st = smem + (size_t)i * stage_bytes + kSub * kABytes;
 #pragma unroll
-        for (uint32_t h = 0; h < kSub; ++h)
-          tma_load_pair(st + kSub * kABytes + h * b_bytes, &tm_b, bar0[i], (kb * (int)kSub + (int)h) * (int)kBlockK, y);
-      };
-      for (int u = pair; u < p.units && ok; u += n_pairs) {
-        const int tile = u / p.passes, row0 = (u - tile * p.passes) * p.nd;
-        const int ya = tile * 256 + rank * 128;
-        const int yb = p.n_cfg == 2 ? rank * p.bt + row0 : row0 + rank * (int)p.b_rows;
-        if (!waited) {
-          const int n_pre = p.kb_total < p.stages ? p.kb_total : p.stages;
-          for (int i = 0; i < n_pre; ++i) {
-            if (rank == 0) mbar_expect_tx(&full_bar[i], 2 * stage_bytes);
-            load_a(smem + (size_t)i * stage_bytes, i, i, ya);
-          }
-          pdl_wait();
-          waited = true;
-          for (int kb = 0; kb < p.kb_total; ++kb) {
-            uint8_t* st = smem + (size_t)stage * stage_bytes;
-            if (kb >= n_pre) {
-              if (!(ok = wait_or_abort(&empty_bar[stage], par, &s_abort, p.status))) break;
-              if (rank == 0) mbar_expect_tx(&full_bar[stage], 2 * stage_bytes);
-              load_a(st, stage, kb, ya);
-            }
-            load_b(st, stage, kb, yb);
-            ++issued;
-            if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1u; }
-          }
-          continue;
-        }
-        for (int kb = 0; kb < p.kb_total; ++kb) {
-          if (!(ok = wait_or_abort(&empty_bar[stage], par, &s_abort, p.status))) break;
-          uint8_t* st = smem + (size_t)stage * stage_bytes;
-          if (rank == 0) mbar_expect_tx(&full_bar[stage], 2 * stage_bytes);
-          load_a(st, stage, kb, ya);
-          load_b(st, stage, kb, yb);
-          ++issued;
-          if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1u; }
-        }
+        for (uint32_t h = 0; h < kSub; ++h) tma_load_pair(st + h * b_bytes, &tm_b, bar0, (kb * (int)kSub + (int)h) * (int)kBlockK, y);
       }
-      if (!ok && rank == 0) {                     // gave up: nothing may be in flight when the pair leaves (bounded)
-        for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
-          for (uint32_t k = 0; k < kSpinLimit && !mbar_try_wait_cluster(&full_bar[i % p.stages], (i / p.stages) & 1); ++k) {}
+    };
+    const int n_pre = p.kb_total < p.stages ? p.kb_total : p.stages;
+    for (int u = pair; u < p.units && ok; u += n_pairs) {
+      const int tile = u / p.passes, row0 = (u - tile * p.passes) * p.nd;
+      const int ya = tile * 256 + rank * 128;
+      const int yb = p.n_cfg == 2 ? rank * p.bt + row0 : row0 + rank * (int)p.b_rows;
+      const int done = u == pair ? n_pre : 0;       // codebook blocks requested already
+      if (done) {
+        for (int i = 0; i < n_pre; ++i) load_a(i, i, ya);
+        pdl_wait();
       }
+      for (int kb = 0; kb < p.kb_total; ++kb) {
+        if (kb >= done) {
+          if (!(ok = __all_sync(0xffffffffu, wait_or_abort(&empty_bar[stage], par, &s_abort, p.status)))) break;
+          load_a(stage, kb, ya);
+        }
+        load_b(stage, kb, yb);
+        ++issued;
+        if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1u; }
+      }
+    }
+    if (!ok && rank == 0) {                       // gave up: nothing may be in flight when the pair leaves (bounded)
+      for (int i = issued > p.stages ? issued - p.stages : 0; i < issued; ++i)
+        for (uint32_t k = 0; k < kSpinLimit && !mbar_try_wait_cluster(&full_bar[i % p.stages], (i / p.stages) & 1); ++k) {}
     }
   } else if (warp == 1 && rank == 0) {
-    if (lane == 0) {
-      // ---- MMA issuer ------------------------------------------------------------------------------------------------
-      const uint32_t n_cols = p.n_cfg == 2 ? 2u * (uint32_t)p.nd : (uint32_t)p.nd;
-      const uint32_t idesc = idesc_bf16_f32(256, n_cols);
-      const uint32_t lo0 = desc_lo_sw128(smem_u32(smem)), stage_lo = stage_bytes >> 4;
-      uint32_t stage = 0, par = 0;
-      int it = 0;
-      bool ok = true;
-      for (int u = pair; u < p.units && ok; u += n_pairs, ++it) {
-        const uint32_t buf = it & 1, d = tmem + buf * 256u;
-        if (!(ok = wait_or_abort(&acc_empty[buf], ((it >> 1) & 1) ^ 1, &s_abort, p.status))) break;
+    // ---- MMA issuer --------------------------------------------------------------------------------------------------
+    const uint32_t n_cols = p.n_cfg == 2 ? 2u * (uint32_t)p.nd : (uint32_t)p.nd;
+    const uint32_t idesc = idesc_bf16_f32(256, n_cols);
+    const uint32_t lo0 = desc_lo_sw128(smem_u32(smem)), stage_lo = stage_bytes >> 4;
+    uint32_t stage = 0, par = 0;
+    int it = 0;
+    bool ok = true;
+    for (int u = pair; u < p.units && ok; u += n_pairs, ++it) {
+      const uint32_t buf = it & 1, d = tmem + buf * 256u;
+      if (!(ok = __all_sync(0xffffffffu, wait_or_abort(&acc_empty[buf], ((it >> 1) & 1) ^ 1, &s_abort, p.status)))) break;
+      tc_fence_after();
+      for (int kb = 0; kb < p.kb_total; ++kb) {
+        if (!(ok = __all_sync(0xffffffffu, wait_or_abort(&full_bar[stage], par, &s_abort, p.status)))) break;
         tc_fence_after();
-        for (int kb = 0; kb < p.kb_total; ++kb) {
-          if (!(ok = wait_or_abort(&full_bar[stage], par, &s_abort, p.status))) break;
-          tc_fence_after();
-          const uint32_t a_lo = lo0 + stage * stage_lo;
+        const uint32_t a_lo = lo0 + stage * stage_lo;
 #pragma unroll
-          for (uint32_t h = 0; h < kSub; ++h)
-            mma_pair_k64(d, a_lo + h * (kABytes >> 4), a_lo + ((kSub * kABytes + h * b_bytes) >> 4), idesc, kb > 0 || h > 0);
-          commit_pair(&empty_bar[stage]);
-          if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1u; }
-        }
-        commit_pair(&acc_full[buf]);
+        for (uint32_t h = 0; h < kSub; ++h)
+          mma_pair_k64(d, a_lo + h * (kABytes >> 4), a_lo + ((kSub * kABytes + h * b_bytes) >> 4), idesc, kb > 0 || h > 0);
+        commit_pair(&empty_bar[stage]);
+        if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1u; }
       }
+      commit_pair(&acc_full[buf]);
     }
   } else if (warp >= 4) {
-    // ---- epilogue: thread = one code; logits out, then partials from a shared tile, two threads per decision row ------
-    const int e = tid - 128, q = warp - 4;
+    // ---- epilogue: a group takes every fourth chunk of 16 decision rows; thread = one code, logits out and to the group's tile
+    // (codes of row r at code ^ 8 (r & 3): no two threads on a bank in either direction), then eight threads per row for the partials
+    const int grp = (warp - 4) >> 2, q = warp & 3, e = q * 32 + lane;
     const uint32_t t_lane = (uint32_t)(q * 32) << 16;
     const uint32_t empty0 = mapa(smem_u32(&acc_empty[0]), 0), empty1 = mapa(smem_u32(&acc_empty[1]), 0);
+    float* tile_s = sL + grp * (kChunk * 128);
+    const int prow = e >> 3, part = e & 7;
+    const unsigned mates = 0xffu << (lane & 24);
     int it = 0;
     pdl_wait();
     for (int u = pair; u < p.units; u += n_pairs, ++it) {
@@ -210,56 +217,56 @@ lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, con
       if (!wait_or_abort(&acc_full[buf], (it >> 1) & 1, &s_abort, p.status)) break;
       tc_fence_after();
       const uint32_t t_row = tmem + (uint32_t)buf * 256u + t_lane;
-      float* dst = p.logits + (size_t)row0 * p.v + n;
-      for (int c0 = 0; c0 < nd; c0 += kChunk) {
+      auto release = [&]() {                      // the accumulator has been read: the next unit but one may have it
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive_remote(buf ? empty1 : empty0);
+      };
+      if (grp * kChunk >= nd) release();
+      for (int c0 = grp * kChunk; c0 < nd; c0 += kGroups * kChunk) {
         const int rows = min(kChunk, nd - c0);
-        for (int c = 0; c < rows; c += 16) {
-          float lc[16], lu[16];
-          tmem_ld16(t_row + c0 + c, lc);
-          if (p.n_cfg == 2) tmem_ld16(t_row + (uint32_t)p.nd + c0 + c, lu);
+        float l[16];
+        tmem_ld16(t_row + c0, l);
+        if (p.n_cfg == 2) {
+          float lu[16];
+          tmem_ld16(t_row + (uint32_t)p.nd + c0, lu);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            if (c + j < rows) {
-              float l = lc[j];
-              if (p.n_cfg == 2) l = lu[j] + p.cfg_scale * (l - lu[j]);
-              l *= p.inv_temp;
-              sL[(c + j) * kLd + e] = n_ok ? l : -CUDART_INF_F;
-              if (n_ok) dst[(size_t)(c0 + c + j) * p.v] = l;
-            }
-          }
+          for (int j = 0; j < 16; ++j) l[j] = lu[j] + p.cfg_scale * (l[j] - lu[j]);
         }
-        if (c0 + kChunk >= nd) {                  // the accumulator has been read: the next unit but one may have it
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) arrive_remote(buf ? empty1 : empty0);
+        if (c0 + kGroups * kChunk >= nd) release();
+        float* dst = p.logits + (size_t)(row0 + c0) * p.v + n;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          l[j] *= p.inv_temp;
+          tile_s[j * 128 + (e ^ (8 * (j & 3)))] = n_ok ? l[j] : -CUDART_INF_F;
+          if (n_ok && j < rows) *dst = l[j];
+          dst += p.v;
         }
-        named_bar_sync(1, 128);
-        if (t128 < p.n_tiles && (e >> 1) < rows) {
-          const float* row = sL + (e >> 1) * kLd + (e & 1) * 64;
-          float m0 = -CUDART_INF_F, m1 = m0, m2 = m0, m3 = m0;
-#pragma unroll 4
-          for (int i = 0; i < 64; i += 4) {
-            m0 = fmaxf(m0, row[i]); m1 = fmaxf(m1, row[i + 1]); m2 = fmaxf(m2, row[i + 2]); m3 = fmaxf(m3, row[i + 3]);
-          }
-          float mx = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
-          const unsigned mate = 3u << (lane & ~1);
-          mx = fmaxf(mx, __shfl_xor_sync(mate, mx, 1));
-          float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+        named_bar_sync(1 + grp, 128);
+        if (t128 < p.n_tiles && prow < rows) {
+          const float* row = tile_s + prow * 128;
+          float x[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) x[i] = row[(part + 8 * i) ^ (8 * (prow & 3))];
+          float mx = x[0];
+#pragma unroll
+          for (int i = 1; i < 16; ++i) mx = fmaxf(mx, x[i]);
+#pragma unroll
+          for (int o = 1; o < 8; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(mates, mx, o));
+          float sum = 0.f;
           if (mx > -CUDART_INF_F) {
-#pragma unroll 4
-            for (int i = 0; i < 64; i += 4) {
-              s0 += expf(row[i] - mx); s1 += expf(row[i + 1] - mx); s2 += expf(row[i + 2] - mx); s3 += expf(row[i + 3] - mx);
-            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) sum += expf(x[i] - mx);
           }
-          float sum = (s0 + s1) + (s2 + s3);
-          sum += __shfl_xor_sync(mate, sum, 1);
-          if ((e & 1) == 0) {
-            const size_t at = (size_t)(row0 + c0 + (e >> 1)) * p.n_tiles + t128;
+#pragma unroll
+          for (int o = 1; o < 8; o <<= 1) sum += __shfl_xor_sync(mates, sum, o);
+          if (part == 0) {
+            const size_t at = (size_t)(row0 + c0 + prow) * p.n_tiles + t128;
             p.part_m[at] = mx;
             p.part_s[at] = sum;
           }
         }
-        named_bar_sync(1, 128);                   // the tile is written again
+        named_bar_sync(1 + grp, 128);             // the tile is written again
       }
     }
   }
@@ -301,8 +308,8 @@ int launch_lmhead_pair(const LmHeadArgs& a, cudaStream_t s) {
   p.b_rows = (uint32_t)lmhead_pair_box_rows(a.bt, a.n_cfg);
   p.cfg_scale = a.cfg_scale; p.inv_temp = a.inv_temp; p.part_m = a.part_m; p.part_s = a.part_s; p.logits = a.logits_out;
   p.status = a.status;
-  const int stage_bytes = (int)(kSub * (kABytes + p.b_rows * kBlockK * 2)), tile_bytes = kChunk * kLd * 4;
-  p.stages = (224 * 1024 - tile_bytes) / stage_bytes;
+  const int stage_bytes = (int)(kSub * (kABytes + p.b_rows * kBlockK * 2));
+  p.stages = (224 * 1024 - kTileBytes) / stage_bytes;
   if (p.stages > kMaxStages) p.stages = kMaxStages;
   if (ensure_dynamic_smem(reinterpret_cast<const void*>(lmhead_pair_kernel), 225 * 1024) != cudaSuccess) return VVS_ERR_CUDA;
   // (all of the SM's shared memory: the two CTAs of a pair wait for each other, so neither may find its tensor memory

@@ -21,3 +21,9 @@ def test_lmhead_edges(d, v, n_images, n_cfg, k):
     assert gpu["status"] == 0
     np.testing.assert_allclose(gpu["target_probs"], ora["target_probs"], rtol=6e-2, atol=2e-4)
     H.check_replay(case, gpu)
+
+
+@pytest.mark.parametrize("d,v,n_images,n_cfg,k", [(64, 300, 69, 2, 12), (200, 129, 10, 2, 12), (72, 4100, 20, 1, 12)])
+def test_lmhead_pair_chunks(d, v, n_images, n_cfg, k):
+    """Passes whose last is one decision row (897 in eight of 128: most epilogue groups have none), 50 (130 in two of 80), 100 of 160."""
+    test_lmhead_edges(d, v, n_images, n_cfg, k)
