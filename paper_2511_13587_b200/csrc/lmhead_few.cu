@@ -4,7 +4,9 @@
 //
 // What bounds it: the stream of codebook rows, if nothing else gets in its way.  Two warps issue, every other k-block each with
 // an accumulator of its own (one issuing lane in a branch of its own reached a k-block every ~600 cycles, which is slower than
-// the stream fills a stage; issued by converged warps 14.4 -> 14.0 us a call of one image and 16384 codes); the pipeline is as deep as shared memory allows and its weights are
+// the stream fills a stage; issued by converged warps 14.4 -> 14.0 us a call of one image and 16384 codes); nor is the loading lane alone:
+// with its ring's 600 cycles a k-block d 4096, 4096 or 8192 codes took 27 to 28 us a call of one image, decision included, 20 as a converged warp
+// (d 2048, 9472 codes 19.9 -> 17.8; d 1280, 8192 codes 16.1 -> 14.8); the pipeline is as deep as shared memory allows and its weights are
 // requested before griddepcontrol.wait.  Up to one tile per SM a CTA takes the whole SM's shared memory; with more, two
 // CTAs share an SM so that one's epilogue runs under the other's stream.  With one issuer and a thread per decision row
 // summing 128 values from shared memory (2.1 us) a call of one image and 16384 codes took 21.8 us, decision included; 15.3
@@ -48,7 +50,7 @@ lmhead_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, cons
   __shared__ float s_m[4][kMaxCols], s_s[4][kMaxCols];    // partials of the tile's four groups of 32 codes
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int tile = blockIdx.x, C = p.n_cfg, nt = p.nd_pad * C;
   const uint32_t half_bytes = (uint32_t)p.nd_pad * kBlockK * 2u, stage_bytes = kATileBytes + half_bytes * (uint32_t)C;
 
@@ -74,32 +76,36 @@ lmhead_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, cons
   pdl_launch_dependents();
 
   const int n_pre = p.kb_total < p.stages ? p.kb_total : p.stages;
-  auto load_b = [&](int i, uint32_t stage, int half) {
-    tma_load_2d(smem + (size_t)stage * stage_bytes + kATileBytes + (half ? half_bytes : 0u), &tm_b, &full_bar[stage], i * (int)kBlockK,
-                half ? p.bt : 0);
-  };
-  if (warp == 0 && lane == 0) {
-    // ---- TMA producer: the weights of the free stages go out before the wait ------------------------------
-    for (int i = 0; i < n_pre; ++i) {
-      mbar_expect_tx(&full_bar[i], stage_bytes);
-      tma_load_2d(smem + (size_t)i * stage_bytes, &tm_a, &full_bar[i], i * (int)kBlockK, tile * (int)kTileRows);
+  // loads by one lane of a converged warp (mma_bf16_k64)
+  auto load_a = [&](int i, uint32_t stage) {
+    if (elect_one()) {
+      mbar_expect_tx(&full_bar[stage], stage_bytes);
+      tma_load_2d(smem + (size_t)stage * stage_bytes, &tm_a, &full_bar[stage], i * (int)kBlockK, tile * (int)kTileRows);
     }
+  };
+  auto load_b = [&](int i, uint32_t stage, int half) {
+    if (elect_one())
+      tma_load_2d(smem + (size_t)stage * stage_bytes + kATileBytes + (half ? half_bytes : 0u), &tm_b, &full_bar[stage], i * (int)kBlockK,
+                  half ? p.bt : 0);
+  };
+  if (warp == 0) {
+    // ---- TMA producer: the weights of the free stages go out before the wait ------------------------------
+    for (int i = 0; i < n_pre; ++i) load_a(i, i);
     pdl_wait();
     for (int i = 0; i < n_pre; ++i) load_b(i, i, 0);
     uint32_t stage = 0, par = 0;
     for (int i = n_pre; i < p.kb_total; ++i) {
-      if (!wait_or_abort(&empty_bar[stage], par, &s_abort)) {
-        atomicOr(p.status, VVS_DEV_TIMEOUT);
+      if (!__all_sync(0xffffffffu, wait_or_abort(&empty_bar[stage], par, &s_abort))) {
+        if (lane == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
         s_abort = 1;
         break;
       }
-      mbar_expect_tx(&full_bar[stage], stage_bytes);
-      tma_load_2d(smem + (size_t)stage * stage_bytes, &tm_a, &full_bar[stage], i * (int)kBlockK, tile * (int)kTileRows);
+      load_a(i, stage);
       load_b(i, stage, 0);
       if (C == 2) load_b(i, stage, 1);
       if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1; }
     }
-  } else if (warp == 3 && lane == 0) {
+  } else if (warp == 3) {
     // the unconditional feature rows of the first stages, beside the producer's conditional ones
     if (C == 2) {
       pdl_wait();
