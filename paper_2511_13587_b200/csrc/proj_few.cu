@@ -434,7 +434,7 @@ int launch_proj_few(int epi, const ProjFewPlan& pl, const ProjArgs& g, cudaStrea
   cudaError_t e;
   switch (epi) {
     case PROJ_QKV: e = pl.splits == 2 ? launch_epi<PROJ_QKV, 1>(pl, kp, g, s) : launch_epi<PROJ_QKV, 0>(pl, kp, g, s); break;
-    case PROJ_ADD: e = pl.splits == 4 ? launch_epi<PROJ_ADD, 2>(pl, kp, g, s) : pl.splits == 2 ? launch_epi<PROJ_ADD, 1>(pl, kp, g, s) : launch_epi<PROJ_ADD, 0>(pl, kp, g, s); break;
+    case PROJ_ADD: e = pl.splits == 4 ? launch_epi<PROJ_ADD, 2>(pl, kp, g, s) : launch_epi<PROJ_ADD, 0>(pl, kp, g, s); break;
     case PROJ_GATEUP: e = launch_epi<PROJ_GATEUP, 0>(pl, kp, g, s); break;
     default: return VVS_ERR_INVALID_ARG;
   }
