@@ -235,7 +235,7 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
   }
   __syncwarp();
   if (warp >= 2) pdl_wait();
-  else if (eid < items) prepare(eid);
+  else prepare(eid);                        // (lanes past the last item too: the epilogue goes by whole warps and asks for their `dst`)
   float2 xo[TPI];
   auto load_x = [&](int idx) {
     const int t0 = (idx >> (log_np + log_sub)) * 4 + sub;

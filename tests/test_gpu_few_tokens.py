@@ -29,6 +29,10 @@ STREAM3 = replace(B7, name="stream3", n_layers=1, d_model=2048, n_heads=16, d_ff
     (FEW64, 1, 2, 1, 3, [199]),                            # 8
     (FEW64, 1, 1, 2, 7, [16]),                             # 9
     (FEW64, 3, 1, 1, 10, [0, 47, 150]),                    # 33
+    (FEW64, 1, 2, 1, 24, [150]),                           # 50 and 58: thirteen and fifteen quads of sixteen items, the last half warp
+    (FEW64, 1, 2, 1, 28, [77]),                            # of them in warps 1 and 0
+    (STREAM3, 1, 2, 1, 24, [513]),
+    (STREAM1, 1, 2, 1, 28, [77]),
     (FEW64, 2, 2, 6, 10, [3, 190]),                        # 64
     (FEW64, 5, 1, 3, 10, [3, 20, 37, 90, 190]),            # 65
     (FEW64, 3, 2, 1, 15, [0, 47, 150]),                    # 96
