@@ -49,13 +49,16 @@ struct Smem {
 };
 
 // The 16 NS keys of a slice against the 16 query rows of an m-tile.  MASKED: bit k of vis[i] = key k is visible to row g + 8 i, of
-// vmem = row k of the V tile holds data (others are zeroed before they are multiplied).  The running maximum is kept unscaled, so that
-// scaling and subtraction are one FMA.
+// vmem = row k of the V tile holds data (others are zeroed before they are multiplied).  Heads of 64 keep the running maximum
+// unscaled, so that scaling and subtraction are one FMA.  Heads of 128 scale, subtract and sum with a rounding each, the arithmetic
+// their results have always had: deep models of such heads (32 layers of d_model 4096) answer any other place of a rounding with
+// features 5.7e-3 away and guided probabilities 1.4e-2 to 4.8e-2, which is more than a caller may see move.
 template <int HD, int NS, bool MASKED>
 __device__ __forceinline__ void att_keys(AttState<HD>& st, const uint32_t (&qa)[HD / 16][4], uint32_t k_base, uint32_t v_base, int lane,
                                          float sl2, const uint32_t (&vis)[2], uint32_t vmem) {
   constexpr uint32_t kChunk = NS * 2048u;                     // 64 columns of all keys
   const int c = lane & 3, mi = lane >> 3, ri = lane & 7;
+  constexpr bool kScaled = HD == 128;                         // the scores and the running maximum are scaled
   float s[2 * NS][4];
 #pragma unroll
   for (int n = 0; n < 2 * NS; ++n)
@@ -77,6 +80,12 @@ __device__ __forceinline__ void att_keys(AttState<HD>& st, const uint32_t (&qa)[
   uint32_t pa[NS][4];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
+    if (kScaled) {
+#pragma unroll
+      for (int n = 0; n < 2 * NS; ++n)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) s[n][2 * i + e] = __fmul_rn(s[n][2 * i + e], sl2);
+    }
     if (MASKED) {
       const uint32_t vb = vis[i] >> (2 * c);
 #pragma unroll
@@ -91,17 +100,18 @@ __device__ __forceinline__ void att_keys(AttState<HD>& st, const uint32_t (&qa)[
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
     const float m_new = fmaxf(st.m[i], mx);
-    const float m_scaled = m_new == -CUDART_INF_F ? 0.f : m_new * sl2;
-    const float alpha = ex2(fmaf(st.m[i], sl2, -m_scaled));
+    const float m_scaled = m_new == -CUDART_INF_F ? 0.f : kScaled ? m_new : m_new * sl2;
+    auto weight = [&](float x) { return ex2(kScaled ? __fsub_rn(x, m_scaled) : fmaf(x, sl2, -m_scaled)); };
+    const float alpha = weight(st.m[i]);
     st.m[i] = m_new;
-    float sum = 0.f;
+    float sum = kScaled ? st.l[i] : 0.f;
 #pragma unroll
     for (int n = 0; n < 2 * NS; ++n) {
-      const float p0 = ex2(fmaf(s[n][2 * i], sl2, -m_scaled)), p1 = ex2(fmaf(s[n][2 * i + 1], sl2, -m_scaled));
-      sum += p0 + p1;
+      const float p0 = weight(s[n][2 * i]), p1 = weight(s[n][2 * i + 1]);
+      sum = kScaled && n == 0 ? fmaf(sum, alpha, p0 + p1) : sum + (p0 + p1);
       pa[n >> 1][i + 2 * (n & 1)] = pack2(p0, p1);
     }
-    st.l[i] = fmaf(st.l[i], alpha, sum);
+    st.l[i] = kScaled ? sum : fmaf(st.l[i], alpha, sum);
 #pragma unroll
     for (int j = 0; j < HD / 8; ++j) {
       st.o[j][2 * i] *= alpha;
@@ -329,7 +339,7 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
             float* dst = s_o + (size_t)(warp * NMT * 16 + row) * L::kLd + 2 * c;
 #pragma unroll
             for (int j = 0; j < NJ; ++j) *reinterpret_cast<float2*>(dst + 8 * j) = make_float2(st[mi].o[j][2 * i], st[mi].o[j][2 * i + 1]);
-            if (c == 0) *reinterpret_cast<float2*>(s_ml + (warp * NMT * 16 + row) * 2) = make_float2(st[mi].m[i] * sl2, l);
+            if (c == 0) *reinterpret_cast<float2*>(s_ml + (warp * NMT * 16 + row) * 2) = make_float2(HD == 128 ? st[mi].m[i] : st[mi].m[i] * sl2, l);
           }
         }
     }
@@ -455,7 +465,8 @@ int launch_variant(const AttentionBlockArgs& a, int split, int per_sm, cudaStrea
 // where they are dealt to two row groups (16: 863), 8 warps with two slots 713); with many, small CTAs: four warps with three slots of 16 keys,
 // three CTAs per SM (16 images 1724, 8 images 1294, 4 images 958; four CTAs per SM with two slots 1716, 1329 and 1021; three with two slots
 // of 32 keys 1766, 1294 and 959), two m-tiles a warp beyond 16 rows (5 images of 27 rows, two slots of 32 keys 1596, three of 16 keys 1624).
-// Heads of 128: 224 items with four warps 1378, with eight 1398.
+// Heads of 128 (see att_keys): up to two items per SM take eight warps, more take four, since the warps' shares of the keys decide in
+// which order the sums are taken (224 items would take 1378 us a step with four, 1398 with eight).
 int launch_attention_block(const AttentionBlockArgs& a, cudaStream_t s) {
   if (a.t_len > kMaxT) return VVS_ERR_SHAPE;
   const long long items = (long long)a.n_heads * a.n_rows;
@@ -465,7 +476,7 @@ int launch_attention_block(const AttentionBlockArgs& a, cudaStream_t s) {
     return a.t_len > 16 ? launch_variant<64, 2, 4, 2, 2, true>(a, split, 2, s) : launch_variant<64, 1, 4, 3, 1, true>(a, split, 3, s);
   }
   if (a.hd == 128)
-    return items <= a.n_sms ? launch_variant<128, 1, 8, 2, 1, true>(a, split, 1, s) : launch_variant<128, 1, 4, 3, 1, true>(a, split, 2, s);
+    return items <= 2LL * a.n_sms ? launch_variant<128, 1, 8, 2, 1, true>(a, split, 1, s) : launch_variant<128, 1, 4, 3, 1, true>(a, split, 2, s);
   return VVS_ERR_SHAPE;
 }
 
