@@ -150,6 +150,8 @@ inline ProjPlan plan_proj(int m, int n, int k, bool dual, int n_sms) {
 // ---- the same for few tokens, proj_few.cu ----------------------------------------------------------
 struct ProjFewPlan {
   int nt, tiles, kb_total, splits, group, stages, ring, recv_off, smem_bytes, tmem_cols;    // stages of `group` k-blocks
+  int parts;                   // slices of plan_proj's per slice, whose sums are kept apart; 0: sums of its own
+  int acc_ld;                  // columns of tensor memory from one accumulator to the next
 };
 
 // partial sums of squares per token an ADD projection writes: one per tile and slice, rounded up to whole float4
@@ -159,14 +161,18 @@ inline int proj_ss_parts(const ProjFewPlan& pl) { return (pl.tiles * pl.splits +
 // measurements; fewer than eight k-blocks are not worth an exchange.
 // in_l2: the model's weights are requested into L2 ahead and a CTA takes as much shared memory as its K range fills.
 // Weights that come from HBM need all CTAs on the device at once, and those of the next projection beside them as they leave: one,
-// two or three CTAs per SM, as many as it takes, rings of stages of two k-blocks.  7B shape, 18 tokens, against proj_tc.cu on 128-row
-// tiles, 2967 us a step: QKV alone here (384 CTAs, three per SM) 2886, with 1 slice and two per SM 2894; output projection (256, two)
-// 2897; gate/up (344, three) 2875, with two per SM, i.e. two waves, 2998; down projection (256, two) 2941; all 2699.  d_model 2048, 24
-// layers, 18 tokens: 960 -> 803, with one CTA per SM and two waves 908, with two per SM everywhere 838; stages of four k-blocks
-// instead of two 858.  More tokens fill shared memory from L2 rather than from HBM: d_model 2048, 64 / 96 tokens 1193 -> 986 / 1166 ->
-// 1147; eight layers of 7B, 64 / 80 / 96 tokens 823 -> 792 / 851 -> 828 / 923 -> 915; of d_model 5120, 18 / 80 / 96 tokens 1019 -> 927 /
-// 1248 -> 1231 / 1502 -> 1524 (hence 80 for matrices beyond 64 MB).  Where even three CTAs per SM are not enough (d_model 8192) proj_tc.cu
-// is the better one, 18 / 48 tokens 1034 / 1080 us against 1033 / 1132 with fewer slices.
+// two or three CTAs per SM, as many as it takes, rings of stages of two k-blocks.  And such models are large and deep: any other order
+// of the sums moves their features by 2.4e-3 (24 layers of d_model 2048) to 5.7e-3 (7B shape) and guided probabilities by more than
+// the 1e-2 that two correct calls may differ by, so the partial sums of plan_proj's slices are kept apart and added in proj_tc.cu's
+// order: the same bits from either kernel.  Hence this kernel takes a projection whose slices each hold whole ones of that plan, an
+// output or down projection only where its four ranks of 16 rows are that plan's eight of 128.  Step with proj_tc.cu alone / with sums of
+// its own, for all projections / so: 7B shape 18 tokens 2851 / 2473 / 2570 us, 64 tokens 3359 / 3154 / 3231; d_model 2048, 24
+// layers, 18 tokens 996 / 792 / 869, 64 tokens 1197 / 928 / 1038, 90 tokens 1396 / 1106 / 1318; four layers of d_model 5120, 18 tokens
+// 541 / 475 / 500, 80 tokens 667 / 621 / 627 (96 tokens lost with sums of its own, hence 80 for matrices beyond 64 MB).  (proj_tc.cu with
+// MMAs from a lone lane; from a converged warp 2 % less.)
+// Which CTAs per SM, with sums of its own: 7B shape, QKV 384 CTAs, three per SM, 2886 us, 1 slice and two per SM 2894; gate/up 344, three
+// 2875, two per SM, i.e. two waves, 2998; d_model 2048, 18 tokens 803, one CTA per SM and two waves 908, two per SM everywhere 838;
+// stages of four k-blocks instead of two 858.  Where even three CTAs per SM are not enough (d_model 8192) proj_tc.cu takes it.
 inline ProjFewPlan plan_proj_few(int m, int n, int k, bool dual, bool add, bool in_l2, int n_sms) {
   using namespace proj;
   ProjFewPlan pl{};
@@ -181,31 +187,39 @@ inline ProjFewPlan plan_proj_few(int m, int n, int k, bool dual, bool add, bool 
     const int ctas = pl.tiles * pl.splits, fit = pl.splits == 4 ? n_sms * 33 / 37 : n_sms;      // (clusters of four: as in plan_proj)
     while (q < 3 && ctas > q * fit) ++q;
     if (ctas > q * fit || (huge && m > 80)) return ProjFewPlan{};
+    const int slices = plan_proj(m, n, k, dual, n_sms).splits;
+    pl.parts = slices / pl.splits;
+    if (pl.parts < 1 || (add && pl.parts * pl.splits != 8)) return ProjFewPlan{};    // (ADD: ranks of 16 rows, a sum of squares each)
   }
+  pl.acc_ld = (pl.nt + 31) & ~31;
+  const int n_acc = pl.parts * (dual ? 1 : 2) > 1 ? pl.parts * (dual ? 1 : 2) : 1;
   const int kb_bytes = 64 * (int)kBlockK * 2 + pl.nt * (int)kBlockK * 2, per_cta = (pl.kb_total + pl.splits - 1) / pl.splits;
   // the tile's rows on their way to the epilogue: unsplit they lie over the drained stages
-  const int recv = (m + 3) / 4 * 64 * 16, beside = pl.splits > 1 ? recv : 0;
-  const int room = (q == 1 ? kFewSmem : 228 * 1024 / q - 2048) - 1024 - beside;      // for stages (a CTA's fixed part and the system's: 2 KB)
+  const int recv = (m + 3) / 4 * 64 * 16 * (pl.splits > 1 && pl.parts > 1 ? pl.parts : 1), beside = pl.splits > 1 ? recv : 0;
+  const int most = q == 1 ? kFewSmem : 228 * 1024 / q - 2048, room = most - 1024 - beside;      // for stages (a CTA's fixed part and the system's: 2 KB)
   // All k-blocks at once where they fit, in stages of four, five or seven: as few blocks beyond the range as there can be, then as
   // few stages.
   auto fit = [&](int g) { return (per_cta + g - 1) / g * g * kb_bytes <= room; };
   pl.group = 4;
   for (int g = 5; g <= 7; g += 2)
     if (fit(g) && (per_cta + g - 1) / g * g <= (per_cta + pl.group - 1) / pl.group * pl.group) pl.group = g;
-  if (!in_l2 && !fit(pl.group)) pl.group = 2;
+  if (!in_l2) pl.group = 2;
   const int stage_bytes = pl.group * kb_bytes, groups = (per_cta + pl.group - 1) / pl.group;
   pl.stages = room / stage_bytes;
   if (pl.stages > kFewStages) pl.stages = kFewStages;
   if (pl.stages > groups) pl.stages = groups;
-  pl.ring = pl.stages < groups;
-  if (pl.ring && pl.stages < 2) return ProjFewPlan{};
+  pl.ring = pl.stages < groups || pl.parts > 0;
+  if (pl.stages < groups && pl.stages < 2) return ProjFewPlan{};
   pl.recv_off = beside ? pl.stages * stage_bytes : 0;
   pl.smem_bytes = pl.stages * stage_bytes + beside + 1024;
   if (pl.smem_bytes < recv + 1024) pl.smem_bytes = recv + 1024;
-  pl.tmem_cols = pl.nt <= 32 ? 32 : pl.nt <= 64 ? 64 : 128;
-  const int share = (int)((228u * 1024u * (unsigned)pl.tmem_cols + 511u) / 512u) - 1024;   // as in plan_proj
+  pl.tmem_cols = 32;
+  while (pl.tmem_cols < (n_acc > 1 ? pl.acc_ld * n_acc : pl.nt)) pl.tmem_cols <<= 1;
+  // as in plan_proj, less the fixed part too: of at most sixteen CTAs the half kilobyte that may be missing from each is less than
+  // 32 columns' share
+  const int share = (int)((228u * 1024u * (unsigned)pl.tmem_cols + 511u) / 512u) - 2048;
   if (pl.smem_bytes < share) pl.smem_bytes = share;
-  return pl;
+  return pl.smem_bytes <= most ? pl : ProjFewPlan{};
 }
 
 // ---- block-vs-cache attention, attention_block.cu -------------------------------------------------

@@ -1,5 +1,6 @@
-// Weight-streaming projections of calls with few tokens (bf16 contexts of wide models whose matrices stay in L2): the same
-// operations as proj_tc.cu on tiles of 64 weight rows.
+// Weight-streaming projections of calls with few tokens (bf16 contexts of wide models): the same operations as proj_tc.cu on
+// tiles of 64 weight rows.  Of models whose weights do not stay in L2 it gives the same bits too (APART below; which projections
+// these are and what it gives: plan_proj_few, launch_plans.h).
 //
 // What bounds such a projection is the chain of one CTA: wait for the kernel before, activations from L2, MMAs, exchange, epilogue.
 // - An MMA of 64 rows reads half the shared memory of one of 128 and takes 24 cycles in the place of 40 (N = 24 or 32), so a CTA
@@ -10,6 +11,7 @@
 // - All stages' weights are requested before tensor memory and the CTA's barrier, then whatever the epilogue needs besides
 //   the sums (rows, places in the cache, rotation) is found, all before griddepcontrol.wait.
 //   QKV, ADD  64 rows of one matrix;  GATEUP  32 rows of gate, then the same 32 of up, in the order of their addresses
+// (All figures here: the XL shape and models like it, whose weights stay in L2.)
 // An accumulator of M = 64 lies in lanes 0-15 of the four lane quarters; its rows go to shared memory as [token quad][rank][row]
 // float4 (split: with st.async to the rank that owns the row, counted on its mbarrier), and the epilogue takes a pair of rows and
 // two tokens per thread (four where 64 rows are finished at once), partial sums in rank order.
@@ -33,7 +35,8 @@ constexpr uint32_t kRows = 64;
 constexpr uint32_t kABytes = kRows * kBlockK * 2;
 
 struct Params {
-  int m, n, nt, kb_total, stages;
+  int m, n, nt, kb_total, stages, parts, log_slices;      // parts: slices of proj_tc.cu's plan per CTA, log2 of all of them, columns
+  int acc_ld;                                          // from one accumulator to the next (APART)
   uint32_t tmem_cols, recv_off;
   int32_t* status;
   const float* ss_in; int ss_parts; float inv_d, eps;                  // QKV, GATEUP: [token][ss_parts], a multiple of 4
@@ -44,17 +47,21 @@ struct Params {
   const uint8_t* ahead[2]; uint32_t ahead_bytes;      // weights of the projection after next, to be brought into L2
 };
 
-// LOG_S: log2 of the slices of K; G: k-blocks per stage; RING: stages are filled again.
+// LOG_S: log2 of the slices of K; G: k-blocks per stage; RING: stages are filled again.  APART: every partial sum that proj_tc.cu's plan
+// would take has an accumulator of its own (each of its slices; of a single matrix every other k-block), they are added in that
+// kernel's order, and an ADD's sums of squares cover its rows in its order: the same bits, whichever of the two kernels runs.
 // The issuing warp is alone in its loop, where every wait, vote and branch shows: 80 MMAs of 64 x 24 x 16 take 27.8 cycles each with
 // ten k-blocks per wait, 31 with four, 47 with one, and 41 with four where a ring's bookkeeping and a test for a partial
 // stage are in the loop.
-template <int EPI, int LOG_S, int G, bool RING>
+template <int EPI, int LOG_S, int G, bool RING, bool APART>
 __global__ void __launch_bounds__(kThreads)
 proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b) {
   constexpr bool DUAL = EPI == PROJ_GATEUP;
   constexpr int NACC = DUAL ? 2 : 1;
   constexpr bool SPLIT = LOG_S > 0;
   constexpr int S = 1 << LOG_S;
+  const int parts = APART ? p.parts : 1;
+  const uint32_t acc_ld = (uint32_t)p.acc_ld;
   constexpr int TPI = DUAL || SPLIT ? 2 : 4;           // tokens per item of the epilogue
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[kFewStages];
@@ -97,7 +104,7 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
       s_abort = 0;
       fence_barrier_init();
       fence_proxy_async();
-      if (SPLIT) mbar_expect_tx(&recv_bar, (uint32_t)nq * kRows * 16u);
+      if (SPLIT) mbar_expect_tx(&recv_bar, (uint32_t)(nq * parts) * kRows * 16u);
     }
     __syncwarp();
     // All stages are free, so the weights go out first of all: a CTA that could only start when the kernel before it drained has
@@ -210,7 +217,30 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
         mma_bf16_k64(tmem_base, a_lo + j * (kABytes >> 4), a_lo + G * (kABytes >> 4) + j * b_lo, idesc, (uint32_t)(i + j));
     };
     pdl_wait();
-    if constexpr (RING) {
+    if constexpr (APART) {
+      // k-block at of slice q, which begins at k-block (rank * parts + q) * kb_total / slices: the boundaries of this CTA's range lie on them
+      uint32_t stage = 0, par = 0, d = tmem_base;
+      int at = 0, q = rank * parts, len = (((q + 1) * p.kb_total) >> p.log_slices) - kb0;
+      for (int i = 0; i < ng; ++i) {
+        wait_full(stage, par);
+        const uint32_t a_lo = lo0 + stage * stage_lo;
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+          if (i * G + j < nkb) {
+            mma_bf16_k64(d + (DUAL || !(at & 1) ? 0u : acc_ld), a_lo + j * (kABytes >> 4), a_lo + G * (kABytes >> 4) + j * b_lo, idesc,
+                         (uint32_t)(DUAL ? at : at >> 1));
+            if (++at == len) {
+              const int begin = (++q * p.kb_total) >> p.log_slices;
+              len = (((q + 1) * p.kb_total) >> p.log_slices) - begin;
+              at = 0;
+              d += (DUAL ? 1u : 2u) * acc_ld;
+            }
+          }
+        }
+        if (i + p.stages < ng) mma_commit_elect(&empty_bar[stage]);  // a group is still to come into this stage
+        if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1; }
+      }
+    } else if constexpr (RING) {
       uint32_t stage = 0, par = 0;
       for (int i = 0; i < ng; ++i) {
         wait_full(stage, par);
@@ -273,19 +303,42 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
   // ---- rows to where the epilogue reads them ---------------------------------------------------------------------------
   {
     const int row_t = (warp & 3) * 16 + (lane & 15), owner = row_t >> (6 - LOG_S);
-    const uint32_t at = smem_u32(recv) + (uint32_t)(SPLIT ? rank * rpr + (row_t & (rpr - 1)) : row_t) * 16u;
+    const uint32_t at = smem_u32(recv) + (uint32_t)(SPLIT ? rank * parts * rpr + (row_t & (rpr - 1)) : row_t) * 16u;
     const uint32_t recv_dst = SPLIT ? mapa(at, (uint32_t)owner) : at, bar_dst = SPLIT ? mapa(smem_u32(&recv_bar), (uint32_t)owner) : 0u;
     const uint32_t t_row = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
     for (int c0 = (warp >> 2) * 2; c0 < nq; c0 += 4) {
       float v[8];
-      tmem_ld8(t_row + (uint32_t)(c0 * 4), v);
+      auto put = [&](uint32_t part) {
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        if (lane < 16 && c0 + j < nq) {
-          const uint32_t dst = recv_dst + (uint32_t)(c0 + j) * (kRows * 16u);
-          if (SPLIT) st_async4(dst, bar_dst, &v[4 * j]);
-          else st_shared4(dst, &v[4 * j]);
+        for (int j = 0; j < 2; ++j) {
+          if (lane < 16 && c0 + j < nq) {
+            const uint32_t dst = recv_dst + (uint32_t)((c0 + j) * (SPLIT ? parts : 1)) * (kRows * 16u) + part * (uint32_t)(rpr * 16);
+            if (SPLIT) st_async4(dst, bar_dst, &v[4 * j]);
+            else st_shared4(dst, &v[4 * j]);
+          }
         }
+      };
+      if constexpr (APART) {
+#pragma unroll 1
+        for (int a = 0; a < parts; ++a) {
+          const uint32_t t_acc = t_row + (uint32_t)(DUAL ? a : 2 * a) * acc_ld + (uint32_t)(c0 * 4);
+          const int q = rank * parts + a;
+          float w[8];
+          tmem_ld8(t_acc, w);
+          if (!DUAL && (((q + 1) * p.kb_total) >> p.log_slices) - ((q * p.kb_total) >> p.log_slices) > 1) {     // every other k-block
+            float z[8];
+            tmem_ld8(t_acc + acc_ld, z);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w[j] += z[j];
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[j] = SPLIT || a == 0 ? w[j] : v[j] + w[j];
+          if (SPLIT) put((uint32_t)a);
+        }
+        if (!SPLIT) put(0u);
+      } else {
+        tmem_ld8(t_row + (uint32_t)(c0 * 4), v);
+        put(0u);
       }
     }
   }
@@ -306,7 +359,7 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
   for (int idx = eid; idx < items_up; idx += kThreads) {
     const int quad = idx >> (log_np + log_sub), t0 = quad * 4 + sub;
     float acc[NACC][2][TPI];                                       // [row][token]
-    const uint8_t* src = recv + (size_t)(idx < items ? quad : 0) * (kRows * 16u) + src_row;
+    const uint8_t* src = recv + (size_t)((idx < items ? quad : 0) * (SPLIT ? parts : 1)) * (kRows * 16u) + src_row;
 #pragma unroll
     for (int a = 0; a < NACC; ++a)
 #pragma unroll
@@ -314,7 +367,7 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
         const uint8_t* at = src + (DUAL ? a ^ p.up_first : 0) * (kRows / 2 * 16u) + i * 16;
         ld_shared_vec(at, acc[a][i]);
 #pragma unroll
-        for (int r = 1; r < S; ++r) {         // rank order
+        for (int r = 1; r < (APART && SPLIT ? S * parts : S); ++r) {         // rank order
           float v[TPI];
           ld_shared_vec(at + r * rpr * 16, v);
 #pragma unroll
@@ -322,12 +375,13 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
         }
       }
     if constexpr (EPI == PROJ_ADD) {
-      float sq[TPI];
+      float sq[TPI], sq1[TPI];                 // APART: of the two rows, added last
       const float2 gsc = make_float2(__uint_as_float(scale2 << 16), __uint_as_float(scale2 & 0xffff0000u));
 #pragma unroll
       for (int j = 0; j < TPI; ++j) {
         const float x0 = xo[j].x + acc[0][0][j], x1 = xo[j].y + acc[0][1][j];
-        sq[j] = dst[j] ? x0 * x0 + x1 * x1 : 0.f;
+        sq[j] = !dst[j] ? 0.f : APART ? __fmul_rn(x0, x0) : x0 * x0 + x1 * x1;
+        sq1[j] = APART && dst[j] ? __fmul_rn(x1, x1) : 0.f;
         if (dst[j]) {
           *reinterpret_cast<float2*>(p.x + (size_t)(t0 + j) * p.d + n) = make_float2(x0, x1);
           *reinterpret_cast<uint32_t*>(dst[j]) = pack_bf16(x0 * gsc.x, x1 * gsc.y);
@@ -343,7 +397,13 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
       } else {
         for (int o = 1 << log_np; o > 1; o >>= 1)
 #pragma unroll
-          for (int j = 0; j < TPI; ++j) sq[j] += __shfl_xor_sync(0xffffffffu, sq[j], o);
+          for (int j = 0; j < TPI; ++j) {
+            sq[j] += __shfl_xor_sync(0xffffffffu, sq[j], o);
+            if (APART) sq1[j] += __shfl_xor_sync(0xffffffffu, sq1[j], o);
+          }
+        if (APART)
+#pragma unroll
+          for (int j = 0; j < TPI; ++j) sq[j] += sq1[j];
         if (idx < items && pair == 0)
 #pragma unroll
           for (int j = 0; j < TPI; ++j)
@@ -381,9 +441,9 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
   }
 }
 
-template <int EPI, int LOG_S, int G, bool RING>
+template <int EPI, int LOG_S, int G, bool RING, bool APART = false>
 cudaError_t launch_one(const ProjFewPlan& pl, const Params& kp, const ProjArgs& g, cudaStream_t s) {
-  auto* fn = proj_few_kernel<EPI, LOG_S, G, RING>;
+  auto* fn = proj_few_kernel<EPI, LOG_S, G, RING, APART>;
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(fn), kFewSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -408,21 +468,31 @@ cudaError_t launch_one(const ProjFewPlan& pl, const Params& kp, const ProjArgs& 
   return cudaLaunchKernelEx(&cfg, fn, kp, *g.tm_a, *g.tm_b);
 }
 
+// (what plan_proj_few has no use for is not compiled: QKV has eight k-blocks or more and is split unless its sums are kept apart, an
+// unsplit ADD has fewer than eight and needs no ring)
 template <int EPI, int LOG_S>
 cudaError_t launch_epi(const ProjFewPlan& pl, const Params& kp, const ProjArgs& g, cudaStream_t s) {
   if (pl.splits != 1 << LOG_S) return cudaErrorInvalidValue;
-  if (pl.ring) return pl.group == 2 ? launch_one<EPI, LOG_S, 2, true>(pl, kp, g, s) : launch_one<EPI, LOG_S, 4, true>(pl, kp, g, s);
-  if (pl.group == 2) return launch_one<EPI, LOG_S, 2, false>(pl, kp, g, s);
-  if (pl.group == 4) return launch_one<EPI, LOG_S, 4, false>(pl, kp, g, s);
-  if (pl.group == 5) return launch_one<EPI, LOG_S, 5, false>(pl, kp, g, s);
-  return launch_one<EPI, LOG_S, 7, false>(pl, kp, g, s);
+  if constexpr (EPI != PROJ_ADD || LOG_S > 0) {
+    if (pl.parts > 0) return pl.group == 2 && pl.ring ? launch_one<EPI, LOG_S, 2, true, true>(pl, kp, g, s) : cudaErrorInvalidValue;
+    if constexpr (EPI != PROJ_QKV || LOG_S > 0)
+      if (pl.ring) return pl.group == 4 ? launch_one<EPI, LOG_S, 4, true>(pl, kp, g, s) : cudaErrorInvalidValue;
+  }
+  if (pl.parts > 0 || pl.ring) return cudaErrorInvalidValue;
+  if constexpr (EPI != PROJ_QKV || LOG_S > 0) {
+    if (pl.group == 4) return launch_one<EPI, LOG_S, 4, false>(pl, kp, g, s);
+    if (pl.group == 5) return launch_one<EPI, LOG_S, 5, false>(pl, kp, g, s);
+    if (pl.group == 7) return launch_one<EPI, LOG_S, 7, false>(pl, kp, g, s);
+  }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
 int launch_proj_few(int epi, const ProjFewPlan& pl, const ProjArgs& g, cudaStream_t s) {
   Params kp{};
-  kp.m = g.m; kp.n = g.n; kp.nt = pl.nt; kp.kb_total = pl.kb_total; kp.stages = pl.stages;
+  kp.m = g.m; kp.n = g.n; kp.nt = pl.nt; kp.kb_total = pl.kb_total; kp.stages = pl.stages; kp.parts = pl.parts; kp.acc_ld = pl.acc_ld;
+  while ((1 << kp.log_slices) < pl.parts * pl.splits) ++kp.log_slices;
   kp.tmem_cols = (uint32_t)pl.tmem_cols; kp.recv_off = (uint32_t)pl.recv_off; kp.status = g.status;
   kp.ss_in = g.ss_in; kp.ss_parts = g.ss_parts; kp.inv_d = 1.f / (float)g.d; kp.eps = g.eps;
   kp.x = g.x; kp.xg = g.xg; kp.scale = g.scale; kp.ss_out = g.ss_out; kp.ss_out_parts = proj_ss_parts(pl); kp.d = g.d;

@@ -1,6 +1,8 @@
 """Results that stay what they were, bit for bit.  Deep models answer any change in the order or place of a rounding with guided
-probabilities that move by more than a caller may see, so heads of 128 keep the arithmetic of their attention.  Inputs are small multiples of powers of two: the same everywhere."""
+probabilities that move by more than a caller may see, so heads of 128 keep the arithmetic of their attention, and a projection whose
+weights do not stay in L2 gives the same bits whichever of its two kernels runs it.  Inputs are small multiples of powers of two: the same everywhere."""
 import hashlib
+from dataclasses import replace
 
 import pytest
 
@@ -64,3 +66,30 @@ def test_attention_of_heads_of_128(n_images, n_cfg, n_forced, k, fills, want):
     """Recorded before its kernel was rewritten for fewer instructions (CUDA 12.9)."""
     out = _step(HEADS128, _weights(HEADS128, 7100), n_images, n_cfg, n_forced, k, fills, 7200 + k)
     assert hashlib.sha256(b"".join(x.numpy().tobytes() for x in out)).hexdigest()[:16] == want
+
+
+# Partial sums kept apart: QKV two slices in each of two CTAs, gate/up four in one, down projection two in each of four; one, two (and the
+# output projection two in each of four); QKV unsplit, two in one CTA.
+MID = ModelShape("mid", 2, 2048, 16, 128, 5504, 512, s_max=600, rope_mode=ROPE_1D, n_prefix=1)
+WIDE = replace(MID, name="wide", d_model=4096, n_heads=32, d_ff=11008)
+UNSPLIT = replace(MID, name="unsplit", n_layers=1, d_model=5120, n_heads=40, d_ff=13824)
+EIGHT = replace(MID, name="eight", d_model=1536, n_heads=12, d_ff=4096)          # gate/up: eight in one CTA
+
+
+@pytest.mark.parametrize("ms,n_images,n_cfg,n_forced,k,fills", [
+    (MID, 1, 1, 1, 1, [300]), (MID, 1, 2, 1, 8, [20]), (MID, 1, 2, 1, 24, [570]), (MID, 1, 2, 6, 24, [99]), (MID, 4, 2, 1, 8, [0, 9, 333, 80]),
+    (WIDE, 1, 1, 1, 8, [40]), (WIDE, 1, 2, 1, 8, [512]), (WIDE, 1, 2, 2, 14, [7]), (WIDE, 3, 2, 1, 7, [0, 9, 333]), (WIDE, 5, 2, 1, 7, [1, 2, 3, 4, 5]),
+    (UNSPLIT, 1, 2, 1, 8, [60]), (UNSPLIT, 3, 2, 1, 8, [0, 9, 333]), (EIGHT, 1, 2, 1, 8, [60]), (EIGHT, 2, 2, 1, 14, [5, 200])])
+def test_either_projection_kernel_gives_the_same_bits(ms, n_images, n_cfg, n_forced, k, fills):
+    """d_ff less eight is no multiple of 64 (one kernel for everything), has the same plans, and with eight rows and columns of zeros
+    is the same model again."""
+    import torch
+    w = _weights(replace(ms, d_ff=ms.d_ff - 8), 7300)
+    want = _step(replace(ms, d_ff=ms.d_ff - 8), w, n_images, n_cfg, n_forced, k, fills, 7400 + k)
+    for layer in w["layers"]:
+        for name in ("w_gate", "w_up", "w_down"):
+            pad = (0, 8) if name == "w_down" else (0, 0, 0, 8)
+            layer[name] = torch.nn.functional.pad(layer[name], pad).contiguous()
+    got = _step(ms, w, n_images, n_cfg, n_forced, k, fills, 7400 + k)
+    for a, b in zip(want, got):
+        assert torch.equal(a, b)

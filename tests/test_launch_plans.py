@@ -11,7 +11,8 @@ CSRC = os.path.join(ROOT, "paper_2511_13587_b200", "csrc")
 N_SMS = 148
 FIELDS = ("nt", "passes", "tiles", "kb_total", "splits", "stages", "alias", "recv_off", "smem_bytes", "tmem_cols", "threads",
           "tiles_on_z")
-FEW_FIELDS = ("nt", "tiles", "kb_total", "splits", "group", "stages", "ring", "recv_off", "smem_bytes", "tmem_cols")
+FEW_FIELDS = ("nt", "tiles", "kb_total", "splits", "group", "stages", "ring", "recv_off", "smem_bytes", "tmem_cols",
+              "parts", "acc_ld")
 SHIM = """
 #include "launch_plans.h"
 extern "C" void proj(int m, int n, int k, int dual, int n_sms, int* o) {
@@ -81,8 +82,8 @@ def test_projection_plans_fit_the_hardware(plans, d, ff):
 
 
 @pytest.mark.parametrize("d,ff,in_l2", [(1024, 320, 1), (1024, 2752, 1), (1152, 3072, 1), (1280, 3456, 1), (1280, 64, 1), (2048, 128, 1),
-                                        (1536, 3008, 0), (2048, 5504, 0), (4096, 11008, 0), (5120, 13824, 0), (8192, 28672, 0),
-                                        (1024, 65536, 0), (16384, 64, 0)])
+                                        (1536, 3008, 0), (1536, 4096, 0), (2048, 5504, 0), (3072, 8192, 0), (4096, 11008, 0),
+                                        (5120, 13824, 0), (8192, 28672, 0), (1024, 65536, 0), (16384, 64, 0)])
 def test_few_token_plans_fit_the_hardware(plans, d, ff, in_l2):
     taken = 0
     for m in range(1, 97):
@@ -96,19 +97,25 @@ def test_few_token_plans_fit_the_hardware(plans, d, ff, in_l2):
             taken += 1
             assert p["nt"] % 8 == 0 and p["nt"] - 8 < m <= p["nt"], at
             assert p["tiles"] == -(-n // (32 if dual else 64)) and p["kb_total"] == k // 64, at
+            # where the sums are kept apart: whole slices of the other kernel's plan, and for an ADD its ranks of 16 rows
+            wide = _proj(plans, m, n, k, dual)["splits"]
+            assert (p["parts"] == 0 if in_l2 else p["parts"] * p["splits"] == wide) and (in_l2 or not add or wide == 8), at
+            n_acc = max(1, p["parts"] * (1 if dual else 2))
             # the kernels that exist: gate/up unsplit, QKV in one or two slices, the others in one or four; rings have stages of two or four
             assert p["splits"] in ((1,) if dual else (1, 4) if add else (1, 2)) and p["splits"] <= p["kb_total"], at
             per_cta = -(-p["kb_total"] // p["splits"])
             groups = -(-per_cta // p["group"])
-            assert p["group"] in (2, 4, 5, 7) and 1 <= p["stages"] <= min(12, groups) and p["ring"] == (p["stages"] < groups), at
-            assert not p["ring"] or (p["group"] == (4 if in_l2 else 2) and p["stages"] >= 2), at
+            assert p["group"] in (2, 4, 5, 7) and 1 <= p["stages"] <= min(12, groups) and p["ring"] == (not in_l2 or p["stages"] < groups), at
+            assert not p["ring"] or p["group"] == (4 if in_l2 else 2), at
+            assert p["stages"] >= min(2, groups), at
             # stages, and the tile's rows beside them (split) or over them
-            stage, recv = p["group"] * (64 + p["nt"]) * 128, -(-m // 4) * 1024
+            stage, recv = p["group"] * (64 + p["nt"]) * 128, -(-m // 4) * 1024 * (max(1, p["parts"]) if p["splits"] > 1 else 1)
             assert p["recv_off"] == (p["stages"] * stage if p["splits"] > 1 else 0), at
             need = p["stages"] * stage + recv if p["splits"] > 1 else max(p["stages"] * stage, recv)
             assert need + 1024 <= p["smem_bytes"] <= 226 * 1024, at
-            assert p["nt"] <= p["tmem_cols"] and p["tmem_cols"] in (32, 64, 128), at
-            assert (p["smem_bytes"] + 1024) * 512 >= p["tmem_cols"] * 228 * 1024 - 512, at
+            assert p["acc_ld"] % 32 == 0 and p["nt"] <= p["acc_ld"] and p["tmem_cols"] in (32, 64, 128, 256, 512), at
+            assert (p["nt"] if n_acc == 1 else p["acc_ld"] * n_acc) <= p["tmem_cols"], at
+            assert (p["smem_bytes"] + 2048) * 512 >= p["tmem_cols"] * 228 * 1024 - 512, at
             # the sums of squares: whole float4, room for d / 8 of them per token
             assert p["ss_parts"] % 4 == 0 and p["tiles"] * p["splits"] <= p["ss_parts"] < p["tiles"] * p["splits"] + 4, at
             assert not add or p["ss_parts"] <= (d + 127) // 128 * 16, at
@@ -116,7 +123,6 @@ def test_few_token_plans_fit_the_hardware(plans, d, ff, in_l2):
                 per_sm = 228 * 1024 // (p["smem_bytes"] + 2048) if p["smem_bytes"] <= 112 * 1024 else 1
                 assert p["tiles"] * p["splits"] <= per_sm * N_SMS * (33 / 37 if p["splits"] == 4 else 1), at
     assert taken == 4 * 96 if in_l2 else taken > 0 or d > 8000
-
 
 
 def test_passes_over_weights_that_exceed_l2(plans):
