@@ -377,8 +377,8 @@ int vvs_device_status(vvs_ctx* ctx, void* stream, int32_t* out_bits);
 /* Self-test of the failure path of the library's bounded device-side waits (no counterpart in the
  * paper).  Launches one tiny kernel in which a thread waits, through the same helpers the tensor-core
  * kernels and the streaming chain kernel use but with a limit of a few hundred polls, on barriers
- * nobody ever arrives on.  Each wait must give up and return: gave_up[0] / gave_up[1] (host int32[2])
- * are set to 1 for the two helpers, the VVS_DEV_TIMEOUT bit is left in the device status word (so
+ * nobody ever arrives on; before that, warps of which half give up and half do not decide as one.  Each wait
+ * must give up and return: gave_up[0] / gave_up[1] (host int32[2]) are set to 1 for the two helpers, the VVS_DEV_TIMEOUT bit is left in the device status word (so
  * the next vvs_device_status returns VVS_ERR_DEVICE_TIMEOUT and clears it), and the context stays
  * usable.  Synchronises `stream`.  Nothing in it can hang: the waits are the bounded ones. */
 int vvs_selftest_bounded_wait(vvs_ctx* ctx, void* stream, int32_t* gave_up);

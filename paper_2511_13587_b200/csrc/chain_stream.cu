@@ -1017,17 +1017,25 @@ chain_pack_kernel(PackLayer wl, const ChainCtaPlan* plans, uint8_t* out_layer, i
 // Self-test of the bounded waits: one thread waits, with a limit of a few hundred polls, on barriers
 // on which nobody ever arrives.  Both helpers must give up, record VVS_DEV_TIMEOUT and return.
 __global__ void bounded_wait_selftest_kernel(int32_t* status, int32_t* report) {
-  __shared__ __align__(8) uint64_t bar[2];
+  __shared__ __align__(8) uint64_t bar[3];
   __shared__ volatile int s_abort;
   if (threadIdx.x == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
+    mbar_init(&bar[2], 1);
     s_abort = 0;
     fence_barrier_init();
+    mbar_arrive(&bar[2]);
+  }
+  __syncthreads();
+  // two warps see their barrier complete and two give up: all four have to come to the same decision
+  const bool stay = named_bar_all(1, 128, threadIdx.x < 64 ? mbar_wait_limited(&bar[2], 0u, 256u) : mbar_wait_limited(&bar[0], 0u, 256u));
+  const bool agreed = !__syncthreads_or(stay ? 1 : 0);
+  if (threadIdx.x == 0) {
     const bool got0 = mbar_wait_limited(&bar[0], 0u, 256u);   // the helper of the tcgen05 kernels
     if (!got0) atomicOr(status, VVS_DEV_TIMEOUT);
     wait_slow(&bar[1], 0u, &s_abort, status, 64u);            // the helper of the streaming chain kernel
-    report[0] = got0 ? 1 : 0;
+    report[0] = got0 || !agreed ? 1 : 0;
     report[1] = s_abort;
   }
 }
@@ -1122,7 +1130,7 @@ int chain_stream_pack(const vvs_model_desc& md, const ChainStreamPlan& plan, con
 
 // keys per attention block: K and V of a block share one 20 KB ring slot (8 KB each)
 void launch_bounded_wait_selftest(int32_t* status, int32_t* report, cudaStream_t s) {
-  bounded_wait_selftest_kernel<<<1, 32, 0, s>>>(status, report);
+  bounded_wait_selftest_kernel<<<1, 128, 0, s>>>(status, report);
 }
 
 int chain_stream_kb(const vvs_model_desc& md) { return md.head_dim == 64 ? 64 : 32; }

@@ -33,8 +33,8 @@ constexpr int kChunk = 16;            // decision rows per epilogue step of a gr
 constexpr int kTileBytes = kGroups * kChunk * 128 * 4;     // the groups' logit tiles
 constexpr uint32_t kBlockK = 64;
 constexpr uint32_t kABytes = 128 * kBlockK * 2;
-// k-blocks per pipeline stage: the issuing thread pays a wait and a commit (~270 cycles) per stage against 64 cycles
-// per MMA, and a k-block's four MMAs run 512 cycles at full width
+// k-blocks per pipeline stage: a wait and a commit of the issuing warp per stage, and a k-block's four MMAs run 512 cycles at
+// full width (chosen when a lone lane issued, which paid some 270 cycles for the two; one k-block a stage was not measured since)
 constexpr uint32_t kSub = 2;
 
 struct Params {
@@ -180,7 +180,7 @@ lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, con
     const uint32_t idesc = idesc_bf16_f32(256, n_cols);
     const uint32_t lo0 = desc_lo_sw128(smem_u32(smem)), stage_lo = stage_bytes >> 4;
     uint32_t stage = 0, par = 0;
-    int it = 0;
+    int it = 0, issued = 0;
     bool ok = true;
     for (int u = pair; u < p.units && ok; u += n_pairs, ++it) {
       const uint32_t buf = it & 1, d = tmem + buf * 256u;
@@ -194,9 +194,14 @@ lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, con
         for (uint32_t h = 0; h < kSub; ++h)
           mma_pair_k64(d, a_lo + h * (kABytes >> 4), a_lo + ((kSub * kABytes + h * b_bytes) >> 4), idesc, kb > 0 || h > 0);
         commit_pair(&empty_bar[stage]);
+        ++issued;
         if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1u; }
       }
-      commit_pair(&acc_full[buf]);
+      if (ok) commit_pair(&acc_full[buf]);        // (half an accumulator is nobody's)
+    }
+    if (!ok && issued > 0) {                      // gave up: the MMAs issued so far end before the pair leaves (bounded)
+      const int i = issued - 1;
+      for (uint32_t k = 0; k < kSpinLimit && !mbar_try_wait_cluster(&empty_bar[i % p.stages], (i / p.stages) & 1); ++k) {}
     }
   } else if (warp >= 4) {
     // ---- epilogue: a group takes every fourth chunk of 16 decision rows; thread = one code, logits out and to the group's tile
@@ -214,7 +219,9 @@ lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, con
       const int nd = min(p.nd, p.bt - row0);
       const int n = tile * 256 + rank * 128 + e, t128 = tile * 2 + rank;
       const bool n_ok = n < p.v;
-      if (!wait_or_abort(&acc_full[buf], (it >> 1) & 1, &s_abort, p.status)) break;
+      // (a thread that saw another role's abort in time may be beside one that saw the accumulator: the group leaves or stays as one,
+      // since it meets at barriers below)
+      if (!named_bar_all(1 + grp, 128, wait_or_abort(&acc_full[buf], (it >> 1) & 1, &s_abort, p.status))) break;
       tc_fence_after();
       const uint32_t t_row = tmem + (uint32_t)buf * 256u + t_lane;
       auto release = [&]() {                      // the accumulator has been read: the next unit but one may have it

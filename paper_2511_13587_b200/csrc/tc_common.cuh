@@ -99,6 +99,17 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
 __device__ __forceinline__ void named_bar_sync(int id, int n_threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n_threads) : "memory");
 }
+// The same barrier, and whether all of its threads said yes: the same answer in each of them.  Threads that wait for something with a
+// limit and then meet at a barrier decide with this whether they go on: some may have given up where others have not.
+__device__ __forceinline__ bool named_bar_all(int id, int n_threads, bool yes) {
+  uint32_t all;
+  __syncwarp();
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %3, 0;\n\t"
+      "bar.red.and.pred p, %1, %2, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(all) : "r"(id), "r"(n_threads), "r"((uint32_t)yes) : "memory");
+  return all != 0;
+}
 __device__ __forceinline__ void fence_barrier_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
