@@ -55,7 +55,7 @@ size_t layout(const vvs_model_desc& d, Workspace& ws, char* base, bool few_logit
       const size_t wide = 3 * dm > 2 * ff ? 3 * dm : 2 * ff;
       const size_t tiles = (wide + 127) / 128, passes = (M + 255) / 256;
       c.take(ws.slot_pos, M * 4);
-      c.take(ws.ss_part, (dm + 127) / 128 * 16 * M * 4);     // (proj_few.cu: eight slices of 64 rows)
+      c.take(ws.ss_part, (dm + 127) / 128 * 8 * M * 4);      // (ranks of 16 rows at most)
       c.take(ws.seq_order, (size_t)d.max_rows * 4);
       c.take(ws.rope_cos, M * (size_t)(d.head_dim / 2) * 4);
       c.take(ws.rope_sin, M * (size_t)(d.head_dim / 2) * 4);

@@ -116,9 +116,9 @@ def test_few_token_plans_fit_the_hardware(plans, d, ff, in_l2):
             assert p["acc_ld"] % 32 == 0 and p["nt"] <= p["acc_ld"] and p["tmem_cols"] in (32, 64, 128, 256, 512), at
             assert (p["nt"] if n_acc == 1 else p["acc_ld"] * n_acc) <= p["tmem_cols"], at
             assert (p["smem_bytes"] + 2048) * 512 >= p["tmem_cols"] * 228 * 1024 - 512, at
-            # the sums of squares: whole float4, room for d / 8 of them per token
+            # the sums of squares: whole float4, room for d / 16 of them per token
             assert p["ss_parts"] % 4 == 0 and p["tiles"] * p["splits"] <= p["ss_parts"] < p["tiles"] * p["splits"] + 4, at
-            assert not add or p["ss_parts"] <= (d + 127) // 128 * 16, at
+            assert not add or p["ss_parts"] <= (d + 127) // 128 * 8, at
             if not in_l2:                                           # all CTAs at once, with 1 KB each for the system and what is static
                 per_sm = 228 * 1024 // (p["smem_bytes"] + 2048) if p["smem_bytes"] <= 112 * 1024 else 1
                 assert p["tiles"] * p["splits"] <= per_sm * N_SMS * (33 / 37 if p["splits"] == 4 else 1), at
