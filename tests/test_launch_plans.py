@@ -80,29 +80,41 @@ def test_projection_plans_fit_the_hardware(plans, d, ff):
             assert p["threads"] in (256, 512) and p["threads"] % (128 // p["splits"]) == 0, at
             assert p["ss_parts"] % 4 == 0 and p["ss_parts"] <= p["tiles"] * 8, at
 
+# Weights from HBM: up to how many tokens each projection is taken (QKV, output, gate/up, down projection).  None where more than
+# three CTAs per SM would be needed (d_model 8192), matrices beyond 64 MB at most 80, otherwise what the ranks of plan_proj allow.
+TAKEN = {(1536, 3008): [96, 83, 96, 80], (1536, 4096): [96, 83, 96, 83], (2048, 5504): [64, 0, 96, 96], (3072, 8192): [32, 0, 80, 64],
+         (4096, 11008): [52, 32, 80, 0], (5120, 13824): [80, 0, 80, 0], (8192, 28672): [0, 0, 0, 0], (1024, 65536): [64, 42, 0, 80],
+         (16384, 64): [0, 0, 64, 0]}
+
 
 @pytest.mark.parametrize("d,ff,in_l2", [(1024, 320, 1), (1024, 2752, 1), (1152, 3072, 1), (1280, 3456, 1), (1280, 64, 1), (2048, 128, 1),
                                         (1536, 3008, 0), (1536, 4096, 0), (2048, 5504, 0), (3072, 8192, 0), (4096, 11008, 0),
                                         (5120, 13824, 0), (8192, 28672, 0), (1024, 65536, 0), (16384, 64, 0)])
 def test_few_token_plans_fit_the_hardware(plans, d, ff, in_l2):
-    taken = 0
+    taken = [0, 0, 0, 0]                                            # calls of up to so many tokens: QKV, output, gate/up, down projection
     for m in range(1, 97):
-        for n, k, dual, add in ((3 * d, d, 0, 0), (d, d, 0, 1), (ff, d, 1, 0), (d, ff, 0, 1)):
+        for i, (n, k, dual, add) in enumerate(((3 * d, d, 0, 0), (d, d, 0, 1), (ff, d, 1, 0), (d, ff, 0, 1))):
             out = (ctypes.c_int * (len(FEW_FIELDS) + 1))()
             plans.few(m, n, k, dual, add, in_l2, N_SMS, out)
             p = dict(zip(FEW_FIELDS + ("ss_parts",), out))
             at = (m, n, k, dual, add, p)
             if not in_l2 and p["stages"] == 0:
                 continue                                            # left to proj_tc.cu
-            taken += 1
+            assert taken[i] == m - 1, at
+            taken[i] = m
             assert p["nt"] % 8 == 0 and p["nt"] - 8 < m <= p["nt"], at
             assert p["tiles"] == -(-n // (32 if dual else 64)) and p["kb_total"] == k // 64, at
             # where the sums are kept apart: whole slices of the other kernel's plan, and for an ADD its ranks of 16 rows
             wide = _proj(plans, m, n, k, dual)["splits"]
             assert (p["parts"] == 0 if in_l2 else p["parts"] * p["splits"] == wide) and (in_l2 or not add or wide == 8), at
             n_acc = max(1, p["parts"] * (1 if dual else 2))
-            # the kernels that exist: gate/up unsplit, QKV in one or two slices, the others in one or four; rings have stages of two or four
+            # the kernels that exist, (slices, k-blocks a stage, ring, sums apart): gate/up unsplit, QKV split unless its sums are kept
+            # apart, an output or down projection split or of less than eight k-blocks
+            kernel = p["splits"], p["group"], bool(p["ring"]), p["parts"] > 0
+            own = [(4, True, False), (4, False, False), (5, False, False), (7, False, False)]
+            assert kernel[1:] in own + [(2, True, True)], at
             assert p["splits"] in ((1,) if dual else (1, 4) if add else (1, 2)) and p["splits"] <= p["kb_total"], at
+            assert dual or p["splits"] > 1 or (kernel[1:] in own[1:] if add else p["parts"] > 0), at
             per_cta = -(-p["kb_total"] // p["splits"])
             groups = -(-per_cta // p["group"])
             assert p["group"] in (2, 4, 5, 7) and 1 <= p["stages"] <= min(12, groups) and p["ring"] == (not in_l2 or p["stages"] < groups), at
@@ -122,7 +134,7 @@ def test_few_token_plans_fit_the_hardware(plans, d, ff, in_l2):
             if not in_l2:                                           # all CTAs at once, with 1 KB each for the system and what is static
                 per_sm = 228 * 1024 // (p["smem_bytes"] + 2048) if p["smem_bytes"] <= 112 * 1024 else 1
                 assert p["tiles"] * p["splits"] <= per_sm * N_SMS * (33 / 37 if p["splits"] == 4 else 1), at
-    assert taken == 4 * 96 if in_l2 else taken > 0 or d > 8000
+    assert taken == ([96] * 4 if in_l2 else TAKEN[d, ff])
 
 
 def test_passes_over_weights_that_exceed_l2(plans):
