@@ -32,8 +32,8 @@ from vvs_synth.configs import CONFIGS, DTYPE_FP32, MODE_RELAXED  # noqa: E402
 # ncu capture summarised under profiles/.  Keyed by (workload, fixed-order sums); each entry names the
 # kernel sources the step runs and the first 16 hex digits of the SHA-256 over their concatenation when
 # the counters were taken: the line reports null, and says why, once any of them has changed.
-STEP_SOURCES = ("proj_tc.cu", "attention_block.cu", "gemm_tc.cu", "lmhead_few.cu", "lmhead_pair.cu", "kernels_generic.cu",
-                "kernels_decide.cu", "launch_plans.h", "tc_common.cuh", "att_mma.cuh")
+STEP_SOURCES = ("vvs_api.cu", "launch_plans.h", "proj_few.cu", "proj_tc.cu", "attention_block.cu", "gemm_tc.cu", "lmhead_few.cu",
+                "lmhead_pair.cu", "kernels_generic.cu", "kernels_decide.cu", "kernels_fcache.cu", "tc_common.cuh", "att_mma.cuh")
 NCU_CAPTURES = {       # (both settings of deterministic run the same kernels here)
     (1, False): ("f8515c40e0eb62c2", 1.588e+09, "profiles/folded_step_launches.txt"),
     (1, True): ("f8515c40e0eb62c2", 1.588e+09, "profiles/folded_step_launches.txt"),
