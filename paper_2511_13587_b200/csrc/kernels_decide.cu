@@ -411,7 +411,8 @@ void launch_sample(const Workspace& ws, const DecideParams& p, cudaStream_t s) {
 // itself (a few dozen gathered values: cheaper than an exchange), then sums its contiguous part of the codebook, warp
 // by warp in index order; the part sums are read through distributed shared memory and the one warp whose part
 // holds the sample point walks it.  Replaces finalize / gather / accept / select / residual / sample, six launches
-// of 3-7 us each on a few hundred kilobytes: the work is a chain of four dependent round trips to L2.  What does not depend
+// of 3-7 us each on a few hundred kilobytes: the work is a chain of four dependent round trips to L2 (drafts; their values;
+// the masses of a row; the range of the sample point), of six with neighbour lists (their places; their columns).  What does not depend
 // on the statistics is requested before them, and the partials of a row come in one trip; sixteen warps take the rows
 // and drafts of a usual block in one turn (16 images 8.4 -> 7.6 us, behind the LM head of one image 15.3 -> 14.1 us).
 namespace {

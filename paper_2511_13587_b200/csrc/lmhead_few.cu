@@ -4,8 +4,8 @@
 //
 // What bounds it: the stream of codebook rows, if nothing else gets in its way.  Two warps issue, every other k-block each with
 // an accumulator of its own (one issuing lane in a branch of its own reached a k-block every ~600 cycles, which is slower than
-// the stream fills a stage; issued by converged warps 14.4 -> 14.0 us a call of one image and 16384 codes); nor is the loading lane alone:
-// with its ring's 600 cycles a k-block d 4096, 4096 or 8192 codes took 27 to 28 us a call of one image, decision included, 20 as a converged warp
+// the stream fills a stage; issuing by converged warps moved a call of one image and 16384 codes no further than its runs
+// differ); nor is the loading lane alone: with its ring's 600 cycles a k-block d 4096, 4096 or 8192 codes took 27 to 28 us a call of one image, decision included, 20 as a converged warp
 // (d 2048, 9472 codes 19.9 -> 17.8; d 1280, 8192 codes 16.1 -> 14.8); the pipeline is as deep as shared memory allows and its weights are
 // requested before griddepcontrol.wait.  Up to one tile per SM a CTA takes the whole SM's shared memory; with more, two
 // CTAs share an SM so that one's epilogue runs under the other's stream.  With one issuer and a thread per decision row
