@@ -157,6 +157,17 @@ struct ProjFewPlan {
 // partial sums of squares per token an ADD projection writes: one per tile and slice, rounded up to whole float4
 inline int proj_ss_parts(const ProjFewPlan& pl) { return (pl.tiles * pl.splits + 3) & ~3; }
 
+// A CTA's part of a later projection's weights, which it requests into L2 in pieces of 4 KB: where it begins (CTA x every) and how
+// much of it is requested.  An SM requests some 160 KB a microsecond, and the kernel behind waits for it: where a gate/up of narrow
+// d_ff has few CTAs for a whole QKV matrix, most of that matrix is left to its own kernel.  18 layers, everything / at most 256 KB a
+// CTA (64 to 512 KB are alike): d_model 2304, d_ff 64, 18 tokens 2282 / 483 us; 2048, 512, 18 tokens 512 / 429, 54 tokens 649 / 554;
+// 2048, 832, 54 tokens 618 / 569; XL shape (at most 147 KB a CTA) 362 / 361.
+struct AheadShare { uint32_t every, bytes; };
+inline AheadShare ahead_share(uint32_t bytes, uint32_t n_cta) {
+  const uint32_t every = ((bytes + n_cta - 1) / n_cta + 4095u) & ~4095u, most = 256u << 10;
+  return {every, every < most ? every : most};
+}
+
 // One pass of at most kFewTok tokens, k a multiple of 64; no stages: proj_tc.cu has to take it.  K slices: proj_few.cu has the
 // measurements; fewer than eight k-blocks are not worth an exchange.
 // in_l2: the model's weights are requested into L2 ahead and a CTA takes as much shared memory as its K range fills.

@@ -44,7 +44,7 @@ struct Params {
   __nv_bfloat16* q; __nv_bfloat16* kv_k; __nv_bfloat16* kv_v; const int32_t* slot_pos;               // QKV
   const float* rope_cos; const float* rope_sin; int n_heads, hd, s_max, layer, kv_rows, t_len;
   __nv_bfloat16* act; int ff, up_first;                                                            // GATEUP
-  const uint8_t* ahead[2]; uint32_t ahead_bytes;      // weights of the projection after next, to be brought into L2
+  const uint8_t* ahead[2]; uint32_t ahead_bytes; AheadShare share;      // weights of the projection after next, to be brought into L2
 };
 
 // LOG_S: log2 of the slices of K; G: k-blocks per stage; RING: stages are filled again.  APART: every partial sum that proj_tc.cu's plan
@@ -167,12 +167,11 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
   if (warp >= 2) prepare(eid);
   if (warp == 2 && p.ahead_bytes > 0) {
     // This CTA's share of a later projection's weights, HBM -> L2 (proj_tc.cu has the measurements)
-    const uint32_t n_cta = gridDim.x * gridDim.y, cta = blockIdx.y * gridDim.x + blockIdx.x;
-    const uint32_t share = ((p.ahead_bytes + n_cta - 1) / n_cta + 4095u) & ~4095u, end = min((cta + 1) * share, p.ahead_bytes);
+    const uint32_t begin = (blockIdx.y * gridDim.x + blockIdx.x) * p.share.every, end = min(begin + p.share.bytes, p.ahead_bytes);
 #pragma unroll
     for (int i = 0; i < 2; ++i)
       if (p.ahead[i])
-        for (uint32_t at = cta * share + lane * 4096u; at < end; at += 32 * 4096u) prefetch_l2(p.ahead[i] + at, min(4096u, end - at));
+        for (uint32_t at = begin + lane * 4096u; at < end; at += 32 * 4096u) prefetch_l2(p.ahead[i] + at, min(4096u, end - at));
   }
   if (warp == 0) {
     // ---- TMA producer: activations, then what the ring had no room for ---------------------------
@@ -501,6 +500,7 @@ int launch_proj_few(int epi, const ProjFewPlan& pl, const ProjArgs& g, cudaStrea
   kp.kv_rows = g.kv_rows; kp.t_len = g.t_len; kp.act = g.act; kp.ff = g.ff; kp.up_first = g.up_first ? 1 : 0;
   kp.ahead[0] = static_cast<const uint8_t*>(g.ahead[0]); kp.ahead[1] = static_cast<const uint8_t*>(g.ahead[1]);
   kp.ahead_bytes = g.ahead[0] ? g.ahead_bytes : 0;
+  kp.share = ahead_share(kp.ahead_bytes, (uint32_t)(pl.tiles * pl.splits));
   cudaError_t e;
   switch (epi) {
     case PROJ_QKV: e = pl.splits == 2 ? launch_epi<PROJ_QKV, 1>(pl, kp, g, s) : launch_epi<PROJ_QKV, 0>(pl, kp, g, s); break;

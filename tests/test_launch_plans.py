@@ -25,6 +25,11 @@ extern "C" void few(int m, int n, int k, int dual, int add, int in_l2, int n_sms
   const int v[] = {%s, vvs::proj_ss_parts(p)};
   for (unsigned i = 0; i < sizeof(v) / sizeof(v[0]); ++i) o[i] = v[i];
 }
+extern "C" void ahead(unsigned bytes, unsigned n_cta, unsigned* o) {
+  const vvs::AheadShare s = vvs::ahead_share(bytes, n_cta);
+  o[0] = s.every;
+  o[1] = s.bytes;
+}
 extern "C" int tree_parts(int vocab, int n_images, int n_sms) { return vvs::tree_walk_parts(vocab, n_images, n_sms); }
 extern "C" int att_split(int hd, int items, int s_max, int n_sms) { return vvs::attention_split(hd, items, s_max, n_sms); }
 """ % (", ".join("p." + f for f in FIELDS), ", ".join("p." + f for f in FEW_FIELDS))
@@ -135,6 +140,17 @@ def test_few_token_plans_fit_the_hardware(plans, d, ff, in_l2):
                 per_sm = 228 * 1024 // (p["smem_bytes"] + 2048) if p["smem_bytes"] <= 112 * 1024 else 1
                 assert p["tiles"] * p["splits"] <= per_sm * N_SMS * (33 / 37 if p["splits"] == 4 else 1), at
     assert taken == ([96] * 4 if in_l2 else TAKEN[d, ff])
+
+
+def test_requests_into_l2_are_shared_out(plans):
+    """Whole requests, all of the weights where there are CTAs enough, and no CTA kept at it for long."""
+    for n_cta in (1, 2, 26, 27, 80, 108, 128, 132, 192):
+        for n_bytes in (0, 16, 4096, 4112, 128 * 1024, 3276800, 9830400, 17694720, 31850496):
+            out = (ctypes.c_uint * 2)()
+            plans.ahead(n_bytes, n_cta, out)
+            every, part = out
+            assert every % 4096 == 0 and n_bytes <= every * n_cta < n_bytes + n_cta * 4096, (n_cta, n_bytes)
+            assert part == min(every, 256 << 10), (n_cta, n_bytes)
 
 
 def test_passes_over_weights_that_exceed_l2(plans):
