@@ -170,7 +170,10 @@ inline AheadShare ahead_share(uint32_t bytes, uint32_t n_cta) {
 
 // One pass of at most kFewTok tokens, k a multiple of 64; no stages: proj_tc.cu has to take it.  K slices: proj_few.cu has the
 // measurements; fewer than eight k-blocks are not worth an exchange.
-// in_l2: the model's weights are requested into L2 ahead and a CTA takes as much shared memory as its K range fills.
+// in_l2: the model's weights are requested into L2 ahead and a CTA takes as much shared memory as its K range fills.  All CTAs have to
+// fit at once here too: a second wave of a few repeats load, MMAs and epilogue in the open.  18 layers, two waves / proj_tc.cu for that
+// projection, 18 and 90 tokens: d_model 1024, d_ff 5120 (gate/up 160 CTAs) 414 / 406 and 632 / 573 us; 1600, 2048 (QKV 150) 432 / 428
+// and 660 / 586; 1792, 1664 (QKV 168) 445 / 422 and 691 / 607 (around 54 tokens gate/up loses 2 %: 1088, 5120 554 / 564).
 // Weights that come from HBM need all CTAs on the device at once, and those of the next projection beside them as they leave: one,
 // two or three CTAs per SM, as many as it takes, rings of stages of two k-blocks.  And such models are large and deep: any other order
 // of the sums moves their features by 2.4e-3 (24 layers of d_model 2048) to 5.7e-3 (7B shape) and guided probabilities by more than
@@ -230,6 +233,10 @@ inline ProjFewPlan plan_proj_few(int m, int n, int k, bool dual, bool add, bool 
   // 32 columns' share
   const int share = (int)((228u * 1024u * (unsigned)pl.tmem_cols + 511u) / 512u) - 2048;
   if (pl.smem_bytes < share) pl.smem_bytes = share;
+  if (in_l2) {
+    const int fit = pl.smem_bytes > 112 * 1024 ? 1 : 228 * 1024 / (pl.smem_bytes + 2048), per_sm = fit < 3 ? fit : 3;
+    if (pl.tiles * pl.splits > per_sm * (pl.splits == 4 ? n_sms * 33 / 37 : n_sms)) return ProjFewPlan{};
+  }
   return pl.smem_bytes <= most ? pl : ProjFewPlan{};
 }
 

@@ -17,7 +17,10 @@ FEW64 = replace(XL, name="few64", n_layers=2, d_model=1024, n_heads=16, d_ff=275
 # heads of two tiles; 18 tiles: sums of squares in rows of 18 and 72 parts; a down projection of 5 k-blocks, unsplit
 FEW128 = replace(B7, name="few128", n_layers=2, d_model=1152, n_heads=9, d_ff=320, vocab=1096, vocab_offset=64, lm_rows=2048,
                  tok_rows=0, s_max=700)
-# gate/up of six CTAs, which request a part of the next QKV matrix only
+# CTAs that would not all fit at once: QKV (150) and gate/up (160) go to proj_tc.cu, the others stay; gate/up of six CTAs, which request
+# a part of the next QKV matrix only
+WAVES_QKV = replace(FEW64, name="waves_qkv", d_model=1600, n_heads=25, d_ff=2048)
+WAVES_GU = replace(FEW64, name="waves_gu", d_ff=5120)
 NARROW = replace(FEW64, name="narrow", d_ff=192)
 # weights that do not stay in L2: rings of two k-blocks, one CTA per SM; 47 k-blocks in four slices
 STREAM1 = replace(XL, name="stream1", n_layers=1, d_model=1536, n_heads=24, d_ff=3008, vocab=1096, lm_rows=0, tok_rows=0, s_max=208)
@@ -42,6 +45,9 @@ STREAM3 = replace(B7, name="stream3", n_layers=1, d_model=2048, n_heads=16, d_ff
     (FEW128, 1, 2, 1, 8, [513]),                           # 18
     (FEW128, 3, 2, 1, 4, [5, 160, 677]),                   # 30
     (FEW128, 4, 1, 3, 20, [5, 160, 333, 64]),              # 92
+    (WAVES_QKV, 1, 2, 1, 8, [199]),
+    (WAVES_GU, 1, 2, 1, 8, [199]),
+    (WAVES_GU, 3, 2, 1, 15, [0, 47, 150]),                 # 96
     (NARROW, 1, 2, 1, 8, [77]),
     (STREAM1, 1, 1, 1, 0, [0]),
     (STREAM1, 1, 2, 1, 8, [199]),

@@ -85,15 +85,17 @@ def test_projection_plans_fit_the_hardware(plans, d, ff):
             assert p["threads"] in (256, 512) and p["threads"] % (128 // p["splits"]) == 0, at
             assert p["ss_parts"] % 4 == 0 and p["ss_parts"] <= p["tiles"] * 8, at
 
-# Weights from HBM: up to how many tokens each projection is taken (QKV, output, gate/up, down projection).  None where more than
-# three CTAs per SM would be needed (d_model 8192), matrices beyond 64 MB at most 80, otherwise what the ranks of plan_proj allow.
-TAKEN = {(1536, 3008): [96, 83, 96, 80], (1536, 4096): [96, 83, 96, 83], (2048, 5504): [64, 0, 96, 96], (3072, 8192): [32, 0, 80, 64],
+# Up to how many tokens each projection is taken (QKV, output, gate/up, down projection): those whose CTAs fit at once.  Weights from
+# HBM: none where more than three CTAs per SM would be needed (d_model 8192), matrices beyond 64 MB at most 80, otherwise what the
+# ranks of plan_proj allow.
+TAKEN = {(1024, 5120): [96, 96, 0, 96], (1600, 2048): [0, 96, 96, 96], (2048, 832): [0, 96, 96, 96], (2048, 128): [0, 96, 96, 96],
+         (1536, 3008): [96, 83, 96, 80], (1536, 4096): [96, 83, 96, 83], (2048, 5504): [64, 0, 96, 96], (3072, 8192): [32, 0, 80, 64],
          (4096, 11008): [52, 32, 80, 0], (5120, 13824): [80, 0, 80, 0], (8192, 28672): [0, 0, 0, 0], (1024, 65536): [64, 42, 0, 80],
          (16384, 64): [0, 0, 64, 0]}
 
 
-@pytest.mark.parametrize("d,ff,in_l2", [(1024, 320, 1), (1024, 2752, 1), (1152, 3072, 1), (1280, 3456, 1), (1280, 64, 1), (2048, 128, 1),
-                                        (1536, 3008, 0), (1536, 4096, 0), (2048, 5504, 0), (3072, 8192, 0), (4096, 11008, 0),
+@pytest.mark.parametrize("d,ff,in_l2", [(1024, 320, 1), (1024, 2752, 1), (1024, 5120, 1), (1600, 2048, 1), (2048, 832, 1),
+                                        (1152, 3072, 1), (1280, 3456, 1), (1280, 64, 1), (2048, 128, 1), (1536, 3008, 0), (1536, 4096, 0), (2048, 5504, 0), (3072, 8192, 0), (4096, 11008, 0),
                                         (5120, 13824, 0), (8192, 28672, 0), (1024, 65536, 0), (16384, 64, 0)])
 def test_few_token_plans_fit_the_hardware(plans, d, ff, in_l2):
     taken = [0, 0, 0, 0]                                            # calls of up to so many tokens: QKV, output, gate/up, down projection
@@ -103,7 +105,7 @@ def test_few_token_plans_fit_the_hardware(plans, d, ff, in_l2):
             plans.few(m, n, k, dual, add, in_l2, N_SMS, out)
             p = dict(zip(FEW_FIELDS + ("ss_parts",), out))
             at = (m, n, k, dual, add, p)
-            if not in_l2 and p["stages"] == 0:
+            if p["stages"] == 0:
                 continue                                            # left to proj_tc.cu
             assert taken[i] == m - 1, at
             taken[i] = m
@@ -136,10 +138,10 @@ def test_few_token_plans_fit_the_hardware(plans, d, ff, in_l2):
             # the sums of squares: whole float4, room for d / 16 of them per token
             assert p["ss_parts"] % 4 == 0 and p["tiles"] * p["splits"] <= p["ss_parts"] < p["tiles"] * p["splits"] + 4, at
             assert not add or p["ss_parts"] <= (d + 127) // 128 * 8, at
-            if not in_l2:                                           # all CTAs at once, with 1 KB each for the system and what is static
-                per_sm = 228 * 1024 // (p["smem_bytes"] + 2048) if p["smem_bytes"] <= 112 * 1024 else 1
-                assert p["tiles"] * p["splits"] <= per_sm * N_SMS * (33 / 37 if p["splits"] == 4 else 1), at
-    assert taken == ([96] * 4 if in_l2 else TAKEN[d, ff])
+            # all CTAs at once, with 1 KB each for the system and what is static
+            per_sm = 228 * 1024 // (p["smem_bytes"] + 2048) if p["smem_bytes"] <= 112 * 1024 else 1
+            assert p["tiles"] * p["splits"] <= min(per_sm, 3) * N_SMS * (33 / 37 if p["splits"] == 4 else 1), at
+    assert taken == TAKEN.get((d, ff), [96] * 4)
 
 
 def test_requests_into_l2_are_shared_out(plans):
