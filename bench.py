@@ -34,11 +34,11 @@ from vvs_synth.configs import CONFIGS, DTYPE_FP32, MODE_RELAXED  # noqa: E402
 # the counters were taken: the line reports null, and says why, once any of them has changed.
 STEP_SOURCES = ("vvs_api.cu", "launch_plans.h", "proj_few.cu", "proj_tc.cu", "attention_block.cu", "gemm_tc.cu", "lmhead_few.cu",
                 "lmhead_pair.cu", "kernels_generic.cu", "kernels_decide.cu", "kernels_fcache.cu", "tc_common.cuh", "att_mma.cuh")
-NCU_CAPTURES = {       # (both settings of deterministic run the same kernels here)
-    (1, False): ("f8515c40e0eb62c2", 1.588e+09, "profiles/folded_step_launches.txt"),
-    (1, True): ("f8515c40e0eb62c2", 1.588e+09, "profiles/folded_step_launches.txt"),
-    (2, False): ("f8515c40e0eb62c2", 3.788e+09, "profiles/folded_step_launches.txt"),
-    (2, True): ("f8515c40e0eb62c2", 3.788e+09, "profiles/folded_step_launches.txt"),
+NCU_CAPTURES = {       # (both settings of deterministic run the same kernels here; mean of the first two trials)
+    (1, False): ("c2f6f0ecc97ffd24", 1.518e+09, "profiles/folded_step_launches.txt"),
+    (1, True): ("c2f6f0ecc97ffd24", 1.518e+09, "profiles/folded_step_launches.txt"),
+    (2, False): ("c2f6f0ecc97ffd24", 3.622e+09, "profiles/folded_step_launches.txt"),
+    (2, True): ("c2f6f0ecc97ffd24", 3.622e+09, "profiles/folded_step_launches.txt"),
 }
 N_TRIALS = 32           # distinct (fill, block, draft) inputs cycled through the steps
 DRAFT_LOGIT_STD = 1.0   # target-independent drafter: q = softmax(N(0, std^2))
