@@ -8,13 +8,16 @@
 //   exchanges partial sums, each pushing 64 rows in the place of 128: a CTA pushes some 32 bytes a cycle into its cluster).
 // - A stage is several k-blocks, loaded by one request and waited for once.  Gate and up are one tensor of two matrices at the distance of
 //   their addresses: as two requests per k-block they took a late CTA 1 us (18 tokens 704 -> 697 us, a tree of 54 868 -> 862).
-// - All stages' weights are requested before tensor memory and the CTA's barrier, then whatever the epilogue needs besides
+// - All stages' weights are requested before tensor memory and the CTA's barrier, the activations as soon as the kernel before has ended, by
+//   a warp that waits for neither, then whatever the epilogue needs besides
 //   the sums (rows, places in the cache, rotation) is found, all before griddepcontrol.wait.
 //   QKV, ADD  64 rows of one matrix;  GATEUP  32 rows of gate, then the same 32 of up, in the order of their addresses
 // (All figures here: the XL shape and models like it, whose weights stay in L2.)
 // An accumulator of M = 64 lies in lanes 0-15 of the four lane quarters; its rows go to shared memory as [token quad][rank][row]
 // float4 (split: with st.async to the rank that owns the row, counted on its mbarrier), and the epilogue takes a pair of rows and
-// two tokens per thread (four where 64 rows are finished at once), partial sums in rank order.
+// two tokens per thread (four where 64 rows are finished at once, one of an output or down projection of up to 32), partial sums in rank order.
+// (18 layers, 8, 18 and 28 tokens: activations requested by a warp that waits for nothing else 340.4 -> 338.8, 359.1 -> 357.1, 381.7 -> 380.0 us;
+// one token a thread 334.6, 357.1, 380.7.)
 //
 // Step of the XL shape against 128-row tiles: 18 tokens 876 -> 709 us, 28 tokens 920 -> 766, 54 tokens (a tree) 1061 -> 881; 18
 // layers of it, 72 tokens 615 -> 538, 90 tokens 657 -> 585, 108 tokens 635 -> 641; of d_model 1024, 72 tokens 515 -> 473, 90
@@ -35,7 +38,7 @@ constexpr uint32_t kRows = 64;
 constexpr uint32_t kABytes = kRows * kBlockK * 2;
 
 struct Params {
-  int m, n, nt, kb_total, stages, parts, log_slices;      // parts: slices of proj_tc.cu's plan per CTA, log2 of all of them, columns
+  int m, n, nt, kb_total, stages, group, parts, log_slices;      // parts: slices of proj_tc.cu's plan per CTA, log2 of all of them, columns
   int acc_ld;                                          // from one accumulator to the next (APART)
   uint32_t tmem_cols, recv_off;
   int32_t* status;
@@ -47,13 +50,16 @@ struct Params {
   const uint8_t* ahead[2]; uint32_t ahead_bytes; AheadShare share;      // weights of the projection after next, to be brought into L2
 };
 
-// LOG_S: log2 of the slices of K; G: k-blocks per stage; RING: stages are filled again.  APART: every partial sum that proj_tc.cu's plan
+// LOG_S: log2 of the slices of K; GROUP: k-blocks per stage (0: the plan's); RING: stages are filled again; TPI: tokens per item of the
+// epilogue.  APART: every partial sum that proj_tc.cu's plan
 // would take has an accumulator of its own (each of its slices; of a single matrix every other k-block), they are added in that
 // kernel's order, and an ADD's sums of squares cover its rows in its order: the same bits, whichever of the two kernels runs.
 // The issuing warp is alone in its loop, where every wait, vote and branch shows: 80 MMAs of 64 x 24 x 16 take 27.8 cycles each with
-// ten k-blocks per wait, 31 with four, 47 with one, and 41 with four where a ring's bookkeeping and a test for a partial
-// stage are in the loop.
-template <int EPI, int LOG_S, int G, bool RING, bool APART>
+// ten k-blocks per wait, 31 with four, 47 with one, and 41 with four where a ring's bookkeeping is in the loop.  The loop over a stage's
+// k-blocks is rolled all the same where all stages are there at once: a layer executes its code once, every line of which has to be
+// fetched, and so the output and the down projection are the same code whatever their stages (18 layers of the XL shape 349.1 -> 341.3
+// us, with the loop of qkv_attention_few.cu; only the down projection's stages as long as the output projection's: 343.3).
+template <int EPI, int LOG_S, int GROUP, bool RING, bool APART, int TPI>
 __global__ void __launch_bounds__(kThreads)
 proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b) {
   constexpr bool DUAL = EPI == PROJ_GATEUP;
@@ -62,7 +68,6 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
   constexpr int S = 1 << LOG_S;
   const int parts = APART ? p.parts : 1;
   const uint32_t acc_ld = (uint32_t)p.acc_ld;
-  constexpr int TPI = DUAL || SPLIT ? 2 : 4;           // tokens per item of the epilogue
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[kFewStages];
   __shared__ __align__(8) uint64_t empty_bar[kFewStages];
@@ -72,6 +77,7 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
   __shared__ volatile int s_abort;
   __shared__ float s_rs[EPI == PROJ_ADD ? 1 : kFewTok];            // 1/rms of the tokens
 
+  const int G = GROUP > 0 ? GROUP : p.group;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int tile = (int)blockIdx.x, rank = SPLIT ? (int)blockIdx.y : 0;
@@ -115,19 +121,32 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
     tmem_alloc(&tmem_slot, p.tmem_cols);
     tmem_relinquish();
   }
-  tc_fence_before();
-  __syncthreads();
+  auto load_act = [&](int i, uint32_t stage) {
+    if (elect_one()) tma_load_3d(smem + (size_t)stage * stage_bytes + G * kABytes, &tm_b, &full_bar[stage], 0, 0, kb0 + i * G);
+  };
+  // The warp that requests does not wait for tensor memory: in a CTA that could only start when the kernel before it had ended, the
+  // activations are requested 0.4 us sooner.
+  if (warp == 0) {
+    named_bar_arrive(1, kThreads);
+    pdl_wait();
+    for (int i = 0; i < n_pre; ++i) load_act(i, i);
+    named_bar_sync(2, kThreads);
+  } else {
+    tc_fence_before();
+    named_bar_sync(1, kThreads);
+    pdl_launch_dependents();  // after this CTA holds its TMEM: a dependent grid cannot take it first
+    named_bar_arrive(2, kThreads);
+  }
   tc_fence_after();
   const uint32_t tmem_base = tmem_slot;
-  pdl_launch_dependents();  // after this CTA holds its TMEM: a dependent grid cannot take it first
   if (SPLIT) cluster_arrive_relaxed();      // this rank's barrier is ready for its peers' pushes (fence_barrier_init above)
 
   // ---- this thread's first item of the epilogue: a pair of rows and TPI tokens, the last warps first (the first ones have other
   // work).  What does not depend on the kernel before is found here, under its tail; nothing waits for a load here.
   constexpr int rpr = (int)kRows >> LOG_S, log_np = (DUAL ? 4 : 5) - LOG_S;     // rows of a rank, log2 of the pairs it finishes
   const int eid = (kThreads / 32 - 1 - warp) * 32 + lane;
-  const int pair = (TPI == 2 ? eid >> 1 : eid) & ((1 << log_np) - 1), sub = TPI == 2 ? (eid & 1) * 2 : 0;
-  constexpr int log_sub = TPI == 2 ? 1 : 0;
+  constexpr int log_sub = TPI == 1 ? 2 : TPI == 2 ? 1 : 0;
+  const int pair = (eid >> log_sub) & ((1 << log_np) - 1), sub = (eid & ((1 << log_sub) - 1)) * TPI;
   const int items = nq << (log_np + log_sub);
   const int row0 = DUAL ? tile * 32 : tile * (int)kRows + rank * rpr;       // first output row of this rank
   const int n = row0 + 2 * pair;
@@ -174,12 +193,6 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
         for (uint32_t at = begin + lane * 4096u; at < end; at += 32 * 4096u) prefetch_l2(p.ahead[i] + at, min(4096u, end - at));
   }
   if (warp == 0) {
-    // ---- TMA producer: activations, then what the ring had no room for ---------------------------
-    auto load_act = [&](int i, uint32_t stage) {
-      if (elect_one()) tma_load_3d(smem + (size_t)stage * stage_bytes + G * kABytes, &tm_b, &full_bar[stage], 0, 0, kb0 + i * G);
-    };
-    pdl_wait();
-    for (int i = 0; i < n_pre; ++i) load_act(i, i);
     if constexpr (RING) {
       uint32_t stage = 0, par = 0;                  // stage of group i, parity of its previous release
       for (int i = n_pre; i < ng; ++i) {
@@ -205,15 +218,8 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
       }
       tc_fence_after();
     };
-    auto whole = [&](uint32_t a_lo, int i) {
-#pragma unroll
-      for (int j = 0; j < G; ++j)
-        mma_bf16_k64(tmem_base, a_lo + j * (kABytes >> 4), a_lo + G * (kABytes >> 4) + j * b_lo, idesc, j > 0 ? 1u : (uint32_t)i);
-    };
-    auto part = [&](uint32_t a_lo, int i) {
-#pragma unroll 1
-      for (int j = 0; j < nkb - i * G; ++j)
-        mma_bf16_k64(tmem_base, a_lo + j * (kABytes >> 4), a_lo + G * (kABytes >> 4) + j * b_lo, idesc, (uint32_t)(i + j));
+    auto block = [&](uint32_t a_lo, int j, uint32_t add) {
+      mma_bf16_k64(tmem_base, a_lo + j * (kABytes >> 4), a_lo + G * (kABytes >> 4) + j * b_lo, idesc, add);
     };
     pdl_wait();
     if constexpr (APART) {
@@ -244,20 +250,23 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
       for (int i = 0; i < ng; ++i) {
         wait_full(stage, par);
         const uint32_t a_lo = lo0 + stage * stage_lo;
-        if (nkb - i * G >= G) whole(a_lo, i);
-        else part(a_lo, i);
+        if (nkb - i * G >= G) {
+#pragma unroll
+          for (int j = 0; j < G; ++j) block(a_lo, j, j > 0 ? 1u : (uint32_t)i);
+        } else {
+#pragma unroll 1
+          for (int j = 0; j < nkb - i * G; ++j) block(a_lo, j, (uint32_t)(i + j));
+        }
         if (i + p.stages < ng) mma_commit_elect(&empty_bar[stage]);  // a group is still to come into this stage
         if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1; }
       }
     } else {
-      const int n_whole = nkb / G;
-      for (int i = 0; i < n_whole; ++i) {
+      for (int i = 0; i < ng; ++i) {
         wait_full(i, 0);
-        whole(lo0 + i * stage_lo, i);
-      }
-      if (n_whole < ng) {
-        wait_full(n_whole, 0);
-        part(lo0 + n_whole * stage_lo, n_whole);
+        const uint32_t a_lo = lo0 + i * stage_lo;
+        const int n = min(G, nkb - i * G);
+#pragma unroll 1
+        for (int j = 0; j < n; ++j) block(a_lo, j, (uint32_t)(i + j));
       }
     }
     mma_commit_elect(&acc_bar);
@@ -394,7 +403,7 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
         const int j = warp_sums_index<4>(lane);
         if ((lane & 7) == 0 && t0 + j < p.m) ss[(size_t)(t0 + j) * p.ss_out_parts] = sq[0];
       } else {
-        for (int o = 1 << log_np; o > 1; o >>= 1)
+        for (int o = 1 << (log_np + log_sub - 1); o >= 1 << log_sub; o >>= 1)
 #pragma unroll
           for (int j = 0; j < TPI; ++j) {
             sq[j] += __shfl_xor_sync(0xffffffffu, sq[j], o);
@@ -440,9 +449,13 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
   }
 }
 
-template <int EPI, int LOG_S, int G, bool RING, bool APART = false>
+template <int EPI, int LOG_S, int GROUP, bool RING, bool APART = false>
 cudaError_t launch_one(const ProjFewPlan& pl, const Params& kp, const ProjArgs& g, cudaStream_t s) {
-  auto* fn = proj_few_kernel<EPI, LOG_S, G, RING, APART>;
+  constexpr int kTpi = EPI == PROJ_GATEUP || LOG_S > 0 ? 2 : 4;
+  auto* fn = proj_few_kernel<EPI, LOG_S, GROUP, RING, APART, kTpi>;
+  if constexpr (EPI == PROJ_ADD && LOG_S > 0)          // up to 32 tokens every thread has one token's item at most
+    if (kp.m <= 32) fn = proj_few_kernel<EPI, LOG_S, GROUP, RING, APART, 1>;
+
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(fn), kFewSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -478,11 +491,7 @@ cudaError_t launch_epi(const ProjFewPlan& pl, const Params& kp, const ProjArgs& 
       if (pl.ring) return pl.group == 4 ? launch_one<EPI, LOG_S, 4, true>(pl, kp, g, s) : cudaErrorInvalidValue;
   }
   if (pl.parts > 0 || pl.ring) return cudaErrorInvalidValue;
-  if constexpr (EPI != PROJ_QKV || LOG_S > 0) {
-    if (pl.group == 4) return launch_one<EPI, LOG_S, 4, false>(pl, kp, g, s);
-    if (pl.group == 5) return launch_one<EPI, LOG_S, 5, false>(pl, kp, g, s);
-    if (pl.group == 7) return launch_one<EPI, LOG_S, 7, false>(pl, kp, g, s);
-  }
+  if constexpr (EPI != PROJ_QKV || LOG_S > 0) return launch_one<EPI, LOG_S, 0, false>(pl, kp, g, s);
   return cudaErrorInvalidValue;
 }
 
@@ -490,7 +499,7 @@ cudaError_t launch_epi(const ProjFewPlan& pl, const Params& kp, const ProjArgs& 
 
 int launch_proj_few(int epi, const ProjFewPlan& pl, const ProjArgs& g, cudaStream_t s) {
   Params kp{};
-  kp.m = g.m; kp.n = g.n; kp.nt = pl.nt; kp.kb_total = pl.kb_total; kp.stages = pl.stages; kp.parts = pl.parts; kp.acc_ld = pl.acc_ld;
+  kp.m = g.m; kp.n = g.n; kp.nt = pl.nt; kp.kb_total = pl.kb_total; kp.stages = pl.stages; kp.group = pl.group; kp.parts = pl.parts; kp.acc_ld = pl.acc_ld;
   while ((1 << kp.log_slices) < pl.parts * pl.splits) ++kp.log_slices;
   kp.tmem_cols = (uint32_t)pl.tmem_cols; kp.recv_off = (uint32_t)pl.recv_off; kp.status = g.status;
   kp.ss_in = g.ss_in; kp.ss_parts = g.ss_parts; kp.inv_d = 1.f / (float)g.d; kp.eps = g.eps;

@@ -99,6 +99,10 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
 __device__ __forceinline__ void named_bar_sync(int id, int n_threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n_threads) : "memory");
 }
+// One of them that does not wait there.
+__device__ __forceinline__ void named_bar_arrive(int id, int n_threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n_threads) : "memory");
+}
 // The same barrier, and whether all of its threads said yes: the same answer in each of them.  Threads that wait for something with a
 // limit and then meet at a barrier decide with this whether they go on: some may have given up where others have not.
 __device__ __forceinline__ bool named_bar_all(int id, int n_threads, bool yes) {
@@ -169,6 +173,7 @@ __device__ __forceinline__ void ld_shared_vec(const uint8_t* p, float (&v)[2]) {
   const float2 t = *reinterpret_cast<const float2*>(p);
   v[0] = t.x; v[1] = t.y;
 }
+__device__ __forceinline__ void ld_shared_vec(const uint8_t* p, float (&v)[1]) { v[0] = *reinterpret_cast<const float*>(p); }
 // HBM -> L2
 __device__ __forceinline__ void prefetch_l2(const void* ptr, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(ptr), "r"(bytes) : "memory");
