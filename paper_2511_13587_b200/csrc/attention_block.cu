@@ -51,96 +51,6 @@ struct Smem {
   static int bytes(int t_len, int s) { return kMain + kQ + (s - 1) * t_len * (HD + 2) * 4; }
 };
 
-// The 16 NS keys of a slice against the 16 query rows of an m-tile.  MASKED: bit k of vis[i] = key k is visible to row g + 8 i, of
-// vmem = row k of the V tile holds data (others are zeroed before they are multiplied).  Heads of 64 keep the running maximum
-// unscaled, so that scaling and subtraction are one FMA.  Heads of 128 scale, subtract and sum with a rounding each, the arithmetic
-// their results have always had: deep models of such heads (32 layers of d_model 4096) answer any other place of a rounding with
-// features 5.7e-3 away and guided probabilities 1.4e-2 to 4.8e-2, which is more than a caller may see move.
-template <int HD, int NS, bool MASKED>
-__device__ __forceinline__ void att_keys(AttState<HD>& st, const uint32_t (&qa)[HD / 16][4], uint32_t k_base, uint32_t v_base, int lane,
-                                         float sl2, const uint32_t (&vis)[2], uint32_t vmem) {
-  constexpr uint32_t kChunk = NS * 2048u;                     // 64 columns of all keys
-  const int c = lane & 3, mi = lane >> 3, ri = lane & 7;
-  constexpr bool kScaled = HD == 128;                         // the scores and the running maximum are scaled
-  float s[2 * NS][4];
-#pragma unroll
-  for (int n = 0; n < 2 * NS; ++n)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) s[n][e] = 0.f;
-#pragma unroll
-  for (int kk = 0; kk < HD / 16; ++kk) {
-    const int cc = 2 * kk + (mi & 1);
-    const uint32_t at = k_base + (cc >> 3) * kChunk + (((mi >> 1) << 3) + ri) * 128 + (((cc & 7) ^ ri) << 4);
-#pragma unroll
-    for (int n = 0; n < NS; ++n) {
-      uint32_t r0, r1, r2, r3;
-      ldsm4(at + n * 2048, r0, r1, r2, r3);
-      mma16816(s[2 * n], qa[kk][0], qa[kk][1], qa[kk][2], qa[kk][3], r0, r1);
-      mma16816(s[2 * n + 1], qa[kk][0], qa[kk][1], qa[kk][2], qa[kk][3], r2, r3);
-    }
-  }
-  // online softmax for rows g (i = 0) and g + 8 (i = 1); this lane holds keys 8 n + 2c, 8 n + 2c + 1
-  uint32_t pa[NS][4];
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    if (kScaled) {
-#pragma unroll
-      for (int n = 0; n < 2 * NS; ++n)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) s[n][2 * i + e] = __fmul_rn(s[n][2 * i + e], sl2);
-    }
-    if (MASKED) {
-      const uint32_t vb = vis[i] >> (2 * c);
-#pragma unroll
-      for (int n = 0; n < 2 * NS; ++n)
-#pragma unroll
-        for (int e = 0; e < 2; ++e)
-          if (!((vb >> (8 * n + e)) & 1u)) s[n][2 * i + e] = -CUDART_INF_F;
-    }
-    float mx = fmaxf(s[0][2 * i], s[0][2 * i + 1]);
-#pragma unroll
-    for (int n = 1; n < 2 * NS; ++n) mx = fmaxf(mx, fmaxf(s[n][2 * i], s[n][2 * i + 1]));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const float m_new = fmaxf(st.m[i], mx);
-    const float m_scaled = m_new == -CUDART_INF_F ? 0.f : kScaled ? m_new : m_new * sl2;
-    auto weight = [&](float x) { return ex2(kScaled ? __fsub_rn(x, m_scaled) : fmaf(x, sl2, -m_scaled)); };
-    const float alpha = weight(st.m[i]);
-    st.m[i] = m_new;
-    float sum = kScaled ? st.l[i] : 0.f;
-#pragma unroll
-    for (int n = 0; n < 2 * NS; ++n) {
-      const float p0 = weight(s[n][2 * i]), p1 = weight(s[n][2 * i + 1]);
-      sum = kScaled && n == 0 ? fmaf(sum, alpha, p0 + p1) : sum + (p0 + p1);
-      pa[n >> 1][i + 2 * (n & 1)] = pack2(p0, p1);
-    }
-    st.l[i] = kScaled ? sum : fmaf(st.l[i], alpha, sum);
-#pragma unroll
-    for (int j = 0; j < HD / 8; ++j) {
-      st.o[j][2 * i] *= alpha;
-      st.o[j][2 * i + 1] *= alpha;
-    }
-  }
-  // O += P V
-#pragma unroll
-  for (int n = 0; n < NS; ++n) {
-    const uint32_t vm = vmem >> (16 * n + 2 * c);
-    const uint32_t vlo = (vm & 1u ? 0x0000ffffu : 0u) | (vm & 2u ? 0xffff0000u : 0u);
-    const uint32_t vhi = (vm & 0x100u ? 0x0000ffffu : 0u) | (vm & 0x200u ? 0xffff0000u : 0u);
-#pragma unroll
-    for (int jj = 0; jj < HD / 16; ++jj) {
-      const int cc = 2 * jj + (mi >> 1);
-      uint32_t r0, r1, r2, r3;
-      ldsm4t(v_base + (cc >> 3) * kChunk + n * 2048 + (((mi & 1) << 3) + ri) * 128 + (((cc & 7) ^ ri) << 4), r0, r1, r2, r3);
-      if (MASKED) {
-        r0 &= vlo; r1 &= vhi; r2 &= vlo; r3 &= vhi;
-      }
-      mma16816(st.o[2 * jj], pa[n][0], pa[n][1], pa[n][2], pa[n][3], r0, r1);
-      mma16816(st.o[2 * jj + 1], pa[n][0], pa[n][1], pa[n][2], pa[n][3], r2, r3);
-    }
-  }
-}
-
 template <int HD, int NMT, int W, int D, int NS, bool MANY>
 __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockArgs a) {
   using L = Smem<HD, NMT, W, D, NS, MANY>;

@@ -255,6 +255,35 @@ inline int attention_split(int hd, long long items, int s_max, int n_sms) {
   return split;
 }
 
+// ---- QKV and attention of few tokens and few sequences, qkv_attention_few.cu ----------------------
+struct QkvAttentionPlan {
+  ProjFewPlan proj;
+  int per_item;                // CTAs of a cluster that share an item; 0: two kernels
+  int part_off, recv_off, new_off, smem_bytes;
+};
+
+// qkv: the projection's plan, in two slices with all k-blocks in shared memory (tiles of 64 rows: a head's q, k or v).  Heads of 64 whose
+// items have a CTA each in attention_block.cu; one to three sequences, since the sixteen warps' parts of an item need two CTAs; and all
+// clusters have to fit at once (of 148 SMs 22 take clusters of six: 132).
+inline QkvAttentionPlan plan_qkv_attention(const ProjFewPlan& qkv, int n_heads, int hd, int d, int n_rows, int t_len, int s_max, int n_sms) {
+  using namespace proj;
+  QkvAttentionPlan pl{};
+  pl.proj = qkv;
+  if (hd != 64 || n_heads * hd != d || n_rows > 3 || t_len > 32 || qkv.stages < 1 || qkv.splits != 2 || qkv.ring || qkv.parts > 0) return pl;
+  if (n_heads * 6 > n_sms * 33 / 37 || attention_split(hd, (long long)n_heads * n_rows, s_max, n_sms) > 1) return pl;
+  const int per_item = 6 / n_rows, slots = (16 + per_item - 1) / per_item, ld_t = t_len < 16 ? t_len : 16;
+  const int stages = qkv.stages * qkv.group * (64 * (int)kBlockK * 2 + qkv.nt * (int)kBlockK * 2), recv = (qkv.nt + 3) / 4 * 64 * 16;
+  // the keys and, in the CTA that folds, the parts lie over the stages
+  pl.part_off = slots * 8192;
+  const int attention = pl.part_off + 16 * ld_t * (100 + 2) * 4;
+  pl.recv_off = ((stages > attention ? stages : attention) + 1023) & ~1023;
+  pl.new_off = pl.recv_off + ((recv + 1023) & ~1023);
+  pl.smem_bytes = pl.new_off + 3 * t_len * 128 + 1024;
+  if (pl.smem_bytes < qkv.smem_bytes) pl.smem_bytes = qkv.smem_bytes;
+  if (pl.smem_bytes <= kFewSmem) pl.per_item = per_item;
+  return pl;
+}
+
 // ---- walk of a candidate tree, kernels_tree.cu ---------------------------------------------------
 // CTAs (a cluster) per image, each with a part of the codes: what a part saves on each residual has to outweigh the cluster's
 // barriers, also where most drafts are accepted and there are few residuals.  26 nodes, one image, most accepted / most

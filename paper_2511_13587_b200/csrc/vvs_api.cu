@@ -394,7 +394,7 @@ struct ProjPick {
   int launch(int epi, const ProjArgs& g, cudaStream_t s) const { return few ? launch_proj_few(epi, small, g, s) : launch_proj(epi, wide, g, s); }
 };
 
-// bf16 contexts of wide models: five kernels per layer (proj_tc.cu, attention_block.cu), each a programmatic dependent of
+// bf16 contexts of wide models: five kernels per layer (proj_tc.cu, attention_block.cu), or four (qkv_attention_few.cu), each a programmatic dependent of
 // the one before.  Every sum is taken in a fixed order, so a call repeats bit for bit.
 int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* o, cudaStream_t s) {
   using T = __nv_bfloat16;
@@ -411,8 +411,13 @@ int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_o
   const size_t layer_bytes = ((size_t)4 * d + (size_t)3 * ff) * d * sizeof(T);
   const bool prefetch = 3 * layer_bytes <= (size_t)ctx->l2_bytes;
   const bool whole = ff % 64 == 0;                  // (proj_few.cu takes whole k-blocks)
-  const ProjPick p_qkv(PROJ_QKV, M, 3 * d, d, prefetch, whole, ctx->n_sms), p_o(PROJ_ADD, M, d, d, prefetch, whole, ctx->n_sms);
+  const ProjPick p_qkv(PROJ_QKV, M, 3 * d, d, prefetch, whole, ctx->n_sms);
+  ProjPick p_o(PROJ_ADD, M, d, d, prefetch, whole, ctx->n_sms);
   const ProjPick p_gu(PROJ_GATEUP, M, ff, d, prefetch, whole && ctx->few_pairs, ctx->n_sms), p_down(PROJ_ADD, M, d, ff, prefetch, whole, ctx->n_sms);
+  const QkvAttentionPlan p_qa = p_qkv.few && prefetch ? plan_qkv_attention(p_qkv.small, md.n_heads, md.head_dim, d, R, Tn, md.s_max, ctx->n_sms)
+                                                      : QkvAttentionPlan{};
+  // (one CTA an SM: qkv_attention_few.cu)
+  if (p_qa.per_item > 0 && p_o.few && p_o.small.smem_bytes < 116 * 1024) p_o.small.smem_bytes = 116 * 1024;
   CUtensorMap tm_xq, tm_xg, tm_attn, tm_act;
   if (p_qkv.make_tmap(&tm_xq, xn, M, d) != VVS_OK || p_gu.make_tmap(&tm_xg, xn, M, d) != VVS_OK ||
       p_o.make_tmap(&tm_attn, attn, M, d) != VVS_OK || p_down.make_tmap(&tm_act, act, M, ff) != VVS_OK)
@@ -444,9 +449,15 @@ int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_o
     g.n = 3 * d; g.tm_a = p_qkv.few ? &F.w_qkv[few_map(p_qkv.small.group)] : &W.w_qkv; g.tm_b = &tm_xq; g.layer = at.layer = l; g.ss_parts = l > 0 ? p_down.ss_parts() : 4;
     g.pdl = ctx->use_pdl && l > 0;
     ahead(L.w_gate, L.w_up, ff, d);
-    VVS_LAUNCH(VVS_PROF_GEMM, rc = p_qkv.launch(PROJ_QKV, g, s));
-    g.pdl = ctx->use_pdl;
-    if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_ATTENTION, rc = launch_attention_block(at, s));
+    if (p_qa.per_item > 0) {
+      at.layer = l;
+      VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_qkv_attention(p_qa, g, at, s));
+      g.pdl = ctx->use_pdl;
+    } else {
+      VVS_LAUNCH(VVS_PROF_GEMM, rc = p_qkv.launch(PROJ_QKV, g, s));
+      g.pdl = ctx->use_pdl;
+      if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_ATTENTION, rc = launch_attention_block(at, s));
+    }
     g.n = d; g.tm_a = p_o.few ? &F.w_o[few_map(p_o.small.group)] : &W.w_o; g.tm_b = &tm_attn; g.scale = static_cast<const T*>(ctx->layers[l].norm2);
     ahead(L.w_down, nullptr, d, ff);
     if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = p_o.launch(PROJ_ADD, g, s));

@@ -321,6 +321,8 @@ struct AttentionBlockArgs {
   bool pdl;
 };
 int launch_attention_block(const AttentionBlockArgs& a, cudaStream_t s);
+// QKV and attention as one kernel, qkv_attention_few.cu (its plan: launch_plans.h)
+int launch_qkv_attention(const QkvAttentionPlan& plan, const ProjArgs& g, const AttentionBlockArgs& at, cudaStream_t s);
 
 // ---- tensor-core attention, attention_tc.cu ----------------------------------------------------------
 struct AttentionTcArgs {

@@ -1,0 +1,101 @@
+"""QKV and attention as one kernel (qkv_attention_few.cu, one to three sequences).  The rows of a sequence do not depend on what else is in a
+call, and four or more sequences take the two kernels: images alone give the bits that they give in a batch.  And the plan over sizes."""
+import ctypes
+import os
+import subprocess
+from dataclasses import replace
+
+import pytest
+
+from test_gpu_same_bits import _ints, _weights
+from vvs_synth.configs import XL
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2511_13587_b200", "csrc")
+SHAPE = replace(XL, name="qkv_attention", n_layers=2, d_model=1024, n_heads=16, d_ff=1024, vocab=512, lm_rows=0, tok_rows=0, s_max=700)
+
+
+def _step(ctx_rows, w, block, parents, fills, n_cfg, kv):
+    """Features and cache rows of one step on the given images (caches: cond rows, then uncond rows)."""
+    import torch
+
+    from paper_2511_13587_b200 import binding as vb
+    b, t_len = block.shape
+    rows = b * n_cfg
+    ctx = vb.vvs_create(vb.make_desc(SHAPE, ctx_rows, t_len, 1))
+    vb.vvs_bind_weights(ctx, w)
+    kv = [x.clone() for x in kv]
+    zeros = lambda *shape: torch.zeros(shape, dtype=torch.int32, device="cuda")  # noqa: E731
+    hidden = torch.zeros((rows, t_len, SHAPE.d_model), dtype=torch.bfloat16, device="cuda")
+    k = t_len - 1
+    more = {} if parents is None else dict(tree_parent=torch.tensor([parents] * b, dtype=torch.int32, device="cuda"),
+                                           target_probs=torch.zeros((b, t_len, SHAPE.vocab), device="cuda"))
+    vb.vvs_verify(ctx, n_images=b, n_cfg=n_cfg, n_forced=1, n_draft_max=k, block=block.contiguous(), kv_k=kv[0], kv_v=kv[1], kv_rows=rows,
+                  cache_len=torch.tensor(fills * n_cfg, dtype=torch.int32, device="cuda"),
+                  draft_probs=torch.full((b, max(k, 1), SHAPE.vocab), 1.0 / SHAPE.vocab, device="cuda"),
+                  uniforms=torch.full((b, k + 1), 0.5, device="cuda"), cfg_scale=2.0 if n_cfg == 2 else 1.0, temperature=1.0, mode=0,
+                  nbr_k=1, hidden=hidden, accept_len=zeros(b), next_token=zeros(b), new_len=zeros(rows), n_commit=zeros(rows),
+                  accept_mask=torch.zeros((b, max(k, 1)), dtype=torch.uint8, device="cuda"), **more)
+    assert vb.vvs_device_status(ctx) == 0
+    vb.vvs_destroy(ctx)
+    out = [hidden] if parents else [hidden, *kv]             # (a tree call moves the accepted rows afterwards)
+    return [x.view(torch.int16).cpu() for x in out]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_cfg,group,t_len,tree,fills", [
+    (2, 1, 9, False, [300, 0]), (2, 1, 9, False, [31, 32]), (2, 1, 9, False, [24, 23]), (2, 1, 1, False, [511, 512]),
+    (2, 1, 9, False, [503, 504]), (2, 1, 9, False, [543, 691]),             # more than sixteen slices: a part takes two
+    (2, 1, 16, False, [495, 497]), (2, 1, 13, True, [7, 640]),
+    (2, 1, 17, False, [250, 239]), (2, 1, 24, False, [231, 668]),           # two row groups, eight parts each
+    (1, 1, 9, False, [5, 570, 64, 200]), (1, 1, 24, False, [511, 256, 0, 668]), (1, 1, 16, True, [511, 256, 0, 668]),
+    (1, 2, 9, False, [5, 570, 64, 200]), (1, 3, 10, False, [1, 33, 544, 690, 0, 100])])
+def test_images_alone_or_in_a_batch(n_cfg, group, t_len, tree, fills):
+    import torch
+    b = len(fills)
+    w = _weights(SHAPE, 8100)
+    g = torch.Generator().manual_seed(8200 + t_len)
+    block = torch.randint(0, SHAPE.vocab, (b, t_len), generator=g, dtype=torch.int32).cuda()
+    parents = [-1] + [int(torch.randint(0, t, (1,), generator=g)) for t in range(1, t_len)] if tree else None
+    kv = [_ints((SHAPE.n_layers, b * n_cfg, SHAPE.n_heads, SHAPE.s_max, SHAPE.head_dim), 96, 32, 8300 + i) for i in range(2)]
+    want = _step(b * n_cfg, w, block, parents, fills, n_cfg, kv)
+    for at in range(0, b, group):
+        images = list(range(at, min(at + group, b)))
+        rows = [c * b + i for c in range(n_cfg) for i in images]
+        got = _step(len(rows), w, block[images], parents, [fills[i] for i in images], n_cfg, [x[:, rows].contiguous() for x in kv])
+        if b * n_cfg * t_len <= 64:                # (the final norm of more rows takes its sums in another order)
+            assert torch.equal(got[0], want[0][rows])
+        for a, e in zip(got[1:], want[1:]):
+            assert torch.equal(a, e[:, rows])
+
+
+def test_plan(tmp_path):
+    """Everything that lies over the stages lies inside the shared memory of a CTA, for every size that the kernel takes."""
+    src, lib = str(tmp_path / "shim.cc"), str(tmp_path / "shim.so")
+    with open(src, "w") as f:
+        f.write("""
+#include "launch_plans.h"
+extern "C" void plan(int rows, int t, int d, int s_max, int* o) {
+  const vvs::ProjFewPlan q = vvs::plan_proj_few(rows * t, 3 * d, d, false, false, true, 148);
+  const vvs::QkvAttentionPlan p = vvs::plan_qkv_attention(q, d / 64, 64, d, rows, t, s_max, 148);
+  const int v[] = {p.per_item, p.part_off, p.recv_off, p.new_off, p.smem_bytes, q.stages * q.group * (8192 + q.nt * 128), q.nt};
+  for (int i = 0; i < 7; ++i) o[i] = v[i];
+}
+""")
+    subprocess.run([os.environ.get("CXX", "g++"), "-std=c++17", "-Wall", "-Werror", "-shared", "-fPIC", "-I", CSRC, src, "-o", lib], check=True)
+    plan, taken = ctypes.CDLL(lib).plan, 0
+    for d in range(1024, 2049, 64):
+        for rows in range(1, 6):
+            for t in range(1, 33):
+                o = (ctypes.c_int * 7)()
+                plan(rows, t, d, 592, o)
+                per_item, part_off, recv_off, new_off, smem, stages, nt = o
+                if per_item == 0:
+                    continue
+                taken += 1
+                assert rows <= 3 and per_item * rows == 6 and d // 64 * 6 <= 132
+                assert -(-16 // per_item) <= 8 and part_off == -(-16 // per_item) * 8192      # a part a warp, a slot each
+                assert part_off + 16 * min(t, 16) * 102 * 4 <= recv_off and stages <= recv_off
+                assert recv_off + (nt + 3) // 4 * 1024 <= new_off and new_off + 384 * t + 1024 <= smem <= 226 * 1024
+                plan(rows, t, d, 4608, o)                                                     # long caches are split over clusters
+                assert o[0] == 0 or rows * d // 64 * 2 > 148
+    assert taken > 100
