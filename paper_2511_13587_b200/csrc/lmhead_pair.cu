@@ -52,30 +52,6 @@ __device__ __forceinline__ void tma_load_pair(void* dst, const CUtensorMap* m, u
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
       ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y) : "memory");
 }
-// mma_bf16_k64 and mma_commit_elect for a pair: called by a converged warp, of which one lane issues; the commit arrives on the same
-// barrier of both CTAs once the MMAs issued so far have completed
-__device__ __forceinline__ void mma_pair_k64(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred e, p, q;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\t"
-      "elect.sync _|e, 0xffffffff;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 q, %5, %5;\n\t"
-      "mov.b64 a, {%1, %5};\n\tmov.b64 b, {%2, %5};\n\t"
-      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, p;\n\t"
-      "add.u32 x, %1, 2;\n\tadd.u32 y, %2, 2;\n\tmov.b64 a, {x, %5};\n\tmov.b64 b, {y, %5};\n\t"
-      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, q;\n\t"
-      "add.u32 x, %1, 4;\n\tadd.u32 y, %2, 4;\n\tmov.b64 a, {x, %5};\n\tmov.b64 b, {y, %5};\n\t"
-      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, q;\n\t"
-      "add.u32 x, %1, 6;\n\tadd.u32 y, %2, 6;\n\tmov.b64 a, {x, %5};\n\tmov.b64 b, {y, %5};\n\t"
-      "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, q;\n\t}"
-      ::"r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHiSw128)
-      : "memory");
-}
-__device__ __forceinline__ void commit_pair(uint64_t* bar) {
-  asm volatile(
-      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
-      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
-      ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
-}
 __device__ __forceinline__ void arrive_remote(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }

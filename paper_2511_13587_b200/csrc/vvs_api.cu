@@ -380,18 +380,21 @@ struct ProjPick {
   bool few;
   ProjPlan wide{};
   ProjFewPlan small{};
+  GateupPairPlan pair{};
   ProjPick(int epi, int m, int n, int k, bool in_l2, bool whole, int n_sms) : few(whole && m <= proj::kFewTok) {
     const bool dual = epi == PROJ_GATEUP;
     if (few) small = plan_proj_few(m, n, k, dual, epi == PROJ_ADD, in_l2, n_sms);
     few = small.stages > 0;
     if (!few) wide = plan_proj(m, n, k, dual, n_sms);
+    if (!few && whole && in_l2 && dual) pair = plan_gateup_pair(m, n, k, n_sms);
   }
   int make_tmap(CUtensorMap* tm, const void* act, int m, int k) const {
+    if (pair.pairs > 0) return make_tmap_bf16_2d(tm, act, (uint64_t)m, (uint64_t)k, (uint32_t)pair.nt / 2);
     return few ? make_tmap_bf16_blocks(tm, act, (uint64_t)m, (uint64_t)k, (uint32_t)small.nt, (uint32_t)small.group)
                : make_tmap_bf16_2d(tm, act, (uint64_t)m, (uint64_t)k, (uint32_t)wide.nt);
   }
   int ss_parts() const { return few ? proj_ss_parts(small) : proj_ss_parts(wide); }
-  int launch(int epi, const ProjArgs& g, cudaStream_t s) const { return few ? launch_proj_few(epi, small, g, s) : launch_proj(epi, wide, g, s); }
+  int launch(int epi, const ProjArgs& g, cudaStream_t s) const { return pair.pairs > 0 ? launch_gateup_pair(pair, g, s) : few ? launch_proj_few(epi, small, g, s) : launch_proj(epi, wide, g, s); }
 };
 
 // bf16 contexts of wide models: five kernels per layer (proj_tc.cu, attention_block.cu), or four (qkv_attention_few.cu), each a programmatic dependent of
@@ -461,7 +464,7 @@ int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_o
     g.n = d; g.tm_a = p_o.few ? &F.w_o[few_map(p_o.small.group)] : &W.w_o; g.tm_b = &tm_attn; g.scale = static_cast<const T*>(ctx->layers[l].norm2);
     ahead(L.w_down, nullptr, d, ff);
     if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = p_o.launch(PROJ_ADD, g, s));
-    g.n = ff; g.tm_a = p_gu.few ? &F.w_gateup[few_map(p_gu.small.group)] : &W.w_gate; g.tm_a2 = &W.w_up; g.up_first = L.w_up < L.w_gate; g.tm_b = &tm_xg; g.ss_parts = p_o.ss_parts();
+    g.n = ff; g.tm_a = p_gu.pair.pairs > 0 ? &F.w_gateup_pair : p_gu.few ? &F.w_gateup[few_map(p_gu.small.group)] : &W.w_gate; g.tm_a2 = &W.w_up; g.up_first = L.w_up < L.w_gate; g.tm_b = &tm_xg; g.ss_parts = p_o.ss_parts();
     ahead(next ? next->w_qkv : nullptr, nullptr, 3 * d, d);
     if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = p_gu.launch(PROJ_GATEUP, g, s));
     g.n = d; g.tm_a = p_down.few ? &F.w_down[few_map(p_down.small.group)] : &W.w_down; g.tm_a2 = nullptr; g.tm_b = &tm_act;
@@ -924,6 +927,7 @@ int vvs_bind_weights(vvs_ctx* ctx, const vvs_weights* w) {
           if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_down[few_map(g)], s.w_down, d, ff, 64, g);
           if (rc == VVS_OK && pair) rc = make_tmap_bf16_pair_blocks(&q.w_gateup[few_map(g)], w0, dist, ff, d, 32, g);
         }
+        if (rc == VVS_OK && pair) rc = make_tmap_bf16_alternating_blocks(&q.w_gateup_pair, w0, dist, ff, d, 64, 1);
       }
     }
     if (rc == VVS_OK)

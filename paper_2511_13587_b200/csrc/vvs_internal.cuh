@@ -130,6 +130,7 @@ struct LayerMaps {
 // the same matrices in the boxes of proj_few.cu: 64 rows (32 of gate and up) of one to several k-blocks
 struct FewMaps {
   CUtensorMap w_qkv[4], w_o[4], w_gateup[4], w_down[4];   // [stages of two, four, five, seven k-blocks]
+  CUtensorMap w_gateup_pair;                              // gateup_pair.cu: 64 rows of both in turns, one k-block
 };
 
 }  // namespace vvs
@@ -268,6 +269,8 @@ struct GemmTcArgs {
 int make_tmap_bf16_blocks(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_blocks);
 int make_tmap_bf16_pair_blocks(CUtensorMap* out, const void* base, uint64_t dist, uint64_t rows, uint64_t cols, uint32_t box_rows,
                                uint32_t box_blocks);
+int make_tmap_bf16_alternating_blocks(CUtensorMap* out, const void* base, uint64_t dist, uint64_t rows, uint64_t cols, uint32_t box_rows,
+                                      uint32_t box_blocks);
 int make_tmap_bf16_2d(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 int make_weight_tmap(CUtensorMap* out, const void* w, int rows, int cols);
 GemmTcPlan plan_gemm_tc(int m, int n, int k, bool dual, bool allow_split, int n_sms, int split_cap = 32);
@@ -306,6 +309,8 @@ struct ProjArgs {
 };
 int launch_proj(int epi, const ProjPlan& plan, const ProjArgs& g, cudaStream_t s);
 int launch_proj_few(int epi, const ProjFewPlan& plan, const ProjArgs& g, cudaStream_t s);   // tensor maps: make_tmap_bf16_blocks, boxes of plan.group blocks; of b plan.nt rows
+
+int launch_gateup_pair(const GateupPairPlan& plan, const ProjArgs& g, cudaStream_t s);   // box rows of b: half of plan.nt
 
 // ---- block-vs-cache attention on rotated queries and appended keys, attention_block.cu ------------------
 struct AttentionBlockArgs {

@@ -1,0 +1,33 @@
+"""Gate/up of many tokens on CTA pairs (gateup_pair.cu) gives the bits of proj_tc.cu.  A d_ff that is no multiple of 64 takes that kernel;
+with eight rows and columns of zeros it is the same model again, in the same plans."""
+from dataclasses import replace
+
+import pytest
+
+from test_gpu_same_bits import _step, _weights
+from vvs_synth.configs import XL
+
+pytestmark = pytest.mark.gpu
+
+XL2 = replace(XL, name="xl2", n_layers=2, vocab=512, lm_rows=0, tok_rows=0, s_max=208)             # 54 CTAs of 64 outputs
+ODD = replace(XL2, name="odd", d_model=1088, n_heads=17, d_ff=2752)                               # 43 of them, the last pair's second idle; 17 k-blocks
+
+
+@pytest.mark.parametrize("ms,n_images,n_cfg,k,up_first", [
+    (XL2, 97, 1, 0, False),                                  # 97 tokens: passes of 64, the last of 33
+    (XL2, 7, 2, 8, True), (XL2, 16, 1, 15, False),           # 126, 256
+    (ODD, 97, 1, 0, False), (ODD, 10, 1, 10, True),          # 110
+    (ODD, 6, 2, 15, False), (ODD, 13, 2, 8, False)])         # 192, 234
+def test_pairs_give_the_same_bits(ms, n_images, n_cfg, k, up_first):
+    import torch
+    fills = [(37 * i) % (ms.s_max - k - 1) for i in range(n_images)]
+    w = _weights(replace(ms, d_ff=ms.d_ff - 8), 8400)
+    want = _step(replace(ms, d_ff=ms.d_ff - 8), w, n_images, n_cfg, 1, k, fills, 8500 + k)
+    for layer in w["layers"]:
+        layer["w_down"] = torch.nn.functional.pad(layer["w_down"], (0, 8)).contiguous()
+        gate, up = (torch.nn.functional.pad(layer[n], (0, 0, 0, 8)) for n in ("w_gate", "w_up"))
+        both = torch.stack([up, gate] if up_first else [gate, up])
+        layer["w_gate"], layer["w_up"] = both[int(up_first)], both[1 - int(up_first)]
+    got = _step(ms, w, n_images, n_cfg, 1, k, fills, 8500 + k)
+    for a, b in zip(want, got):
+        assert torch.equal(a, b)
