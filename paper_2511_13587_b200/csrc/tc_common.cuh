@@ -178,6 +178,7 @@ __device__ __forceinline__ void ld_shared_vec(const uint8_t* p, float (&v)[1]) {
 __device__ __forceinline__ void prefetch_l2(const void* ptr, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(ptr), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ void prefetch_l2_sector(const void* ptr) { asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr) : "memory"); }
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&h);
