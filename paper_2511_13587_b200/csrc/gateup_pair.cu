@@ -4,9 +4,14 @@
 // What bounds it there is the fill of shared memory from L2 (55 bytes a clock and SM): a CTA stages 128 rows of both matrices and all tokens of
 // its pass.  A pair (tcgen05.mma.cta_group::2, M = 256) stages half of the tokens per CTA, and gate and up lie in one tile, row by row in
 // turns, 64 outputs a CTA.  XL shape, 216 tokens: 440 KB a CTA in the place of 760.
-// 18 layers of the XL shape (us): 108 tokens 601.4 -> 584.9, 126 615.6 -> 598.9, 144 637.8 -> 625.3, 180 668.3 -> 660.8, 216 802.6 -> 792.3, 252 856.6 ->
-// 836.1.  Passes of more than 128 tokens gain in the fill what their epilogue of three rounds loses (270 tokens 882.5 / 883.9, 288 895.7 / 896.2;
-// with twenty warps, two rounds, 886, 900), and QKV on pairs gains nothing (144 tokens 637.8 / 636.9, 288 896 / 912): those stay in proj_tc.cu.
+// A stage is two k-blocks where five such stages fit (passes of up to 96 tokens), else one: four stages of two are too coarse for the way from
+// a stage's last MMA to the loads that fill it again (18 layers of the XL shape, two / one: 108 tokens 585.8 / 595.4 us, 144 623.0 / 626.2, 180 660.1 /
+// 662.4; 198 711.4 / 705.5, 252 835.8 / 830.9, 288 880.8 / 879.6).
+// 18 layers of the XL shape, proj_tc.cu / this kernel (us): 108 tokens 604.0 / 587.3, 126 616.6 / 598.4, 144 640.2 / 624.3, 180 670.9 / 659.8, 216 802.6
+// / 789.3, 252 856.6 / 831.5, 288 896.3 / 879.8.  Passes of more than 160 tokens lose in the epilogue what they gain in the fill (of 192: 360 tokens
+// 957.8 / 949.5, 378 961.6 / 966.3, 14 sequences of 27 rows 876.7 / 887.3; of 224: 396 tokens 974.4 / 991.5), and QKV on pairs gains nothing (144 tokens
+// 637.8 / 636.9, 288 896 / 912): those stay in proj_tc.cu.  Other widths: d_model 1024, d_ff 4096, 108 tokens 572.3 / 561.9, 216 644.0 / 646.2; 1152,
+// 3072, 180 tokens 629.8 / 613.3, 288 816.1 / 807.9.
 #include "tc_common.cuh"
 #include "vvs_internal.cuh"
 
@@ -18,11 +23,9 @@ using namespace proj;
 namespace {
 
 constexpr int kThreads = 512;
-constexpr uint32_t kSub = 2;                                         // k-blocks of a stage
-constexpr int kMaxPairTok = 128;                                     // of a pass
 
 struct Params {
-  int m, nt, kb_total, stages, up_first;                          // nt: tokens of a pass; kb_total: stages' worth of k-blocks
+  int m, nt, kb_total, stages, up_first;                          // nt: tokens of a pass; kb_total: stages' worth of k-blocks (SUB each)
   uint32_t tmem_cols;
   int32_t* status;
   const float* ss_in; int ss_parts; float inv_d, eps;
@@ -42,19 +45,20 @@ __device__ __forceinline__ void load_pair_4d(void* dst, const CUtensorMap* m, ui
       ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
 }
 
+template <int SUB>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 gateup_pair_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], acc_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_abort;
-  __shared__ float s_rs[kMaxPairTok];
+  __shared__ float s_rs[kPairTok];
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int rank = (int)(blockIdx.x & 1), tile = (int)blockIdx.x, pass = (int)blockIdx.y;          // tile: of this CTA's rows
   const int tok0 = pass * p.nt, ntok = min(p.nt, p.m - tok0);
-  const uint32_t b_bytes = (uint32_t)p.nt * kBlockK, stage_bytes = kSub * (kATileBytes + b_bytes);  // (half of the tokens)
+  const uint32_t b_bytes = (uint32_t)p.nt * kBlockK, stage_bytes = SUB * (kATileBytes + b_bytes);  // (half of the tokens)
 
   if (tid == 0) {
     for (int i = 0; i < p.stages; ++i) {
@@ -94,16 +98,16 @@ gateup_pair_kernel(const __grid_constant__ Params p, const __grid_constant__ CUt
         uint8_t* st = smem + (size_t)stage * stage_bytes;
         if (rank == 0) mbar_expect_tx(&full_bar[stage], 2 * stage_bytes);
 #pragma unroll
-        for (int h = 0; h < (int)kSub; ++h) load_pair_4d(st + h * kATileBytes, &tm_a, bar0, 0, 0, tile * 64, kb * (int)kSub + h);
+        for (int h = 0; h < SUB; ++h) load_pair_4d(st + h * kATileBytes, &tm_a, bar0, 0, 0, tile * 64, kb * SUB + h);
       }
     };
     auto load_act = [&](uint32_t stage, int kb) {
       if (elect_one()) {
         const uint32_t bar0 = mapa(smem_u32(&full_bar[stage]), 0);
-        uint8_t* st = smem + (size_t)stage * stage_bytes + kSub * kATileBytes;
+        uint8_t* st = smem + (size_t)stage * stage_bytes + SUB * kATileBytes;
 #pragma unroll
-        for (int h = 0; h < (int)kSub; ++h)
-          load_pair_2d(st + h * b_bytes, &tm_b, bar0, (kb * (int)kSub + h) * (int)kBlockK, tok0 + rank * (p.nt >> 1));
+        for (int h = 0; h < SUB; ++h)
+          load_pair_2d(st + h * b_bytes, &tm_b, bar0, (kb * SUB + h) * (int)kBlockK, tok0 + rank * (p.nt >> 1));
       }
     };
     const int n_pre = min(p.kb_total, p.stages);
@@ -141,8 +145,8 @@ gateup_pair_kernel(const __grid_constant__ Params p, const __grid_constant__ CUt
       tc_fence_after();
       const uint32_t a_lo = lo0 + stage * stage_lo;
 #pragma unroll
-      for (uint32_t h = 0; h < kSub; ++h)
-        mma_pair_k64(tmem, a_lo + h * (kATileBytes >> 4), a_lo + ((kSub * kATileBytes + h * b_bytes) >> 4), idesc, (uint32_t)(i | (int)h));
+      for (int h = 0; h < SUB; ++h)
+        mma_pair_k64(tmem, a_lo + h * (kATileBytes >> 4), a_lo + ((SUB * kATileBytes + h * b_bytes) >> 4), idesc, (uint32_t)(i | h));
       commit_pair(&empty_bar[stage]);
       if (++stage == (uint32_t)p.stages) { stage = 0; par ^= 1; }
     }
@@ -166,7 +170,7 @@ gateup_pair_kernel(const __grid_constant__ Params p, const __grid_constant__ CUt
       }
       warp_sums(ss, lane);
       const int j = warp_sums_index<8>(lane);
-      if ((lane & 3) == 0 && t0 + j < kMaxPairTok) s_rs[t0 + j] = rsqrtf(ss[0] * p.inv_d + p.eps);
+      if ((lane & 3) == 0 && t0 + j < kPairTok) s_rs[t0 + j] = rsqrtf(ss[0] * p.inv_d + p.eps);
     }
   }
   const int row_t = (warp & 3) * 32 + lane;   // weight row of this thread in TMEM
@@ -237,9 +241,10 @@ int launch_gateup_pair(const GateupPairPlan& pl, const ProjArgs& g, cudaStream_t
   kp.ahead[0] = static_cast<const uint8_t*>(g.ahead[0]); kp.ahead[1] = static_cast<const uint8_t*>(g.ahead[1]);
   kp.ahead_bytes = g.ahead[0] ? g.ahead_bytes : 0;
   kp.share = ahead_share(kp.ahead_bytes, (uint32_t)(2 * pl.pairs * pl.passes));
-  if (ensure_dynamic_smem(reinterpret_cast<const void*>(gateup_pair_kernel), 222 * 1024) != cudaSuccess) return VVS_ERR_CUDA;
-  return launch_kernel(gateup_pair_kernel, dim3(2 * pl.pairs, pl.passes), dim3(kThreads), (size_t)pl.smem_bytes, g.pdl, s, kp, *g.tm_a, *g.tm_b)
-                 == cudaSuccess ? VVS_OK : VVS_ERR_CUDA;
+  auto* fn = pl.sub == 2 ? gateup_pair_kernel<2> : gateup_pair_kernel<1>;
+  if (ensure_dynamic_smem(reinterpret_cast<const void*>(fn), 222 * 1024) != cudaSuccess) return VVS_ERR_CUDA;
+  return launch_kernel(fn, dim3(2 * pl.pairs, pl.passes), dim3(kThreads), (size_t)pl.smem_bytes, g.pdl, s, kp, *g.tm_a, *g.tm_b) == cudaSuccess
+                 ? VVS_OK : VVS_ERR_CUDA;
 }
 
 }  // namespace vvs

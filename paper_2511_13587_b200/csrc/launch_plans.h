@@ -11,6 +11,7 @@ namespace proj {
 constexpr int kMaxStages = 12;
 constexpr int kMaxThreads = 512;
 constexpr int kMaxTok = 128;              // tokens per pass
+constexpr int kPairTok = 160;             // the same, gate/up on CTA pairs
 constexpr uint32_t kTileRows = 128;       // weight rows per tile = MMA M
 constexpr uint32_t kBlockK = 64;          // bf16 elements per smem row = one 128-byte swizzle row
 constexpr uint32_t kATileBytes = kTileRows * kBlockK * 2;
@@ -242,32 +243,35 @@ inline ProjFewPlan plan_proj_few(int m, int n, int k, bool dual, bool add, bool 
 
 // ---- gate/up of many tokens on CTA pairs, gateup_pair.cu --------------------------------------------
 struct GateupPairPlan {
-  int pairs, passes, nt, kb_total, stages, smem_bytes, tmem_cols;       // kb_total: stages of two k-blocks; pairs 0: proj_tc.cu takes it
+  int pairs, passes, nt, kb_total, sub, stages, smem_bytes, tmem_cols;  // kb_total: stages' worth of sub k-blocks; pairs 0: proj_tc.cu takes it
 };
 
 // Where proj_tc.cu's plan is an unsplit one, of up to 20 MB of weights, and a CTA of a pair stages at most nine tenths of the bytes: the
-// fewest tokens per pass (a multiple of 32, an MMA's on a pair) that leave no second wave, up to 128 (gateup_pair.cu).
+// fewest tokens per pass (a multiple of 32, an MMA's on a pair) that leave no second wave, up to kPairTok (gateup_pair.cu).
 inline GateupPairPlan plan_gateup_pair(int m, int ff, int k, int n_sms) {
   using namespace proj;
   GateupPairPlan pl{};
   const ProjPlan one = plan_proj(m, ff, k, true, n_sms);
   if (one.splits > 1 || one.tiles_on_z || k % (int)kBlockK || (size_t)ff * k * 4 > (size_t)20 << 20) return pl;
   const int pairs = (ff + 127) / 128;
-  for (int passes = (m + 127) / 128; passes * pairs <= n_sms / 2; ++passes) {
+  for (int passes = (m + kPairTok - 1) / kPairTok; passes * pairs <= n_sms / 2; ++passes) {
     const int nt = ((m + passes - 1) / passes + 31) / 32 * 32;
     if ((m + nt - 1) / nt != passes || (pl.passes > 0 && nt >= pl.nt)) continue;
     pl.passes = passes;
     pl.nt = nt;
   }
   if (pl.passes == 0 || (128 + pl.nt / 2) * 10 > (256 + one.nt) * 9) return pl;       // (rows of a k-block that a CTA stages)
-  pl.kb_total = (k / (int)kBlockK + 1) / 2;
-  const int stage_bytes = 2 * ((int)kATileBytes + pl.nt * (int)kBlockK);
-  pl.stages = 200 * 1024 / stage_bytes;
+  // (220 KB: a fifth stage of two k-blocks with 96 tokens a pass, 144 tokens 628.0 -> 623.0 us a step of 18 layers of the XL shape)
+  const int kb_bytes = (int)kATileBytes + pl.nt * (int)kBlockK, room = 220 * 1024;
+  pl.sub = 5 * 2 * kb_bytes <= room ? 2 : 1;
+  pl.kb_total = (k / (int)kBlockK + pl.sub - 1) / pl.sub;
+  const int stage_bytes = pl.sub * kb_bytes;
+  pl.stages = room / stage_bytes;
   if (pl.stages > pl.kb_total) pl.stages = pl.kb_total;
   if (pl.stages > kMaxStages) pl.stages = kMaxStages;
   pl.smem_bytes = pl.stages * stage_bytes + 1024;
   if (pl.smem_bytes < pl.nt * 144 + 1024) pl.smem_bytes = pl.nt * 144 + 1024;         // the finished tile, token-major
-  pl.tmem_cols = pl.nt <= 32 ? 32 : pl.nt <= 64 ? 64 : 128;
+  pl.tmem_cols = pl.nt <= 32 ? 32 : pl.nt <= 64 ? 64 : pl.nt <= 128 ? 128 : 256;
   // (as in plan_proj: as large a share of an SM's shared memory as of its tensor memory)
   const int share = (int)((228u * 1024u * (unsigned)pl.tmem_cols + 511u) / 512u) - 1024;
   if (pl.smem_bytes < share) pl.smem_bytes = share;

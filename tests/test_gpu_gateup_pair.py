@@ -17,7 +17,9 @@ ODD = replace(XL2, name="odd", d_model=1088, n_heads=17, d_ff=2752)             
     (XL2, 97, 1, 0, False),                                  # 97 tokens: passes of 64, the last of 33
     (XL2, 7, 2, 8, True), (XL2, 16, 1, 15, False),           # 126, 256
     (ODD, 97, 1, 0, False), (ODD, 10, 1, 10, True),          # 110
-    (ODD, 6, 2, 15, False), (ODD, 13, 2, 8, False)])         # 192, 234
+    (ODD, 6, 2, 15, False), (ODD, 13, 2, 8, False),          # 192, 234
+    (XL2, 16, 2, 8, True), (XL2, 20, 1, 15, False),          # 288, 320: passes of 160
+    (ODD, 9, 2, 15, False), (ODD, 24, 1, 15, True)])         # 288, 384
 def test_pairs_give_the_same_bits(ms, n_images, n_cfg, k, up_first):
     import torch
     fills = [(37 * i) % (ms.s_max - k - 1) for i in range(n_images)]
