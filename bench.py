@@ -32,13 +32,14 @@ from vvs_synth.configs import CONFIGS, DTYPE_FP32, MODE_RELAXED  # noqa: E402
 # ncu capture summarised under profiles/.  Keyed by (workload, fixed-order sums); each entry names the
 # kernel sources the step runs and the first 16 hex digits of the SHA-256 over their concatenation when
 # the counters were taken: the line reports null, and says why, once any of them has changed.
-STEP_SOURCES = ("vvs_api.cu", "launch_plans.h", "proj_few.cu", "proj_tc.cu", "attention_block.cu", "gemm_tc.cu", "lmhead_few.cu",
-                "lmhead_pair.cu", "kernels_generic.cu", "kernels_decide.cu", "kernels_fcache.cu", "tc_common.cuh", "att_mma.cuh")
+STEP_SOURCES = ("vvs_api.cu", "launch_plans.h", "proj_few.cu", "proj_tc.cu", "gateup_pair.cu", "qkv_attention_few.cu", "attention_block.cu",
+                "gemm_tc.cu", "lmhead_few.cu", "lmhead_pair.cu", "kernels_generic.cu", "kernels_decide.cu", "kernels_fcache.cu",
+                "tc_common.cuh", "att_mma.cuh")
 NCU_CAPTURES = {       # (both settings of deterministic run the same kernels here; mean of the first two trials)
-    (1, False): ("c2f6f0ecc97ffd24", 1.518e+09, "profiles/folded_step_launches.txt"),
-    (1, True): ("c2f6f0ecc97ffd24", 1.518e+09, "profiles/folded_step_launches.txt"),
-    (2, False): ("c2f6f0ecc97ffd24", 3.622e+09, "profiles/folded_step_launches.txt"),
-    (2, True): ("c2f6f0ecc97ffd24", 3.622e+09, "profiles/folded_step_launches.txt"),
+    (1, False): ("cee5dbf395813fd5", 1.522e+09, "profiles/folded_step_launches.txt"),
+    (1, True): ("cee5dbf395813fd5", 1.522e+09, "profiles/folded_step_launches.txt"),
+    (2, False): ("cee5dbf395813fd5", 3.593e+09, "profiles/folded_step_launches.txt"),
+    (2, True): ("cee5dbf395813fd5", 3.593e+09, "profiles/folded_step_launches.txt"),
 }
 N_TRIALS = 32           # distinct (fill, block, draft) inputs cycled through the steps
 DRAFT_LOGIT_STD = 1.0   # target-independent drafter: q = softmax(N(0, std^2))
@@ -58,7 +59,7 @@ def kernels_name(ms, chain_kernels: bool = False) -> str:
         return "whole-chain kernels (previous generation, debug switch)"
     if ms.dtype == DTYPE_FP32:
         return "five float32 kernels per layer, norms and epilogues folded in"
-    return "five kernels per layer, epilogues folded in" if ms.d_model >= 1024 else "nine kernels per layer"
+    return "four or five kernels per layer, epilogues folded in" if ms.d_model >= 1024 else "nine kernels per layer"
 
 
 def metric_name(wl) -> str:

@@ -394,11 +394,14 @@ struct ProjPick {
                : make_tmap_bf16_2d(tm, act, (uint64_t)m, (uint64_t)k, (uint32_t)wide.nt);
   }
   int ss_parts() const { return few ? proj_ss_parts(small) : proj_ss_parts(wide); }
-  int launch(int epi, const ProjArgs& g, cudaStream_t s) const { return pair.pairs > 0 ? launch_gateup_pair(pair, g, s) : few ? launch_proj_few(epi, small, g, s) : launch_proj(epi, wide, g, s); }
+  int launch(int epi, const ProjArgs& g, cudaStream_t s) const {
+    if (pair.pairs > 0) return launch_gateup_pair(pair, g, s);
+    return few ? launch_proj_few(epi, small, g, s) : launch_proj(epi, wide, g, s);
+  }
 };
 
-// bf16 contexts of wide models: five kernels per layer (proj_tc.cu, attention_block.cu), or four (qkv_attention_few.cu), each a programmatic dependent of
-// the one before.  Every sum is taken in a fixed order, so a call repeats bit for bit.
+// bf16 contexts of wide models: five kernels per layer (proj_few.cu, proj_tc.cu, gateup_pair.cu, attention_block.cu), or four
+// (qkv_attention_few.cu), each a programmatic dependent of the one before.  Every sum is taken in a fixed order, so a call repeats bit for bit.
 int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_out* o, cudaStream_t s) {
   using T = __nv_bfloat16;
   const vvs_model_desc& md = ctx->desc;
@@ -464,7 +467,8 @@ int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_o
     g.n = d; g.tm_a = p_o.few ? &F.w_o[few_map(p_o.small.group)] : &W.w_o; g.tm_b = &tm_attn; g.scale = static_cast<const T*>(ctx->layers[l].norm2);
     ahead(L.w_down, nullptr, d, ff);
     if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = p_o.launch(PROJ_ADD, g, s));
-    g.n = ff; g.tm_a = p_gu.pair.pairs > 0 ? &F.w_gateup_pair : p_gu.few ? &F.w_gateup[few_map(p_gu.small.group)] : &W.w_gate; g.tm_a2 = &W.w_up; g.up_first = L.w_up < L.w_gate; g.tm_b = &tm_xg; g.ss_parts = p_o.ss_parts();
+    g.n = ff; g.tm_a = p_gu.pair.pairs > 0 ? &F.w_gateup_pair : p_gu.few ? &F.w_gateup[few_map(p_gu.small.group)] : &W.w_gate;
+    g.tm_a2 = &W.w_up; g.up_first = L.w_up < L.w_gate; g.tm_b = &tm_xg; g.ss_parts = p_o.ss_parts();
     ahead(next ? next->w_qkv : nullptr, nullptr, 3 * d, d);
     if (rc == VVS_OK) VVS_LAUNCH(VVS_PROF_GEMM, rc = p_gu.launch(PROJ_GATEUP, g, s));
     g.n = d; g.tm_a = p_down.few ? &F.w_down[few_map(p_down.small.group)] : &W.w_down; g.tm_a2 = nullptr; g.tm_b = &tm_act;
