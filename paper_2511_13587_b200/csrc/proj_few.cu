@@ -306,6 +306,7 @@ proj_few_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const 
     if (lane == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
     s_abort = 1;
   }
+  __syncwarp();       // each lane left the wait by itself, what follows is for a whole warp at once (.aligned)
   tc_fence_after();
   if (SPLIT) cluster_wait();
   // ---- rows to where the epilogue reads them ---------------------------------------------------------------------------

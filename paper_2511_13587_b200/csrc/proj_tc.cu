@@ -225,7 +225,7 @@ proj_tc_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, const _
   if (!SPLIT && (warp >> 2) * 16 < ntok) operands((warp >> 2) * 16);
 
   // A CTA that gave up pushes whatever its accumulator holds: its peers' waits must still end.
-  if (!wait_or_abort(&acc_bar, 0, &s_abort)) {
+  if (!warp_wait_or_abort(&acc_bar, 0, &s_abort)) {
     if (lane == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
     s_abort = 1;
   }

@@ -263,6 +263,7 @@ qkv_attention_kernel(const __grid_constant__ Params p, const __grid_constant__ C
     if (lane == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
     s_abort = 1;
   }
+  __syncwarp();       // each lane left the wait by itself, what follows is for a whole warp at once (.aligned)
   tc_fence_after();
   cluster_wait();
   // ---- partial sums to the rank that owns the row ------------------------------------------------------------------------
@@ -286,6 +287,7 @@ qkv_attention_kernel(const __grid_constant__ Params p, const __grid_constant__ C
     bool got = false;
     for (uint32_t i = 0; i < 16u * kSpinLimit && !got; ++i) got = mbar_try_wait_cluster(bar, 0);
     if (!got && lane == 0) atomicOr(p.status, VVS_DEV_TIMEOUT);
+    __syncwarp();     // (ldmatrix and the MMAs are .aligned too)
   };
   wait_cluster(&recv_bar);
   // ---- finished sums: 1/rms, rotation, to the CTAs that attend with them; k and v into the cache ------------------------------
@@ -400,15 +402,15 @@ qkv_attention_kernel(const __grid_constant__ Params p, const __grid_constant__ C
   // ---- parts folded in their order ---------------------------------------------------------------------------------------------
   {
     // weights of the parts of each row, sixteen lanes a row; a part past the last one gets none
-    for (int idx = tid; idx < T * kParts; idx += kThreads) {         // (T * 16 is a multiple of sixteen: a row's lanes stay together)
-      const int t = idx >> 4, w = idx & 15, row = groups == 2 ? t & 15 : t;
+#pragma unroll 1
+    for (int idx = tid; idx < (T + 1) / 2 * 32; idx += kThreads) {   // (whole warps: the second half of the last one may have no row)
+      const int t = min(idx >> 4, T - 1), w = idx & 15, row = groups == 2 ? t & 15 : t;
       float2* ml = reinterpret_cast<float2*>(parts_ml) + ((groups == 2 ? (t >> 4) * wpg : 0) + min(w, wpg - 1)) * ld_t + row;
       const float mine = w < busy ? ml->x : -CUDART_INF_F;
-      const uint32_t lanes = __activemask();
       float m = mine;
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(lanes, m, o));
-      if (w < busy) ml->x = ex2(mine - (m == -CUDART_INF_F ? 0.f : m));
+      for (int o = 8; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (w < busy && idx < T * kParts) ml->x = ex2(mine - (m == -CUDART_INF_F ? 0.f : m));
     }
     __syncthreads();
   }

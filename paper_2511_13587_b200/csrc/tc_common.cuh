@@ -85,6 +85,14 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, vo
   }
   return false;
 }
+// The same wait of a whole warp, which goes on as one: what follows may be .aligned (tcgen05.ld, barrier.cluster).
+__device__ __forceinline__ bool warp_wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  for (uint32_t i = 0; i < kSpinLimit; ++i) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if ((i & 1023u) == 1023u && __any_sync(0xffffffffu, *abort_flag)) return false;
+  }
+  return false;
+}
 // The same test for a barrier that other CTAs of the cluster arrive on or write behind.
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
