@@ -392,6 +392,9 @@ class VerifyBench:
         alg = algorithmic_bytes(self.wl, self.trials)
         per_step = {"gemm": cls_ms[0] / n_prof, "attention": cls_ms[1] / n_prof,
                     "other": cls_ms[2] / n_prof, "chain": cls_ms[3] / n_prof}
+        if cls_n[1] == 0 and cls_n[3] == 0:         # one kernel a layer for QKV and attention: its time cannot be told apart
+            del per_step["attention"]
+            per_step["gemm_and_attention"] = per_step.pop("gemm")
         if cls_n[3] > 0:
             # calls of at most 32 tokens: embedding + all decoder layers are ONE persistent kernel, which
             # streams every layer weight once and reads the K/V rows (the LM head is a separate launch)

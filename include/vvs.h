@@ -390,8 +390,11 @@ int vvs_last_launch_count(const vvs_ctx* ctx);
  * vvs_verify / vvs_epilogue is bracketed by CUDA events on the call's stream (this costs time:
  * never enable it around a headline measurement).  Classes: 0 = projection / LM-head GEMMs,
  * 1 = attention, 2 = everything else, 3 = the whole-chain kernel (embedding and every decoder
- * layer in one launch; used by calls of at most 32 block tokens, which then have no class-0 / 1
- * launches except the LM head).  vvs_profile_read synchronises the stream, ADDS the milliseconds
+ * layer in one launch, of contexts created under VVS_DEBUG_CHAIN_KERNELS only; such calls have no
+ * class-0 / 1 launches except the LM head).  Where one kernel does a layer's QKV projection AND its
+ * attention (bf16, few tokens, one to three sequences), that launch counts as class 0 and class 1
+ * has none: a step without class-1 launches has its attention in class 0 (or 3).
+ * vvs_profile_read synchronises the stream, ADDS the milliseconds
  * and launch counts recorded since the last read to ms[4] / launches[4] (host arrays) and forgets
  * them.  Events are created by vvs_profile_enable, not on the verify path. */
 enum { VVS_PROF_GEMM = 0, VVS_PROF_ATTENTION = 1, VVS_PROF_OTHER = 2, VVS_PROF_CHAIN = 3, VVS_PROF_CLASSES = 4 };

@@ -237,7 +237,8 @@ def vvs_profile_enable(ctx: int, on: bool) -> None:
 
 def vvs_profile_read(ctx: int, stream=None):
     """Returns ([ms per class], [launches per class]) accumulated since the last read;
-    classes: 0 GEMM, 1 attention, 2 other, 3 whole-chain kernel."""
+    classes: 0 GEMM (and the attention of steps that do it in the QKV kernel: none in class 1 then), 1 attention, 2 other,
+    3 whole-chain kernel."""
     ms = (C.c_float * 4)(0, 0, 0, 0)
     n = (C.c_int32 * 4)(0, 0, 0, 0)
     _check(lib.vvs_profile_read(ctx, _stream(stream), ms, n), "vvs_profile_read")

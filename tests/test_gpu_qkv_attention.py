@@ -1,5 +1,6 @@
 """QKV and attention as one kernel (qkv_attention_few.cu, one to three sequences).  The rows of a sequence do not depend on what else is in a
-call, and four or more sequences take the two kernels: images alone give the bits that they give in a batch.  And the plan over sizes."""
+call, and four or more sequences take the two kernels: images alone give the bits that they give in a batch.  What the launch counts as.  And the plan
+over sizes."""
 import ctypes
 import os
 import subprocess
@@ -7,6 +8,7 @@ from dataclasses import replace
 
 import pytest
 
+import helpers as H
 from test_gpu_same_bits import _ints, _weights
 from vvs_synth.configs import XL
 
@@ -66,6 +68,23 @@ def test_images_alone_or_in_a_batch(n_cfg, group, t_len, tree, fills):
             assert torch.equal(got[0], want[0][rows])
         for a, e in zip(got[1:], want[1:]):
             assert torch.equal(a, e[:, rows])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_images,one_kernel", [(1, True), (2, False)])
+def test_classes_of_a_profiled_step(n_images, one_kernel):
+    """One launch for QKV and attention of a layer counts with the projections (include/vvs.h); profiling changes no result."""
+    case = H.build_case_independent(SHAPE, 8650, n_images, 2, 1, 8, [77, 300][:n_images], logit_std=0.6)
+    run = H.GpuRunner(SHAPE, case["w"], 2 * n_images, 9)
+    want = run.verify(case)
+    run.vb.vvs_profile_enable(run.ctx, True)
+    got = run.verify(case)
+    ms, launches = run.vb.vvs_profile_read(run.ctx)
+    run.vb.vvs_profile_enable(run.ctx, False)
+    assert (got["hidden"] == want["hidden"]).all() and sum(launches) == want["launches"] == got["launches"]
+    assert launches[:2] == [4 * SHAPE.n_layers + 1, 0 if one_kernel else SHAPE.n_layers] and launches[3] == 0
+    assert ms[0] > 0 and (ms[1] > 0) == (not one_kernel)
+    run.close()
 
 
 def test_plan(tmp_path):
