@@ -10,8 +10,7 @@
 // 18 layers of the XL shape, proj_tc.cu / this kernel (us): 108 tokens 604.0 / 587.3, 126 616.6 / 598.4, 144 640.2 / 624.3, 180 670.9 / 659.8, 216 802.6
 // / 789.3, 252 856.6 / 831.5, 288 896.3 / 879.8.  Passes of more than 160 tokens lose in the epilogue what they gain in the fill (of 192: 360 tokens
 // 957.8 / 949.5, 378 961.6 / 966.3, 14 sequences of 27 rows 876.7 / 887.3; of 224: 396 tokens 974.4 / 991.5), and QKV on pairs gains nothing (144 tokens
-// 637.8 / 636.9, 288 896 / 912): those stay in proj_tc.cu.  Other widths: d_model 1024, d_ff 4096, 108 tokens 572.3 / 561.9, 216 644.0 / 646.2; 1152,
-// 3072, 180 tokens 629.8 / 613.3, 288 816.1 / 807.9.
+// 637.8 / 636.9, 288 896 / 912): those stay in proj_tc.cu.  Other widths, and up to how many tokens a pass each may have: plan_gateup_pair.
 #include "tc_common.cuh"
 #include "vvs_internal.cuh"
 

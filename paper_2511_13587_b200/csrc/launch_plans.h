@@ -247,14 +247,21 @@ struct GateupPairPlan {
 };
 
 // Where proj_tc.cu's plan is an unsplit one, of up to 20 MB of weights, and a CTA of a pair stages at most nine tenths of the bytes: the
-// fewest tokens per pass (a multiple of 32, an MMA's on a pair) that leave no second wave, up to kPairTok (gateup_pair.cu).
+// fewest tokens per pass (a multiple of 32, an MMA's on a pair) that leave no second wave.  How many that may be: a pass has about twice
+// the tokens of proj_tc.cu's, and its epilogue the time they take, which short K ranges do not earn back.  18 layers, steps against
+// proj_tc.cu, 337 calls of 97 to 1200 tokens in chains of 9, 16 and 18 rows, 100 and 300 cached: up to 64 tokens a pass -0.4 to -5 % at every
+// width; 96 and 128 from 18 k-blocks on -0.3 to -3.6 %, at 16 of them (d_model 1024) -1.5 to +1.0 %, 0 on average; 160 where weights x k-blocks
+// reach 270 MB (MB x blocks of 64: d_model 1280, d_ff 3456 338; 1536, 2048 288; below 1280, 2560 250; 1024, 4096 256) -2.7 to 0 %, below
+// +0.1 to +2.6 %.  Of what this takes 1280, 3456 with passes of 160 loses while caches are short: 288 tokens, 20 cached +0.2 to +0.8 %, 100
+// -0.2 to +0.4, 300 -1.6 to 0, 550 -1.2 to -0.6.
 inline GateupPairPlan plan_gateup_pair(int m, int ff, int k, int n_sms) {
   using namespace proj;
   GateupPairPlan pl{};
   const ProjPlan one = plan_proj(m, ff, k, true, n_sms);
   if (one.splits > 1 || one.tiles_on_z || k % (int)kBlockK || (size_t)ff * k * 4 > (size_t)20 << 20) return pl;
-  const int pairs = (ff + 127) / 128;
-  for (int passes = (m + kPairTok - 1) / kPairTok; passes * pairs <= n_sms / 2; ++passes) {
+  const int pairs = (ff + 127) / 128, blocks = k / (int)kBlockK;
+  const int most = (size_t)ff * k * 4 * blocks >= (size_t)270 << 20 ? kPairTok : blocks >= 18 ? 128 : 64;
+  for (int passes = (m + most - 1) / most; passes * pairs <= n_sms / 2; ++passes) {
     const int nt = ((m + passes - 1) / passes + 31) / 32 * 32;
     if ((m + nt - 1) / nt != passes || (pl.passes > 0 && nt >= pl.nt)) continue;
     pl.passes = passes;

@@ -13,6 +13,7 @@ FIELDS = ("nt", "passes", "tiles", "kb_total", "splits", "stages", "alias", "rec
           "tiles_on_z")
 FEW_FIELDS = ("nt", "tiles", "kb_total", "splits", "group", "stages", "ring", "recv_off", "smem_bytes", "tmem_cols",
               "parts", "acc_ld")
+PAIR_FIELDS = ("pairs", "passes", "nt", "kb_total", "sub", "stages", "smem_bytes", "tmem_cols")
 SHIM = """
 #include "launch_plans.h"
 extern "C" void proj(int m, int n, int k, int dual, int n_sms, int* o) {
@@ -25,6 +26,11 @@ extern "C" void few(int m, int n, int k, int dual, int add, int in_l2, int n_sms
   const int v[] = {%s, vvs::proj_ss_parts(p)};
   for (unsigned i = 0; i < sizeof(v) / sizeof(v[0]); ++i) o[i] = v[i];
 }
+extern "C" void pair(int m, int ff, int k, int n_sms, int* o) {
+  const vvs::GateupPairPlan p = vvs::plan_gateup_pair(m, ff, k, n_sms);
+  const int v[] = {%s, vvs::proj::kPairTok};
+  for (unsigned i = 0; i < sizeof(v) / sizeof(v[0]); ++i) o[i] = v[i];
+}
 extern "C" void ahead(unsigned bytes, unsigned n_cta, unsigned* o) {
   const vvs::AheadShare s = vvs::ahead_share(bytes, n_cta);
   o[0] = s.every;
@@ -32,7 +38,7 @@ extern "C" void ahead(unsigned bytes, unsigned n_cta, unsigned* o) {
 }
 extern "C" int tree_parts(int vocab, int n_images, int n_sms) { return vvs::tree_walk_parts(vocab, n_images, n_sms); }
 extern "C" int att_split(int hd, int items, int s_max, int n_sms) { return vvs::attention_split(hd, items, s_max, n_sms); }
-""" % (", ".join("p." + f for f in FIELDS), ", ".join("p." + f for f in FEW_FIELDS))
+""" % (", ".join("p." + f for f in FIELDS), ", ".join("p." + f for f in FEW_FIELDS), ", ".join("p." + f for f in PAIR_FIELDS))
 
 # (d_model, d_ff): the benchmark shapes, one between them, one below and one above
 WIDTHS = [(1024, 2752), (1280, 3456), (1536, 2744), (2048, 5504), (4096, 11008), (8192, 22016)]
@@ -142,6 +148,49 @@ def test_few_token_plans_fit_the_hardware(plans, d, ff, in_l2):
             per_sm = 228 * 1024 // (p["smem_bytes"] + 2048) if p["smem_bytes"] <= 112 * 1024 else 1
             assert p["tiles"] * p["splits"] <= min(per_sm, 3) * N_SMS * (33 / 37 if p["splits"] == 4 else 1), at
     assert taken == TAKEN.get((d, ff), [96] * 4)
+
+
+def _pair(plans, m, ff, k):
+    out = (ctypes.c_int * (len(PAIR_FIELDS) + 1))()
+    plans.pair(m, ff, k, N_SMS, out)
+    return dict(zip(PAIR_FIELDS + ("most",), out))
+
+
+@pytest.mark.parametrize("d", [1024, 1088, 1280, 1408, 1536, 2048])
+def test_pair_plans_fit_the_hardware(plans, d):
+    """Gate/up on CTA pairs: one wave of passes, none of them empty, everything inside a CTA's shared and tensor memory."""
+    taken = 0
+    for ff in (64, 512, 1024, 1536, 2048, 2560, 2752, 3072, 3456, 4096, 4800, 5120, 6144):
+        for m in list(range(1, 400)) + list(range(400, 1300, 13)):
+            p = _pair(plans, m, ff, d)
+            if p["pairs"] == 0:
+                continue
+            taken += 1
+            at = (m, ff, d, p)
+            one = _proj(plans, m, ff, d, True)                       # the kernel whose place it takes: unsplit, weights that stay in L2
+            assert one["splits"] == 1 and not one["tiles_on_z"] and ff * d * 4 <= 20 << 20, at
+            assert p["pairs"] == -(-ff // 128) and p["pairs"] * p["passes"] <= N_SMS // 2, at
+            assert p["nt"] % 32 == 0 and 32 <= p["nt"] <= p["most"] and (p["passes"] - 1) * p["nt"] < m <= p["passes"] * p["nt"], at
+            assert p["sub"] in (1, 2) and p["kb_total"] * p["sub"] >= d // 64 > (p["kb_total"] - 1) * p["sub"], at
+            assert min(2, p["kb_total"]) <= p["stages"] <= min(12, p["kb_total"]), at
+            stage = p["sub"] * (128 + p["nt"] // 2) * 128            # a CTA's rows of gate and up, half of the tokens
+            assert max(p["stages"] * stage, p["nt"] * 144) + 1024 <= p["smem_bytes"] <= 222 * 1024, at
+            assert p["nt"] <= p["tmem_cols"] and p["tmem_cols"] in (32, 64, 128, 256), at
+            assert (p["smem_bytes"] + 1024) * 512 >= p["tmem_cols"] * 228 * 1024 - 512, at
+            # passes no longer than the K range pays for
+            assert p["nt"] <= (160 if ff * d * 4 * (d // 64) >= 270 << 20 else 128 if d >= 1152 else 64), at
+    assert taken > 100, taken
+
+
+def test_pairs_are_taken_where_their_bits_are_compared(plans):
+    from test_gpu_gateup_pair import CASES, NOT_TAKEN
+    widths = set()
+    for ms, n_images, n_cfg, k, _ in CASES:
+        m = n_images * n_cfg * (1 + k)
+        p = _pair(plans, m, ms.d_ff, ms.d_model)
+        assert (p["pairs"] == 0) == ((ms.name, m) in NOT_TAKEN), (ms.name, m, p)
+        widths.add((p["sub"], p["nt"]))
+    assert {(2, 64), (2, 96), (1, 128), (1, 160)} <= widths, widths
 
 
 def test_requests_into_l2_are_shared_out(plans):
