@@ -30,11 +30,6 @@ namespace {
 using bf16 = __nv_bfloat16;
 constexpr int kMaxT = 32;      // block rows per sequence
 
-__device__ __forceinline__ void st_async2(uint32_t addr, uint32_t bar, float a, float b) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
-               ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
-}
-
 // Shared memory: the rings of the W warps, [slot][warp]; the merge buffer lies over the last slot of them; then, in a cluster,
 // the states of ranks 1 .. S-1 (written by them into rank 0).  A slice is 16 NS keys.
 template <int HD, int NMT, int W, int D, int NS, bool MANY>
@@ -310,8 +305,8 @@ __global__ void __launch_bounds__(32 * W) attention_block_kernel(AttentionBlockA
       if constexpr (CP == 2) {
         if (rank > 0) {
           const uint32_t dst = xbuf0 + (uint32_t)(((rank - 1) * T + t) * (HD + 2)) * 4u;
-          st_async2(dst + (uint32_t)cp * 8u, x_bar0, o[0], o[1]);
-          if (cp == 0) st_async2(dst + HD * 4u, x_bar0, m, l);
+          tc::st_async2(dst + (uint32_t)cp * 8u, x_bar0, o[0], o[1]);
+          if (cp == 0) tc::st_async2(dst + HD * 4u, x_bar0, m, l);
           continue;
         }
         if (!waited) {

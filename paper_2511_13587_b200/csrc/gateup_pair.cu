@@ -32,18 +32,6 @@ struct Params {
   const uint8_t* ahead[2]; uint32_t ahead_bytes; AheadShare share;
 };
 
-// loads into this CTA, bytes counted on a barrier of the pair (cluster address)
-__device__ __forceinline__ void load_pair_2d(void* dst, const CUtensorMap* m, uint32_t bar, int x, int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y) : "memory");
-}
-__device__ __forceinline__ void load_pair_4d(void* dst, const CUtensorMap* m, uint32_t bar, int x, int y, int z, int w) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
-}
-
 template <int SUB>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 gateup_pair_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b) {
@@ -97,7 +85,7 @@ gateup_pair_kernel(const __grid_constant__ Params p, const __grid_constant__ CUt
         uint8_t* st = smem + (size_t)stage * stage_bytes;
         if (rank == 0) mbar_expect_tx(&full_bar[stage], 2 * stage_bytes);
 #pragma unroll
-        for (int h = 0; h < SUB; ++h) load_pair_4d(st + h * kATileBytes, &tm_a, bar0, 0, 0, tile * 64, kb * SUB + h);
+        for (int h = 0; h < SUB; ++h) tma_load_pair_4d(st + h * kATileBytes, &tm_a, bar0, 0, 0, tile * 64, kb * SUB + h);
       }
     };
     auto load_act = [&](uint32_t stage, int kb) {
@@ -106,7 +94,7 @@ gateup_pair_kernel(const __grid_constant__ Params p, const __grid_constant__ CUt
         uint8_t* st = smem + (size_t)stage * stage_bytes + SUB * kATileBytes;
 #pragma unroll
         for (int h = 0; h < SUB; ++h)
-          load_pair_2d(st + h * b_bytes, &tm_b, bar0, (kb * SUB + h) * (int)kBlockK, tok0 + rank * (p.nt >> 1));
+          tma_load_pair_2d(st + h * b_bytes, &tm_b, bar0, (kb * SUB + h) * (int)kBlockK, tok0 + rank * (p.nt >> 1));
       }
     };
     const int n_pre = min(p.kb_total, p.stages);

@@ -588,34 +588,23 @@ int make_tmap_bf16_blocks(CUtensorMap* out, const void* base, uint64_t rows, uin
 }
 
 // Two such matrices, the second `dist` bytes behind the first (a multiple of 16 below 2^40): a box holds `box_rows` rows of both, one
-// after the other in each block.
+// after the other in each block, or (in_turns) row r of the first, row r of the second, row r + 1 of the first.
 int make_tmap_bf16_pair_blocks(CUtensorMap* out, const void* base, uint64_t dist, uint64_t rows, uint64_t cols, uint32_t box_rows,
-                               uint32_t box_blocks) {
+                               uint32_t box_blocks, bool in_turns) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return VVS_ERR_CUDA;
-  cuuint64_t dims[4] = {kBlockK, rows, 2, cols / kBlockK};
-  cuuint64_t strides[3] = {cols * 2, dist, kBlockK * 2};
-  cuuint32_t box[4] = {kBlockK, box_rows, 2, box_blocks};
-  cuuint32_t estr[4] = {1, 1, 1, 1};
-  CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+  const int r = in_turns ? 2 : 1, two = in_turns ? 1 : 2;        // dimensions of rows and of the two matrices
+  cuuint64_t dims[4] = {kBlockK, 0, 0, cols / kBlockK}, strides[3] = {0, 0, kBlockK * 2};
+  cuuint32_t box[4] = {kBlockK, 0, 0, box_blocks}, estr[4] = {1, 1, 1, 1};
+  dims[r] = rows;
+  strides[r - 1] = cols * 2;
+  box[r] = box_rows;
+  dims[two] = box[two] = 2;
+  strides[two - 1] = dist;
+  CUresult e = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? VVS_OK : VVS_ERR_CUDA;
-}
-
-// The same two matrices row by row: row r of the first, row r of the second, row r + 1 of the first.
-int make_tmap_bf16_alternating_blocks(CUtensorMap* out, const void* base, uint64_t dist, uint64_t rows, uint64_t cols, uint32_t box_rows,
-                                      uint32_t box_blocks) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return VVS_ERR_CUDA;
-  cuuint64_t dims[4] = {kBlockK, 2, rows, cols / kBlockK};
-  cuuint64_t strides[3] = {dist, cols * 2, kBlockK * 2};
-  cuuint32_t box[4] = {kBlockK, 2, box_rows, box_blocks};
-  cuuint32_t estr[4] = {1, 1, 1, 1};
-  CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? VVS_OK : VVS_ERR_CUDA;
+  return e == CUDA_SUCCESS ? VVS_OK : VVS_ERR_CUDA;
 }
 
 int make_weight_tmap(CUtensorMap* out, const void* w, int rows, int cols) {

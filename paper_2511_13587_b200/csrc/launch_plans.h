@@ -310,12 +310,12 @@ struct QkvAttentionPlan {
 
 // qkv: the projection's plan, in two slices with all k-blocks in shared memory (tiles of 64 rows: a head's q, k or v).  Heads of 64 whose
 // items have a CTA each in attention_block.cu; one to three sequences, since the sixteen warps' parts of an item need two CTAs; and all
-// clusters have to fit at once (of 148 SMs 22 take clusters of six: 132).
+// clusters have to fit at once (of 148 SMs 22 take clusters of six: 132).  A token has at most 128 sums of squares (d / 16 of them).
 inline QkvAttentionPlan plan_qkv_attention(const ProjFewPlan& qkv, int n_heads, int hd, int d, int n_rows, int t_len, int s_max, int n_sms) {
   using namespace proj;
   QkvAttentionPlan pl{};
   pl.proj = qkv;
-  if (hd != 64 || n_heads * hd != d || n_rows > 3 || t_len > 32 || qkv.stages < 1 || qkv.splits != 2 || qkv.ring || qkv.parts > 0) return pl;
+  if (hd != 64 || n_heads * hd != d || d > 2048 || n_rows > 3 || t_len > 32 || qkv.stages < 1 || qkv.splits != 2 || qkv.ring || qkv.parts > 0) return pl;
   if (n_heads * 6 > n_sms * 33 / 37 || attention_split(hd, (long long)n_heads * n_rows, s_max, n_sms) > 1) return pl;
   const int per_item = 6 / n_rows, slots = (16 + per_item - 1) / per_item, ld_t = t_len < 16 ? t_len : 16;
   const int stages = qkv.stages * qkv.group * (64 * (int)kBlockK * 2 + qkv.nt * (int)kBlockK * 2), recv = (qkv.nt + 3) / 4 * 64 * 16;

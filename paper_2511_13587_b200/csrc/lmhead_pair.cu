@@ -46,12 +46,6 @@ struct Params {
   int32_t* status;
 };
 
-// load into this CTA, bytes counted on a barrier of the pair (cluster address)
-__device__ __forceinline__ void tma_load_pair(void* dst, const CUtensorMap* m, uint32_t bar, int x, int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y) : "memory");
-}
 __device__ __forceinline__ void arrive_remote(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -115,7 +109,7 @@ lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, con
         uint8_t* st = smem + (size_t)i * stage_bytes;
         if (rank == 0) mbar_expect_tx(&full_bar[i], 2 * stage_bytes);
 #pragma unroll
-        for (uint32_t h = 0; h < kSub; ++h) tma_load_pair(st + h * kABytes, &tm_a, bar0, (kb * (int)kSub + (int)h) * (int)kBlockK, y);
+        for (uint32_t h = 0; h < kSub; ++h) tma_load_pair_2d(st + h * kABytes, &tm_a, bar0, (kb * (int)kSub + (int)h) * (int)kBlockK, y);
       }
     };
     auto load_b = [&](uint32_t i, int kb, int y) {
@@ -123,7 +117,7 @@ lmhead_pair_kernel(const Params p, const __grid_constant__ CUtensorMap tm_a, con
         const uint32_t bar0 = mapa(smem_u32(&full_bar[i]), 0);
         uint8_t* st = smem + (size_t)i * stage_bytes + kSub * kABytes;
 #pragma unroll
-        for (uint32_t h = 0; h < kSub; ++h) tma_load_pair(st + h * b_bytes, &tm_b, bar0, (kb * (int)kSub + (int)h) * (int)kBlockK, y);
+        for (uint32_t h = 0; h < kSub; ++h) tma_load_pair_2d(st + h * b_bytes, &tm_b, bar0, (kb * (int)kSub + (int)h) * (int)kBlockK, y);
       }
     };
     const int n_pre = p.kb_total < p.stages ? p.kb_total : p.stages;

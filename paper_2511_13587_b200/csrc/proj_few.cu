@@ -16,8 +16,10 @@
 // An accumulator of M = 64 lies in lanes 0-15 of the four lane quarters; its rows go to shared memory as [token quad][rank][row]
 // float4 (split: with st.async to the rank that owns the row, counted on its mbarrier), and the epilogue takes a pair of rows and
 // two tokens per thread (four where 64 rows are finished at once, one of an output or down projection of up to 32), partial sums in rank order.
-// (18 layers, 8, 18 and 28 tokens: activations requested by a warp that waits for nothing else 340.4 -> 338.8, 359.1 -> 357.1, 381.7 -> 380.0 us;
-// one token a thread 334.6, 357.1, 380.7.)
+// (18 layers, 8, 18 and 28 tokens: activations requested by a warp that waits for nothing else 340.4 -> 338.8, 359.1 -> 357.1, 381.7 -> 380.0 us.
+// One token a thread up to 32 tokens, 146 calls of 1 to 32 tokens at five widths: -0.4 % on average, -2.5 to +0.75 %; two tokens / one: XL shape,
+// 12 tokens 323.1 / 321.1, 18 333.9 / 333.2, 28 349.0 / 346.6, 32 354.8 / 353.6; d_model 1024, 4 tokens 285.4 / 282.2, 32 323.5 / 324.3; 1536, d_ff
+// 3008, 8 tokens 412.3 / 415.0, 18 442.3 / 437.5, 24 layers of 2048, 18 tokens 869.4 / 865.7.)
 //
 // Step of the XL shape against 128-row tiles: 18 tokens 876 -> 709 us, 28 tokens 920 -> 766, 54 tokens (a tree) 1061 -> 881; 18
 // layers of it, 72 tokens 615 -> 538, 90 tokens 657 -> 585, 108 tokens 635 -> 641; of d_model 1024, 72 tokens 515 -> 473, 90

@@ -8,10 +8,12 @@
 //   the last was finished.  The cache gets its rows as before; q is nowhere else.
 // - A sequence's head is shared by 6 / n_rows of the six CTAs.  The sixteen warps that attention_block.cu gives an item are dealt to them,
 //   each with its slot of 32 keys, which lies over the stages, drained by then (old keys are requested into L2 before the wait and into
-//   the slots behind the exchange): a CTA of 120 KB in the place of 172.
+//   the slots behind the exchange).  XL shape, two sequences: 120 KB a CTA with 9 rows each, 152 with 14, 175 with 27 (from 10 rows on the parts
+//   that one CTA folds set the size); with slots of their own 172 with 9.
 // - One of these CTAs gathers the warps' parts, also by st.async, and folds them in the order of the sixteen; the others end.
 // - The output projection takes more than half of an SM's shared memory then (vvs_api.cu): its CTAs would all start on the 28 SMs that this
-//   kernel leaves free, three to an SM (18 tokens 18 layers 364 us with 80 KB, 350 with 116 or 200).
+//   kernel leaves free, three to an SM (18 layers, 18 tokens 348.0 us with what it needs, 332.5 with 116 KB; 28 tokens 358.7, 346.7; a tree
+//   of 54 437.4, 423.4; one sequence of 9 tokens 344.1, 345.1).
 // - Loops are rolled and code is not repeated where a layer executes it once: a rolled loop of MMAs 343.3 -> 338.8 us.
 // 18 layers of the XL shape, two kernels / this one (us): guidance, 3 / 9 / 16 rows a sequence, 500 cached 355 / 334, 369 / 355, 399 / 388; 50 cached
 // 344 / 327, 356 / 341, 372 / 358; trees of 20 and 32 rows, 500 cached 492 / 442, 535 / 490; without guidance, 9 rows, 570 cached 377 / 353; 24 layers
@@ -46,14 +48,6 @@ struct Params {
   int n_heads, s_max, layer, kv_rows, t_len, per_item;                  // per_item: CTAs that share an item
   const uint8_t* ahead[2]; uint32_t ahead_bytes; AheadShare share;
 };
-
-__device__ __forceinline__ void st_async1(uint32_t addr, uint32_t bar, uint32_t v) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void st_async2(uint32_t addr, uint32_t bar, float a, float b) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
-               ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
-}
 
 __global__ void __launch_bounds__(kThreads, 1)
 qkv_attention_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b) {
@@ -229,19 +223,12 @@ qkv_attention_kernel(const __grid_constant__ Params p, const __grid_constant__ C
     for (int t0 = (warp - 3) * 8; t0 < p.m; t0 += 8 * (kThreads / 32 - 3)) {
       const int t = t0 + (lane >> 2);
       const float4* row = reinterpret_cast<const float4*>(p.ss_in + (size_t)min(t, p.m - 1) * p.ss_parts);
+      float4 v[8];                          // (at most 128 sums a token: plan_qkv_attention)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = q + 4 * k < n4 ? __ldcg(row + q + 4 * k) : make_float4(0.f, 0.f, 0.f, 0.f);
       float a[8];
-      auto take = [&](int at, bool first) {
-        float4 v[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = at + q + 4 * k < n4 ? __ldcg(row + at + q + 4 * k) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const float s = (v[k].x + v[k].y) + (v[k].z + v[k].w);
-          a[k] = first ? s : a[k] + s;
-        }
-      };
-      take(0, true);
-      for (int at = 32; at < n4; at += 32) take(at, false);
+      for (int k = 0; k < 8; ++k) a[k] = (v[k].x + v[k].y) + (v[k].z + v[k].w);
 #pragma unroll
       for (int o = 4; o > 0; o >>= 1)
 #pragma unroll

@@ -456,7 +456,6 @@ int run_verify_folded(vvs_ctx* ctx, const vvs_verify_args* a, const vvs_verify_o
     g.pdl = ctx->use_pdl && l > 0;
     ahead(L.w_gate, L.w_up, ff, d);
     if (p_qa.per_item > 0) {
-      at.layer = l;
       VVS_LAUNCH(VVS_PROF_GEMM, rc = launch_qkv_attention(p_qa, g, at, s));
       g.pdl = ctx->use_pdl;
     } else {
@@ -929,9 +928,9 @@ int vvs_bind_weights(vvs_ctx* ctx, const vvs_weights* w) {
           if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_qkv[few_map(g)], s.w_qkv, 3 * (uint64_t)d, d, 64, g);
           if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_o[few_map(g)], s.w_o, d, d, 64, g);
           if (rc == VVS_OK) rc = make_tmap_bf16_blocks(&q.w_down[few_map(g)], s.w_down, d, ff, 64, g);
-          if (rc == VVS_OK && pair) rc = make_tmap_bf16_pair_blocks(&q.w_gateup[few_map(g)], w0, dist, ff, d, 32, g);
+          if (rc == VVS_OK && pair) rc = make_tmap_bf16_pair_blocks(&q.w_gateup[few_map(g)], w0, dist, ff, d, 32, g, false);
         }
-        if (rc == VVS_OK && pair) rc = make_tmap_bf16_alternating_blocks(&q.w_gateup_pair, w0, dist, ff, d, 64, 1);
+        if (rc == VVS_OK && pair) rc = make_tmap_bf16_pair_blocks(&q.w_gateup_pair, w0, dist, ff, d, 64, 1, true);
       }
     }
     if (rc == VVS_OK)

@@ -268,9 +268,7 @@ struct GemmTcArgs {
 };
 int make_tmap_bf16_blocks(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_blocks);
 int make_tmap_bf16_pair_blocks(CUtensorMap* out, const void* base, uint64_t dist, uint64_t rows, uint64_t cols, uint32_t box_rows,
-                               uint32_t box_blocks);
-int make_tmap_bf16_alternating_blocks(CUtensorMap* out, const void* base, uint64_t dist, uint64_t rows, uint64_t cols, uint32_t box_rows,
-                                      uint32_t box_blocks);
+                               uint32_t box_blocks, bool in_turns);
 int make_tmap_bf16_2d(CUtensorMap* out, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 int make_weight_tmap(CUtensorMap* out, const void* w, int rows, int cols);
 GemmTcPlan plan_gemm_tc(int m, int n, int k, bool dual, bool allow_split, int n_sms, int split_cap = 32);

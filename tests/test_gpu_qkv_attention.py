@@ -176,7 +176,7 @@ extern "C" void plan(int rows, int t, int d, int s_max, int* o) {
                 if per_item == 0:
                     continue
                 taken += 1
-                assert rows <= 3 and per_item * rows == 6 and d // 64 * 6 <= 132
+                assert rows <= 3 and per_item * rows == 6 and d // 64 * 6 <= 132 and d // 16 <= 128   # (sums of squares of a token)
                 assert -(-16 // per_item) <= 8 and part_off == -(-16 // per_item) * 8192      # a part a warp, a slot each
                 assert part_off + 16 * min(t, 16) * 102 * 4 <= recv_off and stages <= recv_off
                 assert recv_off + (nt + 3) // 4 * 1024 <= new_off and new_off + 384 * t + 1024 <= smem <= 226 * 1024
