@@ -41,3 +41,23 @@ def test_pairs_give_the_same_bits(ms, n_images, n_cfg, k, up_first):
     got = _step(ms, w, n_images, n_cfg, 1, k, fills, 8500 + k)
     for a, b in zip(want, got):
         assert torch.equal(a, b)
+
+
+# where proj_few.cu refuses gate/up (its 160 CTAs would not all fit at once) and takes the other projections
+FEW = replace(XL2, name="few", d_model=1024, n_heads=16, d_ff=4800)
+FEW_CASES = [(FEW, 5, 1, 7), (FEW, 4, 2, 7), (FEW, 5, 2, 8), (FEW, 6, 2, 7)]         # 40, 64, 90, 96 tokens: one pass of 64 and 96
+
+
+@pytest.mark.parametrize("ms,n_images,n_cfg,k", FEW_CASES)
+def test_few_tokens_give_the_same_bits(ms, n_images, n_cfg, k):
+    """One matrix as both gate and up takes proj_tc.cu, two copies of it take the pairs."""
+    fills = [(37 * i) % (ms.s_max - k - 1) for i in range(n_images)]
+    w = _weights(ms, 8450)
+    for layer in w["layers"]:
+        layer["w_up"] = layer["w_gate"]
+    want = _step(ms, w, n_images, n_cfg, 1, k, fills, 8550 + k)
+    for layer in w["layers"]:
+        layer["w_up"] = layer["w_gate"].clone()
+    got = _step(ms, w, n_images, n_cfg, 1, k, fills, 8550 + k)
+    for a, b in zip(want, got):
+        assert (a == b).all()

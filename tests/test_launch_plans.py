@@ -183,7 +183,7 @@ def test_pair_plans_fit_the_hardware(plans, d):
 
 
 def test_pairs_are_taken_where_their_bits_are_compared(plans):
-    from test_gpu_gateup_pair import CASES, NOT_TAKEN
+    from test_gpu_gateup_pair import CASES, FEW_CASES, NOT_TAKEN
     widths = set()
     for ms, n_images, n_cfg, k, _ in CASES:
         m = n_images * n_cfg * (1 + k)
@@ -191,6 +191,10 @@ def test_pairs_are_taken_where_their_bits_are_compared(plans):
         assert (p["pairs"] == 0) == ((ms.name, m) in NOT_TAKEN), (ms.name, m, p)
         widths.add((p["sub"], p["nt"]))
     assert {(2, 64), (2, 96), (1, 128), (1, 160)} <= widths, widths
+    for ms, n_images, n_cfg, k in FEW_CASES:
+        m, out = n_images * n_cfg * (1 + k), (ctypes.c_int * (len(FEW_FIELDS) + 1))()
+        plans.few(m, ms.d_ff, ms.d_model, 1, 0, 1, N_SMS, out)
+        assert dict(zip(FEW_FIELDS, out))["stages"] == 0 and _pair(plans, m, ms.d_ff, ms.d_model)["pairs"] > 0, (ms.name, m)
 
 
 def test_requests_into_l2_are_shared_out(plans):
